@@ -20,6 +20,7 @@
 
 #include "internal.h"
 #include "taps.cuh"
+#include "wide.cuh"
 
 namespace gbst {
 std::atomic<int64_t> g_launches{0};
@@ -119,6 +120,7 @@ struct stencil_plan_s {
   bool varcoef = false;
   Shape shape = Shape::kStar;
   HostTaps taps;
+  WideTaps wide;  // the weights split for the integer form of the sum (n = 0: FMA chain)
   // library-owned device buffers
   double* d_tmp = nullptr;     // ping-pong partner of the caller's grid
   double* d_stage = nullptr;   // host-entry staging (grid, then kappa)
@@ -211,6 +213,16 @@ void build_taps(stencil_plan_s* p, const double* w) {
     p->taps.dx[i] = (int8_t)off[2];
   }
 }
+
+// The stencil classes whose kernels have the integer form of the sum.  All
+// kernels of a class take it, so its results do not depend on the kernel.
+bool uses_wide(int ndim, int radius) {
+  return ndim == 3 && radius == 1;
+}
+
+// Whether a 3D grid that the TMA-fed kernels do not take is streamed all the
+// same (asynchronous copies instead of TMA boxes) or swept cell by cell.
+bool wide3d_worth(const Geom& g) { return g.nx >= 32 && g.ny >= 8; }
 
 std::string device_name();
 
@@ -570,6 +582,7 @@ int launch_exchange_block(stencil_plan_s* p, const double* a, double* b, int Tb,
   L.counters = p->d_xcnt;
   L.status = p->d_status;
   L.wdev = p->d_w;
+  L.wide = p->wide;
   L.Tb = Tb;
   L.spin_limit = kSpinLimitNs;
   for (const ExchangeBand& band : bands) {
@@ -604,19 +617,21 @@ int run_steps(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, int variant,
       e = cudaSuccess;
       steps = Tb;
     } else if (variant == kVariantTemporal && T - t >= Tb) {
-      e = launch_temporal(p->ndim, p->radius, p->shape, p->boundary, Tb, p->g, p->d_w, a, b, sms, s,
+      e = launch_temporal(p->ndim, p->radius, p->shape, p->boundary, Tb, p->g, p->wide, p->d_w, a, b, sms, s,
                           equal_box && p->ndim == 2 && p->radius == 1);
       steps = Tb;
     } else {
       const int v = variant == kVariantTemporal || variant == kVariantExchange ? single : variant;
       if (v == kVariantStream && p->ndim == 3)
-        e = launch_stream3d(p->shape, p->boundary, p->g, p->taps, p->d_w, a, b, p->d_status, sms, s,
+        e = launch_stream3d(p->shape, p->boundary, p->g, p->taps, p->wide, p->d_w, a, b, p->d_status, sms, s,
                             (unsigned long long)kSpinLimitNs, -1, tile_y);
       else if (v == kVariantStream)
         e = launch_stream2d(p->shape, p->radius, p->boundary, equal_box && p->radius == 1, p->g, p->taps,
                             p->d_w, a, b, p->d_status, sms, s);
+      else if (p->wide.n && p->ndim == 3 && p->radius == 1 && wide3d_worth(p->g))
+        e = launch_wide3d(p->shape, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, 0, false);
       else
-        e = launch_direct(p->ndim, p->radius, p->shape, p->boundary, p->g, p->taps, p->d_w, a, b, s);
+        e = launch_direct(p->ndim, p->radius, p->shape, p->boundary, p->g, p->taps, p->wide, p->d_w, a, b, s);
     }
     if (e != cudaSuccess) return cuda_fail(e, "launching the sweep");
     std::swap(a, b);
@@ -931,6 +946,7 @@ int stencil_create(int ndim, const int64_t* dims, int radius, const double* weig
   p->boundary = boundary;
   p->shape = (star || ndim == 1) ? Shape::kStar : Shape::kBox;
   build_taps(p, weights);
+  if (uses_wide(ndim, radius)) make_wide(p->taps.w, p->taps.n, p->wide);
   *out = p;
   return STENCIL_OK;
 }
@@ -1736,7 +1752,7 @@ int stencil_selftest_tma_timeout(double limit_ms, void* cuda_stream) {
   cudaMemsetAsync(status, 0, sizeof(int), s);
   cudaMemcpyAsync(w, hw.data(), hw.size() * sizeof(double), cudaMemcpyHostToDevice, s);
   int rc = STENCIL_OK;
-  cudaError_t e = launch_stream3d(Shape::kStar, kPeriodic, g, taps, w, a, b, status, sm_count(), s,
+  cudaError_t e = launch_stream3d(Shape::kStar, kPeriodic, g, taps, WideTaps{}, w, a, b, status, sm_count(), s,
                                   (unsigned long long)(limit_ms * 1e6), 1);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   int st = 0;

@@ -7,6 +7,7 @@
 // Operation: one step of u'(x) = sum_o w_o u~(x+o) (paper Sec. 2.1, Listing 1).
 #include "internal.h"
 #include "taps.cuh"
+#include "wide.cuh"
 
 namespace gbst {
 namespace {
@@ -30,6 +31,16 @@ __device__ __forceinline__ bool axis_index(int c, int n, int& out) {
   }
 }
 
+template <int MODE>
+__device__ __forceinline__ double direct_value(const double* __restrict__ src, int z, int y, int x, int nz, int ny,
+                                               int nx) {
+  int zz, yy, xx;
+  bool in = axis_index<MODE>(z, nz, zz);
+  in &= axis_index<MODE>(y, ny, yy);
+  in &= axis_index<MODE>(x, nx, xx);
+  return in ? __ldg(src + ((int64_t)zz * ny + yy) * nx + xx) : 0.0;
+}
+
 template <int NT, int MODE>
 __global__ void __launch_bounds__(256) k_direct(const double* __restrict__ src,
                                                 double* __restrict__ dst, int nz, int ny, int nx,
@@ -50,18 +61,34 @@ __global__ void __launch_bounds__(256) k_direct(const double* __restrict__ src,
     double acc = 0.0;
 #pragma unroll
     for (int k = 0; k < NT; ++k) {
-      int zz, yy, xx;
-      bool in = axis_index<MODE>(z + tp.dz[k], nz, zz);
-      in &= axis_index<MODE>(y + tp.dy[k], ny, yy);
-      in &= axis_index<MODE>(x + tp.dx[k], nx, xx);
-      double v = 0.0;
-      if (in) v = __ldg(src + ((int64_t)zz * ny + yy) * nx + xx);
+      const double v = direct_value<MODE>(src, z + tp.dz[k], y + tp.dy[k], x + tp.dx[k], nz, ny, nx);
       if constexpr (kRegs)
         W.tap(acc, k, v, 0);
       else
         acc = fma(tp.w[k], v, k == 0 ? zero : acc);
     }
     dst[((int64_t)z * ny + y) * nx + x] = acc;
+  }
+}
+
+// The same sweep with the weighted sum in the integer form (wide.cuh).
+template <int NT, int MODE>
+__global__ void __launch_bounds__(256) k_direct_wide(const double* __restrict__ src, double* __restrict__ dst, int nz,
+                                                     int ny, int nx, int zper,
+                                                     const __grid_constant__ TapList<NT> tp,
+                                                     const __grid_constant__ WideTaps wide,
+                                                     const double* __restrict__ wdev) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  if (x >= nx || y >= ny) return;
+  const int z0 = blockIdx.z * zper;
+  const int z1 = min(nz, z0 + zper);
+  for (int z = z0; z < z1; ++z) {
+    WideVal u[NT];
+#pragma unroll
+    for (int k = 0; k < NT; ++k)
+      u[k] = wide_unpack(direct_value<MODE>(src, z + tp.dz[k], y + tp.dy[k], x + tp.dx[k], nz, ny, nx));
+    dst[((int64_t)z * ny + y) * nx + x] = wide_sum<NT>(u, wide, wdev);
   }
 }
 
@@ -96,6 +123,7 @@ __global__ void __launch_bounds__(256) k_direct_f32(const float* __restrict__ sr
   }
 }
 
+// Enough blocks for every SM several times over; the rest of z is walked.
 void direct_shape(const Geom& g, dim3& grid, dim3& block, int& zper) {
   zper = 1;
   if (g.ny == 1 && g.nz == 1) {
@@ -138,7 +166,7 @@ cudaError_t launch_nt_f32(int mode, const Geom& g, const HostTaps& ht, const flo
 }
 
 template <int NT>
-cudaError_t launch_nt(int mode, const Geom& g, const HostTaps& ht, const double* wdev,
+cudaError_t launch_nt(int mode, const Geom& g, const HostTaps& ht, const WideTaps& wide, const double* wdev,
                       const double* src, double* dst, cudaStream_t stream) {
   TapList<NT> tp;
   for (int k = 0; k < NT; ++k) {
@@ -148,22 +176,18 @@ cudaError_t launch_nt(int mode, const Geom& g, const HostTaps& ht, const double*
     tp.dx[k] = ht.dx[k];
   }
   dim3 block, grid;
-  int zper = 1;
-  if (g.ny == 1 && g.nz == 1) {
-    block = dim3(256, 1, 1);
-    grid = dim3((g.nx + 255) / 256, 1, 1);
-  } else {
-    block = dim3(32, 8, 1);
-    unsigned gx = (g.nx + 31) / 32, gy = (g.ny + 7) / 8;
-    // enough blocks for every SM several times over; the rest of z is walked
-    int64_t tiles = (int64_t)gx * gy;
-    int64_t want = 152 * 16;
-    int64_t zchunks = (want + tiles - 1) / tiles;
-    if (zchunks > g.nz) zchunks = g.nz;
-    if (zchunks < 1) zchunks = 1;
-    zper = (int)((g.nz + zchunks - 1) / zchunks);
-    zchunks = (g.nz + zper - 1) / zper;
-    grid = dim3(gx, gy, (unsigned)zchunks);
+  int zper;
+  direct_shape(g, grid, block, zper);
+  if constexpr (NT <= kWideMaxTaps) {
+    if (wide.n) {
+      switch (mode) {
+        case 0: k_direct_wide<NT, 0><<<grid, block, 0, stream>>>(src, dst, g.nz, g.ny, g.nx, zper, tp, wide, wdev); break;
+        case 1: k_direct_wide<NT, 1><<<grid, block, 0, stream>>>(src, dst, g.nz, g.ny, g.nx, zper, tp, wide, wdev); break;
+        default: k_direct_wide<NT, 2><<<grid, block, 0, stream>>>(src, dst, g.nz, g.ny, g.nx, zper, tp, wide, wdev); break;
+      }
+      g_launches.fetch_add(1, std::memory_order_relaxed);
+      return cudaGetLastError();
+    }
   }
   switch (mode) {
     case 0: k_direct<NT, 0><<<grid, block, 0, stream>>>(src, dst, g.nz, g.ny, g.nx, zper, tp, wdev); break;
@@ -177,7 +201,7 @@ cudaError_t launch_nt(int mode, const Geom& g, const HostTaps& ht, const double*
 }  // namespace
 
 cudaError_t launch_direct(int ndim, int radius, Shape shape, int boundary, const Geom& g,
-                          const HostTaps& taps, const double* wdev, const double* src, double* dst,
+                          const HostTaps& taps, const WideTaps& wide, const double* wdev, const double* src, double* dst,
                           cudaStream_t stream) {
   int mode = 0;
   if (boundary == kPeriodic) {
@@ -185,14 +209,14 @@ cudaError_t launch_direct(int ndim, int radius, Shape shape, int boundary, const
     mode = small ? 2 : 1;
   }
   switch (taps.n) {
-    case 3: return launch_nt<3>(mode, g, taps, wdev, src, dst, stream);
-    case 5: return launch_nt<5>(mode, g, taps, wdev, src, dst, stream);
-    case 7: return launch_nt<7>(mode, g, taps, wdev, src, dst, stream);
-    case 9: return launch_nt<9>(mode, g, taps, wdev, src, dst, stream);
-    case 13: return launch_nt<13>(mode, g, taps, wdev, src, dst, stream);
-    case 25: return launch_nt<25>(mode, g, taps, wdev, src, dst, stream);
-    case 27: return launch_nt<27>(mode, g, taps, wdev, src, dst, stream);
-    case 125: return launch_nt<125>(mode, g, taps, wdev, src, dst, stream);
+    case 3: return launch_nt<3>(mode, g, taps, wide, wdev, src, dst, stream);
+    case 5: return launch_nt<5>(mode, g, taps, wide, wdev, src, dst, stream);
+    case 7: return launch_nt<7>(mode, g, taps, wide, wdev, src, dst, stream);
+    case 9: return launch_nt<9>(mode, g, taps, wide, wdev, src, dst, stream);
+    case 13: return launch_nt<13>(mode, g, taps, wide, wdev, src, dst, stream);
+    case 25: return launch_nt<25>(mode, g, taps, wide, wdev, src, dst, stream);
+    case 27: return launch_nt<27>(mode, g, taps, wide, wdev, src, dst, stream);
+    case 125: return launch_nt<125>(mode, g, taps, wide, wdev, src, dst, stream);
     default: return cudaErrorInvalidValue;
   }
   (void)shape;

@@ -83,6 +83,7 @@
 #include "internal.h"
 #include "ptx.cuh"
 #include "taps.cuh"
+#include "wide.cuh"
 
 namespace gbst {
 
@@ -102,9 +103,10 @@ constexpr int kMaps = 5;           // TMA box heights: 1, h_lo, h_lo+1, h_lo+2, 
 constexpr int kMaxStages = 8;      // largest Tb; progress counters per CTA
 constexpr unsigned long long kWaitNs = 2000000000ull;
 // Stage skew L in planes: 4 at Tb = 2 (a level is published 3 Tb units
-// before it is needed instead of Tb), else 2 (a skew of 3 measured the same
-// at Tb = 4 and 8, with a larger ring).
-inline int stage_lag(int Tb) { return Tb == 2 ? 4 : 2; }
+// before it is needed instead of Tb), 3 at Tb = 4 (512^3 in the integer form of
+// the sum: 85.0 against 82.6 GStencil/s at 2, 85.7 at 4; the FMA chain the same at
+// 2 and 3), 2 at Tb = 8 (a larger ring would leave L2).
+inline int stage_lag(int Tb) { return Tb == 2 ? 4 : Tb == 4 ? 3 : 2; }
 // Ring planes per stage for skew L (see the slot-reuse rule above).
 inline int ring_k(bool box, int lag) { return box ? 2 * lag + 2 : 2 * lag + 1; }
 
@@ -176,6 +178,7 @@ struct XParams {
   int Tb, iters, qoff;
   int lag, K;  // stage skew in planes; ring planes per stage
   long long spin_limit;
+  WideTaps wide;
 };
 
 __device__ __forceinline__ int wrapi(int c, int n) {
@@ -246,6 +249,103 @@ __device__ __forceinline__ void unit_rows(const XSlot& sl, const RegWeights<NT>&
         }
       }
     }
+  }
+}
+
+// The same cells of one row by the integer form (false: it does not take both,
+// see unit_chain).  The values are unpacked from the unit's planes, their rows
+// read twice: for the largest exponents, then for the sums (the 36 values of a
+// box's pair would not fit the registers).
+template <int NT, bool BOX>
+__device__ __forceinline__ bool unit_row_wide(const XSlot& sl, const WideTaps& T, int r, int lane, double (&out)[2]) {
+  auto row = [&](int dz, int dy, double (&v)[4]) {  // columns x-1 .. x+2
+    const double2 p = *reinterpret_cast<const double2*>(&sl.plane[dz + 1][r + 1 + dy][2 * lane]);
+    v[1] = p.x;
+    v[2] = p.y;
+    if (BOX || (dz == 0 && dy == 0)) {
+      v[0] = __shfl_up_sync(0xffffffffu, p.y, 1);
+      v[3] = __shfl_down_sync(0xffffffffu, p.x, 1);
+      if (lane == 0) v[0] = sl.halo[dz + 1][r + 1 + dy][0].y;
+      if (lane == 31) v[3] = sl.halo[dz + 1][r + 1 + dy][1].x;
+    }
+  };
+  if constexpr (!BOX) {
+    double zm[4], n[4], c[4], s[4], zp[4];
+    row(-1, 0, zm);
+    row(0, -1, n);
+    row(0, 0, c);
+    row(0, 1, s);
+    row(1, 0, zp);
+    WideVal x[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = wide_unpack(c[k]);
+    bool all = true;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const WideVal u[7] = {wide_unpack(zm[1 + i]), wide_unpack(n[1 + i]), x[i], x[i + 1], x[i + 2],
+                            wide_unpack(s[1 + i]), wide_unpack(zp[1 + i])};
+      bool ok;
+      out[i] = wide_sum<7>(u, T, ok);
+      all = all && ok;
+    }
+    return all;
+  } else {
+    int E[2] = {-0x7fffffff, -0x7fffffff};
+#pragma unroll
+    for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+      for (int dy = -1; dy <= 1; ++dy) {
+        double v[4];
+        row(dz, dy, v);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int e = wide_unpack(v[k]).e;
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+            if (k - i >= 0 && k - i <= 2) E[i] = max(E[i], e + T.ex[tap_at<BOX>(dz, dy, k - i - 1)]);
+        }
+      }
+    WideAcc acc[2];
+#pragma unroll
+    for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+      for (int dy = -1; dy <= 1; ++dy) {
+        double v[4];
+        row(dz, dy, v);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const WideVal u = wide_unpack(v[k]);
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+            if (k - i >= 0 && k - i <= 2) {
+              const int t = tap_at<BOX>(dz, dy, k - i - 1);
+              acc[i].add(u, t, E[i] - u.e - T.ex[t], T);
+            }
+        }
+      }
+    out[0] = acc[0].get(E[0], T);
+    out[1] = acc[1].get(E[1], T);
+    return wide_covers(E[0], T) && wide_covers(E[1], T);
+  }
+}
+
+// Those of the two cells that the integer form does not take, by the FMA chain,
+// written at out.  Out of line: rarely run.
+template <int NT, bool BOX>
+__device__ __noinline__ void unit_chain(const XSlot& sl, const WideTaps& T, const double* wdev, int r, int lane,
+                                        double* out) {
+  for (int i = 0; i < 2; ++i) {
+    double v[NT];
+    int E = -0x7fffffff;
+    for (int k = 0; k < 27; ++k) {
+      const int dz = k / 9 - 1, dy = k / 3 % 3 - 1, dx = k % 3 - 1;
+      if (!BOX && (dz != 0) + (dy != 0) + (dx != 0) > 1) continue;
+      const int t = tap_at<BOX>(dz, dy, dx), x = 2 * lane + i + dx;
+      v[t] = x < 0 ? sl.halo[dz + 1][r + 1 + dy][0].y : x >= kXW ? sl.halo[dz + 1][r + 1 + dy][1].x
+                                                                 : sl.plane[dz + 1][r + 1 + dy][x];
+      E = max(E, wide_unpack(v[t]).e + T.ex[t]);
+    }
+    if (!wide_covers(E, T)) out[i] = wide_chain(v, wdev, NT);
   }
 }
 
@@ -330,7 +430,7 @@ __device__ int build_segs(const XParams& P, int ra, int rb, int ytop, int wrap, 
   return ns;
 }
 
-template <int NT, bool BOX, bool PERIODIC>
+template <int NT, bool BOX, bool PERIODIC, bool WIDE>
 __global__ void __launch_bounds__(kThreadsX, 1) k_exchange3d(const __grid_constant__ XParams P) {
   const int K = P.K;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -552,8 +652,8 @@ __global__ void __launch_bounds__(kThreadsX, 1) k_exchange3d(const __grid_consta
   }
 
   // -------------------------------------------------------------- consumers
-  RegWeights<NT> W;
-  W.load(P.wdev);
+  RegWeights<WIDE ? 1 : NT> W;
+  if constexpr (!WIDE) W.load(P.wdev);
   // the ring is re-read within a few iterations: keep its lines in L2; the
   // output is not re-read: streaming stores
   const uint64_t keep = policy_evict_last();
@@ -590,29 +690,35 @@ __global__ void __launch_bounds__(kThreadsX, 1) k_exchange3d(const __grid_consta
       const int64_t base = (last ? ((int64_t)q * P.ny + y0) * P.nx
                                  : (((int64_t)(s - 1) * K + wrapi(q, K)) * P.nyb + yl0) * P.nx) +
                            x0 + 2 * lane;
-      if (r0 + kWarps < h) {
+      auto put = [&](int r, double v0, double v1) {  // row r of the tile
+        const int64_t off = base + (int64_t)r * P.nx;
+        if (!last) st_global_v2_hint(P.ring + off, v0, v1, keep);
+        else if (y0 + r >= P.own_lo && y0 + r < P.own_hi) st_global_v2_cs(P.dst + off, v0, v1);
+      };
+      if constexpr (WIDE) {
+#pragma unroll 1
+        for (int r = r0; r < h; r += kWarps) {
+          double v[2];
+          const bool all = unit_row_wide<NT, BOX>(sl, P.wide, r, lane, v);
+          if (xin) {
+            put(r, v[0], v[1]);
+            if (!all && (!last || (y0 + r >= P.own_lo && y0 + r < P.own_hi)))
+              unit_chain<NT, BOX>(sl, P.wide, P.wdev, r, lane, (last ? P.dst : P.ring) + base + (int64_t)r * P.nx);
+          }
+        }
+      } else if (r0 + kWarps < h) {
         const int rr[2] = {r0, r0 + kWarps};
         double a[2][2];
         unit_rows<NT, BOX, 2>(sl, W, rr, lane, a);
         if (xin) {
-#pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            const int64_t off = base + (int64_t)rr[k] * P.nx;
-            if (!last) st_global_v2_hint(P.ring + off, a[k][0], a[k][1], keep);
-            else if (y0 + rr[k] >= P.own_lo && y0 + rr[k] < P.own_hi) st_global_v2_cs(P.dst + off, a[k][0], a[k][1]);
-          }
+          put(rr[0], a[0][0], a[0][1]);
+          put(rr[1], a[1][0], a[1][1]);
         }
       } else if (r0 < h) {
         const int rr[1] = {r0};
         double a[1][2];
         unit_rows<NT, BOX, 1>(sl, W, rr, lane, a);
-        const int64_t off = base + (int64_t)r0 * P.nx;
-        if (!xin) {
-        } else if (!last) {
-          st_global_v2_hint(P.ring + off, a[0][0], a[0][1], keep);
-        } else if (y0 + r0 >= P.own_lo && y0 + r0 < P.own_hi) {
-          st_global_v2_cs(P.dst + off, a[0][0], a[0][1]);
-        }
+        if (xin) put(r0, a[0][0], a[0][1]);
       }
       // this thread's share of unit (i, s) is written (stage Tb: the output).
       // Its stores are generic-proxy writes that TMA (the async proxy) reads
@@ -656,12 +762,12 @@ bool encode_ring(CUtensorMap* map, const double* base, int nx, int nyb, int K, i
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int NT, bool BOX, bool PERIODIC>
+template <int NT, bool BOX, bool PERIODIC, bool WIDE>
 int x_occupancy() {
   static std::atomic<int> cache[kMaxDeviceOrdinals];
   return cached_per_device(cache, [] {
     int occ = 0;
-    auto kern = k_exchange3d<NT, BOX, PERIODIC>;
+    auto kern = k_exchange3d<NT, BOX, PERIODIC, WIDE>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(XSmem)) !=
             cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreadsX, sizeof(XSmem)) != cudaSuccess)
@@ -670,9 +776,9 @@ int x_occupancy() {
   });
 }
 
-template <int NT, bool BOX, bool PERIODIC>
+template <int NT, bool BOX, bool PERIODIC, bool WIDE>
 cudaError_t launch_x(const ExchangeLaunch& L, cudaStream_t stream) {
-  if (x_occupancy<NT, BOX, PERIODIC>() < 1) return cudaErrorInvalidConfiguration;
+  if (x_occupancy<NT, BOX, PERIODIC, WIDE>() < 1) return cudaErrorInvalidConfiguration;
   XParams P;
   const Geom& g = L.g;
   const ExchangeBand& b = L.band;
@@ -717,6 +823,7 @@ cudaError_t launch_x(const ExchangeLaunch& L, cudaStream_t stream) {
   // iteration nz - 1 - qoff + lag (Tb - 1)
   P.iters = g.nz - P.qoff + P.lag * (L.Tb - 1);
   P.spin_limit = L.spin_limit;
+  P.wide = L.wide;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(L.tiles_x * b.tiles_y), 1, 1);
   cfg.blockDim = dim3(kThreadsX, 1, 1);
@@ -727,7 +834,7 @@ cudaError_t launch_x(const ExchangeLaunch& L, cudaStream_t stream) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_exchange3d<NT, BOX, PERIODIC>, P);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, k_exchange3d<NT, BOX, PERIODIC, WIDE>, P);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return e;
 }
@@ -778,8 +885,11 @@ cudaError_t launch_exchange(Shape shape, int boundary, const ExchangeLaunch& L, 
   const bool per = boundary == kPeriodic;
   if (L.Tb < 2 || L.Tb > kMaxStages || L.tiles_x < 1 || L.band.tiles_y < 1) return cudaErrorInvalidValue;
   if (shape == Shape::kBox)
-    return per ? launch_x<27, true, true>(L, stream) : launch_x<27, true, false>(L, stream);
-  return per ? launch_x<7, false, true>(L, stream) : launch_x<7, false, false>(L, stream);
+    return L.wide.n ? (per ? launch_x<27, true, true, true>(L, stream) : launch_x<27, true, false, true>(L, stream))
+                    : (per ? launch_x<27, true, true, false>(L, stream) : launch_x<27, true, false, false>(L, stream));
+  if (L.wide.n)
+    return per ? launch_x<7, false, true, true>(L, stream) : launch_x<7, false, false, true>(L, stream);
+  return per ? launch_x<7, false, true, false>(L, stream) : launch_x<7, false, false, false>(L, stream);
 }
 
 }  // namespace gbst

@@ -57,12 +57,27 @@ struct HostTaps {
   int8_t dz[kMaxTaps], dy[kMaxTaps], dx[kMaxTaps];
 };
 
+// The weights split for the integer form of the weighted sum (wide.cuh); n = 0
+// when that form does not cover them.
+constexpr int kWideMaxTaps = 27;
+struct WideTaps {
+  int n = 0;
+  int hi[kWideMaxTaps], lo[kWideMaxTaps];  // limbs of the significand: hi * 2^26 + lo
+  int hi2[kWideMaxTaps];                   // 2 * hi
+  int ex[kWideMaxTaps];                    // exponent below the largest weight's (<= 0)
+  int heat;                                // one weight at the centre tap (n / 2), one at all others
+  int bias;                                // exponent of the result: E - bias above R's
+  int e_min;                               // E in [e_min, e_min + e_span], else the FMA chain
+  unsigned int e_span;
+};
+
 // Launchers implemented in the .cu files.  Each returns a cudaError_t from
 // the launch (cudaSuccess when nothing failed) and enqueues on `stream`.
 // wdev: the plan's weights on the device (taps.n weights in tap order, then
-// zero and one slots; see taps.cuh).
+// zero and one slots; see taps.cuh).  wide: the same weights split for the
+// integer form of the sum; n = 0 selects the FMA chain.
 cudaError_t launch_direct(int ndim, int radius, Shape shape, int boundary, const Geom& g,
-                          const HostTaps& taps, const double* wdev, const double* src, double* dst,
+                          const HostTaps& taps, const WideTaps& wide, const double* wdev, const double* src, double* dst,
                           cudaStream_t stream);
 
 // FP32 twin of the direct sweep (accuracy studies only; up to 27 taps).
@@ -81,10 +96,17 @@ bool stream3d_shape_ok(int ndim, int radius, Shape shape, int boundary, const Ge
 int stream3d_tile_y(Shape shape, int tile_y);
 // wait_ns bounds every mbarrier wait (kSpinLimitNs in normal runs); skip_plane
 // >= 0 is the self-test's starved plane (the producer posts no copy for it).
-cudaError_t launch_stream3d(Shape shape, int boundary, const Geom& g, const HostTaps& taps,
+cudaError_t launch_stream3d(Shape shape, int boundary, const Geom& g, const HostTaps& taps, const WideTaps& wide,
                             const double* wdev, const double* src, double* dst, int* status,
                             int sms, cudaStream_t stream, unsigned long long wait_ns = 2000000000ull,
                             long long skip_plane = -1, int tile_y = 0);
+
+// 3D radius-1 sweep with the weighted sum in the integer form (wide.n != 0):
+// tiles of 64 columns by 16 rows (8 for tile_y = 8).  tma: the grid is one that
+// stream3d_eligible takes; false: any shape, alignment and boundary.
+cudaError_t launch_wide3d(Shape shape, int boundary, const Geom& g, const WideTaps& wide, const double* wdev,
+                          const double* src, double* dst, int* status, int sms, cudaStream_t stream, int tile_y,
+                          bool tma);
 
 // 2D radius-1 or radius-2 streaming sweep (TMA-fed ring of 16-row blocks).  Same
 // eligibility rules with ny % 16 == 0 for periodic grids.  `equal` selects
@@ -103,7 +125,7 @@ bool temporal_supported(int ndim, int radius, int Tb);
 // equal: a 2D box whose weights are all equal takes the shared-partial-sum
 // form (within rounding of the tap-order kernels, not bitwise equal).
 cudaError_t launch_temporal(int ndim, int radius, Shape shape, int boundary, int Tb, const Geom& g,
-                            const double* wdev, const double* src, double* dst, int sms,
+                            const WideTaps& wide, const double* wdev, const double* src, double* dst, int sms,
                             cudaStream_t stream, bool equal = false);
 
 // Temporal blocking without recomputation (3D radius 1, star or box, Tb >= 2):
@@ -129,6 +151,7 @@ struct ExchangeLaunch {
   unsigned int* counters;  // exchange_counter_words(tiles) words, zero before the launch
   int* status;
   const double* wdev;
+  WideTaps wide;
   int Tb;
   int tiles_x;             // exchange_tiles_x(g): ceil(nx / 64)
   ExchangeBand band;

@@ -28,6 +28,7 @@
 // Dirichlet ghost cells (outside the grid, at every time level) stay zero.
 #include "internal.h"
 #include "taps.cuh"
+#include "wide.cuh"
 
 namespace gbst {
 namespace {
@@ -111,6 +112,7 @@ struct TParams {
   int tiles_x, tiles_y;
   long long work;       // tiles * nw
   const double* wdev;
+  WideTaps wide;
 };
 
 __device__ __forceinline__ int wrapn(int c, int n) {
@@ -176,11 +178,12 @@ __device__ __forceinline__ constexpr int tidx(int dw, int dv, int du) {
 // instead of 18 (additions as FMAs against a register holding 1).  The sum
 // is taken in another order than the tap list, so the result is within
 // rounding of the other kernels, not bitwise equal to them.
-template <int NDIM, int NT, bool BOX, bool EQ = false>
-__device__ __forceinline__ void pair_update(const RegWeights<NT>& W, const double* pm, const double* p0,
+template <int NDIM, int NT, bool BOX, bool EQ, bool WIDE>
+__device__ __forceinline__ void pair_update(const TapSum<NT, WIDE>& S, const double* pm, const double* p0,
                                             const double* pp, int sw, int ly, int lx, double& a0,
                                             double& a1) {
   if constexpr (NDIM == 2 && EQ) {
+    const RegWeights<NT>& W = S.W;
     double C[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -192,6 +195,7 @@ __device__ __forceinline__ void pair_update(const RegWeights<NT>& W, const doubl
     a1 = fma(W.w[8], C[3], wt);
     return;
   }
+  typename TapSum<NT, WIDE>::Acc s0, s1;
   const double* pl[3] = {pm, p0, pp};
   const int de = NDIM == 3 ? sw : 1;  // the second cell
 #pragma unroll
@@ -204,18 +208,20 @@ __device__ __forceinline__ void pair_update(const RegWeights<NT>& W, const doubl
         if (!BOX && (dw != 0) + (dv != 0) + (du != 0) > 1) continue;
         const double* q = pl[dw + 1] + (ly + dv) * sw + lx + du;
         const int t = tidx<NDIM, BOX>(dw, dv, du);
-        W.tap(a0, t, q[0], 0);
-        W.tap(a1, t, q[de], 1);
+        S.tap(s0, t, q[0], 0);
+        S.tap(s1, t, q[de], 1);
       }
     }
   }
+  a0 = S.get(s0);
+  a1 = S.get(s1);
 }
 
 // Pair c of stage s's region, plane i: computed from the three planes of
 // stage s-1 around it and written to stage s's ring, or (s = Tb) to global
 // memory.
-template <int NDIM, int NT, bool BOX, bool PERIODIC, int TB, bool EQ = false>
-__device__ __forceinline__ void stage_pair(const TParams& P, const RegWeights<NT>& W, double* sm, int s,
+template <int NDIM, int NT, bool BOX, bool PERIODIC, int TB, bool EQ, bool WIDE>
+__device__ __forceinline__ void stage_pair(const TParams& P, const TapSum<NT, WIDE>& W, double* sm, int s,
                                            int c, int i, int wa, int y0, int x0) {
   using L = Lay<NDIM, TB, BOX>;
   const int ws = L::W(s);
@@ -234,7 +240,7 @@ __device__ __forceinline__ void stage_pair(const TParams& P, const RegWeights<NT
   const double* p0 = src + L::slot(s - 1, i) * sn;
   const double* pp = src + L::slot(s - 1, i + 1) * sn;
   double a0, a1;
-  pair_update<NDIM, NT, BOX, EQ>(W, pm, p0, pp, L::W(s - 1), NDIM == 3 ? qy + 1 : 0, qx + 1, a0, a1);
+  pair_update<NDIM, NT, BOX, EQ, WIDE>(W, pm, p0, pp, L::W(s - 1), NDIM == 3 ? qy + 1 : 0, qx + 1, a0, a1);
   const int w = wa - TB + i;
   const int x = x0 - TB + s + qx;
   const int y = NDIM == 3 ? y0 - TB + s + qy : 0;
@@ -274,16 +280,15 @@ __device__ __forceinline__ void stage_pair(const TParams& P, const RegWeights<NT
   }
 }
 
-template <int NDIM, int NT, bool BOX, bool PERIODIC, int TB, bool EQ = false>
+template <int NDIM, int NT, bool BOX, bool PERIODIC, int TB, bool EQ, bool WIDE>
 __global__ void __launch_bounds__(temporal_threads<NDIM, BOX, TB>(), temporal_min_blocks<NDIM, BOX, TB>())
-    k_temporal(const TParams P) {
+    k_temporal(const __grid_constant__ TParams P) {
   using L = Lay<NDIM, TB, BOX>;
   constexpr int NTH = temporal_threads<NDIM, BOX, TB>();
   constexpr int LAG = temporal_lag<NDIM, TB, BOX>();
   constexpr int TX = Geo<NDIM, TB, BOX>::TX, TY = Geo<NDIM, TB, BOX>::TY;
   extern __shared__ __align__(16) double sm[];
-  RegWeights<NT> W;
-  W.load(P.wdev);
+  const TapSum<NT, WIDE> W(P.wdev, P.wide);
 
   const long long G = gridDim.x;
   const long long f_begin = P.work * blockIdx.x / G;
@@ -320,7 +325,7 @@ __global__ void __launch_bounds__(temporal_threads<NDIM, BOX, TB>(), temporal_mi
             c -= L::pairs(s);
             ++s;
           }
-          stage_pair<NDIM, NT, BOX, PERIODIC, TB, EQ>(P, W, sm, s, c, k - 2 * s, wa, y0, x0);
+          stage_pair<NDIM, NT, BOX, PERIODIC, TB, EQ, WIDE>(P, W, sm, s, c, k - 2 * s, wa, y0, x0);
         }
       } else {
         // stage by stage: plane k - s - 1 is in range for s <= (k - 1) / 2
@@ -328,7 +333,7 @@ __global__ void __launch_bounds__(temporal_threads<NDIM, BOX, TB>(), temporal_mi
         for (int s = 1; s <= s_hi; ++s) {
           if (s > 1) __syncthreads();  // stage s-1's plane of this iteration is written
           for (int j = threadIdx.x; j < L::pairs(s); j += NTH)
-            stage_pair<NDIM, NT, BOX, PERIODIC, TB, EQ>(P, W, sm, s, j, k - s - 1, wa, y0, x0);
+            stage_pair<NDIM, NT, BOX, PERIODIC, TB, EQ, WIDE>(P, W, sm, s, j, k - s - 1, wa, y0, x0);
         }
       }
     }
@@ -336,13 +341,13 @@ __global__ void __launch_bounds__(temporal_threads<NDIM, BOX, TB>(), temporal_mi
   }
 }
 
-template <int NDIM, int NT, bool BOX, bool PERIODIC, int TB, bool EQ = false>
-cudaError_t launch_tb(const Geom& g, const double* wdev, const double* src, double* dst, int sms,
+template <int NDIM, int NT, bool BOX, bool PERIODIC, int TB, bool EQ, bool WIDE>
+cudaError_t launch_tb(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst, int sms,
                       cudaStream_t stream) {
   using L = Lay<NDIM, TB, BOX>;
   constexpr int NTH = temporal_threads<NDIM, BOX, TB>();
   static_assert(L::bytes <= 227 * 1024, "stage rings exceed shared memory");
-  auto kern = k_temporal<NDIM, NT, BOX, PERIODIC, TB, EQ>;
+  auto kern = k_temporal<NDIM, NT, BOX, PERIODIC, TB, EQ, WIDE>;
   static std::atomic<int> cache[kMaxDeviceOrdinals];
   const int occ = cached_per_device(cache, [kern] {
     int n = 0;
@@ -362,6 +367,7 @@ cudaError_t launch_tb(const Geom& g, const double* wdev, const double* src, doub
   P.tiles_y = NDIM == 3 ? (g.ny + Geo<NDIM, TB, BOX>::TY - 1) / Geo<NDIM, TB, BOX>::TY : 1;
   P.work = (long long)P.tiles_x * P.tiles_y * P.nw;
   P.wdev = wdev;
+  P.wide = wide;
   long long grid = (long long)sms * occ;
   if (grid > P.work) grid = P.work;
   kern<<<(unsigned)grid, NTH, L::bytes, stream>>>(P);
@@ -369,13 +375,13 @@ cudaError_t launch_tb(const Geom& g, const double* wdev, const double* src, doub
   return cudaGetLastError();
 }
 
-template <int NDIM, int NT, bool BOX, bool PERIODIC, bool EQ = false>
-cudaError_t by_tb(int Tb, const Geom& g, const double* wdev, const double* src, double* dst, int sms,
+template <int NDIM, int NT, bool BOX, bool PERIODIC, bool EQ = false, bool WIDE = false>
+cudaError_t by_tb(int Tb, const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst, int sms,
                   cudaStream_t stream) {
   switch (Tb) {
-    case 2: return launch_tb<NDIM, NT, BOX, PERIODIC, 2, EQ>(g, wdev, src, dst, sms, stream);
-    case 4: return launch_tb<NDIM, NT, BOX, PERIODIC, 4, EQ>(g, wdev, src, dst, sms, stream);
-    case 8: return launch_tb<NDIM, NT, BOX, PERIODIC, 8, EQ>(g, wdev, src, dst, sms, stream);
+    case 2: return launch_tb<NDIM, NT, BOX, PERIODIC, 2, EQ, WIDE>(g, wide, wdev, src, dst, sms, stream);
+    case 4: return launch_tb<NDIM, NT, BOX, PERIODIC, 4, EQ, WIDE>(g, wide, wdev, src, dst, sms, stream);
+    case 8: return launch_tb<NDIM, NT, BOX, PERIODIC, 8, EQ, WIDE>(g, wide, wdev, src, dst, sms, stream);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -458,7 +464,7 @@ bool temporal_supported(int ndim, int radius, int Tb) {
 }
 
 cudaError_t launch_temporal(int ndim, int radius, Shape shape, int boundary, int Tb, const Geom& g,
-                            const double* wdev, const double* src, double* dst, int sms,
+                            const WideTaps& wide, const double* wdev, const double* src, double* dst, int sms,
                             cudaStream_t stream, bool equal) {
   const bool per = boundary == kPeriodic;
   const bool box = shape == Shape::kBox;
@@ -472,17 +478,21 @@ cudaError_t launch_temporal(int ndim, int radius, Shape shape, int boundary, int
                : launch_1d<1, false>(Tb, g, wdev, src, dst, stream);
   }
   if (ndim == 3) {
-    if (box) return per ? by_tb<3, 27, true, true>(Tb, g, wdev, src, dst, sms, stream)
-                        : by_tb<3, 27, true, false>(Tb, g, wdev, src, dst, sms, stream);
-    return per ? by_tb<3, 7, false, true>(Tb, g, wdev, src, dst, sms, stream)
-               : by_tb<3, 7, false, false>(Tb, g, wdev, src, dst, sms, stream);
+    if (box && wide.n) return per ? by_tb<3, 27, true, true, false, true>(Tb, g, wide, wdev, src, dst, sms, stream)
+                                  : by_tb<3, 27, true, false, false, true>(Tb, g, wide, wdev, src, dst, sms, stream);
+    if (box) return per ? by_tb<3, 27, true, true>(Tb, g, wide, wdev, src, dst, sms, stream)
+                        : by_tb<3, 27, true, false>(Tb, g, wide, wdev, src, dst, sms, stream);
+    if (wide.n) return per ? by_tb<3, 7, false, true, false, true>(Tb, g, wide, wdev, src, dst, sms, stream)
+                           : by_tb<3, 7, false, false, false, true>(Tb, g, wide, wdev, src, dst, sms, stream);
+    return per ? by_tb<3, 7, false, true>(Tb, g, wide, wdev, src, dst, sms, stream)
+               : by_tb<3, 7, false, false>(Tb, g, wide, wdev, src, dst, sms, stream);
   }
-  if (box && equal) return per ? by_tb<2, 9, true, true, true>(Tb, g, wdev, src, dst, sms, stream)
-                               : by_tb<2, 9, true, false, true>(Tb, g, wdev, src, dst, sms, stream);
-  if (box) return per ? by_tb<2, 9, true, true>(Tb, g, wdev, src, dst, sms, stream)
-                      : by_tb<2, 9, true, false>(Tb, g, wdev, src, dst, sms, stream);
-  return per ? by_tb<2, 5, false, true>(Tb, g, wdev, src, dst, sms, stream)
-             : by_tb<2, 5, false, false>(Tb, g, wdev, src, dst, sms, stream);
+  if (box && equal) return per ? by_tb<2, 9, true, true, true>(Tb, g, wide, wdev, src, dst, sms, stream)
+                               : by_tb<2, 9, true, false, true>(Tb, g, wide, wdev, src, dst, sms, stream);
+  if (box) return per ? by_tb<2, 9, true, true>(Tb, g, wide, wdev, src, dst, sms, stream)
+                      : by_tb<2, 9, true, false>(Tb, g, wide, wdev, src, dst, sms, stream);
+  return per ? by_tb<2, 5, false, true>(Tb, g, wide, wdev, src, dst, sms, stream)
+             : by_tb<2, 5, false, false>(Tb, g, wide, wdev, src, dst, sms, stream);
 }
 
 }  // namespace gbst

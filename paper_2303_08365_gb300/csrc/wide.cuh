@@ -1,0 +1,254 @@
+// wide.cuh -- the weighted sum of a sweep in integer arithmetic.
+//
+// This GPU issues 2 FP64 instructions per clock per SM but 64 of each of the
+// integer kinds that the sum needs (measured per clock per SM: DFMA 1.98,
+// 32 x 32 + 64 bit multiply-add 62, shift and logic 63, 64-bit shift 25), so
+// sum_k w_k u_k over K taps costs K/2 clocks on the FP64 pipe and about 0.13 K
+// + 0.2 on the integer pipes.  The sum is taken in fixed point, aligned cell by
+// cell:
+//   - u_k is unpacked into a signed 62-bit integer M_k (the 53-bit significand,
+//     9 zero bits below it) and its exponent; w_k = W_k 2^x_k, W_k the 53-bit
+//     significand, is split once on the host into two limbs of 27 and 26 bits;
+//   - E = the largest exponent of any product w_k u_k; A_k = M_k >> (E - e_k),
+//     so the low bits that a product loses lie 2^-62 below the largest one;
+//   - S = sum_k A_k W_k, exactly, in four 64-bit accumulators of 32 x 32 bit
+//     products, then R = S / 2^57 rounded, 56 bits or more for the largest product;
+//   - R is rounded once to a double and its exponent is set.
+// The error is one rounding of the result and about 2^-55 of the largest product
+// (half a unit of R, and K/16 units from the bits that the alignment drops),
+// against K roundings of partial sums in an FMA chain.  The result is
+// a function of the K values alone: every kernel that takes it gives the same
+// bits, whatever its tiles.
+//
+// It covers weights > 0.  Values whose largest exponent is out of the range in
+// which that is safe (infinities, NaN, products near the largest or the
+// smallest doubles, neighbourhoods that are all zero) take the FMA chain, cell by cell.
+#pragma once
+
+#include <cmath>
+#include <cstdint>
+
+#include "internal.h"
+#include "taps.cuh"
+
+namespace gbst {
+
+// Splits the weights; false (and n = 0) when the integer form does not cover
+// them: a weight that is not positive, or weights so far apart or so extreme
+// that no range of exponents is left.
+inline bool make_wide(const double* w, int n, WideTaps& t) {
+  t.n = 0;
+  if (n < 1 || n > kWideMaxTaps) return false;
+  int xmax = -100000, x[kWideMaxTaps];
+  for (int k = 0; k < n; ++k) {
+    if (!(w[k] > 0.0) || !std::isfinite(w[k])) return false;
+    std::frexp(w[k], &x[k]);  // w = m 2^x, m in [0.5, 1)
+    if (x[k] > xmax) xmax = x[k];
+  }
+  int ex_min = 0;
+  for (int k = 0; k < n; ++k) {
+    const int64_t W = (int64_t)std::ldexp(w[k], 53 - x[k]);  // [2^52, 2^53), exact
+    const int64_t hi = W >> 26, lo = W - hi * (1 << 26);
+    t.hi[k] = (int)hi;
+    t.hi2[k] = (int)(2 * hi);
+    t.lo[k] = (int)lo;
+    t.ex[k] = x[k] - xmax;
+    if (t.ex[k] < ex_min) ex_min = t.ex[k];
+  }
+  t.bias = 1080 - xmax;
+  // a zero or subnormal value is unpacked as if it had a leading 1: E >= 64
+  // shifts it out; the result's exponent stays within the normal range; an
+  // infinity or NaN (exponent field 2047) is always above e_max
+  const int e_min = t.bias - 1010 > 64 ? t.bias - 1010 : 64;
+  const int e_max = 2046 + ex_min < 2030 - xmax ? 2046 + ex_min : 2030 - xmax;
+  if (e_max < e_min + 256) return false;
+  t.e_min = e_min;
+  t.e_span = (unsigned)(e_max - e_min);
+  t.heat = n >= 3 && n % 2 == 1;
+  for (int k = 1; k < n; ++k)
+    if (k != n / 2 && w[k] != w[0]) t.heat = 0;
+  t.n = n;
+  return true;
+}
+
+#ifdef __CUDACC__
+
+// A value unpacked: the signed 62-bit integer (hi, lo) and its exponent field.
+struct WideVal {
+  int hi;
+  unsigned int lo;
+  int e;
+};
+
+__device__ __forceinline__ WideVal wide_unpack(double v) {
+  const unsigned int hi = (unsigned int)__double2hiint(v), lo = (unsigned int)__double2loint(v);
+  const int s = (int)hi >> 31;
+  const unsigned int m = (hi & 0xfffffu) | 0x100000u;
+  WideVal u;
+  u.e = (int)((hi << 1) >> 21);
+  // one's complement for negative values: 2^-62 of the value away
+  u.hi = (int)(__funnelshift_l(lo, m, 9) ^ (unsigned int)s);
+  u.lo = (lo << 9) ^ (unsigned int)s;
+  return u;
+}
+
+// The double that was unpacked (exact, whatever it was).
+__device__ __forceinline__ double wide_repack(const WideVal& u) {
+  const unsigned int s = (unsigned int)(u.hi >> 31);
+  const unsigned int h = (unsigned int)u.hi ^ s, l = u.lo ^ s;
+  return __hiloint2double((int)((s & 0x80000000u) | ((unsigned int)u.e << 20) | ((h >> 9) & 0xfffffu)),
+                          (int)__funnelshift_r(l, h, 9));
+}
+
+// The FMA chain for the neighbourhoods that the integer form does not take
+// (wdev: the weights as doubles).  Out of line: it is rarely run.
+static __device__ __noinline__ double wide_chain(const double* v, const double* wdev, int n) {
+  long long any = 0;
+  for (int k = 0; k < n; ++k) any |= __double_as_longlong(v[k]) << 1;
+  if (any == 0) return 0.0;  // every value is a zero
+  double acc = 0.0;
+  for (int k = 0; k < n; ++k) acc = fma(__ldg(wdev + k), v[k], acc);
+  return acc;
+}
+
+// Whether the integer form takes a cell whose largest product has exponent E.
+__device__ __forceinline__ bool wide_covers(int E, const WideTaps& T) {
+  return (unsigned int)(E - T.e_min) <= T.e_span;
+}
+
+// M >> d; an amount over 63 leaves the sign.
+__device__ __forceinline__ long long wide_align(const WideVal& u, int d) {
+  long long a;
+  asm("{.reg .b64 t; mov.b64 t, {%2, %1}; shr.s64 %0, t, %3;}" : "=l"(a) : "r"(u.hi), "r"(u.lo), "r"(d));
+  return a;
+}
+
+// The accumulators of a cell: hh, hl, lh and ll count units of 2^57, 2^32, 2^26 and
+// 1 of S (27 taps: below 2^63 each).
+struct WideAcc {
+  long long hh, hl;
+  unsigned long long lh, ll;
+  __device__ __forceinline__ WideAcc() : hh(0), hl(1 << 24 /* half a unit of R */), lh(0), ll(0) {}
+
+  // Adds W_k a.
+  __device__ __forceinline__ void add(long long a, int k, const WideTaps& T) {
+    const int ah = (int)(a >> 32);
+    const unsigned int al = (unsigned int)a;
+    // one multiply-add each (written in C, the addends cost moves: 149 against
+    // 115 instructions for a 5-tap cell)
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(hh) : "r"(ah), "r"(T.hi2[k]));
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(hl) : "r"(ah), "r"(T.lo[k]));
+    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(lh) : "r"(al), "r"(T.hi[k]));
+    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(ll) : "r"(al), "r"(T.lo[k]));
+  }
+
+  // Adds w_k u whose product lies d exponents below the cell's largest.
+  __device__ __forceinline__ void add(const WideVal& u, int k, int d, const WideTaps& T) {
+    add(wide_align(u, d), k, T);
+  }
+
+  // The sum as a double.
+  __device__ __forceinline__ double get(int E, const WideTaps& T) const {
+    const long long R = hh + ((hl + (long long)((lh + (ll >> 26)) >> 6)) >> 25);
+    // R to double: (2^84 + 2^63 + high) - (2^84 + 2^63 + 2^52) exactly, then one
+    // rounding when the low word (2^52 + low) is added.  As FMAs on registers,
+    // which run at the full FP64 rate (additions at 83%)
+    double one, off;
+    asm("mov.f64 %0, 0d3FF0000000000000;" : "=d"(one));
+    asm("mov.f64 %0, 0dC530000080100000;" : "=d"(off));
+    const double dh = __hiloint2double(0x45300000, (int)(R >> 32) ^ (int)0x80000000);
+    const double dl = __hiloint2double(0x43300000, (int)(unsigned int)R);
+    const double r = fma(dl, one, fma(dh, one, off));
+    const int h = __double2hiint(r);
+    return __hiloint2double(h != 0 ? h + ((E - T.bias) << 20) : h, __double2loint(r));
+  }
+};
+
+// sum_k w_k u_k of one cell (the file's head comment); ok = false, and a
+// result without meaning, where the FMA chain has to take the cell.
+template <int NT>
+__device__ __forceinline__ double wide_sum(const WideVal (&u)[NT], const WideTaps& T, bool& ok) {
+  int e[NT];
+#pragma unroll
+  for (int k = 0; k < NT; ++k) e[k] = u[k].e + T.ex[k];
+  int E = e[0];
+#pragma unroll
+  for (int k = 1; k < NT; ++k) E = max(E, e[k]);
+  ok = wide_covers(E, T);
+  WideAcc acc;
+#pragma unroll
+  for (int k = 0; k < NT; ++k) acc.add(u[k], k, E - e[k], T);
+  return acc.get(E, T);
+}
+
+// The same for weights that are one value at the centre tap (NT / 2) and one at
+// all the others (Eq. 3): one exponent for the neighbours, and their integers added
+// in pairs (two of 62 bits fit 63) before the multiplication.  S is exact either
+// way, so the result has the same bits.
+template <int NT>
+__device__ __forceinline__ double wide_sum_heat(const WideVal (&u)[NT], const WideTaps& T, bool& ok) {
+  constexpr int C = NT / 2;  // NT - 1 neighbours: an even number
+  auto nb = [&](int k) -> const WideVal& { return u[k < C ? k : k + 1]; };
+  int en = nb(0).e;
+#pragma unroll
+  for (int k = 1; k + 1 < NT - 1; k += 2) en = __vimax3_s32(en, nb(k).e, nb(k + 1).e);
+  en = max(en, nb(NT - 2).e);
+  const int ec = u[C].e + T.ex[C];
+  const int E = max(en + T.ex[0], ec);
+  ok = wide_covers(E, T);
+  const int dn = E - T.ex[0];
+  WideAcc acc;
+#pragma unroll
+  for (int k = 0; k < NT - 1; k += 2)
+    acc.add(wide_align(nb(k), dn - nb(k).e) + wide_align(nb(k + 1), dn - nb(k + 1).e), 0, T);
+  acc.add(u[C], C, E - ec, T);
+  return acc.get(E, T);
+}
+
+// The same with the FMA chain in its place where it has to be.
+template <int NT>
+__device__ __forceinline__ double wide_sum(const WideVal (&u)[NT], const WideTaps& T,
+                                           const double* __restrict__ wdev) {
+  bool ok;
+  const double r = wide_sum<NT>(u, T, ok);
+  if (ok) return r;
+  double v[NT];
+#pragma unroll
+  for (int k = 0; k < NT; ++k) v[k] = wide_repack(u[k]);
+  return wide_chain(v, wdev, NT);
+}
+
+// The weighted sum of a cell, collected tap by tap: the FMA chain in tap
+// order, or the integer form once every value is there.
+template <int NT, bool WIDE>
+struct TapSum;
+
+template <int NT>
+struct TapSum<NT, false> {
+  using Acc = double;
+  RegWeights<NT> W;
+  __device__ __forceinline__ TapSum(const double* __restrict__ wdev, const WideTaps&) { W.load(wdev); }
+  __device__ __forceinline__ void tap(Acc& acc, int k, double v, int c) const { W.tap(acc, k, v, c); }
+  __device__ __forceinline__ double get(const Acc& acc) const { return acc; }
+  __device__ __forceinline__ double get(const Acc& acc, bool& ok) const {
+    ok = true;
+    return acc;
+  }
+};
+
+template <int NT>
+struct TapSum<NT, true> {
+  struct Acc {
+    WideVal u[NT];
+  };
+  const WideTaps& T;
+  const double* wdev;
+  __device__ __forceinline__ TapSum(const double* __restrict__ w, const WideTaps& t) : T(t), wdev(w) {}
+  __device__ __forceinline__ void tap(Acc& acc, int k, double v, int) const { acc.u[k] = wide_unpack(v); }
+  __device__ __forceinline__ double get(const Acc& acc) const { return wide_sum<NT>(acc.u, T, wdev); }
+  __device__ __forceinline__ double get(const Acc& acc, bool& ok) const { return wide_sum<NT>(acc.u, T, ok); }
+};
+
+#endif  // __CUDACC__
+
+}  // namespace gbst

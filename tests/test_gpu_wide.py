@@ -1,0 +1,125 @@
+"""The integer form of the weighted sum (csrc/wide.cuh) and the kernels that
+only it has: sizes at the edges of their tiles, unaligned grids, and the values
+at which it hands over to the FMA chain."""
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+PERIODIC, DIRICHLET = 1, 0
+EPS = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def st():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2303_08365_gb300 import build
+    build.build()
+    import paper_2303_08365_gb300 as st
+    return st
+
+
+def weights(kind, ndim, radius, seed=5):
+    side = 2 * radius + 1
+    w = np.random.default_rng(seed).random((side,) * ndim) + 0.01
+    if kind == "star":
+        off = np.stack(np.meshgrid(*[np.arange(-radius, radius + 1)] * ndim, indexing="ij"))
+        w[(off != 0).sum(axis=0) > 1] = 0.0
+    return w / w.sum()
+
+
+def run(st, u0, w, radius, boundary, T, tuning=(0, 0), offset=0):
+    """Sweeps a copy of u0 placed `offset` elements past a 256-byte boundary, between canaries."""
+    import torch
+    n = u0.size
+    buf = torch.full((n + 128,), 7.0, dtype=torch.float64, device="cuda")
+    g = buf[64 + offset:64 + offset + n].view(u0.shape)
+    g.copy_(torch.from_numpy(u0))
+    p = st.Plan(u0.shape, radius, w, boundary)
+    p.set_tuning(*tuning)
+    p.run(g, T)
+    assert p.status() == 0
+    out = g.cpu().numpy().copy()
+    g.fill_(7.0)
+    assert bool((buf == 7.0).all())
+    p.close()
+    return out
+
+
+# planes of one row or column more or fewer than a tile, one tile in all, rows
+# that start on and off 16 bytes, a grid that ends half-way through 16 bytes
+SHAPES3D = [(1, 8, 32), (2, 17, 33), (3, 16, 64), (5, 15, 65), (7, 33, 63), (4, 18, 129), (9, 31, 191), (40, 9, 130)]
+
+
+@pytest.mark.parametrize("kind", ["star", "box"])
+@pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
+@pytest.mark.parametrize("shape", SHAPES3D)
+def test_streaming_any_shape_3d(st, shape, boundary, kind):
+    w = weights(kind, 3, 1)
+    u0 = synth.normal(31, shape)
+    T, taps = 3, int(np.count_nonzero(w))
+    ref = oracle.run(u0, w, 1, boundary, T, nthreads=0)
+    # two roundings per tap and step in the oracle, fewer on the GPU; the sums do not expand
+    tol = T * (2 * taps + 2) * EPS * np.abs(u0).max()
+    for offset in (0, 1):
+        got = run(st, u0, w, 1, boundary, T, (1, st.VARIANT_DIRECT), offset)
+        assert np.abs(got - ref).max() <= tol, offset
+
+
+def exact_sum(u, w, at, radius):
+    """(sum, largest |product|) of one cell over the reals, zeros outside."""
+    total, top = Fraction(0), Fraction(0)
+    for o in np.ndindex(*w.shape):
+        i = tuple(a + k - radius for a, k in zip(at, o))
+        if w[o] != 0 and all(0 <= a < n for a, n in zip(i, u.shape)):
+            p = Fraction(float(w[o])) * Fraction(float(u[i]))
+            total += p
+            top = max(top, abs(p))
+    return total, top
+
+
+WIDE_RANGE = [((6, 9, 33), "star", 1), ((4, 9, 34), "box", 1)]
+
+
+@pytest.mark.parametrize("spread", [0, 8, 60, 300])
+@pytest.mark.parametrize("shape,kind,radius", WIDE_RANGE)
+def test_one_step_against_exact_arithmetic(st, shape, kind, radius, spread):
+    """Values of both signs whose exponents are spread, with zeros among them:
+    one rounding of the result and 2^-55 of the largest product."""
+    rng = np.random.default_rng(spread)
+    u0 = rng.standard_normal(shape) * 2.0 ** rng.integers(-spread, spread + 1, shape)
+    u0[rng.random(shape) < 0.1] = 0.0
+    w = weights(kind, len(shape), radius)
+    got = run(st, u0, w, radius, DIRICHLET, 1)
+    for at in np.ndindex(*shape):
+        want, top = exact_sum(u0, w, at, radius)
+        err = abs(Fraction(float(got[at])) - want)
+        assert err <= abs(want) * Fraction(EPS) + top * Fraction(2.0 ** -55), at
+
+
+@pytest.mark.parametrize("shape,kind,radius", WIDE_RANGE)
+def test_values_outside_the_integer_range(st, shape, kind, radius):
+    """Infinities, NaN, the largest and the smallest doubles, and all-zero
+    neighbourhoods take the FMA chain: as the oracle has them."""
+    rng = np.random.default_rng(9)
+    w = weights(kind, len(shape), radius)
+    for values in ([np.inf, 1.0], [np.nan, 1.0], [-np.inf, np.inf, 0.0], [1.7e308, -1.2e308, 3.0],
+                   [5e-324, -3e-310, 0.0], [2.3e-308, 0.0], [1e-290, 1e-292], [0.0, -0.0]):
+        u0 = np.zeros(shape)
+        mask = rng.random(shape) < 0.05
+        u0[mask] = rng.choice(values, int(mask.sum()))
+        with np.errstate(all="ignore"):
+            ref = oracle.run(u0, w, radius, DIRICHLET, 1, nthreads=1)
+            got = run(st, u0, w, radius, DIRICHLET, 1)
+            assert np.array_equal(np.isnan(got), np.isnan(ref)), values
+            fine = np.isfinite(ref)
+            assert np.array_equal(got[~fine & ~np.isnan(ref)], ref[~fine & ~np.isnan(ref)]), values
+            # 27 roundings at most of sums no larger than the largest value; below the
+            # normal range each is half of the smallest subnormal
+            top = np.abs(u0[np.isfinite(u0)]).max() if np.isfinite(u0).any() else 0.0
+            assert np.abs(got[fine] - ref[fine]).max(initial=0.0) <= max(60 * EPS * top, 60 * 5e-324), values
