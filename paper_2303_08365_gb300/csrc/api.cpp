@@ -217,12 +217,19 @@ void build_taps(stencil_plan_s* p, const double* w) {
 // The stencil classes whose kernels have the integer form of the sum.  All
 // kernels of a class take it, so its results do not depend on the kernel.
 bool uses_wide(int ndim, int radius) {
-  return ndim == 3 && radius == 1;
+  return (ndim == 3 && radius == 1) || (ndim == 2 && radius == 2);
 }
 
-// Whether a 3D grid that the TMA-fed kernels do not take is streamed all the
-// same (asynchronous copies instead of TMA boxes) or swept cell by cell.
-bool wide3d_worth(const Geom& g) { return g.nx >= 32 && g.ny >= 8; }
+// Whether a grid that the TMA-fed kernels do not take is streamed all the same
+// (by bulk copies) or swept cell by cell.  Streaming takes longer to start: on
+// GB300, us a step, cell by cell against streamed: 2D radius 2, 257^2 6.3 / 6.3,
+// 513^2 11.4 / 8.3, 129^2 4.2 / 6.3; 3D star 97^3 22.9 / 24.8, 129^3 43 / 41;
+// 27-point box 49^3 16.6 / 14.7, 33^3 10.5 / 12.5.
+bool streamed_any_shape(const stencil_plan_s* p) {
+  if (!p->wide.n || p->g.nx < 32 || p->g.ny < 8) return false;
+  if (p->ndim == 2) return p->cells() >= (int64_t)1 << 17;
+  return p->ndim == 3 && p->radius == 1 && p->cells() >= (int64_t)1 << (p->shape == Shape::kBox ? 17 : 21);
+}
 
 std::string device_name();
 
@@ -622,14 +629,20 @@ int run_steps(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, int variant,
       steps = Tb;
     } else {
       const int v = variant == kVariantTemporal || variant == kVariantExchange ? single : variant;
-      if (v == kVariantStream && p->ndim == 3)
-        e = launch_stream3d(p->shape, p->boundary, p->g, p->taps, p->wide, p->d_w, a, b, p->d_status, sms, s,
+      if (v == kVariantStream && p->ndim == 3 && p->wide.n)
+        e = launch_wide3d(p->shape, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, tile_y, true);
+      else if (v == kVariantStream && p->ndim == 2 && p->wide.n && !(equal_box && p->radius == 1))
+        e = launch_wide2d(p->shape, p->radius, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, true);
+      else if (v == kVariantStream && p->ndim == 3)
+        e = launch_stream3d(p->shape, p->boundary, p->g, p->taps, p->d_w, a, b, p->d_status, sms, s,
                             (unsigned long long)kSpinLimitNs, -1, tile_y);
       else if (v == kVariantStream)
         e = launch_stream2d(p->shape, p->radius, p->boundary, equal_box && p->radius == 1, p->g, p->taps,
                             p->d_w, a, b, p->d_status, sms, s);
-      else if (p->wide.n && p->ndim == 3 && p->radius == 1 && wide3d_worth(p->g))
+      else if (p->ndim == 3 && streamed_any_shape(p))
         e = launch_wide3d(p->shape, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, 0, false);
+      else if (p->ndim == 2 && streamed_any_shape(p))
+        e = launch_wide2d(p->shape, p->radius, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, false);
       else
         e = launch_direct(p->ndim, p->radius, p->shape, p->boundary, p->g, p->taps, p->wide, p->d_w, a, b, s);
     }
@@ -1752,7 +1765,7 @@ int stencil_selftest_tma_timeout(double limit_ms, void* cuda_stream) {
   cudaMemsetAsync(status, 0, sizeof(int), s);
   cudaMemcpyAsync(w, hw.data(), hw.size() * sizeof(double), cudaMemcpyHostToDevice, s);
   int rc = STENCIL_OK;
-  cudaError_t e = launch_stream3d(Shape::kStar, kPeriodic, g, taps, WideTaps{}, w, a, b, status, sm_count(), s,
+  cudaError_t e = launch_stream3d(Shape::kStar, kPeriodic, g, taps, w, a, b, status, sm_count(), s,
                                   (unsigned long long)(limit_ms * 1e6), 1);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   int st = 0;

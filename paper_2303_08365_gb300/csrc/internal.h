@@ -96,7 +96,7 @@ bool stream3d_shape_ok(int ndim, int radius, Shape shape, int boundary, const Ge
 int stream3d_tile_y(Shape shape, int tile_y);
 // wait_ns bounds every mbarrier wait (kSpinLimitNs in normal runs); skip_plane
 // >= 0 is the self-test's starved plane (the producer posts no copy for it).
-cudaError_t launch_stream3d(Shape shape, int boundary, const Geom& g, const HostTaps& taps, const WideTaps& wide,
+cudaError_t launch_stream3d(Shape shape, int boundary, const Geom& g, const HostTaps& taps,
                             const double* wdev, const double* src, double* dst, int* status,
                             int sms, cudaStream_t stream, unsigned long long wait_ns = 2000000000ull,
                             long long skip_plane = -1, int tile_y = 0);
@@ -118,6 +118,13 @@ bool taps_all_equal(const HostTaps& t);
 cudaError_t launch_stream2d(Shape shape, int radius, int boundary, bool equal, const Geom& g,
                             const HostTaps& taps, const double* wdev, const double* src, double* dst,
                             int* status, int sms, cudaStream_t stream);
+
+// 2D sweep (radius 1 or 2, star or box) with the weighted sum in the integer
+// form (wide.n != 0), tiles of 64 columns by 16 rows.  tma: the grid is one that
+// stream2d_eligible takes; false: any shape, alignment and boundary.
+cudaError_t launch_wide2d(Shape shape, int radius, int boundary, const Geom& g, const WideTaps& wide,
+                          const double* wdev, const double* src, double* dst, int* status, int sms,
+                          cudaStream_t stream, bool tma);
 
 // Temporal blocking: Tb fused steps per launch (2D and 3D: radius 1, any
 // shape and boundary; 1D: radius 1 or 2; Tb in {2, 4, 8}).

@@ -383,13 +383,12 @@ cudaError_t launch_ty(int ty, const Geom& g, const double* wdev, const double* s
 }
 }  // namespace
 
-cudaError_t launch_stream3d(Shape shape, int boundary, const Geom& g, const HostTaps& taps, const WideTaps& wide,
+cudaError_t launch_stream3d(Shape shape, int boundary, const Geom& g, const HostTaps& taps,
                             const double* wdev, const double* src, double* dst, int* status,
                             int sms, cudaStream_t stream, unsigned long long wait_ns, long long skip_plane,
                             int tile_y) {
   const bool per = boundary == kPeriodic;
   const int ty = stream3d_tile_y(shape, tile_y);
-  if (wide.n) return launch_wide3d(shape, boundary, g, wide, wdev, src, dst, status, sms, stream, ty, true);
   if (shape == Shape::kBox) {
     if (taps.n != 27) return cudaErrorInvalidValue;
     return per ? launch_ty<27, true, true>(ty, g, wdev, src, dst, status, sms, stream, wait_ns, skip_plane)

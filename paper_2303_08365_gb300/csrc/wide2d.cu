@@ -1,0 +1,451 @@
+// wide2d.cu -- 2D sweep (radius 1 or 2, star or box) with the weighted sum in the
+// integer form (wide.cuh).
+//
+// One step of u'(x) = sum_o w_o u~(x+o) (paper Sec. 2.1, Listing 1).  The grid is
+// cut into tiles of 64 columns by 16 rows, taken down each column of tiles.  As in
+// wide3d.cu a tile's values are unpacked once, into shared memory:
+//   - the raw tile (its columns, RAD rows more above and below) arrives up to
+//     three tiles ahead: by TMA where the grid allows it (out-of-range parts read
+//     zeros, the Dirichlet ghosts), else row by row by bulk copies, which take any
+//     size, alignment and wrap;
+//   - iteration g: every consumer warp unpacks its own two rows of tile g into ring
+//     slot g % 3 (the producer warp the rows and columns around the tile), arrives
+//     on conv[g % 3], and computes its rows of tile g-1, which is complete
+//     (waited for before tile g is unpacked; every warp has then also finished
+//     tile g-3, whose slot tile g takes).
+// The rows between two tiles are unpacked twice (18 or 20 rows for 16).
+//
+// Measured at 8192^2, periodic, general weights (FMA chain before): 25-point box
+// 52 GStencil/s (23.6), radius-2 star 113 (67).
+//
+// Work split: the tiles are cut into equal contiguous ranges, one per CTA.
+#include <cudaTypedefs.h>
+
+#include "internal.h"
+#include "ptx.cuh"
+#include "taps.cuh"
+#include "wide.cuh"
+#include "widestream.cuh"
+
+namespace gbst {
+
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();  // stream.cu
+
+namespace {
+
+constexpr int kTX = kWTX, kRaw = kWRaw, kWarps = kWWarps, kThreads = kWThreads;
+constexpr int kTC = 16;                // tile rows
+constexpr int kR = kTC / kWarps;       // rows of a consumer warp
+constexpr int kU = 3;
+
+template <int RAD>
+using Plane = WidePlane<kTC + 2 * RAD>;
+
+template <int RAD, bool TMA>
+struct __align__(128) Smem {
+  double raw[kRaw][kTC + 2 * RAD][raw_col<TMA>()];
+  int shift[kRaw][kTC + 2 * RAD];  // bulk copies: position of column x0 in the row (0 or 1)
+  Plane<RAD> u[kU];
+  uint64_t full[kRaw];   // raw tile has landed
+  uint64_t empty[kRaw];  // raw tile is unpacked: 8 consumer warps, the producer
+  uint64_t conv[kU];     // tile is unpacked: the same 9 arrivals
+};
+static_assert(kU == kRaw, "one ring position serves both");
+
+struct Params {
+  CUtensorMap map_row;   // box {64, 1} over src
+  CUtensorMap map_tile;  // box {64, 16 + 2 RAD} over src
+  const double* src;
+  double* dst;
+  int ny, nx;
+  int tiles_y;
+  int work;  // tiles
+  int vec;   // rows start on 16 bytes
+  int* status;
+  const double* wdev;
+  WideTaps wide;
+};
+
+// Position of offset (dy, dx) in the lexicographic tap list of the class.
+template <bool BOX, int RAD>
+__device__ __forceinline__ constexpr int tap_at(int dy, int dx) {
+  if (BOX) return (dy + RAD) * (2 * RAD + 1) + (dx + RAD);
+  return dy < 0 ? dy + RAD : dy > 0 ? 3 * RAD + dy : 2 * RAD + dx;
+}
+
+// Columns c-RAD .. c+1+RAD of a row.
+template <int RAD>
+__device__ __forceinline__ void get_row(const Plane<RAD>& u, int row, int c, WideVal (&v)[2 * RAD + 2]) {
+  get_pair(&u.m[row][c], &u.e[row][c], v[RAD], v[RAD + 1]);
+  if constexpr (RAD == 1) {
+    v[0] = get(&u.m[row][c - 1], &u.e[row][c - 1]);
+    v[3] = get(&u.m[row][c + 2], &u.e[row][c + 2]);
+  } else {
+    get_pair(&u.m[row][c - 2], &u.e[row][c - 2], v[0], v[1]);
+    get_pair(&u.m[row][c + 2], &u.e[row][c + 2], v[4], v[5]);
+  }
+}
+
+// The cells of a lane that the integer form does not take, by the FMA chain:
+// `cols` columns from c0 on of rows row0 .. row0+rows-1.  Out of line: rarely run.
+template <bool BOX, int RAD>
+__device__ __noinline__ void chain_cells(const Plane<RAD>& u, int row0, int rows, int cols, int c0, const WideTaps& T,
+                                         const double* wdev, double* out, int nx) {
+  constexpr int NT = BOX ? (2 * RAD + 1) * (2 * RAD + 1) : 4 * RAD + 1;
+  for (int r = 0; r < rows; ++r)
+    for (int i = 0; i < cols; ++i) {
+      double v[NT];
+      int E = -0x7fffffff;
+      for (int dy = -RAD; dy <= RAD; ++dy)
+        for (int dx = -RAD; dx <= RAD; ++dx) {
+          if (!BOX && dy != 0 && dx != 0) continue;
+          const int t = tap_at<BOX, RAD>(dy, dx), row = row0 + r + dy, c = c0 + i + dx;
+          const WideVal x = get(&u.m[row][c], &u.e[row][c]);
+          v[t] = wide_repack(x);
+          E = max(E, x.e + T.ex[t]);
+        }
+      if (!wide_covers(E, T)) out[(int64_t)r * nx + i] = wide_chain(v, wdev, NT);
+    }
+}
+
+template <bool BOX, int RAD>
+constexpr int wide2d_ctas() { return RAD == 1 && !BOX ? 3 : 2; }
+
+template <bool BOX, int RAD, bool HEAT, bool PERIODIC, bool TMA>
+__global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(const __grid_constant__ Params P) {
+  constexpr int kRows = kTC + 2 * RAD;
+  constexpr unsigned long long kWaitNs = (unsigned long long)kSpinLimitNs;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  Smem<RAD, TMA>& S = *reinterpret_cast<Smem<RAD, TMA>*>(smem_raw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kRaw; ++s) {
+      mbar_init(&S.full[s], 1);
+      mbar_init(&S.empty[s], kWarps + 1);
+      mbar_init(&S.conv[s], kWarps + 1);
+    }
+    fence_mbar_init();
+    if (TMA) {
+      prefetch_tmap(&P.map_row);
+      prefetch_tmap(&P.map_tile);
+    }
+  }
+  __syncthreads();
+  // a bounded wait; false: it gave up (the other warps' waits on this one then do the same)
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    if (mbar_wait_bounded(bar, parity, kWaitNs)) return true;
+    atomicCAS(P.status, 0, -5 /* STENCIL_ERR_TIMEOUT */);
+    return false;
+  };
+  const int64_t pitch = P.nx;
+  const int t0 = (int)((long long)P.work * blockIdx.x / gridDim.x);
+  const int t1 = (int)((long long)P.work * (blockIdx.x + 1) / gridDim.x);
+  RingPos<kU> pos;       // of tile g
+  int u1 = kU - 1;       // slot of tile g-1
+  uint32_t ph1 = 1;      // its phase (a fresh barrier lets a wait for phase 1 pass)
+  auto next = [&] {
+    u1 = pos.s;
+    ph1 = pos.ph;
+    pos.next();
+  };
+  if (warp == kWarps) {
+    // ------------------------------------------------------------ producer
+    RingPos<kU> post;  // of the next tile to post
+    int posted = t0;
+    // copies tile t into its raw slot, once the slot's earlier tile is unpacked
+    auto post_tile = [&](int t) {
+      if (!wait(&S.empty[post.s], post.ph ^ 1)) return false;
+      const int x0 = t / P.tiles_y * kTX, y0 = t % P.tiles_y * kTC;
+      const int r = lane;
+      int y = y0 - RAD + r;
+      if (TMA) {
+        const bool whole = !PERIODIC || (y0 >= RAD && y0 + kTC + RAD <= P.ny);
+        fence_proxy_async_smem();
+        if (lane == 0) {
+          mbar_arrive_expect_tx(&S.full[post.s], (uint32_t)sizeof(S.raw[0]));
+          if (whole) tma_load_2d(&S.raw[post.s][0][0], &P.map_tile, x0, y0 - RAD, &S.full[post.s]);
+        }
+        __syncwarp();
+        if (!whole && r < kRows)
+          tma_load_2d(&S.raw[post.s][r][0], &P.map_row, x0, wrapn(y, P.ny), &S.full[post.s]);
+      } else {
+        bool in = r < kRows;
+        if (PERIODIC) {
+          in = in && y < P.ny + RAD;  // rows past the ghosts of a ragged tile are not read
+          y = wrapn(y, P.ny);
+        } else {
+          in = in && y >= 0 && y < P.ny;
+        }
+        RowCopy cp;
+        if (in) {
+          cp.plan(S.raw[post.s][r], P.src + (y * pitch + x0), min(kTX, P.nx - x0), P.src, P.src + P.ny * pitch);
+          fence_proxy_async_smem();
+        }
+        if (r < kRows) S.shift[post.s][r] = cp.shift;
+        // rows outside the grid are zeros
+        unsigned int out = __ballot_sync(0xffffffffu, r < kRows && !in);
+        while (out) {
+          const int q = __ffs((int)out) - 1;
+          out &= out - 1;
+          S.raw[post.s][q][lane] = 0.0;
+          S.raw[post.s][q][lane + 32] = 0.0;
+        }
+        const uint32_t total = __reduce_add_sync(0xffffffffu, cp.bytes);
+        __syncwarp();  // the lanes' own writes come before lane 0's arrival
+        if (lane == 0) mbar_arrive_expect_tx(&S.full[post.s], total);
+        __syncwarp();
+        if (cp.bytes) bulk_load(&S.raw[post.s][r][cp.to], cp.from, cp.bytes, &S.full[post.s]);
+      }
+      post.next();
+      ++posted;
+      return true;
+    };
+    // the columns beside a tile: RAD on either side of every row that has
+    // them (star: the tile's own rows), HN values per lane
+    constexpr int HR = BOX ? kRows : kTC, H0 = BOX ? 0 : RAD, HALL = 2 * RAD * HR, HN = (HALL + 31) / 32;
+    auto halo = [&](int t, double (&h)[HN]) {
+      const int x0 = t / P.tiles_y * kTX, y0 = t % P.tiles_y * kTC;
+      const int cols = TMA ? kTX : min(kTX, P.nx - x0);
+#pragma unroll
+      for (int q = 0; q < HN; ++q) {
+        const int k = lane + 32 * q, j = k / HR;  // j: the column, west to east
+        int x = j < RAD ? x0 - RAD + j : x0 + cols + (j - RAD), y = y0 - RAD + H0 + k % HR;
+        bool in = k < HALL;
+        if (PERIODIC) {
+          x = wrapn(x, P.nx);
+          y = wrapn(y, P.ny);
+        } else {
+          in = in && x >= 0 && x < P.nx && y >= 0 && y < P.ny;
+        }
+        h[q] = in ? __ldg(P.src + (y * pitch + x)) : 0.0;
+      }
+    };
+    // a wait that gave up: the copies already posted land (bounded) before the warp leaves
+    auto leave = [&](int t) {
+      RingPos<kU> q = pos;
+      for (int k = t; k < posted; ++k, q.next()) mbar_wait_bounded(&S.full[q.s], q.ph, kWaitNs);
+    };
+    double h[HN], hn[HN];
+    if (t0 < t1) halo(t0, h);
+    for (int t = t0; t < t1; ++t) {
+      while (posted < t1 && posted < t + kRaw)
+        if (!post_tile(posted)) return leave(t);
+      if (t + 1 < t1) halo(t + 1, hn);
+      if (!wait(&S.conv[u1], ph1)) return leave(t);
+      Plane<RAD>& u = S.u[pos.s];
+      const int cols = TMA ? kTX : min(kTX, P.nx - t / P.tiles_y * kTX);
+#pragma unroll
+      for (int q = 0; q < HN; ++q) {
+        const int k = lane + 32 * q, j = k / HR, row = H0 + k % HR;
+        const int c = 2 + (j < RAD ? j - RAD : cols + (j - RAD));
+        if (k < HALL) put(&u.m[row][c], &u.e[row][c], wide_unpack(h[q]));
+      }
+      if (!wait(&S.full[pos.s], pos.ph)) return leave(t);
+      WideVal v[2];
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) {
+        unpack_row<TMA, kRows>(S.raw[pos.s], S.shift[pos.s], u, r, lane, cols, v);
+        unpack_row<TMA, kRows>(S.raw[pos.s], S.shift[pos.s], u, kTC + RAD + r, lane, cols, v);
+      }
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&S.empty[pos.s]);
+        mbar_arrive(&S.conv[pos.s]);
+      }
+#pragma unroll
+      for (int q = 0; q < HN; ++q) h[q] = hn[q];
+      next();
+    }
+    return;
+  }
+  // -------------------------------------------------------------- consumers
+  const int row0 = RAD + warp * kR;  // the warp's first row in the planes
+  const int c = 2 + 2 * lane;
+  for (int t = t0; t <= t1 && t0 < t1; ++t) {  // (the last iteration unpacks nothing)
+    if (!wait(&S.conv[u1], ph1)) return;
+    if (t < t1) {
+      if (!wait(&S.full[pos.s], pos.ph)) return;
+      const int cols = TMA ? kTX : min(kTX, P.nx - t / P.tiles_y * kTX);
+      WideVal v[2];
+#pragma unroll
+      for (int r = 0; r < kR; ++r)
+        unpack_row<TMA, kRows>(S.raw[pos.s], S.shift[pos.s], S.u[pos.s], row0 + r, lane, cols, v);
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&S.empty[pos.s]);
+        mbar_arrive(&S.conv[pos.s]);
+      }
+    }
+    if (t > t0) {
+      const Plane<RAD>& u = S.u[u1];
+      const int xa = (t - 1) / P.tiles_y * kTX + 2 * lane, ya = (t - 1) % P.tiles_y * kTC + warp * kR;
+      const int rows = xa < P.nx ? min(kR, P.ny - ya) : 0;  // rows that the lane stores
+      double* out = P.dst + ya * pitch + xa;
+      auto store = [&](int r, double v0, double v1) {
+        if (r >= rows) return;
+        double* o = out + r * pitch;
+        if (TMA || (P.vec && xa + 1 < P.nx)) {  // (TMA grids: nx even, rows on 16 bytes)
+          st_global_v2(o, v0, v1);
+        } else {
+          o[0] = v0;
+          if (xa + 1 < P.nx) o[1] = v1;
+        }
+      };
+      // the integer form takes every cell that is stored (the others may hold anything)
+      bool all = true;
+      auto covers = [&](bool ok, int r, int i) { return ok || r >= rows || (!TMA && i == 1 && xa + 1 >= P.nx); };
+      if constexpr (!BOX) {
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+          const int row = row0 + r;
+          WideVal y[2 * RAD][2], x[2 * RAD + 2];
+#pragma unroll
+          for (int k = 0; k < 2 * RAD; ++k) {
+            const int rr = row + (k < RAD ? k - RAD : k - RAD + 1);
+            get_pair(&u.m[rr][c], &u.e[rr][c], y[k][0], y[k][1]);
+          }
+          get_row<RAD>(u, row, c, x);
+          double v[2];
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            WideVal w[4 * RAD + 1];
+#pragma unroll
+            for (int k = 0; k < RAD; ++k) {
+              w[k] = y[k][i];
+              w[3 * RAD + 1 + k] = y[RAD + k][i];
+            }
+#pragma unroll
+            for (int k = 0; k <= 2 * RAD; ++k) w[RAD + k] = x[i + k];
+            bool ok;
+            if constexpr (HEAT) v[i] = wide_sum_heat<4 * RAD + 1>(w, P.wide, ok);
+            else v[i] = wide_sum<4 * RAD + 1>(w, P.wide, ok);
+            all = all && covers(ok, r, i);
+          }
+          store(r, v[0], v[1]);
+        }
+      } else {
+        // row by row; the largest exponents first, then the sums: a pair's values would
+        // not fit the registers, so their rows are read twice
+#pragma unroll 1
+        for (int r = 0; r < kR; ++r) {
+          int E[2] = {-0x7fffffff, -0x7fffffff};
+#pragma unroll
+          for (int dy = -RAD; dy <= RAD; ++dy) {
+            const int* er = &u.e[row0 + r + dy][c];
+            int e[2 * RAD + 2];
+#pragma unroll
+            for (int k = 0; k < RAD + 1; ++k) {
+              if (RAD == 1 && k != 0) continue;
+              const int2 m = *reinterpret_cast<const int2*>(er + (RAD == 1 ? 0 : 2 * k - 2));
+              e[RAD == 1 ? 1 : 2 * k] = m.x;
+              e[RAD == 1 ? 2 : 2 * k + 1] = m.y;
+            }
+            if (RAD == 1) {
+              e[0] = er[-1];
+              e[3] = er[2];
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+              for (int dx = -RAD; dx <= RAD; ++dx)
+                E[i] = max(E[i], e[RAD + i + dx] + P.wide.ex[tap_at<true, RAD>(dy, dx)]);
+          }
+          WideAcc acc[2];
+#pragma unroll
+          for (int dy = -RAD; dy <= RAD; ++dy) {
+            WideVal v[2 * RAD + 2];
+            get_row<RAD>(u, row0 + r + dy, c, v);
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+              for (int dx = -RAD; dx <= RAD; ++dx) {
+                const int k = tap_at<true, RAD>(dy, dx);
+                acc[i].add(v[RAD + i + dx], k, E[i] - v[RAD + i + dx].e - P.wide.ex[k], P.wide);
+              }
+          }
+          all = all && covers(wide_covers(E[0], P.wide), r, 0) && covers(wide_covers(E[1], P.wide), r, 1);
+          store(r, acc[0].get(E[0], P.wide), acc[1].get(E[1], P.wide));
+        }
+      }
+      if (!all) chain_cells<BOX, RAD>(u, row0, rows, min(2, P.nx - xa), c, P.wide, P.wdev, out, P.nx);
+      __syncwarp();
+    }
+    if (t < t1) next();
+  }
+}
+
+bool encode_2d(CUtensorMap* map, const double* base, const Geom& g, int rows) {
+  auto enc = tensor_map_encoder();
+  if (!enc) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny};
+  cuuint64_t strides[1] = {(cuuint64_t)g.nx * sizeof(double)};
+  cuuint32_t box[2] = {(cuuint32_t)kTX, (cuuint32_t)rows};
+  cuuint32_t estr[2] = {1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, const_cast<double*>(base), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <bool BOX, int RAD, bool HEAT, bool PERIODIC, bool TMA>
+cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst,
+                     int* status, int sms, cudaStream_t stream) {
+  auto kern = k_wide2d<BOX, RAD, HEAT, PERIODIC, TMA>;
+  constexpr size_t bytes = sizeof(Smem<RAD, TMA>);
+  static std::atomic<int> cache[kMaxDeviceOrdinals];
+  const int occ = cached_per_device(cache, [kern] {
+    int n = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kThreads, bytes) != cudaSuccess)
+      n = 0;
+    return n;
+  });
+  if (occ < 1) return cudaErrorInvalidConfiguration;
+  Params P;
+  if (TMA && (!encode_2d(&P.map_row, src, g, 1) || !encode_2d(&P.map_tile, src, g, kTC + 2 * RAD)))
+    return cudaErrorInvalidValue;
+  P.src = src;
+  P.dst = dst;
+  P.ny = g.ny;
+  P.nx = g.nx;
+  P.tiles_y = (g.ny + kTC - 1) / kTC;
+  const int64_t work = (int64_t)((g.nx + kTX - 1) / kTX) * P.tiles_y;
+  if (work > INT32_MAX) return cudaErrorInvalidValue;
+  P.work = (int)work;
+  P.vec = g.nx % 2 == 0 && ((uintptr_t)dst & 15) == 0;
+  P.status = status;
+  P.wdev = wdev;
+  P.wide = wide;
+  int64_t grid = (int64_t)sms * occ;
+  if (grid > work) grid = work;
+  kern<<<(unsigned)grid, kThreads, bytes, stream>>>(P);
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  return cudaGetLastError();
+}
+
+template <bool BOX, int RAD, bool HEAT>
+cudaError_t launch_p(bool per, bool tma, const Geom& g, const WideTaps& wide, const double* wdev, const double* src,
+                     double* dst, int* status, int sms, cudaStream_t stream) {
+  if (tma)
+    return per ? launch_t<BOX, RAD, HEAT, true, true>(g, wide, wdev, src, dst, status, sms, stream)
+               : launch_t<BOX, RAD, HEAT, false, true>(g, wide, wdev, src, dst, status, sms, stream);
+  return per ? launch_t<BOX, RAD, HEAT, true, false>(g, wide, wdev, src, dst, status, sms, stream)
+             : launch_t<BOX, RAD, HEAT, false, false>(g, wide, wdev, src, dst, status, sms, stream);
+}
+
+}  // namespace
+
+cudaError_t launch_wide2d(Shape shape, int radius, int boundary, const Geom& g, const WideTaps& wide,
+                          const double* wdev, const double* src, double* dst, int* status, int sms,
+                          cudaStream_t stream, bool tma) {
+  const bool per = boundary == kPeriodic, box = shape == Shape::kBox;
+  const int side = 2 * radius + 1;
+  if (wide.n != (box ? side * side : 4 * radius + 1)) return cudaErrorInvalidValue;
+  if (radius == 2)
+    return box ? launch_p<true, 2, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream)
+               : launch_p<false, 2, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream);
+  if (box) return launch_p<true, 1, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream);
+  return wide.heat ? launch_p<false, 1, true>(per, tma, g, wide, wdev, src, dst, status, sms, stream)
+                   : launch_p<false, 1, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream);
+}
+
+}  // namespace gbst

@@ -32,6 +32,7 @@
 #include "ptx.cuh"
 #include "taps.cuh"
 #include "wide.cuh"
+#include "widestream.cuh"
 
 namespace gbst {
 
@@ -39,11 +40,9 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();  // stream.cu
 
 namespace {
 
-constexpr int kTX = 64;
-constexpr int kCol = kTX + 4;  // unpacked row: columns x0-2 .. x0+65 (the pair (x0, x0+1) on 16 bytes)
-constexpr int kRaw = 3;        // raw planes in flight
-constexpr int kWarps = 8;      // consumers
-constexpr int kThreads = (kWarps + 1) * 32;
+constexpr int kTX = kWTX, kRaw = kWRaw, kWarps = kWWarps, kThreads = kWThreads;
+template <int TC>
+using Plane = WidePlane<TC + 2>;
 
 // Unpacked planes.  Star: the three that are read.  Box: a warp reads other
 // warps' rows of all three, the oldest (g-4 in iteration g-1) while another warp
@@ -51,15 +50,6 @@ constexpr int kThreads = (kWarps + 1) * 32;
 template <bool BOX>
 constexpr int ring() { return BOX ? 5 : 3; }
 
-template <int TC>
-struct __align__(16) Plane {
-  long long m[TC + 2][kCol];
-  int e[TC + 2][kCol];
-};
-// A raw row: the tile's 64 columns, or (bulk copies) up to one element more on
-// either side.
-template <bool TMA>
-constexpr int raw_col() { return TMA ? kTX : kTX + 2; }
 template <bool BOX, bool TMA, int TC>
 struct __align__(128) Smem {
   double raw[kRaw][TC + 2][raw_col<TMA>()];
@@ -84,64 +74,12 @@ struct Params {
   WideTaps wide;
 };
 
-__device__ __forceinline__ int wrapn(int c, int n) {
-  const int m = c % n;
-  return m < 0 ? m + n : m;
-}
-__device__ __forceinline__ int wrap1(int c, int n, bool periodic) {  // -n <= c < 2 n
-  return !periodic ? c : c < 0 ? c + n : c >= n ? c - n : c;
-}
-
-// Bulk copy global -> shared (both 16-byte aligned, bytes a multiple of 16).
-__device__ __forceinline__ void bulk_load(double* dst, const double* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-
-__device__ __forceinline__ void put(long long* m, int* e, const WideVal& u) {
-  *m = (long long)(((unsigned long long)(unsigned int)u.hi << 32) | u.lo);
-  *e = u.e;
-}
-__device__ __forceinline__ WideVal get(const long long* m, const int* e) {
-  const long long v = *m;
-  return {(int)(v >> 32), (unsigned int)v, *e};
-}
-__device__ __forceinline__ void get_pair(const long long* m, const int* e, WideVal& a, WideVal& b) {
-  const int4 v = *reinterpret_cast<const int4*>(m);
-  const int2 x = *reinterpret_cast<const int2*>(e);
-  a = {v.y, (unsigned int)v.x, x.x};
-  b = {v.w, (unsigned int)v.z, x.y};
-}
 // Columns c-1 .. c+2 of a row.
 template <int TC>
 __device__ __forceinline__ void get_row(const Plane<TC>& u, int row, int c, WideVal (&v)[4]) {
   v[0] = get(&u.m[row][c - 1], &u.e[row][c - 1]);
   get_pair(&u.m[row][c], &u.e[row][c], v[1], v[2]);
   v[3] = get(&u.m[row][c + 2], &u.e[row][c + 2]);
-}
-
-// Unpacks row `row` of a raw plane (two columns per lane; those at or beyond
-// column `cols` of the tile are the producer's or nobody's).
-template <bool TMA, int TC>
-__device__ __forceinline__ void unpack_row(const double (&raw)[TC + 2][raw_col<TMA>()], const int (&shift)[TC + 2],
-                                           Plane<TC>& u, int row, int lane, int cols, WideVal (&v)[2]) {
-  double2 p;
-  if (TMA) {
-    p = *reinterpret_cast<const double2*>(&raw[row][2 * lane]);
-  } else {
-    const double* r = &raw[row][2 * lane + shift[row]];
-    p = make_double2(r[0], r[1]);
-  }
-  v[0] = wide_unpack(p.x);
-  v[1] = wide_unpack(p.y);
-  if (TMA || 2 * lane + 1 < cols) {
-    *reinterpret_cast<int4*>(&u.m[row][2 + 2 * lane]) = make_int4((int)v[0].lo, v[0].hi, (int)v[1].lo, v[1].hi);
-    *reinterpret_cast<int2*>(&u.e[row][2 + 2 * lane]) = make_int2(v[0].e, v[1].e);
-  } else if (2 * lane < cols) {
-    put(&u.m[row][2 + 2 * lane], &u.e[row][2 + 2 * lane], v[0]);
-  }
 }
 
 // Tap index of offset (dz, dy, dx) in the class's lexicographic tap list.
@@ -176,19 +114,6 @@ __device__ __noinline__ void chain_cells(const Plane<TC>& um, const Plane<TC>& u
       if (!wide_covers(E, T)) out[(int64_t)r * nx + i] = wide_chain(v, wdev, NT);
     }
 }
-
-// A slot and phase that advance plane by plane.
-template <int N>
-struct RingPos {
-  int s = 0;
-  uint32_t ph = 0;
-  __device__ __forceinline__ void next() {
-    if (++s == N) {
-      s = 0;
-      ph ^= 1;
-    }
-  }
-};
 
 template <bool BOX, bool HEAT, bool PERIODIC, bool TMA, int TC>
 __global__ void __launch_bounds__(kThreads, BOX || !TMA ? 2 : 3) k_wide3d(const __grid_constant__ Params P) {
@@ -267,41 +192,17 @@ __global__ void __launch_bounds__(kThreads, BOX || !TMA ? 2 : 3) k_wide3d(const 
                         &S.full[post.s]);
           }
         } else {
-          // lane r copies row r: from the 16-byte boundary at or before column x0
-          // to the one at or after the last column, within the grid; the grid's
-          // first or last element, when it has no whole 16 bytes, by itself
-          const int r = lane;
+          const int r = lane;  // lane r copies row r
           int y = y0 - 1 + r;
           bool in = r < TC + 2 && y <= P.ny && z >= 0 && z < P.nz;
           if (PERIODIC) y = y < 0 ? P.ny - 1 : y >= P.ny ? 0 : y;
           else in = in && y >= 0 && y < P.ny;
-          uint32_t bytes = 0;
-          const double* from = nullptr;
-          int sh = 0;
+          RowCopy cp;
           if (in) {
-            const double* row = P.src + (z * plane + y * pitch + x0);
-            const double* const end = P.src + P.nz * plane;
-            const int n = cols;
-            sh = (int)(((uintptr_t)row >> 3) & 1);
-            from = row - sh;
-            int k0 = 0;
-            if (from < P.src) {  // the grid starts half-way through 16 bytes
-              from += 2;
-              k0 = 2;
-              S.raw[post.s][r][1] = row[0];
-            }
-            int k1 = (sh + n + 1) & ~1;  // one past the last element copied
-            if (from + (k1 - k0) > end) {  // the grid ends half-way through 16 bytes
-              k1 -= 2;
-              S.raw[post.s][r][sh + n - 1] = row[n - 1];
-            }
-            bytes = k1 > k0 ? (uint32_t)(k1 - k0) * 8 : 0;
-            S.shift[post.s][r] = sh;
+            cp.plan(S.raw[post.s][r], P.src + (z * plane + y * pitch + x0), cols, P.src, P.src + P.nz * plane);
             fence_proxy_async_smem();
-            sh = k0;
-          } else if (r < TC + 2) {
-            S.shift[post.s][r] = 0;
           }
+          if (r < TC + 2) S.shift[post.s][r] = cp.shift;
           // rows outside the grid are zeros (those below a ragged tile are not read)
           unsigned int out = __ballot_sync(0xffffffffu, r < TC + 2 && !in);
           while (out) {
@@ -310,11 +211,11 @@ __global__ void __launch_bounds__(kThreads, BOX || !TMA ? 2 : 3) k_wide3d(const 
             S.raw[post.s][q][lane] = 0.0;
             S.raw[post.s][q][lane + 32] = 0.0;
           }
-          const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+          const uint32_t total = __reduce_add_sync(0xffffffffu, cp.bytes);
           __syncwarp();  // the lanes' own writes come before lane 0's arrival
           if (lane == 0) mbar_arrive_expect_tx(&S.full[post.s], total);
           __syncwarp();
-          if (bytes) bulk_load(&S.raw[post.s][r][sh], from, bytes, &S.full[post.s]);
+          if (cp.bytes) bulk_load(&S.raw[post.s][r][cp.to], cp.from, cp.bytes, &S.full[post.s]);
         }
         post.next();
         ++posted;
@@ -366,8 +267,8 @@ __global__ void __launch_bounds__(kThreads, BOX || !TMA ? 2 : 3) k_wide3d(const 
           if (hrow[q] >= 0) put(&u.m[hrow[q]][hcol[q]], &u.e[hrow[q]][hcol[q]], wide_unpack(h[q]));
         if (!wait(&S.full[raw.s], raw.ph)) return leave(j);
         WideVal v[2];
-        unpack_row<TMA, TC>(S.raw[raw.s], S.shift[raw.s], u, 0, lane, cols, v);
-        unpack_row<TMA, TC>(S.raw[raw.s], S.shift[raw.s], u, TC + 1, lane, cols, v);
+        unpack_row<TMA, TC + 2>(S.raw[raw.s], S.shift[raw.s], u, 0, lane, cols, v);
+        unpack_row<TMA, TC + 2>(S.raw[raw.s], S.shift[raw.s], u, TC + 1, lane, cols, v);
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(&S.empty[raw.s]);
@@ -401,7 +302,7 @@ __global__ void __launch_bounds__(kThreads, BOX || !TMA ? 2 : 3) k_wide3d(const 
       if (j < nplanes) {
         if (!wait(&S.full[raw.s], raw.ph)) return;
 #pragma unroll
-        for (int r = 0; r < R; ++r) unpack_row<TMA, TC>(S.raw[raw.s], S.shift[raw.s], S.u[con().s], row0 + r, lane, cols, zp[r]);
+        for (int r = 0; r < R; ++r) unpack_row<TMA, TC + 2>(S.raw[raw.s], S.shift[raw.s], S.u[con().s], row0 + r, lane, cols, zp[r]);
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(&S.empty[raw.s]);

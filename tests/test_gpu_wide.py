@@ -56,6 +56,11 @@ def run(st, u0, w, radius, boundary, T, tuning=(0, 0), offset=0):
 SHAPES3D = [(1, 8, 32), (2, 17, 33), (3, 16, 64), (5, 15, 65), (7, 33, 63), (4, 18, 129), (9, 31, 191), (40, 9, 130)]
 
 
+# the smallest that are streamed (2^17 and 2^21 cells), a last tile of one column and
+# one row, of 63 and 15
+SHAPES3D += [(17, 97, 129), (15, 95, 127), (130, 129, 129)]
+
+
 @pytest.mark.parametrize("kind", ["star", "box"])
 @pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
 @pytest.mark.parametrize("shape", SHAPES3D)
@@ -71,6 +76,23 @@ def test_streaming_any_shape_3d(st, shape, boundary, kind):
         assert np.abs(got - ref).max() <= tol, offset
 
 
+SHAPES2D = [(8, 33), (17, 64), (90, 1460), (1025, 129), (1009, 191), (481, 449), (480, 448), (20, 6593)]
+
+
+@pytest.mark.parametrize("kind,radius", [("star", 2), ("box", 2)])
+@pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
+@pytest.mark.parametrize("shape", SHAPES2D)
+def test_streaming_any_shape_2d(st, shape, boundary, kind, radius):
+    w = weights(kind, 2, radius)
+    u0 = synth.normal(32, shape)
+    T, taps = 3, int(np.count_nonzero(w))
+    ref = oracle.run(u0, w, radius, boundary, T, nthreads=0)
+    tol = T * (2 * taps + 2) * EPS * np.abs(u0).max()
+    for variant, offset in ((st.VARIANT_DIRECT, 0), (st.VARIANT_DIRECT, 1), (0, 0)):
+        got = run(st, u0, w, radius, boundary, T, (1, variant), offset)
+        assert np.abs(got - ref).max() <= tol, (variant, offset)
+
+
 def exact_sum(u, w, at, radius):
     """(sum, largest |product|) of one cell over the reals, zeros outside."""
     total, top = Fraction(0), Fraction(0)
@@ -83,7 +105,7 @@ def exact_sum(u, w, at, radius):
     return total, top
 
 
-WIDE_RANGE = [((6, 9, 33), "star", 1), ((4, 9, 34), "box", 1)]
+WIDE_RANGE = [((6, 9, 33), "star", 1), ((4, 9, 34), "box", 1), ((19, 70), "star", 2), ((19, 70), "box", 2)]
 
 
 @pytest.mark.parametrize("spread", [0, 8, 60, 300])
