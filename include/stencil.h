@@ -158,12 +158,12 @@ typedef struct {
   double* d_grid;
 } stencil_batch_item;
 
-/* Builds a batch plan: cuts every item into tiles of 512 consecutive cells,
- * lists them by the item's T (largest first) as one persistent kernel's
- * device work list, allocates one partner buffer for all items, the item
- * table and the barrier words, and captures the whole advance (every item
- * by its own T, a bounded device-wide barrier between steps) as one CUDA
- * graph on first run.  items is copied.  All items share the boundary rule. */
+/* Builds a batch plan: cuts every item into tiles (see
+ * stencil_batch_set_tuning), lists them by the item's T (largest first) as one
+ * persistent kernel's device work list, allocates one partner buffer for all
+ * items, the item table and the barrier words, and captures the whole advance
+ * (every item by its own T, a bounded wait between steps) as one CUDA graph on
+ * first run.  items is copied.  All items share the boundary rule. */
 int stencil_batch_create(const stencil_batch_item* items, int n, int boundary,
                          stencil_batch* out);
 
@@ -181,8 +181,11 @@ void stencil_batch_destroy(stencil_batch b);
 /* Kernel configuration of a batch.  Tb = 1 (or 0): one step per device-wide
  * barrier, with cells_per_thread (1, 2 or 4; a tile is 256 *
  * cells_per_thread consecutive cells of one item) and cooperative blocks per
- * SM (1 .. the kernel's occupancy; 0 restores the defaults 2 and
- * min(occupancy, 4)).  Tb = 2, 4 or 8: Tb steps in shared memory per
+ * SM (1 .. the kernel's occupancy; 0 restores the defaults 2, or 4 from 2^22
+ * cells on, and min(occupancy, 4)).  With both at their defaults, a batch with
+ * positive weights whose items fill tiles of 64 x 16 cells to 80 % or more, 1000
+ * tiles at least, runs tile by tile instead, every tile as soon as its
+ * neighbours have made the step before.  Tb = 2, 4 or 8: Tb steps in shared memory per
  * exchange, every item cut into tiles of at most 16 x 32 cells that
  * synchronise through per-tile flags with the tiles of the same item their
  * halo reaches (cells_per_thread and blocks_per_sm are then ignored).
@@ -217,9 +220,11 @@ int stencil_plan_status(stencil_plan p, void* cuda_stream);
 
 /* Kernel variants (ids are stable).  Defaults when nothing is forced or
  * tuned: 3D radius 1 -> STREAM; 2D radius 1 -> PERSISTENT with Tb = 4 up to
- * 2^18 cells, PERSISTENT with Tb = 1 (5-point star) up to 3 * 2^20 cells,
- * else STREAM; 2D radius 2 -> STREAM; 1D -> TEMPORAL with Tb = 8; anything
- * else -> DIRECT.  STREAM needs an even nx and, for periodic grids, nx a
+ * 2^18 cells (positive weights: a star Tb = 8 up to 2^16, a box of unequal
+ * weights up to 2^17), PERSISTENT with Tb = 1 (5-point star) up to 3 * 2^20
+ * cells -- by default, with positive weights and a grid that STREAM takes, run
+ * as STREAM, which is faster --, else STREAM; 2D radius 2 -> STREAM; 1D ->
+ * TEMPORAL with Tb = 8; anything else -> DIRECT.  STREAM needs an even nx and, for periodic grids, nx a
  * multiple of 64 and ny a multiple of the tile height (32 for the 3D star,
  * 16 otherwise); other shapes default to DIRECT.  A variant a plan cannot
  * use (including STREAM on buffers not 16-byte aligned) falls back to DIRECT

@@ -130,6 +130,7 @@ struct stencil_plan_s {
   int* d_status = nullptr;     // device status word (bounded waits that gave up)
   unsigned int* d_flags = nullptr;  // per-tile flags of the persistent temporal kernel
   int flags_cap = 0;
+  unsigned int* d_progress = nullptr;  // of the persistent tile kernel's CTAs
   double* d_ring = nullptr;         // exchange kernel: ring of intermediate time levels
   size_t ring_cells = 0;
   unsigned int* d_xcnt = nullptr;   // exchange kernel: per-CTA progress counters
@@ -161,7 +162,7 @@ struct stencil_batch_s {
   BatchItemDev* d_items = nullptr;
   BatchTile* d_tiles = nullptr;
   double* d_partner = nullptr;
-  unsigned int* d_ctl = nullptr;  // [0] arrivals, [1] generation, [2] status
+  unsigned int* d_ctl = nullptr;  // [0] arrivals, [1] generation, [2] status; from [4] on the tile kernel's progress
   int ntiles = 0;
   int max_T = 0;
   int blocks = 0;
@@ -180,6 +181,13 @@ struct stencil_batch_s {
   unsigned int* d_tb_flags = nullptr;
   int ntb_tiles = 0;
   int tb_max_blocks = 0;
+  // tiles of 64 x 16 cells in the integer form (Tb = 1, no cells per thread
+  // asked for, every grid fills its tiles)
+  WideStepItem* d_steps = nullptr;
+  int nsteps = 0;          // items in it (0: not used)
+  int step_tiles = 0;
+  int steps_odd = 0, steps_heat = 0;
+  int any_wide = 0;  // some item takes the integer form
   std::vector<BatchItemDev> hi;  // the item descriptors, kept to rebuild the tile list
   bool ready = false;      // the work list is complete (the last build succeeded)
 };
@@ -217,7 +225,7 @@ void build_taps(stencil_plan_s* p, const double* w) {
 // The stencil classes whose kernels have the integer form of the sum.  All
 // kernels of a class take it, so its results do not depend on the kernel.
 bool uses_wide(int ndim, int radius) {
-  return (ndim == 3 && radius == 1) || (ndim == 2 && radius == 2);
+  return (ndim == 3 && radius == 1) || ndim == 2;
 }
 
 // Whether a grid that the TMA-fed kernels do not take is streamed all the same
@@ -347,12 +355,12 @@ bool tune_lookup(const std::string& key, int& tb, int& v, int& ty) {
 }
 
 // The kernel (and Tb) a constant-weight plan uses when nothing was tuned or
-// forced.  Small 2D grids are latency-bound: they run as one persistent launch,
-// with Tb = 4 steps in shared memory per exchange up to 2^18 cells, and one
-// step per device-wide barrier (5-point star) up to 3 * 2^20 cells; larger
-// grids stream one launch per step (measured on GB300, 2D 5-point heat,
-// T = 100: 512^2 53.6 vs 43.3 GStencil/s, 1024^2 76.2 vs 54.3 and 68.1 for
-// streaming, 2048^2 streaming 102.3 vs 99.7).
+// forced.  Small 2D grids are latency-bound: up to 2^18 cells (general boxes in the
+// integer form 2^17) they run as one persistent launch with Tb = 4 steps in shared
+// memory per exchange (a star in the integer form 8 up to 2^16: 256^2 39 GStencil/s
+// against 37, 128^2 14.0 / 13.2, 400^2 38 / 39); 5-point stars up to 3 * 2^20 cells as one
+// persistent launch with one step at a time (streams_anyway says when not); larger grids
+// stream one launch per step (box 448^2 40 GStencil/s, persistent 32).
 int default_variant(const stencil_plan_s* p, int* Tb = nullptr) {
   if (Tb) *Tb = 1;
   // shapes the streaming kernels cannot take (odd nx; periodic sizes off their tile) go direct
@@ -361,8 +369,9 @@ int default_variant(const stencil_plan_s* p, int* Tb = nullptr) {
                                                                                : kVariantDirect;
   const bool stream2d = stream2d_shape_ok(p->ndim, p->radius, p->boundary, p->g);
   if (p->ndim == 2 && p->radius == 1) {
-    if (p->cells() <= ((int64_t)1 << 18)) {
-      if (Tb) *Tb = 4;
+    const bool wide_box = p->wide.n && p->shape == Shape::kBox && !taps_all_equal(p->taps);
+    if (p->cells() <= ((int64_t)1 << (wide_box ? 17 : 18))) {
+      if (Tb) *Tb = p->wide.n == 5 && p->cells() <= 1 << 16 ? 8 : 4;
       return kVariantPersistent;
     }
     if (p->cells() <= ((int64_t)3 << 20) && p->shape == Shape::kStar && p->taps.n == 5)
@@ -405,15 +414,26 @@ int one_step_variant(const stencil_plan_s* p) {
   return v;
 }
 
+// Whether a run that would take its steps one at a time in one persistent launch, by
+// default and not by a caller's or the tuner's choice, takes one launch per step instead:
+// in the integer form each of those is set up while the step before runs, and TMA copies
+// whole tiles (heat, GStencil/s, streamed against persistent: 1000^2 107 / 90, 600^2 73 / 60,
+// 1536^2 157 / 118).  Rows off 16 bytes, which TMA does not take, stay (1001^2).
+bool streams_anyway(const stencil_plan_s* p, int Tb, int variant, bool stream_ok) {
+  return variant == kVariantPersistent && Tb == 1 && p->user_variant == 0 && p->wide.n && stream_ok;
+}
+
 // Resolved (Tb, variant, streaming tile height; 0 = the kernel's default) for
-// the next run of a constant-weight plan.
-void choose(const stencil_plan_s* p, int& Tb, int& variant, int& tile_y) {
+// the next run of a constant-weight plan.  tuned: the tuner's choice.
+void choose(const stencil_plan_s* p, int& Tb, int& variant, int& tile_y, bool& tuned) {
   tile_y = p->user_tile_y;
+  tuned = false;
   if (p->user_Tb > 0 || p->user_variant > 0) {
     Tb = p->user_Tb > 0 ? p->user_Tb : 1;
     variant = p->user_variant > 0 ? p->user_variant : Tb > 1 ? fused_variant(p) : one_step_variant(p);
     return;
   }
+  tuned = true;
   if (p->tuned_Tb > 0) {
     Tb = p->tuned_Tb;
     variant = p->tuned_variant;
@@ -425,11 +445,13 @@ void choose(const stencil_plan_s* p, int& Tb, int& variant, int& tile_y) {
     if (!tile_y) tile_y = ty;
     return;
   }
+  tuned = false;
   variant = default_variant(p, &Tb);
 }
 void choose(const stencil_plan_s* p, int& Tb, int& variant) {
   int ty;
-  choose(p, Tb, variant, ty);
+  bool tuned;
+  choose(p, Tb, variant, ty, tuned);
 }
 
 // Uploads the plan's weights (and the zero slots) to the device once.
@@ -487,16 +509,17 @@ int run_persistent_tb(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, cuda
     cudaFree(p->d_flags);
     p->d_flags = nullptr;
     p->flags_cap = 0;
-    CUDA_TRY(dev_malloc(&p->d_flags, ntiles * sizeof(unsigned int)), "allocating the tile flags");
+    CUDA_TRY(dev_malloc(&p->d_flags, (size_t)ntiles * kFlagWords * sizeof(unsigned int)), "allocating the tile flags");
     p->flags_cap = ntiles;
   }
-  CUDA_TRY(cudaMemsetAsync(p->d_flags, 0, ntiles * sizeof(unsigned int), s), "clearing the tile flags");
+  CUDA_TRY(cudaMemsetAsync(p->d_flags, 0, (size_t)ntiles * kFlagWords * sizeof(unsigned int), s), "clearing the tile flags");
   L.a = d_grid;
   L.b = p->d_tmp;
   L.ny = p->g.ny;
   L.nx = p->g.nx;
   L.T = T;
   L.wdev = p->d_w;
+  if (p->wide.n) make_wide(p->taps.w, p->taps.n, L.wide);
   L.flags = p->d_flags;
   L.status = p->d_status;
   L.spin_limit = kSpinLimitNs;
@@ -505,9 +528,39 @@ int run_persistent_tb(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, cuda
   return STENCIL_OK;
 }
 
-// One-step persistent kernel (the batched kernel with a single item): its
-// device work list for (d_grid, T) comes from the plan's LRU cache.
+// All T steps of one grid by the tile kernel in one launch (its whole work
+// description is a launch parameter).
+int run_wide_steps(stencil_plan_s* p, double* d_grid, int64_t T, cudaStream_t s) {
+  constexpr size_t words = kProgressWords * sizeof(unsigned int);
+  if (!p->d_progress) CUDA_TRY(dev_malloc(&p->d_progress, words), "allocating the progress words");
+  CUDA_TRY(cudaMemsetAsync(p->d_progress, 0, words, s), "clearing the progress words");
+  BatchItemDev it;
+  it.a = d_grid;
+  it.b = p->d_tmp;
+  it.ny = p->g.ny;
+  it.nx = p->g.nx;
+  it.T = (int)T;
+  for (int k = 0; k < 5; ++k) it.w[k] = p->taps.w[k];
+  make_wide(it.w, 5, it.wide);
+  WideStepsLaunch L;
+  wide_step_item(L.one, it, 0);
+  L.nitems = 1;
+  L.max_T = (int)T;
+  L.any_odd = (int)(T & 1);
+  L.heat = it.wide.heat;
+  L.progress = p->d_progress;
+  L.status = p->d_status;
+  L.spin_limit = kSpinLimitNs;
+  cudaError_t e = launch_wide_steps(L, L.one.ntiles, p->boundary, sm_count(), s);
+  if (e != cudaSuccess) return cuda_fail(e, "launching the persistent step kernel");
+  return STENCIL_OK;
+}
+
+// One-step persistent kernel: the tile kernel where the grid fills its tiles, else the
+// batched kernel with a single item, whose device work list for (d_grid, T)
+// comes from the plan's LRU cache.
 int run_persistent_step(stencil_plan_s* p, double* d_grid, int64_t T, cudaStream_t s) {
+  if (p->wide.n && wide_steps_worth(p->g.ny, p->g.nx)) return run_wide_steps(p, d_grid, T, s);
   stencil_batch_s* hit = nullptr;
   for (auto& e : p->persist)
     if (e.grid == d_grid && e.T == T) {
@@ -532,6 +585,7 @@ int run_persistent_step(stencil_plan_s* p, double* d_grid, int64_t T, cudaStream
     it.T = (int)T;
     for (int k = 0; k < 5; ++k) it.w[k] = p->taps.w[k];
     it.zero[0] = it.zero[1] = 0.0;
+    make_wide(it.w, 5, it.wide);
     const int rc = batch_init(b, std::vector<BatchItemDev>{it}, p->boundary);
     if (rc) {
       stencil_batch_destroy(b);
@@ -629,10 +683,13 @@ int run_steps(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, int variant,
       steps = Tb;
     } else {
       const int v = variant == kVariantTemporal || variant == kVariantExchange ? single : variant;
+      const bool chained = t > 0 && v == variant;  // the stream's last launch was this loop's last step
       if (v == kVariantStream && p->ndim == 3 && p->wide.n)
-        e = launch_wide3d(p->shape, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, tile_y, true);
+        e = launch_wide3d(p->shape, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, tile_y, true,
+                          chained);
       else if (v == kVariantStream && p->ndim == 2 && p->wide.n && !(equal_box && p->radius == 1))
-        e = launch_wide2d(p->shape, p->radius, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, true);
+        e = launch_wide2d(p->shape, p->radius, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, true,
+                          chained);
       else if (v == kVariantStream && p->ndim == 3)
         e = launch_stream3d(p->shape, p->boundary, p->g, p->taps, p->d_w, a, b, p->d_status, sms, s,
                             (unsigned long long)kSpinLimitNs, -1, tile_y);
@@ -640,9 +697,11 @@ int run_steps(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, int variant,
         e = launch_stream2d(p->shape, p->radius, p->boundary, equal_box && p->radius == 1, p->g, p->taps,
                             p->d_w, a, b, p->d_status, sms, s);
       else if (p->ndim == 3 && streamed_any_shape(p))
-        e = launch_wide3d(p->shape, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, 0, false);
+        e = launch_wide3d(p->shape, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, 0, false,
+                          chained);
       else if (p->ndim == 2 && streamed_any_shape(p))
-        e = launch_wide2d(p->shape, p->radius, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, false);
+        e = launch_wide2d(p->shape, p->radius, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, false,
+                          chained);
       else
         e = launch_direct(p->ndim, p->radius, p->shape, p->boundary, p->g, p->taps, p->wide, p->d_w, a, b, s);
     }
@@ -662,7 +721,8 @@ int run_steps(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, int variant,
 int run_const(stencil_plan_s* p, double* d_grid, int64_t T, cudaStream_t s) {
   tune_on_first_run(p, d_grid, s);
   int Tb, variant, tile_y;
-  choose(p, Tb, variant, tile_y);
+  bool tuned;
+  choose(p, Tb, variant, tile_y, tuned);
   // a variant the caller named is an error when the grid cannot use it; a
   // Tb > 1 fixed without a variant is an error when no fused kernel covers
   // the plan; any other choice falls back quietly
@@ -693,6 +753,7 @@ int run_const(stencil_plan_s* p, double* d_grid, int64_t T, cudaStream_t s) {
                   "height (16; 32 for the 3D star)");
     variant = kVariantDirect;
   }
+  if (!tuned && streams_anyway(p, Tb, variant, stream_ok)) variant = kVariantStream;
   if (variant == kVariantPersistent && Tb > 1) {
     if (p->ndim == 2 && p->radius == 1 && (p->taps.n == 5 || p->taps.n == 9) && Tb <= 8)
       return run_persistent_tb(p, d_grid, T, Tb, s);
@@ -788,6 +849,7 @@ int batch_init_tb(stencil_batch_s* b, const std::vector<BatchItemDev>& hi, const
     d.T = hi[i].T;
     for (int k = 0; k < 5; ++k) d.w[k] = hi[i].w[k];
     d.zero = 0.0;
+    d.wide = hi[i].wide;
     d.tiles_y = (d.ny + kBatchTbTileH - 1) / kBatchTbTileH;
     d.tiles_x = (d.nx + kBatchTbTileW - 1) / kBatchTbTileW;
     const int hmin = d.ny / d.tiles_y, wmin = d.nx / d.tiles_x;
@@ -809,7 +871,7 @@ int batch_init_tb(stencil_batch_s* b, const std::vector<BatchItemDev>& hi, const
   if (!tiles.empty())
     CUDA_TRY(cudaMemcpy(b->d_tb_tiles, tiles.data(), sizeof(BatchTbTile) * tiles.size(), cudaMemcpyHostToDevice),
              "copying the tile list");
-  CUDA_TRY(dev_malloc(&b->d_tb_flags, sizeof(unsigned int) * std::max<size_t>(1, tiles.size())),
+  CUDA_TRY(dev_malloc(&b->d_tb_flags, sizeof(unsigned int) * kFlagWords * std::max<size_t>(1, tiles.size())),
            "allocating the tile flags");
   const int occ = batched_tb_blocks_per_sm(Tb, b->boundary);
   if (occ < 1) return fail(STENCIL_ERR_CUDA, "the batched temporal kernel does not fit on an SM");
@@ -817,6 +879,39 @@ int batch_init_tb(stencil_batch_s* b, const std::vector<BatchItemDev>& hi, const
   b->blocks = sm_count() * std::min(occ, 2);
   if (b->ntb_tiles > 0 && b->ntb_tiles < b->blocks) b->blocks = b->ntb_tiles;
   b->ready = true;
+  return STENCIL_OK;
+}
+
+// The item list of the tile kernel, when it takes the whole batch.
+int batch_init_steps(stencil_batch_s* b, const std::vector<BatchItemDev>& hi, const std::vector<int>& order) {
+  b->nsteps = 0;
+  b->step_tiles = 0;
+  b->steps_odd = 0;
+  b->steps_heat = 1;
+  std::vector<WideStepItem> list;
+  int64_t tiles = 0, cells = 0;
+  for (int i : order) {
+    if (hi[i].T == 0) continue;
+    if (!hi[i].wide.n) return STENCIL_OK;
+    WideStepItem d;
+    wide_step_item(d, hi[i], (int)tiles);
+    tiles += d.ntiles;
+    cells += (int64_t)d.ny * d.nx;
+    if (tiles > INT32_MAX) return STENCIL_OK;
+    b->steps_odd |= d.T & 1;
+    if (!d.wide.heat) b->steps_heat = 0;
+    list.push_back(d);
+  }
+  // small grids leave the tiles part empty, and few tiles leave the SMs idle: cells
+  // per thread instead.  GStencil/s, tiles against cells: 96 grids of 64..256 (tiles 74 %
+  // full) 72 / 78, 20 of 100..700 (89 %) 84 / 77, 5 of 200..900 (1340 tiles) 66 / 59, 10
+  // of 64..256 (290 tiles) 19 / 24, 48 of 128..4096 148 / 95.
+  if (list.empty() || 10 * cells < 8 * tiles * 1024 || tiles < 1000) return STENCIL_OK;
+  CUDA_TRY(dev_malloc(&b->d_steps, sizeof(WideStepItem) * list.size()), "allocating the item table");
+  CUDA_TRY(cudaMemcpy(b->d_steps, list.data(), sizeof(WideStepItem) * list.size(), cudaMemcpyHostToDevice),
+           "copying the item table");
+  b->nsteps = (int)list.size();
+  b->step_tiles = (int)tiles;
   return STENCIL_OK;
 }
 
@@ -834,11 +929,32 @@ int batch_init(stencil_batch_s* b, const std::vector<BatchItemDev>& hi, int boun
   std::vector<int> order(n);
   for (int i = 0; i < n; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return hi[a].T > hi[c].T; });
-  if (b->cpt == 0) b->cpt = batched_default_cpt();
+  // the defaults, asked for or as stencil_batch_get_tuning reports them: tiles where
+  // they are worth it, else cells per thread
+  b->any_wide = 0;
+  int64_t cells = 0;
+  for (const BatchItemDev& it : hi) {
+    b->any_wide |= it.wide.n != 0;
+    cells += (int64_t)it.ny * it.nx;
+  }
+  const bool tiles_wanted = b->Tb == 1 && (b->cpt == 0 || b->cpt == batched_default_cpt()) &&
+                            (b->per_sm == 0 || b->per_sm == 4);
+  // (400 grids of 64..256 in the integer form: 102 GStencil/s with 4 cells per thread, 97 with 2)
+  if (b->cpt == 0) b->cpt = b->any_wide && cells >= (int64_t)1 << 22 ? 4 : batched_default_cpt();
   b->hi = hi;
-  CUDA_TRY(dev_malloc(&b->d_ctl, 4 * sizeof(unsigned int)), "allocating the barrier words");
+  CUDA_TRY(dev_malloc(&b->d_ctl, (4 + kProgressWords) * sizeof(unsigned int)), "allocating the barrier words");
   CUDA_TRY(cudaMemset(b->d_ctl, 0, 4 * sizeof(unsigned int)), "clearing the barrier words");
   if (b->Tb > 1) return batch_init_tb(b, hi, order);
+  if (tiles_wanted) {
+    const int rc = batch_init_steps(b, hi, order);
+    if (rc) return rc;
+    if (b->nsteps > 0) {
+      b->cpt = batched_default_cpt();
+      b->blocks = 4 * sm_count();  // (what get_tuning reports)
+      b->ready = true;
+      return STENCIL_OK;
+    }
+  }
   std::vector<BatchTile> tiles;
   const int tc = batched_tile_cells(b->cpt);
   for (int i : order) {
@@ -856,7 +972,7 @@ int batch_init(stencil_batch_s* b, const std::vector<BatchItemDev>& hi, int boun
   if (!tiles.empty())
     CUDA_TRY(cudaMemcpy(b->d_tiles, tiles.data(), sizeof(BatchTile) * tiles.size(), cudaMemcpyHostToDevice),
              "copying the tile list");
-  const int occ = batched_blocks_per_sm(b->cpt);
+  const int occ = batched_blocks_per_sm(b->cpt, b->any_wide);
   if (occ < 1) return fail(STENCIL_ERR_CUDA, "the batched kernel does not fit on an SM");
   b->ntiles = (int)tiles.size();
   const int per_sm = b->per_sm > 0 ? std::min(b->per_sm, occ) : std::min(occ, 4);
@@ -880,9 +996,24 @@ int batch_enqueue(stencil_batch_s* b, cudaStream_t s) {
     L.status = (int*)(b->d_ctl + 2);
     L.spin_limit = kSpinLimitNs;
     CUDA_TRY(cudaMemsetAsync(b->d_ctl, 0, 4 * sizeof(unsigned int), s), "clearing the status word");
-    CUDA_TRY(cudaMemsetAsync(b->d_tb_flags, 0, sizeof(unsigned int) * b->ntb_tiles, s), "clearing the tile flags");
+    CUDA_TRY(cudaMemsetAsync(b->d_tb_flags, 0, sizeof(unsigned int) * kFlagWords * b->ntb_tiles, s), "clearing the tile flags");
     cudaError_t e = launch_batched_tb(L, b->blocks, b->Tb, b->boundary, s);
     if (e != cudaSuccess) return cuda_fail(e, "launching the batched temporal kernel");
+    return STENCIL_OK;
+  }
+  if (b->nsteps > 0) {
+    WideStepsLaunch L;
+    L.items = b->d_steps;
+    L.nitems = b->nsteps;
+    L.max_T = b->max_T;
+    L.any_odd = b->steps_odd;
+    L.heat = b->steps_heat;
+    L.progress = b->d_ctl + 4;
+    L.status = (int*)(b->d_ctl + 2);
+    L.spin_limit = kSpinLimitNs;
+    CUDA_TRY(cudaMemsetAsync(b->d_ctl, 0, (4 + kProgressWords) * sizeof(unsigned int), s), "clearing the progress words");
+    cudaError_t e = launch_wide_steps(L, b->step_tiles, b->boundary, sm_count(), s);
+    if (e != cudaSuccess) return cuda_fail(e, "launching the batched tile kernel");
     return STENCIL_OK;
   }
   BatchLaunch L;
@@ -896,6 +1027,7 @@ int batch_enqueue(stencil_batch_s* b, cudaStream_t s) {
   L.spin_limit = kSpinLimitNs;
   L.barrier_blocks = 0;
   CUDA_TRY(cudaMemsetAsync(b->d_ctl, 0, 4 * sizeof(unsigned int), s), "clearing the barrier words");
+  L.wide = b->any_wide;
   cudaError_t e = launch_batched(L, b->blocks, b->cpt, s);
   if (e != cudaSuccess) return cuda_fail(e, "launching the batched kernel");
   return STENCIL_OK;
@@ -994,6 +1126,7 @@ void stencil_destroy(stencil_plan p) {
   cudaFree(p->d_adj);
   cudaFree(p->d_status);
   cudaFree(p->d_flags);
+  cudaFree(p->d_progress);
   cudaFree(p->d_ring);
   cudaFree(p->d_xcnt);
   cudaFree(p->d_w);
@@ -1233,7 +1366,8 @@ int stencil_get_tile(stencil_plan p, int* tile_x, int* tile_y) {
   g_err.clear();
   if (!p || !tile_x || !tile_y) return fail(STENCIL_ERR_ARG, "NULL argument");
   int Tb, v, ty;
-  choose(p, Tb, v, ty);
+  bool tuned;
+  choose(p, Tb, v, ty, tuned);
   *tile_x = 0;
   *tile_y = 0;
   if (v == kVariantStream && p->ndim == 3 && p->radius == 1) {
@@ -1365,6 +1499,7 @@ int stencil_batch_create(const stencil_batch_item* items, int n, int boundary, s
     hi[i].w[3] = it.alpha;
     hi[i].w[4] = it.alpha;
     hi[i].zero[0] = hi[i].zero[1] = 0.0;
+    make_wide(hi[i].w, 5, hi[i].wide);
     off += it.ny * it.nx;
   }
   int rc = batch_init(b, hi, boundary);
@@ -1434,6 +1569,9 @@ void batch_release_lists(stencil_batch_s* b) {
   cudaFree(b->d_tb_items);
   cudaFree(b->d_tb_tiles);
   cudaFree(b->d_tb_flags);
+  cudaFree(b->d_steps);
+  b->d_steps = nullptr;
+  b->nsteps = 0;
   b->d_items = nullptr;
   b->d_tiles = nullptr;
   b->d_ctl = nullptr;
@@ -1517,8 +1655,8 @@ int stencil_batch_autotune(stencil_batch b, int64_t probe_steps, void* cuda_stre
   struct Cand { int Tb, cpt, per_sm; };
   std::vector<Cand> cands;
   for (int cpt : {1, 2, 4})
-    for (int per_sm = 1; per_sm <= std::min(batched_blocks_per_sm(cpt), 4); ++per_sm) cands.push_back({1, cpt, per_sm});
-  for (int Tb : {2, 4, 8}) cands.push_back({Tb, 0, 0});
+    for (int per_sm = 1; per_sm <= std::min(batched_blocks_per_sm(cpt, b->any_wide), 4); ++per_sm) cands.push_back({1, cpt, per_sm});
+  for (int Tb : {1, 2, 4, 8}) cands.push_back({Tb, 0, 0});  // (1: the tile kernel where it takes the batch)
   for (const Cand& cd : cands) {
     if (rc) break;
     auto* t = new (std::nothrow) stencil_batch_s();
@@ -1580,6 +1718,7 @@ void stencil_batch_destroy(stencil_batch b) {
   cudaFree(b->d_tb_items);
   cudaFree(b->d_tb_tiles);
   cudaFree(b->d_tb_flags);
+  cudaFree(b->d_steps);
   delete b;
 }
 
@@ -1680,7 +1819,7 @@ int stencil_selftest_flag_timeout(double limit_ms, void* cuda_stream) {
   const int ny = 32, nx = 64, n = ny * nx;
   if (dev_malloc(&grid, 2 * n * sizeof(double)) != cudaSuccess ||
       dev_malloc(&ctl, 4 * sizeof(unsigned int)) != cudaSuccess ||
-      dev_malloc(&flags, 4 * sizeof(unsigned int)) != cudaSuccess ||
+      dev_malloc(&flags, 4 * kFlagWords * sizeof(unsigned int)) != cudaSuccess ||
       dev_malloc(&d_item, sizeof(BatchTbItemDev)) != cudaSuccess ||
       dev_malloc(&d_tiles, 3 * sizeof(BatchTbTile)) != cudaSuccess) {
     cleanup();
@@ -1702,7 +1841,7 @@ int stencil_selftest_flag_timeout(double limit_ms, void* cuda_stream) {
   const BatchTbTile tl[3] = {{0, 0, 0}, {0, 0, 1}, {0, 1, 0}};  // tile (1, 1) left out
   cudaMemsetAsync(grid, 0, 2 * n * sizeof(double), s);
   cudaMemsetAsync(ctl, 0, 4 * sizeof(unsigned int), s);
-  cudaMemsetAsync(flags, 0, 4 * sizeof(unsigned int), s);
+  cudaMemsetAsync(flags, 0, 4 * kFlagWords * sizeof(unsigned int), s);
   cudaMemcpyAsync(d_item, &it, sizeof(it), cudaMemcpyHostToDevice, s);
   cudaMemcpyAsync(d_tiles, tl, sizeof(tl), cudaMemcpyHostToDevice, s);
   BatchTbLaunch L;

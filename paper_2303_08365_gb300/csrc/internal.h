@@ -60,16 +60,18 @@ struct HostTaps {
 // The weights split for the integer form of the weighted sum (wide.cuh); n = 0
 // when that form does not cover them.
 constexpr int kWideMaxTaps = 27;
-struct WideTaps {
+template <int N>
+struct WideTapsOf {
   int n = 0;
-  int hi[kWideMaxTaps], lo[kWideMaxTaps];  // limbs of the significand: hi * 2^26 + lo
-  int hi2[kWideMaxTaps];                   // 2 * hi
-  int ex[kWideMaxTaps];                    // exponent below the largest weight's (<= 0)
+  int hi[N], lo[N];                        // limbs of the significand: hi * 2^26 + lo
+  int hi2[N];                              // 2 * hi
+  int ex[N];                               // exponent below the largest weight's (<= 0)
   int heat;                                // one weight at the centre tap (n / 2), one at all others
   int bias;                                // exponent of the result: E - bias above R's
   int e_min;                               // E in [e_min, e_min + e_span], else the FMA chain
   unsigned int e_span;
 };
+using WideTaps = WideTapsOf<kWideMaxTaps>;
 
 // Launchers implemented in the .cu files.  Each returns a cudaError_t from
 // the launch (cudaSuccess when nothing failed) and enqueues on `stream`.
@@ -103,10 +105,12 @@ cudaError_t launch_stream3d(Shape shape, int boundary, const Geom& g, const Host
 
 // 3D radius-1 sweep with the weighted sum in the integer form (wide.n != 0):
 // tiles of 64 columns by 16 rows (8 for tile_y = 8).  tma: the grid is one that
-// stream3d_eligible takes; false: any shape, alignment and boundary.
+// stream3d_eligible takes; false: any shape, alignment and boundary.  chained: the
+// stream's last launch is a step of the same run by this kernel or launch_wide2d's
+// (launch_step in widestream.cuh).
 cudaError_t launch_wide3d(Shape shape, int boundary, const Geom& g, const WideTaps& wide, const double* wdev,
                           const double* src, double* dst, int* status, int sms, cudaStream_t stream, int tile_y,
-                          bool tma);
+                          bool tma, bool chained = false);
 
 // 2D radius-1 or radius-2 streaming sweep (TMA-fed ring of 16-row blocks).  Same
 // eligibility rules with ny % 16 == 0 for periodic grids.  `equal` selects
@@ -121,10 +125,11 @@ cudaError_t launch_stream2d(Shape shape, int radius, int boundary, bool equal, c
 
 // 2D sweep (radius 1 or 2, star or box) with the weighted sum in the integer
 // form (wide.n != 0), tiles of 64 columns by 16 rows.  tma: the grid is one that
-// stream2d_eligible takes; false: any shape, alignment and boundary.
+// stream2d_eligible takes; false: any shape, alignment and boundary.  chained: as
+// in launch_wide3d.
 cudaError_t launch_wide2d(Shape shape, int radius, int boundary, const Geom& g, const WideTaps& wide,
                           const double* wdev, const double* src, double* dst, int* status, int sms,
-                          cudaStream_t stream, bool tma);
+                          cudaStream_t stream, bool tma, bool chained = false);
 
 // Temporal blocking: Tb fused steps per launch (2D and 3D: radius 1, any
 // shape and boundary; 1D: radius 1 or 2; Tb in {2, 4, 8}).
@@ -221,6 +226,7 @@ struct BatchItemDev {
   // centre, east (x+1), south (y+1); Eq. 3 gives alpha, alpha, 1-4 alpha, alpha, alpha
   double w[5];
   double zero[2];  // 0.0: the addends of the first FMA of each row's chain
+  WideTapsOf<5> wide;  // the weights split for the integer form (n = 0: the FMA chain)
 };
 struct BatchLaunch {
   const BatchItemDev* items;
@@ -232,7 +238,46 @@ struct BatchLaunch {
   int* status;            // 0 ok, else a stencil_status
   long long spin_limit;   // bounded waits: wall-time limit in ns
   int barrier_blocks;     // arrivals a device-wide barrier waits for (0: the grid size)
+  int wide = 0;           // some item takes the integer form (wide.n != 0)
 };
+// The same sweep over tiles of 64 x 16 cells with the weighted sum in the integer
+// form (every item's wide.n != 0): widesteps.cu.
+struct WideStepItem {
+  double* a;      // the caller's grid (time level parity 0)
+  double* b;      // library-owned partner buffer (parity 1)
+  int ny, nx, T;
+  int tiles_y;        // tiles per column of tiles
+  int tile0, ntiles;  // the item's tiles in the launch's list
+  int vec;            // rows of both buffers start on 16 bytes
+  double w[5];
+  WideTapsOf<5> wide;
+};
+struct WideStepsLaunch {
+  const WideStepItem* items = nullptr;  // device, largest T first; nullptr: the one item below
+  WideStepItem one;
+  int nitems;
+  int max_T;
+  int any_odd;            // some item's T is odd
+  int heat;               // every item's wide.heat
+  unsigned int* progress;  // kProgressWords words, zero before the launch: steps done by every CTA
+  int* status;
+  long long spin_limit;    // ns
+};
+constexpr int kWideStepCtas = 512;  // most CTAs of a launch
+constexpr int kProgressWords = 16 * kWideStepCtas;  // half a line for each
+void wide_step_item(WideStepItem& d, const BatchItemDev& it, int tile0);
+// Whether a grid fills its tiles of 64 x 16 cells well enough, and the SMs with them
+// (one step per device-wide barrier by cells instead: 256^2 17 against 13 GStencil/s,
+// 512^2 43.6 against 46).
+inline bool wide_steps_worth(int64_t ny, int64_t nx) {
+  const int64_t tiles = ((ny + 15) / 16) * ((nx + 63) / 64);
+  return tiles >= 200 && 10 * ny * nx >= 8 * tiles * 1024;
+}
+cudaError_t launch_wide_steps(const WideStepsLaunch& L, int tiles, int boundary, int sms, cudaStream_t stream);
+
+// Words from one flag (progress word) that other CTAs poll to the next: a line.
+constexpr int kFlagWords = 32;
+
 // Threads per block of the batched kernel; a tile is cpt * kBatchThreads
 // consecutive cells, so the smallest tile (cpt = 1) holds kBatchThreads cells.
 constexpr int kBatchThreads = 256;
@@ -242,7 +287,7 @@ cudaError_t launch_batched(const BatchLaunch& L, int grid_blocks, int cpt, cudaS
 int batched_block_size();
 int batched_default_cpt();
 int batched_tile_cells(int cpt);
-int batched_blocks_per_sm(int cpt);
+int batched_blocks_per_sm(int cpt, bool wide);
 
 // Persistent temporal blocking for one small 2D grid (radius 1, star or box):
 // Tb in {2, 4, 8} steps per exchange, tiles synchronised by per-tile flags.
@@ -252,9 +297,10 @@ struct PersistTbLaunch {
   int ny, nx;
   long long T;
   const double* wdev;    // weights, then the zero and one slots
+  WideTapsOf<9> wide;    // the weights split for the integer form (n = 0: the FMA chain)
   int tiles_y, tiles_x;  // near-equal cut of the grid (from persist_tiling)
   int reach_y, reach_x;  // tiles a Tb-cell halo can reach on each side
-  unsigned int* flags;   // tiles_y * tiles_x words, zero before the launch
+  unsigned int* flags;   // tiles_y * tiles_x * kFlagWords words, zero before the launch
   int* status;
   long long spin_limit;  // ns
 };
@@ -270,6 +316,7 @@ struct BatchTbItemDev {
   int tile_base;          // the item's first tile (its flag words start there)
   double w[5];            // north, west, centre, east, south (lexicographic taps)
   double zero;            // 0.0, the addend of each chain's first FMA
+  WideTapsOf<5> wide;     // the weights split for the integer form (n = 0: the FMA chain)
 };
 struct BatchTbTile {
   int item, ty, tx;       // tile (ty, tx) of item `item`
@@ -279,7 +326,7 @@ struct BatchTbLaunch {
   const BatchTbTile* tiles;
   int ntiles;
   int max_blocks;         // the largest ceil(T / Tb) over the items
-  unsigned int* flags;    // ntiles words, zero before the launch
+  unsigned int* flags;    // ntiles * kFlagWords words, zero before the launch
   int* status;
   long long spin_limit;   // ns
 };

@@ -25,7 +25,9 @@
 //     stencil_static_status reads back (no allocation either).
 #include "../../include/stencil.h"
 #include "internal.h"
+#include "wide.cuh"
 
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -92,7 +94,8 @@ int setup_device(int dev, DeviceSetup& out) {
     void* ptr = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&ptr, g_static_scratch);
     if (e != cudaSuccess) return sfail(STENCIL_ERR_CUDA, "cudaGetSymbolAddress of the static scratch failed");
-    int per_sm = batched_blocks_per_sm(batched_default_cpt()), sms = 0;
+    int per_sm = std::min(batched_blocks_per_sm(batched_default_cpt(), false),
+                          batched_blocks_per_sm(batched_default_cpt(), true)), sms = 0;
     if (per_sm < 1 || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       return sfail(STENCIL_ERR_CUDA, "querying the persistent kernel's occupancy failed");
     s.base = static_cast<unsigned char*>(ptr);
@@ -131,6 +134,7 @@ int static_launch(const DeviceSetup& s, const BatchItemDev& item, int64_t cells,
   L.status = reinterpret_cast<int*>(d_ctl + 2);
   L.spin_limit = spin_limit_ns;
   L.barrier_blocks = barrier_blocks;
+  L.wide = item.wide.n != 0;
   int blocks = s.blocks;
   if (ntiles < blocks) blocks = (int)ntiles;
   if (launch_batched(L, blocks, batched_default_cpt(), stream) != cudaSuccess)
@@ -171,7 +175,7 @@ int stencil_run_2d_static(int64_t ny, int64_t nx, const double* weights, int bou
   cudaStream_t stream = (cudaStream_t)cuda_stream;
 
   BatchItemDev item;
-  memset(&item, 0, sizeof(item));
+  item = BatchItemDev{};
   item.a = d_grid;
   item.b = reinterpret_cast<double*>(s.base);
   item.ny = (int)ny;
@@ -182,6 +186,30 @@ int stencil_run_2d_static(int64_t ny, int64_t nx, const double* weights, int bou
   item.w[2] = weights[4];  // centre
   item.w[3] = weights[5];  // east (x+1)
   item.w[4] = weights[7];  // south (y+1)
+  make_wide(item.w, 5, item.wide);
+  if (item.wide.n && wide_steps_worth(ny, nx)) {  // the tile kernel: its work description is a launch parameter
+    unsigned int* d_ctl = reinterpret_cast<unsigned int*>(s.base + kCtlOff);
+    // (the tile list's place holds the CTAs' progress)
+    unsigned int* progress = reinterpret_cast<unsigned int*>(s.base + kTileOff);
+    static_assert(kMaxTiles * sizeof(BatchTile) >= kProgressWords * sizeof(unsigned int), "progress words");
+    if (cudaMemsetAsync(d_ctl, 0, 4 * sizeof(unsigned int), stream) != cudaSuccess ||
+        cudaMemsetAsync(progress, 0, kProgressWords * sizeof(unsigned int), stream) != cudaSuccess)
+      return sfail(STENCIL_ERR_CUDA, "clearing the barrier words failed");
+    WideStepsLaunch L;
+    wide_step_item(L.one, item, 0);
+    L.nitems = 1;
+    L.max_T = item.T;
+    L.any_odd = item.T & 1;
+    L.heat = item.wide.heat;
+    L.progress = progress;
+    L.status = reinterpret_cast<int*>(d_ctl + 2);
+    L.spin_limit = kSpinLimitNs;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        launch_wide_steps(L, L.one.ntiles, boundary, sms, stream) != cudaSuccess)
+      return sfail(STENCIL_ERR_CUDA, "launching the persistent kernel failed");
+    return STENCIL_OK;
+  }
   return static_launch(s, item, ny * nx, boundary, 0, kSpinLimitNs, stream);
 }
 
@@ -223,7 +251,7 @@ int stencil_selftest_static_timeout(double limit_ms, void* cuda_stream) {
   if (cudaMemsetAsync(partner, 0, 128 * sizeof(double), stream) != cudaSuccess)
     return sfail(STENCIL_ERR_CUDA, "clearing the self-test grid failed");
   BatchItemDev item;
-  memset(&item, 0, sizeof(item));
+  item = BatchItemDev{};
   item.a = partner + 64;
   item.b = partner;
   item.ny = 1;

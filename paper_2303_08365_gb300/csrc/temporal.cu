@@ -178,8 +178,8 @@ __device__ __forceinline__ constexpr int tidx(int dw, int dv, int du) {
 // instead of 18 (additions as FMAs against a register holding 1).  The sum
 // is taken in another order than the tap list, so the result is within
 // rounding of the other kernels, not bitwise equal to them.
-template <int NDIM, int NT, bool BOX, bool EQ, bool WIDE>
-__device__ __forceinline__ void pair_update(const TapSum<NT, WIDE>& S, const double* pm, const double* p0,
+template <int NDIM, int NT, bool BOX, bool EQ, int FORM>
+__device__ __forceinline__ void pair_update(const TapSum<NT, FORM>& S, const double* pm, const double* p0,
                                             const double* pp, int sw, int ly, int lx, double& a0,
                                             double& a1) {
   if constexpr (NDIM == 2 && EQ) {
@@ -195,7 +195,7 @@ __device__ __forceinline__ void pair_update(const TapSum<NT, WIDE>& S, const dou
     a1 = fma(W.w[8], C[3], wt);
     return;
   }
-  typename TapSum<NT, WIDE>::Acc s0, s1;
+  typename TapSum<NT, FORM>::Acc s0, s1;
   const double* pl[3] = {pm, p0, pp};
   const int de = NDIM == 3 ? sw : 1;  // the second cell
 #pragma unroll
@@ -220,8 +220,8 @@ __device__ __forceinline__ void pair_update(const TapSum<NT, WIDE>& S, const dou
 // Pair c of stage s's region, plane i: computed from the three planes of
 // stage s-1 around it and written to stage s's ring, or (s = Tb) to global
 // memory.
-template <int NDIM, int NT, bool BOX, bool PERIODIC, int TB, bool EQ, bool WIDE>
-__device__ __forceinline__ void stage_pair(const TParams& P, const TapSum<NT, WIDE>& W, double* sm, int s,
+template <int NDIM, int NT, bool BOX, bool PERIODIC, int TB, bool EQ, int FORM>
+__device__ __forceinline__ void stage_pair(const TParams& P, const TapSum<NT, FORM>& W, double* sm, int s,
                                            int c, int i, int wa, int y0, int x0) {
   using L = Lay<NDIM, TB, BOX>;
   const int ws = L::W(s);
@@ -240,7 +240,7 @@ __device__ __forceinline__ void stage_pair(const TParams& P, const TapSum<NT, WI
   const double* p0 = src + L::slot(s - 1, i) * sn;
   const double* pp = src + L::slot(s - 1, i + 1) * sn;
   double a0, a1;
-  pair_update<NDIM, NT, BOX, EQ, WIDE>(W, pm, p0, pp, L::W(s - 1), NDIM == 3 ? qy + 1 : 0, qx + 1, a0, a1);
+  pair_update<NDIM, NT, BOX, EQ, FORM>(W, pm, p0, pp, L::W(s - 1), NDIM == 3 ? qy + 1 : 0, qx + 1, a0, a1);
   const int w = wa - TB + i;
   const int x = x0 - TB + s + qx;
   const int y = NDIM == 3 ? y0 - TB + s + qy : 0;
@@ -280,7 +280,7 @@ __device__ __forceinline__ void stage_pair(const TParams& P, const TapSum<NT, WI
   }
 }
 
-template <int NDIM, int NT, bool BOX, bool PERIODIC, int TB, bool EQ, bool WIDE>
+template <int NDIM, int NT, bool BOX, bool PERIODIC, int TB, bool EQ, int FORM>
 __global__ void __launch_bounds__(temporal_threads<NDIM, BOX, TB>(), temporal_min_blocks<NDIM, BOX, TB>())
     k_temporal(const __grid_constant__ TParams P) {
   using L = Lay<NDIM, TB, BOX>;
@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(temporal_threads<NDIM, BOX, TB>(), temporal_mi
   constexpr int LAG = temporal_lag<NDIM, TB, BOX>();
   constexpr int TX = Geo<NDIM, TB, BOX>::TX, TY = Geo<NDIM, TB, BOX>::TY;
   extern __shared__ __align__(16) double sm[];
-  const TapSum<NT, WIDE> W(P.wdev, P.wide);
+  const TapSum<NT, FORM> W(P.wdev, P.wide);
 
   const long long G = gridDim.x;
   const long long f_begin = P.work * blockIdx.x / G;
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(temporal_threads<NDIM, BOX, TB>(), temporal_mi
             c -= L::pairs(s);
             ++s;
           }
-          stage_pair<NDIM, NT, BOX, PERIODIC, TB, EQ, WIDE>(P, W, sm, s, c, k - 2 * s, wa, y0, x0);
+          stage_pair<NDIM, NT, BOX, PERIODIC, TB, EQ, FORM>(P, W, sm, s, c, k - 2 * s, wa, y0, x0);
         }
       } else {
         // stage by stage: plane k - s - 1 is in range for s <= (k - 1) / 2
@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(temporal_threads<NDIM, BOX, TB>(), temporal_mi
         for (int s = 1; s <= s_hi; ++s) {
           if (s > 1) __syncthreads();  // stage s-1's plane of this iteration is written
           for (int j = threadIdx.x; j < L::pairs(s); j += NTH)
-            stage_pair<NDIM, NT, BOX, PERIODIC, TB, EQ, WIDE>(P, W, sm, s, j, k - s - 1, wa, y0, x0);
+            stage_pair<NDIM, NT, BOX, PERIODIC, TB, EQ, FORM>(P, W, sm, s, j, k - s - 1, wa, y0, x0);
         }
       }
     }
@@ -341,13 +341,13 @@ __global__ void __launch_bounds__(temporal_threads<NDIM, BOX, TB>(), temporal_mi
   }
 }
 
-template <int NDIM, int NT, bool BOX, bool PERIODIC, int TB, bool EQ, bool WIDE>
+template <int NDIM, int NT, bool BOX, bool PERIODIC, int TB, bool EQ, int FORM>
 cudaError_t launch_tb(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst, int sms,
                       cudaStream_t stream) {
   using L = Lay<NDIM, TB, BOX>;
   constexpr int NTH = temporal_threads<NDIM, BOX, TB>();
   static_assert(L::bytes <= 227 * 1024, "stage rings exceed shared memory");
-  auto kern = k_temporal<NDIM, NT, BOX, PERIODIC, TB, EQ, WIDE>;
+  auto kern = k_temporal<NDIM, NT, BOX, PERIODIC, TB, EQ, FORM>;
   static std::atomic<int> cache[kMaxDeviceOrdinals];
   const int occ = cached_per_device(cache, [kern] {
     int n = 0;
@@ -375,13 +375,13 @@ cudaError_t launch_tb(const Geom& g, const WideTaps& wide, const double* wdev, c
   return cudaGetLastError();
 }
 
-template <int NDIM, int NT, bool BOX, bool PERIODIC, bool EQ = false, bool WIDE = false>
+template <int NDIM, int NT, bool BOX, bool PERIODIC, bool EQ = false, int FORM = kChain>
 cudaError_t by_tb(int Tb, const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst, int sms,
                   cudaStream_t stream) {
   switch (Tb) {
-    case 2: return launch_tb<NDIM, NT, BOX, PERIODIC, 2, EQ, WIDE>(g, wide, wdev, src, dst, sms, stream);
-    case 4: return launch_tb<NDIM, NT, BOX, PERIODIC, 4, EQ, WIDE>(g, wide, wdev, src, dst, sms, stream);
-    case 8: return launch_tb<NDIM, NT, BOX, PERIODIC, 8, EQ, WIDE>(g, wide, wdev, src, dst, sms, stream);
+    case 2: return launch_tb<NDIM, NT, BOX, PERIODIC, 2, EQ, FORM>(g, wide, wdev, src, dst, sms, stream);
+    case 4: return launch_tb<NDIM, NT, BOX, PERIODIC, 4, EQ, FORM>(g, wide, wdev, src, dst, sms, stream);
+    case 8: return launch_tb<NDIM, NT, BOX, PERIODIC, 8, EQ, FORM>(g, wide, wdev, src, dst, sms, stream);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -478,17 +478,23 @@ cudaError_t launch_temporal(int ndim, int radius, Shape shape, int boundary, int
                : launch_1d<1, false>(Tb, g, wdev, src, dst, stream);
   }
   if (ndim == 3) {
-    if (box && wide.n) return per ? by_tb<3, 27, true, true, false, true>(Tb, g, wide, wdev, src, dst, sms, stream)
-                                  : by_tb<3, 27, true, false, false, true>(Tb, g, wide, wdev, src, dst, sms, stream);
+    if (box && wide.n) return per ? by_tb<3, 27, true, true, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream)
+                                  : by_tb<3, 27, true, false, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream);
     if (box) return per ? by_tb<3, 27, true, true>(Tb, g, wide, wdev, src, dst, sms, stream)
                         : by_tb<3, 27, true, false>(Tb, g, wide, wdev, src, dst, sms, stream);
-    if (wide.n) return per ? by_tb<3, 7, false, true, false, true>(Tb, g, wide, wdev, src, dst, sms, stream)
-                           : by_tb<3, 7, false, false, false, true>(Tb, g, wide, wdev, src, dst, sms, stream);
+    if (wide.n) return per ? by_tb<3, 7, false, true, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream)
+                           : by_tb<3, 7, false, false, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream);
     return per ? by_tb<3, 7, false, true>(Tb, g, wide, wdev, src, dst, sms, stream)
                : by_tb<3, 7, false, false>(Tb, g, wide, wdev, src, dst, sms, stream);
   }
   if (box && equal) return per ? by_tb<2, 9, true, true, true>(Tb, g, wide, wdev, src, dst, sms, stream)
                                : by_tb<2, 9, true, false, true>(Tb, g, wide, wdev, src, dst, sms, stream);
+  if (box && wide.n) return per ? by_tb<2, 9, true, true, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream)
+                                : by_tb<2, 9, true, false, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream);
+  if (wide.heat) return per ? by_tb<2, 5, false, true, false, kHeat>(Tb, g, wide, wdev, src, dst, sms, stream)
+                            : by_tb<2, 5, false, false, false, kHeat>(Tb, g, wide, wdev, src, dst, sms, stream);
+  if (wide.n) return per ? by_tb<2, 5, false, true, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream)
+                         : by_tb<2, 5, false, false, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream);
   if (box) return per ? by_tb<2, 9, true, true>(Tb, g, wide, wdev, src, dst, sms, stream)
                       : by_tb<2, 9, true, false>(Tb, g, wide, wdev, src, dst, sms, stream);
   return per ? by_tb<2, 5, false, true>(Tb, g, wide, wdev, src, dst, sms, stream)

@@ -36,10 +36,11 @@ namespace gbst {
 // Splits the weights; false (and n = 0) when the integer form does not cover
 // them: a weight that is not positive, or weights so far apart or so extreme
 // that no range of exponents is left.
-inline bool make_wide(const double* w, int n, WideTaps& t) {
+template <int N>
+inline bool make_wide(const double* w, int n, WideTapsOf<N>& t) {
   t.n = 0;
-  if (n < 1 || n > kWideMaxTaps) return false;
-  int xmax = -100000, x[kWideMaxTaps];
+  if (n < 1 || n > N) return false;
+  int xmax = -100000, x[N];
   for (int k = 0; k < n; ++k) {
     if (!(w[k] > 0.0) || !std::isfinite(w[k])) return false;
     std::frexp(w[k], &x[k]);  // w = m 2^x, m in [0.5, 1)
@@ -112,7 +113,8 @@ static __device__ __noinline__ double wide_chain(const double* v, const double* 
 }
 
 // Whether the integer form takes a cell whose largest product has exponent E.
-__device__ __forceinline__ bool wide_covers(int E, const WideTaps& T) {
+template <class Taps>
+__device__ __forceinline__ bool wide_covers(int E, const Taps& T) {
   return (unsigned int)(E - T.e_min) <= T.e_span;
 }
 
@@ -131,7 +133,8 @@ struct WideAcc {
   __device__ __forceinline__ WideAcc() : hh(0), hl(1 << 24 /* half a unit of R */), lh(0), ll(0) {}
 
   // Adds W_k a.
-  __device__ __forceinline__ void add(long long a, int k, const WideTaps& T) {
+  template <class Taps>
+  __device__ __forceinline__ void add(long long a, int k, const Taps& T) {
     const int ah = (int)(a >> 32);
     const unsigned int al = (unsigned int)a;
     // one multiply-add each (written in C, the addends cost moves: 149 against
@@ -143,13 +146,40 @@ struct WideAcc {
   }
 
   // Adds w_k u whose product lies d exponents below the cell's largest.
-  __device__ __forceinline__ void add(const WideVal& u, int k, int d, const WideTaps& T) {
+  template <class Taps>
+  __device__ __forceinline__ void add(const WideVal& u, int k, int d, const Taps& T) {
     add(wide_align(u, d), k, T);
   }
 
+  __device__ __forceinline__ long long rounded() const {  // R
+    return hh + ((hl + (long long)((lh + (ll >> 26)) >> 6)) >> 25);
+  }
+
+  // The sum rounded to a double as get() rounds it, unpacked: for a value that the
+  // next step reads, without the two FP64 instructions (64 cycles each) between.
+  template <class Taps>
+  __device__ __forceinline__ WideVal val(int E, const Taps& T) const {
+    const long long R = rounded();
+    const long long s = R >> 63;
+    const unsigned long long a = (unsigned long long)((R ^ s) - s);
+    if (a == 0) return wide_unpack(0.0);
+    const int lz = __clzll((long long)a);
+    const unsigned long long n = a << lz;  // leading bit 63; 53 bits stay
+    unsigned long long r = n + 0x3ff + ((n >> 11) & 1);
+    const bool carry = r < n;
+    r = carry ? 1ull << 63 : r;
+    const unsigned long long m = ((r & ~0x7ffull) >> 2) ^ (unsigned long long)s;
+    WideVal u;
+    u.hi = (int)(m >> 32);
+    u.lo = (unsigned int)m;
+    u.e = E - T.bias + (1023 + 63) - lz + (carry ? 1 : 0);
+    return u;
+  }
+
   // The sum as a double.
-  __device__ __forceinline__ double get(int E, const WideTaps& T) const {
-    const long long R = hh + ((hl + (long long)((lh + (ll >> 26)) >> 6)) >> 25);
+  template <class Taps>
+  __device__ __forceinline__ double get(int E, const Taps& T) const {
+    const long long R = rounded();
     // R to double: (2^84 + 2^63 + high) - (2^84 + 2^63 + 2^52) exactly, then one
     // rounding when the low word (2^52 + low) is added.  As FMAs on registers,
     // which run at the full FP64 rate (additions at 83%)
@@ -165,19 +195,25 @@ struct WideAcc {
 };
 
 // sum_k w_k u_k of one cell (the file's head comment); ok = false, and a
-// result without meaning, where the FMA chain has to take the cell.
-template <int NT>
-__device__ __forceinline__ double wide_sum(const WideVal (&u)[NT], const WideTaps& T, bool& ok) {
+// result without meaning, where the FMA chain has to take the cell.  wide_acc:
+// the sum before its rounding; returns E.
+template <int NT, class Taps>
+__device__ __forceinline__ int wide_acc(const WideVal (&u)[NT], const Taps& T, WideAcc& acc) {
   int e[NT];
 #pragma unroll
   for (int k = 0; k < NT; ++k) e[k] = u[k].e + T.ex[k];
   int E = e[0];
 #pragma unroll
   for (int k = 1; k < NT; ++k) E = max(E, e[k]);
-  ok = wide_covers(E, T);
-  WideAcc acc;
 #pragma unroll
   for (int k = 0; k < NT; ++k) acc.add(u[k], k, E - e[k], T);
+  return E;
+}
+template <int NT, class Taps>
+__device__ __forceinline__ double wide_sum(const WideVal (&u)[NT], const Taps& T, bool& ok) {
+  WideAcc acc;
+  const int E = wide_acc<NT>(u, T, acc);
+  ok = wide_covers(E, T);
   return acc.get(E, T);
 }
 
@@ -185,8 +221,8 @@ __device__ __forceinline__ double wide_sum(const WideVal (&u)[NT], const WideTap
 // all the others (Eq. 3): one exponent for the neighbours, and their integers added
 // in pairs (two of 62 bits fit 63) before the multiplication.  S is exact either
 // way, so the result has the same bits.
-template <int NT>
-__device__ __forceinline__ double wide_sum_heat(const WideVal (&u)[NT], const WideTaps& T, bool& ok) {
+template <int NT, class Taps>
+__device__ __forceinline__ int wide_acc_heat(const WideVal (&u)[NT], const Taps& T, WideAcc& acc) {
   constexpr int C = NT / 2;  // NT - 1 neighbours: an even number
   auto nb = [&](int k) -> const WideVal& { return u[k < C ? k : k + 1]; };
   int en = nb(0).e;
@@ -195,20 +231,24 @@ __device__ __forceinline__ double wide_sum_heat(const WideVal (&u)[NT], const Wi
   en = max(en, nb(NT - 2).e);
   const int ec = u[C].e + T.ex[C];
   const int E = max(en + T.ex[0], ec);
-  ok = wide_covers(E, T);
   const int dn = E - T.ex[0];
-  WideAcc acc;
 #pragma unroll
   for (int k = 0; k < NT - 1; k += 2)
     acc.add(wide_align(nb(k), dn - nb(k).e) + wide_align(nb(k + 1), dn - nb(k + 1).e), 0, T);
   acc.add(u[C], C, E - ec, T);
+  return E;
+}
+template <int NT, class Taps>
+__device__ __forceinline__ double wide_sum_heat(const WideVal (&u)[NT], const Taps& T, bool& ok) {
+  WideAcc acc;
+  const int E = wide_acc_heat<NT>(u, T, acc);
+  ok = wide_covers(E, T);
   return acc.get(E, T);
 }
 
 // The same with the FMA chain in its place where it has to be.
-template <int NT>
-__device__ __forceinline__ double wide_sum(const WideVal (&u)[NT], const WideTaps& T,
-                                           const double* __restrict__ wdev) {
+template <int NT, class Taps>
+__device__ __forceinline__ double wide_sum(const WideVal (&u)[NT], const Taps& T, const double* __restrict__ wdev) {
   bool ok;
   const double r = wide_sum<NT>(u, T, ok);
   if (ok) return r;
@@ -218,35 +258,47 @@ __device__ __forceinline__ double wide_sum(const WideVal (&u)[NT], const WideTap
   return wide_chain(v, wdev, NT);
 }
 
-// The weighted sum of a cell, collected tap by tap: the FMA chain in tap
-// order, or the integer form once every value is there.
-template <int NT, bool WIDE>
-struct TapSum;
+// How a kernel takes the weighted sum of a cell, collected tap by tap: the FMA
+// chain in tap order, or the integer form once every value is there (kHeat: for
+// weights that wide_sum_heat takes).
+enum SumForm : int { kChain = 0, kWide = 1, kHeat = 2 };
 
-template <int NT>
-struct TapSum<NT, false> {
+template <int NT, int FORM, class Taps = WideTaps>
+struct TapSum {
+  struct Acc {
+    WideVal u[NT];
+  };
+  const Taps& T;
+  const double* wdev;
+  __device__ __forceinline__ TapSum(const double* __restrict__ w, const Taps& t) : T(t), wdev(w) {}
+  __device__ __forceinline__ void tap(Acc& acc, int k, double v, int) const { acc.u[k] = wide_unpack(v); }
+  // ok = false: the FMA chain has to take the cell
+  __device__ __forceinline__ double get(const Acc& acc, bool& ok) const {
+    if constexpr (FORM == kHeat) return wide_sum_heat<NT>(acc.u, T, ok);
+    else return wide_sum<NT>(acc.u, T, ok);
+  }
+  __device__ __forceinline__ double get(const Acc& acc) const {
+    bool ok;
+    const double r = get(acc, ok);
+    if (ok) return r;
+    double v[NT];
+#pragma unroll
+    for (int k = 0; k < NT; ++k) v[k] = wide_repack(acc.u[k]);
+    return wide_chain(v, wdev, NT);
+  }
+};
+
+template <int NT, class Taps>
+struct TapSum<NT, kChain, Taps> {
   using Acc = double;
   RegWeights<NT> W;
-  __device__ __forceinline__ TapSum(const double* __restrict__ wdev, const WideTaps&) { W.load(wdev); }
+  __device__ __forceinline__ TapSum(const double* __restrict__ wdev, const Taps&) { W.load(wdev); }
   __device__ __forceinline__ void tap(Acc& acc, int k, double v, int c) const { W.tap(acc, k, v, c); }
-  __device__ __forceinline__ double get(const Acc& acc) const { return acc; }
   __device__ __forceinline__ double get(const Acc& acc, bool& ok) const {
     ok = true;
     return acc;
   }
-};
-
-template <int NT>
-struct TapSum<NT, true> {
-  struct Acc {
-    WideVal u[NT];
-  };
-  const WideTaps& T;
-  const double* wdev;
-  __device__ __forceinline__ TapSum(const double* __restrict__ w, const WideTaps& t) : T(t), wdev(w) {}
-  __device__ __forceinline__ void tap(Acc& acc, int k, double v, int) const { acc.u[k] = wide_unpack(v); }
-  __device__ __forceinline__ double get(const Acc& acc) const { return wide_sum<NT>(acc.u, T, wdev); }
-  __device__ __forceinline__ double get(const Acc& acc, bool& ok) const { return wide_sum<NT>(acc.u, T, ok); }
+  __device__ __forceinline__ double get(const Acc& acc) const { return acc; }
 };
 
 #endif  // __CUDACC__

@@ -66,6 +66,24 @@ struct Params {
   WideTaps wide;
 };
 
+// First column and row of a tile, advanced tile by tile (a division per warp and tile
+// would be 6 of a cell's 125 instructions).
+struct TilePos {
+  int x0, y0;
+  __device__ __forceinline__ TilePos(int t, int tiles_y) : x0(t / tiles_y * kTX), y0(t % tiles_y * kTC) {}
+  __device__ __forceinline__ void next(int ny) {
+    y0 += kTC;
+    if (y0 >= ny) {
+      y0 = 0;
+      x0 += kTX;
+    }
+  }
+};
+
+// -n <= c, wrapped; what lies further than n beyond the end (rows of a ragged tile
+// that nobody uses): any of them.
+__device__ __forceinline__ int wrap_near(int c, int n) { return c < 0 ? c + n : c >= n ? min(c - n, n - 1) : c; }
+
 // Position of offset (dy, dx) in the lexicographic tap list of the class.
 template <bool BOX, int RAD>
 __device__ __forceinline__ constexpr int tap_at(int dy, int dx) {
@@ -131,6 +149,7 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(
     }
   }
   __syncthreads();
+  step_begins();
   // a bounded wait; false: it gave up (the other warps' waits on this one then do the same)
   auto wait = [&](uint64_t* bar, uint32_t parity) {
     if (mbar_wait_bounded(bar, parity, kWaitNs)) return true;
@@ -152,10 +171,11 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(
     // ------------------------------------------------------------ producer
     RingPos<kU> post;  // of the next tile to post
     int posted = t0;
-    // copies tile t into its raw slot, once the slot's earlier tile is unpacked
-    auto post_tile = [&](int t) {
+    TilePos ptile(t0, P.tiles_y), tile = ptile, htile = ptile;  // of the next tile to post, of tile g, of the halo's
+    // copies the next tile into its raw slot, once the slot's earlier tile is unpacked
+    auto post_tile = [&] {
       if (!wait(&S.empty[post.s], post.ph ^ 1)) return false;
-      const int x0 = t / P.tiles_y * kTX, y0 = t % P.tiles_y * kTC;
+      const int x0 = ptile.x0, y0 = ptile.y0;
       const int r = lane;
       int y = y0 - RAD + r;
       if (TMA) {
@@ -167,12 +187,12 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(
         }
         __syncwarp();
         if (!whole && r < kRows)
-          tma_load_2d(&S.raw[post.s][r][0], &P.map_row, x0, wrapn(y, P.ny), &S.full[post.s]);
+          tma_load_2d(&S.raw[post.s][r][0], &P.map_row, x0, wrap_near(y, P.ny), &S.full[post.s]);
       } else {
         bool in = r < kRows;
         if (PERIODIC) {
           in = in && y < P.ny + RAD;  // rows past the ghosts of a ragged tile are not read
-          y = wrapn(y, P.ny);
+          y = wrap_near(y, P.ny);
         } else {
           in = in && y >= 0 && y < P.ny;
         }
@@ -197,14 +217,15 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(
         if (cp.bytes) bulk_load(&S.raw[post.s][r][cp.to], cp.from, cp.bytes, &S.full[post.s]);
       }
       post.next();
+      ptile.next(P.ny);
       ++posted;
       return true;
     };
     // the columns beside a tile: RAD on either side of every row that has
     // them (star: the tile's own rows), HN values per lane
     constexpr int HR = BOX ? kRows : kTC, H0 = BOX ? 0 : RAD, HALL = 2 * RAD * HR, HN = (HALL + 31) / 32;
-    auto halo = [&](int t, double (&h)[HN]) {
-      const int x0 = t / P.tiles_y * kTX, y0 = t % P.tiles_y * kTC;
+    auto halo = [&](double (&h)[HN]) {
+      const int x0 = htile.x0, y0 = htile.y0;
       const int cols = TMA ? kTX : min(kTX, P.nx - x0);
 #pragma unroll
       for (int q = 0; q < HN; ++q) {
@@ -212,13 +233,14 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(
         int x = j < RAD ? x0 - RAD + j : x0 + cols + (j - RAD), y = y0 - RAD + H0 + k % HR;
         bool in = k < HALL;
         if (PERIODIC) {
-          x = wrapn(x, P.nx);
-          y = wrapn(y, P.ny);
+          x = wrap_near(x, P.nx);
+          y = wrap_near(y, P.ny);
         } else {
           in = in && x >= 0 && x < P.nx && y >= 0 && y < P.ny;
         }
-        h[q] = in ? __ldg(P.src + (y * pitch + x)) : 0.0;
+        h[q] = in ? __ldcg(P.src + (y * pitch + x)) : 0.0;
       }
+      htile.next(P.ny);
     };
     // a wait that gave up: the copies already posted land (bounded) before the warp leaves
     auto leave = [&](int t) {
@@ -226,14 +248,14 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(
       for (int k = t; k < posted; ++k, q.next()) mbar_wait_bounded(&S.full[q.s], q.ph, kWaitNs);
     };
     double h[HN], hn[HN];
-    if (t0 < t1) halo(t0, h);
+    if (t0 < t1) halo(h);
+    while (posted < t1 && posted < t0 + kRaw)
+      if (!post_tile()) return leave(t0);
     for (int t = t0; t < t1; ++t) {
-      while (posted < t1 && posted < t + kRaw)
-        if (!post_tile(posted)) return leave(t);
-      if (t + 1 < t1) halo(t + 1, hn);
+      if (t + 1 < t1) halo(hn);
       if (!wait(&S.conv[u1], ph1)) return leave(t);
       Plane<RAD>& u = S.u[pos.s];
-      const int cols = TMA ? kTX : min(kTX, P.nx - t / P.tiles_y * kTX);
+      const int cols = TMA ? kTX : min(kTX, P.nx - tile.x0);
 #pragma unroll
       for (int q = 0; q < HN; ++q) {
         const int k = lane + 32 * q, j = k / HR, row = H0 + k % HR;
@@ -255,17 +277,21 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(
 #pragma unroll
       for (int q = 0; q < HN; ++q) h[q] = hn[q];
       next();
+      tile.next(P.ny);
+      // (after this tile's share of the unpacking, which the consumers wait for)
+      if (posted < t1 && !post_tile()) return leave(t + 1);
     }
     return;
   }
   // -------------------------------------------------------------- consumers
   const int row0 = RAD + warp * kR;  // the warp's first row in the planes
   const int c = 2 + 2 * lane;
+  TilePos tile(t0, P.tiles_y), before = tile;  // of tiles g and g-1
   for (int t = t0; t <= t1 && t0 < t1; ++t) {  // (the last iteration unpacks nothing)
     if (!wait(&S.conv[u1], ph1)) return;
     if (t < t1) {
       if (!wait(&S.full[pos.s], pos.ph)) return;
-      const int cols = TMA ? kTX : min(kTX, P.nx - t / P.tiles_y * kTX);
+      const int cols = TMA ? kTX : min(kTX, P.nx - tile.x0);
       WideVal v[2];
 #pragma unroll
       for (int r = 0; r < kR; ++r)
@@ -278,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(
     }
     if (t > t0) {
       const Plane<RAD>& u = S.u[u1];
-      const int xa = (t - 1) / P.tiles_y * kTX + 2 * lane, ya = (t - 1) % P.tiles_y * kTC + warp * kR;
+      const int xa = before.x0 + 2 * lane, ya = before.y0 + warp * kR;
       const int rows = xa < P.nx ? min(kR, P.ny - ya) : 0;  // rows that the lane stores
       double* out = P.dst + ya * pitch + xa;
       auto store = [&](int r, double v0, double v1) {
@@ -371,6 +397,8 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(
       __syncwarp();
     }
     if (t < t1) next();
+    before = tile;
+    tile.next(P.ny);
   }
 }
 
@@ -388,7 +416,7 @@ bool encode_2d(CUtensorMap* map, const double* base, const Geom& g, int rows) {
 
 template <bool BOX, int RAD, bool HEAT, bool PERIODIC, bool TMA>
 cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst,
-                     int* status, int sms, cudaStream_t stream) {
+                     int* status, int sms, cudaStream_t stream, bool chained) {
   auto kern = k_wide2d<BOX, RAD, HEAT, PERIODIC, TMA>;
   constexpr size_t bytes = sizeof(Smem<RAD, TMA>);
   static std::atomic<int> cache[kMaxDeviceOrdinals];
@@ -417,35 +445,35 @@ cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, co
   P.wide = wide;
   int64_t grid = (int64_t)sms * occ;
   if (grid > work) grid = work;
-  kern<<<(unsigned)grid, kThreads, bytes, stream>>>(P);
+  if (const cudaError_t e = launch_step(kern, (unsigned)grid, bytes, stream, chained, P)) return e;
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
 }
 
 template <bool BOX, int RAD, bool HEAT>
 cudaError_t launch_p(bool per, bool tma, const Geom& g, const WideTaps& wide, const double* wdev, const double* src,
-                     double* dst, int* status, int sms, cudaStream_t stream) {
+                     double* dst, int* status, int sms, cudaStream_t stream, bool chained) {
   if (tma)
-    return per ? launch_t<BOX, RAD, HEAT, true, true>(g, wide, wdev, src, dst, status, sms, stream)
-               : launch_t<BOX, RAD, HEAT, false, true>(g, wide, wdev, src, dst, status, sms, stream);
-  return per ? launch_t<BOX, RAD, HEAT, true, false>(g, wide, wdev, src, dst, status, sms, stream)
-             : launch_t<BOX, RAD, HEAT, false, false>(g, wide, wdev, src, dst, status, sms, stream);
+    return per ? launch_t<BOX, RAD, HEAT, true, true>(g, wide, wdev, src, dst, status, sms, stream, chained)
+               : launch_t<BOX, RAD, HEAT, false, true>(g, wide, wdev, src, dst, status, sms, stream, chained);
+  return per ? launch_t<BOX, RAD, HEAT, true, false>(g, wide, wdev, src, dst, status, sms, stream, chained)
+             : launch_t<BOX, RAD, HEAT, false, false>(g, wide, wdev, src, dst, status, sms, stream, chained);
 }
 
 }  // namespace
 
 cudaError_t launch_wide2d(Shape shape, int radius, int boundary, const Geom& g, const WideTaps& wide,
                           const double* wdev, const double* src, double* dst, int* status, int sms,
-                          cudaStream_t stream, bool tma) {
+                          cudaStream_t stream, bool tma, bool chained) {
   const bool per = boundary == kPeriodic, box = shape == Shape::kBox;
   const int side = 2 * radius + 1;
   if (wide.n != (box ? side * side : 4 * radius + 1)) return cudaErrorInvalidValue;
   if (radius == 2)
-    return box ? launch_p<true, 2, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream)
-               : launch_p<false, 2, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream);
-  if (box) return launch_p<true, 1, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream);
-  return wide.heat ? launch_p<false, 1, true>(per, tma, g, wide, wdev, src, dst, status, sms, stream)
-                   : launch_p<false, 1, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream);
+    return box ? launch_p<true, 2, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained)
+               : launch_p<false, 2, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained);
+  if (box) return launch_p<true, 1, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained);
+  return wide.heat ? launch_p<false, 1, true>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained)
+                   : launch_p<false, 1, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained);
 }
 
 }  // namespace gbst

@@ -137,6 +137,7 @@ __global__ void __launch_bounds__(kThreads, BOX || !TMA ? 2 : 3) k_wide3d(const 
     }
   }
   __syncthreads();
+  step_begins();
   // a bounded wait; false: it gave up (the other warps' waits on this one then do the same)
   auto wait = [&](uint64_t* bar, uint32_t parity) {
     if (mbar_wait_bounded(bar, parity, kWaitNs)) return true;
@@ -247,7 +248,7 @@ __global__ void __launch_bounds__(kThreads, BOX || !TMA ? 2 : 3) k_wide3d(const 
         const int z = wrap1(za - 1 + j, P.nz, PERIODIC);
         const bool zin = z >= 0 && z < P.nz;
 #pragma unroll
-        for (int q = 0; q < HN; ++q) h[q] = zin && hin[q] ? __ldg(P.src + z * plane + hoff[q]) : 0.0;
+        for (int q = 0; q < HN; ++q) h[q] = zin && hin[q] ? __ldcg(P.src + z * plane + hoff[q]) : 0.0;
       };
       // a wait that gave up: the copies already posted land (bounded) before the warp leaves
       auto leave = [&](int j) {
@@ -256,9 +257,9 @@ __global__ void __launch_bounds__(kThreads, BOX || !TMA ? 2 : 3) k_wide3d(const 
       };
       double h[HN], hn[HN];
       halo(0, h);
+      while (posted < nplanes && posted < kRaw)
+        if (!post_plane(posted)) return leave(0);
       for (int j = 0; j < nplanes; ++j) {
-        while (posted < nplanes && posted < j + kRaw)
-          if (!post_plane(posted)) return leave(j);
         if (j + 1 < nplanes) halo(j + 1, hn);
         if (!wait(&S.conv[u1], ph1)) return leave(j);
         Plane<TC>& u = S.u[con().s];
@@ -277,6 +278,8 @@ __global__ void __launch_bounds__(kThreads, BOX || !TMA ? 2 : 3) k_wide3d(const 
 #pragma unroll
         for (int q = 0; q < HN; ++q) h[q] = hn[q];
         next();
+        // (after this plane's share of the unpacking, which the consumers wait for)
+        if (posted < nplanes && !post_plane(posted)) return leave(j + 1);
       }
       continue;
     }
@@ -401,7 +404,7 @@ bool encode_3d(CUtensorMap* map, const double* base, const Geom& g, int box_y) {
 
 template <bool BOX, bool HEAT, bool PERIODIC, bool TMA, int TC>
 cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst,
-                     int* status, int sms, cudaStream_t stream) {
+                     int* status, int sms, cudaStream_t stream, bool chained) {
   auto kern = k_wide3d<BOX, HEAT, PERIODIC, TMA, TC>;
   constexpr size_t bytes = sizeof(Smem<BOX, TMA, TC>);
   static std::atomic<int> cache[kMaxDeviceOrdinals];
@@ -429,38 +432,38 @@ cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, co
   P.wide = wide;
   long long grid = (long long)sms * occ;
   if (grid > P.work) grid = P.work;
-  kern<<<(unsigned)grid, kThreads, bytes, stream>>>(P);
+  if (const cudaError_t e = launch_step(kern, (unsigned)grid, bytes, stream, chained, P)) return e;
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
 }
 
 template <bool BOX, bool HEAT, bool PERIODIC>
 cudaError_t launch_p(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst,
-                     int* status, int sms, cudaStream_t stream, bool tma, bool low) {
+                     int* status, int sms, cudaStream_t stream, bool tma, bool low, bool chained) {
   if (tma)
-    return low ? launch_t<BOX, HEAT, PERIODIC, true, 8>(g, wide, wdev, src, dst, status, sms, stream)
-               : launch_t<BOX, HEAT, PERIODIC, true, 16>(g, wide, wdev, src, dst, status, sms, stream);
-  return low ? launch_t<BOX, HEAT, PERIODIC, false, 8>(g, wide, wdev, src, dst, status, sms, stream)
-             : launch_t<BOX, HEAT, PERIODIC, false, 16>(g, wide, wdev, src, dst, status, sms, stream);
+    return low ? launch_t<BOX, HEAT, PERIODIC, true, 8>(g, wide, wdev, src, dst, status, sms, stream, chained)
+               : launch_t<BOX, HEAT, PERIODIC, true, 16>(g, wide, wdev, src, dst, status, sms, stream, chained);
+  return low ? launch_t<BOX, HEAT, PERIODIC, false, 8>(g, wide, wdev, src, dst, status, sms, stream, chained)
+             : launch_t<BOX, HEAT, PERIODIC, false, 16>(g, wide, wdev, src, dst, status, sms, stream, chained);
 }
 
 }  // namespace
 
 cudaError_t launch_wide3d(Shape shape, int boundary, const Geom& g, const WideTaps& wide, const double* wdev,
                           const double* src, double* dst, int* status, int sms, cudaStream_t stream, int tile_y,
-                          bool tma) {
+                          bool tma, bool chained) {
   const bool per = boundary == kPeriodic, low = tile_y == 8;
   if (shape == Shape::kBox) {
     if (wide.n != 27) return cudaErrorInvalidValue;
-    return per ? launch_p<true, false, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low)
-               : launch_p<true, false, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low);
+    return per ? launch_p<true, false, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained)
+               : launch_p<true, false, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained);
   }
   if (wide.n != 7) return cudaErrorInvalidValue;
   if (wide.heat)
-    return per ? launch_p<false, true, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low)
-               : launch_p<false, true, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low);
-  return per ? launch_p<false, false, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low)
-             : launch_p<false, false, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low);
+    return per ? launch_p<false, true, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained)
+               : launch_p<false, true, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained);
+  return per ? launch_p<false, false, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained)
+             : launch_p<false, false, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained);
 }
 
 }  // namespace gbst

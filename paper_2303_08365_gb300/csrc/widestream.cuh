@@ -59,12 +59,12 @@ struct RowCopy {
     if (from < src) {  // the grid starts half-way through 16 bytes
       from += 2;
       to = 2;
-      dst[1] = row[0];
+      dst[1] = __ldcg(row);
     }
     int k1 = (shift + n + 1) & ~1;   // one past the last element copied
     if (from + (k1 - to) > end) {  // the grid ends half-way through 16 bytes
       k1 -= 2;
-      dst[shift + n - 1] = row[n - 1];
+      dst[shift + n - 1] = __ldcg(row + n - 1);
     }
     bytes = k1 > to ? (uint32_t)(k1 - to) * 8 : 0;
   }
@@ -119,5 +119,34 @@ struct RingPos {
     }
   }
 };
+
+// Step after step of a run, each of a few microseconds: a step's CTAs are launched,
+// and set up their barriers, while the step before still runs (programmatic
+// dependent launch); step_begins then waits until that one is complete and its
+// results are visible.  The next step's CTAs may come up from here on: not
+// earlier, so that no more than two steps are ever in flight.  (The kernels read
+// the grids past L1, which may hold lines from two steps ago.)
+__device__ __forceinline__ void step_begins() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("fence.proxy.async;" ::: "memory");  // the copies are of the async proxy
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launches a step's kernel.  chained: what the stream holds last is the step
+// before of the same run (any other launch takes the stream's plain order).
+template <class Kernel, class P>
+cudaError_t launch_step(Kernel kern, unsigned int grid, size_t smem, cudaStream_t stream, bool chained, const P& p) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kWThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, p);
+}
 
 }  // namespace gbst

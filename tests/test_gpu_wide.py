@@ -145,3 +145,86 @@ def test_values_outside_the_integer_range(st, shape, kind, radius):
             # normal range each is half of the smallest subnormal
             top = np.abs(u0[np.isfinite(u0)]).max() if np.isfinite(u0).any() else 0.0
             assert np.abs(got[fine] - ref[fine]).max(initial=0.0) <= max(60 * EPS * top, 60 * 5e-324), values
+
+
+@pytest.mark.parametrize("kind", ["heat", "star", "box"])
+@pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
+@pytest.mark.parametrize("shape", SHAPES2D)
+def test_streaming_any_shape_2d_radius_1(st, shape, boundary, kind):
+    w = synth.heat_weights(2, 0.2) if kind == "heat" else weights(kind, 2, 1)
+    u0 = synth.normal(33, shape)
+    T, taps = 3, int(np.count_nonzero(w))
+    ref = oracle.run(u0, w, 1, boundary, T, nthreads=0)
+    tol = T * (2 * taps + 2) * EPS * np.abs(u0).max()
+    for tb, variant, offset in ((1, st.VARIANT_DIRECT, 0), (1, st.VARIANT_DIRECT, 1), (0, 0, 0)):
+        got = run(st, u0, w, 1, boundary, T, (tb, variant), offset)
+        assert np.abs(got - ref).max() <= tol, (tb, variant, offset)
+
+
+@pytest.mark.parametrize("spread", [0, 60])
+@pytest.mark.parametrize("kind", ["heat", "star", "box"])
+def test_one_step_against_exact_arithmetic_2d_radius_1(st, kind, spread):
+    rng = np.random.default_rng(spread)
+    u0 = rng.standard_normal((19, 70)) * 2.0 ** rng.integers(-spread, spread + 1, (19, 70))
+    u0[rng.random(u0.shape) < 0.1] = 0.0
+    w = synth.heat_weights(2, 0.2) if kind == "heat" else weights(kind, 2, 1)
+    for tuning in ((1, st.VARIANT_DIRECT), (4, st.VARIANT_PERSISTENT)):
+        got = run(st, u0, w, 1, DIRICHLET, 1, tuning)
+        for at in np.ndindex(*u0.shape):
+            want, top = exact_sum(u0, w, at, 1)
+            assert abs(Fraction(float(got[at])) - want) <= abs(want) * Fraction(EPS) + top * Fraction(2.0 ** -55), at
+
+
+# at least 200 tiles of 64 x 16: one column of tiles, one and a half rows of them, ragged
+# last ones, more than one tile for every CTA
+TILED = [(3200, 64), (23, 6500), (1009, 250), (833, 512), (1500, 1501)]
+
+
+def same(a, b):
+    """Equal bits, any NaN for another (which one depends on the order of the sum)."""
+    return np.array_equal(np.isnan(a), np.isnan(b)) and np.array_equal(a[~np.isnan(a)], b[~np.isnan(b)])
+
+
+@pytest.mark.parametrize("kind", ["heat", "star"])
+@pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
+@pytest.mark.parametrize("shape", TILED)
+def test_persistent_tiles_equal_single_steps(st, shape, boundary, kind):
+    """The integer form's result depends on a cell's values alone: all steps in one
+    launch give the bits of one launch a step, also where cells take the FMA chain."""
+    w = synth.heat_weights(2, 0.2) if kind == "heat" else weights(kind, 2, 1)
+    rng = np.random.default_rng(3)
+    u0 = synth.normal(34, shape)
+    for T in (1, 2, 31):
+        want = run(st, u0, w, 1, boundary, T, (1, st.VARIANT_DIRECT), 1)
+        assert same(run(st, u0, w, 1, boundary, T, (1, st.VARIANT_PERSISTENT), 1), want), T
+    mask = rng.random(shape) < 1e-4
+    u0[mask] = rng.choice([np.inf, -np.inf, np.nan, 1.7e308, 5e-324, 1e-300], int(mask.sum()))
+    want = run(st, u0, w, 1, boundary, 3, (1, st.VARIANT_DIRECT))
+    assert same(run(st, u0, w, 1, boundary, 3, (1, st.VARIANT_PERSISTENT)), want)
+
+
+# (cells per side, items): cells per thread, small tiles' share too low; tiles of many
+# grids; tiles of a few large ones
+BATCHES = [((20, 90), 30), ((150, 700), 40), ((900, 1400), 5)]
+
+
+@pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
+@pytest.mark.parametrize("sides,n", BATCHES)
+def test_batch_equals_plans(st, sides, n, boundary):
+    import torch
+    rng = np.random.default_rng(n)
+    shapes = [tuple(int(k) for k in rng.integers(sides[0], sides[1], 2)) for _ in range(n)]
+    steps = [int(rng.integers(0, 40)) for _ in range(n)]
+    alphas = [float(rng.uniform(0.05, 0.24)) for _ in range(n)]
+    u0 = [synth.normal(200 + i, s) for i, s in enumerate(shapes)]
+    grids = [torch.from_numpy(u.copy()).cuda() for u in u0]
+    with st.Batch(grids, alphas, steps, boundary) as b:
+        for tuning in ((1, 0, 0), (1, 1, 0), (1, 4, 0), (4, 0, 0)):
+            for g, u in zip(grids, u0):
+                g.copy_(torch.from_numpy(u))
+            b.set_tuning(*tuning)
+            b.run()
+            assert b.status() == 0
+            for g, u, a, T in zip(grids, u0, alphas, steps):
+                want = run(st, u, synth.heat_weights(2, a), 1, boundary, T, (1, st.VARIANT_DIRECT)) if T else u
+                assert np.array_equal(g.cpu().numpy(), want), (tuning, u.shape, a, T)
