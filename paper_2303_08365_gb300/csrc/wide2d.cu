@@ -104,25 +104,52 @@ __device__ __forceinline__ void get_row(const Plane<RAD>& u, int row, int c, Wid
   }
 }
 
-// The cells of a lane that the integer form does not take, by the FMA chain:
+// A lane's cells where all that they read are zeros (false: they are not).  Out of line,
+// and apart from chain_cells, whose frame would cost more than this does.
+template <bool BOX, int RAD>
+__device__ __noinline__ bool zero_cells(const Plane<RAD>& u, int row0, int rows, int cols, int c0, double* out, int nx) {
+  constexpr int RX = BOX ? RAD : 0;  // (nobody writes a star's corner columns)
+  if (!zero_rows<kR, RAD>(u, row0, c0, cols) || !zero_rows<RAD, RX>(u, row0 - RAD, c0, cols) ||
+      !zero_rows<RAD, RX>(u, row0 + kR, c0, cols))
+    return false;
+  put_zeros(out, rows, cols, nx);
+  return true;
+}
+
+// One cell by the FMA chain.
+template <bool BOX, int RAD>
+__device__ __noinline__ double chain_cell(const Plane<RAD>& u, int row, int c, const double* wdev) {
+  constexpr int NT = BOX ? (2 * RAD + 1) * (2 * RAD + 1) : 4 * RAD + 1;
+  double v[NT];
+  for (int dy = -RAD; dy <= RAD; ++dy)
+    for (int dx = -RAD; dx <= RAD; ++dx) {
+      if (!BOX && dy != 0 && dx != 0) continue;
+      v[tap_at<BOX, RAD>(dy, dx)] = wide_repack(get(&u.m[row + dy][c + dx], &u.e[row + dy][c + dx]));
+    }
+  return wide_chain(v, wdev, NT);
+}
+
+// The cells of a lane that the integer form does not take: zeros, or by the FMA chain:
 // `cols` columns from c0 on of rows row0 .. row0+rows-1.  Out of line: rarely run.
 template <bool BOX, int RAD>
 __device__ __noinline__ void chain_cells(const Plane<RAD>& u, int row0, int rows, int cols, int c0, const WideTaps& T,
                                          const double* wdev, double* out, int nx) {
-  constexpr int NT = BOX ? (2 * RAD + 1) * (2 * RAD + 1) : 4 * RAD + 1;
   for (int r = 0; r < rows; ++r)
     for (int i = 0; i < cols; ++i) {
-      double v[NT];
+      const int row = row0 + r, c = c0 + i;
+      unsigned int any = 0;
       int E = -0x7fffffff;
+#pragma unroll
       for (int dy = -RAD; dy <= RAD; ++dy)
+#pragma unroll
         for (int dx = -RAD; dx <= RAD; ++dx) {
           if (!BOX && dy != 0 && dx != 0) continue;
-          const int t = tap_at<BOX, RAD>(dy, dx), row = row0 + r + dy, c = c0 + i + dx;
-          const WideVal x = get(&u.m[row][c], &u.e[row][c]);
-          v[t] = wide_repack(x);
-          E = max(E, x.e + T.ex[t]);
+          const WideVal x = get(&u.m[row + dy][c + dx], &u.e[row + dy][c + dx]);
+          any |= wide_nonzero(x);
+          E = max(E, x.e + T.ex[tap_at<BOX, RAD>(dy, dx)]);
         }
-      if (!wide_covers(E, T)) out[(int64_t)r * nx + i] = wide_chain(v, wdev, NT);
+      if (any == 0) out[(int64_t)r * nx + i] = 0.0;
+      else if (!wide_covers(E, T)) out[(int64_t)r * nx + i] = chain_cell<BOX, RAD>(u, row, c, wdev);
     }
 }
 
@@ -393,7 +420,8 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(
           store(r, acc[0].get(E[0], P.wide), acc[1].get(E[1], P.wide));
         }
       }
-      if (!all) chain_cells<BOX, RAD>(u, row0, rows, min(2, P.nx - xa), c, P.wide, P.wdev, out, P.nx);
+      if (!all && !zero_cells<BOX, RAD>(u, row0, rows, min(2, P.nx - xa), c, out, P.nx))
+        chain_cells<BOX, RAD>(u, row0, rows, min(2, P.nx - xa), c, P.wide, P.wdev, out, P.nx);
       __syncwarp();
     }
     if (t < t1) next();

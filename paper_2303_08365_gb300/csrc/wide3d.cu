@@ -89,7 +89,39 @@ __device__ __forceinline__ constexpr int tap_at(int dz, int dy, int dx) {
   return dz < 0 ? 0 : dz > 0 ? 6 : dy < 0 ? 1 : dy > 0 ? 5 : 3 + dx;
 }
 
-// The cells of a lane that the integer form does not take, by the FMA chain:
+// A lane's cells where all that they read are zeros (false: they are not).  Out of line,
+// and apart from chain_cells, whose frame would cost more than this does.
+template <bool BOX, int TC>
+__device__ __noinline__ bool zero_cells(const Plane<TC>& um, const Plane<TC>& u0, const Plane<TC>& up, int row0,
+                                        int rows, int cols, int c0, double* out, int nx) {
+  constexpr int R = TC / kWarps;
+  if (!zero_rows<R, 1>(u0, row0, c0, cols)) return false;
+  if (BOX ? !zero_rows<1, 1>(u0, row0 - 1, c0, cols) || !zero_rows<1, 1>(u0, row0 + R, c0, cols) ||
+                !zero_rows<R + 2, 1>(um, row0 - 1, c0, cols) || !zero_rows<R + 2, 1>(up, row0 - 1, c0, cols)
+          // (nobody writes a star's corner columns)
+          : !zero_rows<1, 0>(u0, row0 - 1, c0, cols) || !zero_rows<1, 0>(u0, row0 + R, c0, cols) ||
+                !zero_rows<R, 0>(um, row0, c0, cols) || !zero_rows<R, 0>(up, row0, c0, cols))
+    return false;
+  put_zeros(out, rows, cols, nx);
+  return true;
+}
+
+// One cell by the FMA chain.
+template <bool BOX, int TC>
+__device__ __noinline__ double chain_cell(const Plane<TC>& um, const Plane<TC>& u0, const Plane<TC>& up, int row, int c,
+                                          const double* wdev) {
+  constexpr int NT = BOX ? 27 : 7;
+  const Plane<TC>* const pl[3] = {&um, &u0, &up};
+  double v[NT];
+  for (int k = 0; k < 27; ++k) {
+    const int dz = k / 9 - 1, dy = k / 3 % 3 - 1, dx = k % 3 - 1;
+    if (!BOX && (dz != 0) + (dy != 0) + (dx != 0) > 1) continue;
+    v[tap_at<BOX>(dz, dy, dx)] = wide_repack(get(&pl[dz + 1]->m[row + dy][c + dx], &pl[dz + 1]->e[row + dy][c + dx]));
+  }
+  return wide_chain(v, wdev, NT);
+}
+
+// The cells of a lane that the integer form does not take: zeros, or by the FMA chain:
 // `cols` columns from c0 on of rows row0 .. row0+rows-1.  Out of line, one call for
 // a lane's cells: rarely run, and a call within the sum's code costs every cell
 // 19 instructions.
@@ -97,21 +129,22 @@ template <bool BOX, int TC>
 __device__ __noinline__ void chain_cells(const Plane<TC>& um, const Plane<TC>& u0, const Plane<TC>& up, int row0,
                                          int rows, int cols, int c0, const WideTaps& T, const double* wdev,
                                          double* out, int nx) {
-  constexpr int NT = BOX ? 27 : 7;
-  const Plane<TC>* const pl[3] = {&um, &u0, &up};
   for (int r = 0; r < rows; ++r)
     for (int i = 0; i < cols; ++i) {
-      double v[NT];
+      const int row = row0 + r, c = c0 + i;
+      unsigned int any = 0;
       int E = -0x7fffffff;
+#pragma unroll
       for (int k = 0; k < 27; ++k) {
         const int dz = k / 9 - 1, dy = k / 3 % 3 - 1, dx = k % 3 - 1;
         if (!BOX && (dz != 0) + (dy != 0) + (dx != 0) > 1) continue;
-        const int t = tap_at<BOX>(dz, dy, dx), row = row0 + r + dy, c = c0 + i + dx;
-        const WideVal u = get(&pl[dz + 1]->m[row][c], &pl[dz + 1]->e[row][c]);
-        v[t] = wide_repack(u);
-        E = max(E, u.e + T.ex[t]);
+        const Plane<TC>& p = dz < 0 ? um : dz > 0 ? up : u0;
+        const WideVal u = get(&p.m[row + dy][c + dx], &p.e[row + dy][c + dx]);
+        any |= wide_nonzero(u);
+        E = max(E, u.e + T.ex[tap_at<BOX>(dz, dy, dx)]);
       }
-      if (!wide_covers(E, T)) out[(int64_t)r * nx + i] = wide_chain(v, wdev, NT);
+      if (any == 0) out[(int64_t)r * nx + i] = 0.0;
+      else if (!wide_covers(E, T)) out[(int64_t)r * nx + i] = chain_cell<BOX, TC>(um, u0, up, row, c, wdev);
     }
 }
 
@@ -380,7 +413,7 @@ __global__ void __launch_bounds__(kThreads, BOX || !TMA ? 2 : 3) k_wide3d(const 
             store(r, acc[0].get(E[0], P.wide), acc[1].get(E[1], P.wide));
           }
         }
-        if (!all)
+        if (!all && !zero_cells<BOX, TC>(um, u0, up, row0, rows, min(2, P.nx - xa), c, out, P.nx))
           chain_cells<BOX, TC>(um, u0, up, row0, rows, min(2, P.nx - xa), c, P.wide, P.wdev, out, P.nx);
         __syncwarp();
         out += plane;

@@ -95,21 +95,34 @@ struct __align__(128) Smem {
   uint64_t done;         // the step's tiles are stored: 8 consumer warps
 };
 
-// The cells of a lane that the integer form does not take, by the FMA chain.  Out
-// of line: rarely run.
+// A lane's cells where all that they read are zeros (false: they are not).
+__device__ __noinline__ bool zero_cells(const Plane& u, int row0, int rows, int cols, int c0, double* out, int pitch) {
+  if (!zero_rows<kR, 1>(u, row0, c0, cols) || !zero_rows<1, 0>(u, row0 - 1, c0, cols) ||
+      !zero_rows<1, 0>(u, row0 + kR, c0, cols))
+    return false;
+  put_zeros(out, rows, cols, pitch);
+  return true;
+}
+
+// The cells of a lane that the integer form does not take: zeros, or by the FMA chain.
+// Out of line: rarely run.
 __device__ __noinline__ void chain_cells(const Plane& u, int row0, int rows, int cols, int c0, const Taps& T,
                                          const double* w, double* out, int pitch) {
-  const int dy[5] = {-1, 0, 0, 0, 1}, dx[5] = {0, -1, 0, 1, 0};
   for (int r = 0; r < rows; ++r)
     for (int i = 0; i < cols; ++i) {
-      double v[5];
+      const int row = row0 + r, c = c0 + i;
+      const WideVal x[5] = {get(&u.m[row - 1][c], &u.e[row - 1][c]), get(&u.m[row][c - 1], &u.e[row][c - 1]),
+                            get(&u.m[row][c], &u.e[row][c]), get(&u.m[row][c + 1], &u.e[row][c + 1]),
+                            get(&u.m[row + 1][c], &u.e[row + 1][c])};
       int E = -0x7fffffff;
+      double v[5];
+#pragma unroll
       for (int k = 0; k < 5; ++k) {
-        const WideVal x = get(&u.m[row0 + r + dy[k]][c0 + i + dx[k]], &u.e[row0 + r + dy[k]][c0 + i + dx[k]]);
-        v[k] = wide_repack(x);
-        E = max(E, x.e + T.ex[k]);
+        E = max(E, x[k].e + T.ex[k]);
+        v[k] = wide_repack(x[k]);
       }
-      if (!wide_covers(E, T)) out[(int64_t)r * pitch + i] = wide_chain(v, w, 5);
+      if (wide_zeros<5>(x)) out[(int64_t)r * pitch + i] = 0.0;
+      else if (!wide_covers(E, T)) out[(int64_t)r * pitch + i] = wide_chain(v, w, 5);
     }
 }
 
@@ -433,6 +446,16 @@ __global__ void __launch_bounds__(kThreads, 3) k_wide_steps(const __grid_constan
     const bool vec = d.vec && left > 1;
     const int64_t pitch = d.pitch;
     double* out = d.out + warp * kR * pitch + 2 * lane;
+    auto store = [&](int r, double v0, double v1) {
+      if (r >= rows) return;
+      double* o = out + r * pitch;
+      if (vec) {
+        st_global_v2(o, v0, v1);
+      } else {
+        o[0] = v0;
+        if (left > 1) o[1] = v1;
+      }
+    };
     bool all = true;  // the integer form takes every cell that is stored
 #pragma unroll
     for (int r = 0; r < kR; ++r) {
@@ -452,17 +475,10 @@ __global__ void __launch_bounds__(kThreads, 3) k_wide_steps(const __grid_constan
         else v[i] = wide_sum<5>(w, T, ok);
         all = all && (ok || r >= rows || (i == 1 && left < 2));
       }
-      if (r < rows) {
-        double* o = out + r * pitch;
-        if (vec) {
-          st_global_v2(o, v[0], v[1]);
-        } else {
-          o[0] = v[0];
-          if (left > 1) o[1] = v[1];
-        }
-      }
+      store(r, v[0], v[1]);
     }
-    if (!all) chain_cells(u, row0, rows, min(2, left), c, d.wide, items[d.item].w, out, d.pitch);
+    if (!all && !zero_cells(u, row0, rows, min(2, left), c, out, d.pitch))
+      chain_cells(u, row0, rows, min(2, left), c, d.wide, items[d.item].w, out, d.pitch);
     __syncwarp();
   };
   // the next tile, or the stop: a CTA that has no tile left waits for the other

@@ -107,6 +107,40 @@ __device__ __forceinline__ void unpack_row(const double (&raw)[ROWS][raw_col<TMA
   }
 }
 
+// Whether rows row0 .. row0+N-1 of a plane are zeros in column c (cols = 2: and c + 1)
+// and RAD columns on either side.
+template <int N, int RAD, int ROWS>
+__device__ __forceinline__ bool zero_rows(const WidePlane<ROWS>& u, int row0, int c, int cols) {
+  const unsigned int second = cols == 2 ? ~0u : 0u;
+  unsigned int any = 0;
+#pragma unroll
+  for (int r = 0; r < N; ++r) {
+    const int row = row0 + r;
+    WideVal a, b;
+    get_pair(&u.m[row][c], &u.e[row][c], a, b);
+    any |= wide_nonzero(a) | (RAD == 0 ? wide_nonzero(b) & second : wide_nonzero(b));
+    if constexpr (RAD == 1) {
+      any |= wide_nonzero(get(&u.m[row][c - 1], &u.e[row][c - 1]));
+      any |= wide_nonzero(get(&u.m[row][c + 2], &u.e[row][c + 2])) & second;
+    }
+    if constexpr (RAD == 2) {
+      get_pair(&u.m[row][c - 2], &u.e[row][c - 2], a, b);
+      any |= wide_nonzero(a) | wide_nonzero(b);
+      get_pair(&u.m[row][c + 2], &u.e[row][c + 2], a, b);
+      any |= wide_nonzero(a) | (wide_nonzero(b) & second);
+    }
+  }
+  return any == 0;
+}
+
+// Zeros for the pair's first `cols` columns of `rows` rows.
+__device__ __forceinline__ void put_zeros(double* out, int rows, int cols, int64_t pitch) {
+  for (int r = 0; r < rows; ++r, out += pitch) {
+    out[0] = 0.0;
+    if (cols > 1) out[1] = 0.0;
+  }
+}
+
 // A slot and phase that advance plane by plane.
 template <int N>
 struct RingPos {

@@ -228,3 +228,32 @@ def test_batch_equals_plans(st, sides, n, boundary):
             for g, u, a, T in zip(grids, u0, alphas, steps):
                 want = run(st, u, synth.heat_weights(2, a), 1, boundary, T, (1, st.VARIANT_DIRECT)) if T else u
                 assert np.array_equal(g.cpu().numpy(), want), (tuning, u.shape, a, T)
+
+
+# TMA tiles, bulk copies with a last tile of 45 and of one column, both directions' ragged
+# tiles; persistent tiles; 16 x 32 tiles
+ZEROS = [((20, 64, 128), "heat", 1, (0, 0)), ((18, 127, 1005), "heat", 1, (1, 1)), ((17, 97, 129), "box", 1, (1, 1)),
+         ((16, 64, 64), "box", 1, (0, 0)), ((320, 512), "heat", 1, (1, 2)), ((411, 557), "box", 2, (1, 1)),
+         ((411, 557), "star", 1, (1, 1)), ((833, 513), "heat", 1, (1, 4)), ((90, 130), "heat", 1, (4, 4)),
+         ((20, 64, 128), "heat", 1, (4, 5))]
+
+
+@pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
+@pytest.mark.parametrize("shape,kind,radius,tuning", ZEROS)
+def test_a_few_values_among_zeros(st, shape, kind, radius, tuning, boundary):
+    """Zeros of either sign stay zeros where nothing else reaches; tiny values beside them."""
+    if tuning[0] == 0 and boundary == PERIODIC and shape[-1] % 64:
+        pytest.skip("no streamed form")
+    rng = np.random.default_rng(12)
+    w = synth.heat_weights(len(shape), 0.12) if kind == "heat" else weights(kind, len(shape), radius)
+    u0 = np.where(rng.random(shape) < 0.5, 0.0, -0.0)
+    at = rng.integers(0, u0.size, 40)
+    u0.reshape(-1)[at] = rng.standard_normal(40) * 10.0 ** rng.integers(-320, 5, 40)
+    T = 4
+    ref = oracle.run(u0, w, radius, boundary, T, nthreads=0)
+    got = run(st, u0, w, radius, boundary, T, tuning)
+    taps = int(np.count_nonzero(w))
+    assert np.array_equal(got == 0.0, ref == 0.0) or np.abs(got[(got == 0.0) != (ref == 0.0)]).max() <= 1e-320
+    # relative to what a cell's neighbourhood holds: the largest value that reaches it
+    top = oracle.run(np.abs(u0), (w > 0).astype(float), radius, boundary, T, nthreads=0)
+    assert (np.abs(got - ref) <= T * (2 * taps + 2) * EPS * top + 60 * T * 5e-324).all()
