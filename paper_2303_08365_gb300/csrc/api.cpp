@@ -230,13 +230,22 @@ bool uses_wide(int ndim, int radius) {
 
 // Whether a grid that the TMA-fed kernels do not take is streamed all the same
 // (by bulk copies) or swept cell by cell.  Streaming takes longer to start: on
-// GB300, us a step, cell by cell against streamed: 2D radius 2, 257^2 6.3 / 6.3,
-// 513^2 11.4 / 8.3, 129^2 4.2 / 6.3; 3D star 97^3 22.9 / 24.8, 129^3 43 / 41;
-// 27-point box 49^3 16.6 / 14.7, 33^3 10.5 / 12.5.
+// GB300, us a step, cell by cell against streamed: 2D radius-2 star 193^2 4.2 / 5.0,
+// 257^2 5.9 / 5.0, 513^2 8.2 / 6.3; 25-point box 257^2 6.2 / 6.6, 361^2 10.3 / 6.9;
+// 3D star 129^3 28.7 / 35.7, 145^3 34.9 / 41.3, 161^3 50.5 / 49.9, 27-point box 49^3
+// 16.6 / 14.7, 33^3 9.3 / 10.5.
 bool streamed_any_shape(const stencil_plan_s* p) {
   if (!p->wide.n || p->g.nx < 32 || p->g.ny < 8) return false;
+  const bool box = p->shape == Shape::kBox;
+  if (p->ndim == 2 && p->radius == 2) return p->cells() >= (int64_t)(box ? 3 : 2) << 15;
   if (p->ndim == 2) return p->cells() >= (int64_t)1 << 17;
-  return p->ndim == 3 && p->radius == 1 && p->cells() >= (int64_t)1 << (p->shape == Shape::kBox ? 17 : 21);
+  return p->ndim == 3 && p->radius == 1 && p->cells() >= (int64_t)1 << (box ? 17 : 22);
+}
+
+// The tile height of those: 16 rows, 8 for small 27-point boxes, whose planes are too
+// few for the chip otherwise (16 against 8 rows: 65^3 28.4 / 22.8 us a step, 97^3 44.4 / 41.0).
+int any_shape_tile_y(const stencil_plan_s* p) {
+  return p->shape == Shape::kBox && p->cells() < (int64_t)1 << 20 ? 8 : 16;
 }
 
 std::string device_name();
@@ -697,8 +706,8 @@ int run_steps(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, int variant,
         e = launch_stream2d(p->shape, p->radius, p->boundary, equal_box && p->radius == 1, p->g, p->taps,
                             p->d_w, a, b, p->d_status, sms, s);
       else if (p->ndim == 3 && streamed_any_shape(p))
-        e = launch_wide3d(p->shape, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, 0, false,
-                          chained);
+        e = launch_wide3d(p->shape, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s,
+                          any_shape_tile_y(p), false, chained);
       else if (p->ndim == 2 && streamed_any_shape(p))
         e = launch_wide2d(p->shape, p->radius, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, false,
                           chained);

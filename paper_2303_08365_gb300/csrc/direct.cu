@@ -5,12 +5,166 @@
 // streaming and temporal-blocking kernels are measured against.
 //
 // Operation: one step of u'(x) = sum_o w_o u~(x+o) (paper Sec. 2.1, Listing 1).
+//
+// The taps are a compile-time list and the wraps of an axis are worked out once per
+// thread: a tap is one address addition and a load.  Us a step, against a list of
+// offsets in the parameters with a wrap test for each: 113 x 28 x 118 star 8.3 (12.4;
+// FMA chain 10.3), 27 x 242 x 31 125-point box 61 (99), 101^3 336 (656), 97^3
+// star 16.4 (22.9).  The 125-point box is bound by the FP64 pipe (62 clocks a cell and
+// SM: 231 us of the 336 at 101^3), the others by the integer pipes and the launch.
 #include "internal.h"
 #include "taps.cuh"
 #include "wide.cuh"
 
 namespace gbst {
 namespace {
+
+// The lexicographic tap list of a stencil class, at compile time.
+template <int NDIM, int RAD, bool BOX>
+struct Taps {
+  static constexpr int kSide = 2 * RAD + 1;
+  static constexpr int kN = !BOX ? 2 * NDIM * RAD + 1 : NDIM == 3 ? kSide * kSide * kSide : kSide * kSide;
+  // offset of tap k along x (axis 0), y (1) or z (2)
+  static __host__ __device__ constexpr int off(int k, int axis) {
+    if (BOX) return axis == 0 ? k % kSide - RAD : axis == 1 ? k / kSide % kSide - RAD : NDIM == 3 ? k / (kSide * kSide) - RAD : 0;
+    // star: the slowest axis's lower half, ..., the fastest axis, ..., the slowest axis's upper half
+    int d = NDIM - 1;
+    while (d > 0) {
+      const int lo = (NDIM - 1 - d) * RAD, hi = kN - 1 - lo;
+      if (k < lo + RAD) return axis == d ? k - lo - RAD : 0;
+      if (k > hi - RAD) return axis == d ? k - hi + RAD : 0;
+      --d;
+    }
+    return axis == 0 ? k - (NDIM - 1) * RAD - RAD : 0;
+  }
+};
+
+// The 2 RAD + 1 positions around coordinate c of an axis of length n, as distances from
+// c in elements (step: the axis's stride), and whether they are in the grid.
+template <int RAD, bool PERIODIC, class Int>
+struct Axis {
+  Int at[2 * RAD + 1];
+  bool in[2 * RAD + 1];
+  __device__ __forceinline__ Axis(int c, int n, Int step) {
+#pragma unroll
+    for (int k = 0; k < 2 * RAD + 1; ++k) {
+      int d = k - RAD;
+      in[k] = true;
+      if (d != 0) {
+        if (PERIODIC) {
+          if (n < RAD) d = ((c + d) % n + n) % n - c;  // (uniform) an axis shorter than the radius
+          else d = c + d < 0 ? d + n : c + d >= n ? d - n : d;
+        } else {
+          in[k] = (unsigned)(c + d) < (unsigned)n;
+        }
+      }
+      at[k] = (Int)d * step;
+    }
+  }
+};
+
+// Weights as kernel parameters (the constant bank).
+template <int NT>
+struct Weights {
+  double w[NT];
+};
+
+struct DirectParams {
+  const double* src;
+  double* dst;
+  int nz, ny, nx;
+  int zper;
+  const double* wdev;
+};
+
+// The thread's cells, plane by plane: body(v, cell) with the cell's NT values.
+template <int NDIM, int RAD, bool BOX, bool PERIODIC, class Body>
+__device__ __forceinline__ void each_cell(const DirectParams& P, const Body& body) {
+  using T = Taps<NDIM, RAD, BOX>;
+  constexpr int RZ = NDIM >= 3 ? RAD : 0, RY = NDIM >= 2 ? RAD : 0;
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  if (x >= P.nx || y >= P.ny) return;
+  const int64_t plane = (int64_t)P.ny * P.nx;
+  const Axis<RAD, PERIODIC, int> X(x, P.nx, 1);
+  const Axis<RY, PERIODIC, int64_t> Y(y, P.ny, P.nx);
+  const int z0 = blockIdx.z * P.zper, z1 = min(P.nz, z0 + P.zper);
+  for (int z = z0; z < z1; ++z) {
+    const Axis<RZ, PERIODIC, int64_t> Z(z, P.nz, plane);
+    const int64_t cell = z * plane + (int64_t)y * P.nx + x;
+    double v[T::kN];
+#pragma unroll
+    for (int k = 0; k < T::kN; ++k) {
+      const int kx = T::off(k, 0) + RAD, ky = T::off(k, 1) + RY, kz = T::off(k, 2) + RZ;
+      const double* row = P.src + cell + (Z.at[kz] + Y.at[ky]);
+      v[k] = Z.in[kz] && Y.in[ky] && X.in[kx] ? __ldg(row + X.at[kx]) : 0.0;
+    }
+    P.dst[cell] = body(v);
+  }
+}
+
+template <int NDIM, int RAD, bool BOX, bool PERIODIC>
+__global__ void __launch_bounds__(256) k_direct(const __grid_constant__ DirectParams P) {
+  constexpr int NT = Taps<NDIM, RAD, BOX>::kN;
+  RegWeights<NT> W;  // the weights live in registers (full FP64 rate)
+  W.load(P.wdev);
+  each_cell<NDIM, RAD, BOX, PERIODIC>(P, [&](const double (&v)[NT]) {
+    double acc = 0.0;
+#pragma unroll
+    for (int k = 0; k < NT; ++k) W.tap(acc, k, v[k], 0);
+    return acc;
+  });
+}
+
+// The 125-tap box: plane by plane of its taps, so that neither 125 values nor as many
+// weights (in the constant bank) have to be held at once.
+template <bool PERIODIC>
+__global__ void __launch_bounds__(256) k_direct_box125(const __grid_constant__ DirectParams P,
+                                                       const __grid_constant__ Weights<125> W) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  if (x >= P.nx || y >= P.ny) return;
+  const int64_t plane = (int64_t)P.ny * P.nx;
+  const Axis<2, PERIODIC, int> X(x, P.nx, 1);
+  const Axis<2, PERIODIC, int64_t> Y(y, P.ny, P.nx);
+  const int z0 = blockIdx.z * P.zper, z1 = min(P.nz, z0 + P.zper);
+  for (int z = z0; z < z1; ++z) {
+    double acc = 0.0;
+#pragma unroll 1
+    for (int kz = 0; kz < 5; ++kz) {
+      int zz = z + kz - 2;
+      if (PERIODIC) zz = P.nz < 2 ? 0 : zz < 0 ? zz + P.nz : zz >= P.nz ? zz - P.nz : zz;
+      const bool zin = PERIODIC || (unsigned)zz < (unsigned)P.nz;
+      const double* p = P.src + (zz * plane + (int64_t)y * P.nx + x);
+      double v[25];
+#pragma unroll
+      for (int k = 0; k < 25; ++k)
+        v[k] = zin && Y.in[k / 5] && X.in[k % 5] ? __ldg(p + Y.at[k / 5] + X.at[k % 5]) : 0.0;
+#pragma unroll
+      for (int k = 0; k < 25; ++k) acc = fma(W.w[25 * kz + k], v[k], acc);
+    }
+    P.dst[z * plane + (int64_t)y * P.nx + x] = acc;
+  }
+}
+
+// The same sweep with the weighted sum in the integer form (wide.cuh).
+template <int NDIM, int RAD, bool BOX, bool PERIODIC, bool HEAT>
+__global__ void __launch_bounds__(256) k_direct_wide(const __grid_constant__ DirectParams P,
+                                                     const __grid_constant__ WideTaps wide) {
+  constexpr int NT = Taps<NDIM, RAD, BOX>::kN;
+  each_cell<NDIM, RAD, BOX, PERIODIC>(P, [&](const double (&v)[NT]) {
+    WideVal u[NT];
+#pragma unroll
+    for (int k = 0; k < NT; ++k) u[k] = wide_unpack(v[k]);
+    bool ok;
+    double r;
+    if constexpr (HEAT) r = wide_sum_heat<NT>(u, wide, ok);
+    else r = wide_sum<NT>(u, wide, ok);
+    if (ok) return r;
+    if (wide_zeros<NT>(u)) return 0.0;
+    return wide_chain(v, P.wdev, NT);
+  });
+}
 
 // Index of a neighbour along one axis under each boundary mode.
 //   MODE 0: Dirichlet zero -- returns false when outside [0, n)
@@ -28,67 +182,6 @@ __device__ __forceinline__ bool axis_index(int c, int n, int& out) {
     int m = c % n;
     out = m < 0 ? m + n : m;
     return true;
-  }
-}
-
-template <int MODE>
-__device__ __forceinline__ double direct_value(const double* __restrict__ src, int z, int y, int x, int nz, int ny,
-                                               int nx) {
-  int zz, yy, xx;
-  bool in = axis_index<MODE>(z, nz, zz);
-  in &= axis_index<MODE>(y, ny, yy);
-  in &= axis_index<MODE>(x, nx, xx);
-  return in ? __ldg(src + ((int64_t)zz * ny + yy) * nx + xx) : 0.0;
-}
-
-template <int NT, int MODE>
-__global__ void __launch_bounds__(256) k_direct(const double* __restrict__ src,
-                                                double* __restrict__ dst, int nz, int ny, int nx,
-                                                int zper, const __grid_constant__ TapList<NT> tp,
-                                                const double* __restrict__ wdev) {
-  // up to 27 taps the weights live in registers (full FP64 rate); the
-  // 125-tap radius-2 box keeps them in the constant bank instead of spilling
-  constexpr bool kRegs = NT <= 27;
-  RegWeights<kRegs ? NT : 1> W;
-  if (kRegs) W.load(wdev);
-  const double zero = kRegs ? W.z[0] : 0.0;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  if (x >= nx || y >= ny) return;
-  const int z0 = blockIdx.z * zper;
-  const int z1 = min(nz, z0 + zper);
-  for (int z = z0; z < z1; ++z) {
-    double acc = 0.0;
-#pragma unroll
-    for (int k = 0; k < NT; ++k) {
-      const double v = direct_value<MODE>(src, z + tp.dz[k], y + tp.dy[k], x + tp.dx[k], nz, ny, nx);
-      if constexpr (kRegs)
-        W.tap(acc, k, v, 0);
-      else
-        acc = fma(tp.w[k], v, k == 0 ? zero : acc);
-    }
-    dst[((int64_t)z * ny + y) * nx + x] = acc;
-  }
-}
-
-// The same sweep with the weighted sum in the integer form (wide.cuh).
-template <int NT, int MODE>
-__global__ void __launch_bounds__(256) k_direct_wide(const double* __restrict__ src, double* __restrict__ dst, int nz,
-                                                     int ny, int nx, int zper,
-                                                     const __grid_constant__ TapList<NT> tp,
-                                                     const __grid_constant__ WideTaps wide,
-                                                     const double* __restrict__ wdev) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  if (x >= nx || y >= ny) return;
-  const int z0 = blockIdx.z * zper;
-  const int z1 = min(nz, z0 + zper);
-  for (int z = z0; z < z1; ++z) {
-    WideVal u[NT];
-#pragma unroll
-    for (int k = 0; k < NT; ++k)
-      u[k] = wide_unpack(direct_value<MODE>(src, z + tp.dz[k], y + tp.dy[k], x + tp.dx[k], nz, ny, nx));
-    dst[((int64_t)z * ny + y) * nx + x] = wide_sum<NT>(u, wide, wdev);
   }
 }
 
@@ -165,37 +258,44 @@ cudaError_t launch_nt_f32(int mode, const Geom& g, const HostTaps& ht, const flo
   return cudaGetLastError();
 }
 
-template <int NT>
-cudaError_t launch_nt(int mode, const Geom& g, const HostTaps& ht, const WideTaps& wide, const double* wdev,
-                      const double* src, double* dst, cudaStream_t stream) {
-  TapList<NT> tp;
-  for (int k = 0; k < NT; ++k) {
-    tp.w[k] = ht.w[k];
-    tp.dz[k] = ht.dz[k];
-    tp.dy[k] = ht.dy[k];
-    tp.dx[k] = ht.dx[k];
-  }
+template <int NDIM, int RAD, bool BOX, bool PERIODIC>
+cudaError_t launch_p(const Geom& g, const HostTaps& ht, const WideTaps& wide, const double* wdev, const double* src,
+                     double* dst, cudaStream_t stream) {
+  constexpr int NT = Taps<NDIM, RAD, BOX>::kN;
   dim3 block, grid;
-  int zper;
-  direct_shape(g, grid, block, zper);
-  if constexpr (NT <= kWideMaxTaps) {
+  DirectParams P{src, dst, g.nz, g.ny, g.nx, 1, wdev};
+  direct_shape(g, grid, block, P.zper);
+  bool done = false;
+  if constexpr (NDIM == 2 || (NDIM == 3 && RAD == 1)) {  // the classes that have the integer form
     if (wide.n) {
-      switch (mode) {
-        case 0: k_direct_wide<NT, 0><<<grid, block, 0, stream>>>(src, dst, g.nz, g.ny, g.nx, zper, tp, wide, wdev); break;
-        case 1: k_direct_wide<NT, 1><<<grid, block, 0, stream>>>(src, dst, g.nz, g.ny, g.nx, zper, tp, wide, wdev); break;
-        default: k_direct_wide<NT, 2><<<grid, block, 0, stream>>>(src, dst, g.nz, g.ny, g.nx, zper, tp, wide, wdev); break;
+      done = true;
+      if constexpr (!BOX && RAD == 1) {
+        if (wide.heat) k_direct_wide<NDIM, RAD, BOX, PERIODIC, true><<<grid, block, 0, stream>>>(P, wide);
+        else k_direct_wide<NDIM, RAD, BOX, PERIODIC, false><<<grid, block, 0, stream>>>(P, wide);
+      } else {
+        k_direct_wide<NDIM, RAD, BOX, PERIODIC, false><<<grid, block, 0, stream>>>(P, wide);
       }
-      g_launches.fetch_add(1, std::memory_order_relaxed);
-      return cudaGetLastError();
     }
   }
-  switch (mode) {
-    case 0: k_direct<NT, 0><<<grid, block, 0, stream>>>(src, dst, g.nz, g.ny, g.nx, zper, tp, wdev); break;
-    case 1: k_direct<NT, 1><<<grid, block, 0, stream>>>(src, dst, g.nz, g.ny, g.nx, zper, tp, wdev); break;
-    default: k_direct<NT, 2><<<grid, block, 0, stream>>>(src, dst, g.nz, g.ny, g.nx, zper, tp, wdev); break;
+  if (!done) {
+    if constexpr (NT == 125) {
+      Weights<NT> w;
+      for (int k = 0; k < NT; ++k) w.w[k] = ht.w[k];
+      k_direct_box125<PERIODIC><<<grid, block, 0, stream>>>(P, w);
+    } else {
+      k_direct<NDIM, RAD, BOX, PERIODIC><<<grid, block, 0, stream>>>(P);
+    }
   }
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
+}
+
+template <int NDIM, int RAD, bool BOX>
+cudaError_t launch_c(int boundary, const Geom& g, const HostTaps& ht, const WideTaps& wide, const double* wdev,
+                     const double* src, double* dst, cudaStream_t stream) {
+  if (ht.n != Taps<NDIM, RAD, BOX>::kN) return cudaErrorInvalidValue;
+  return boundary == kPeriodic ? launch_p<NDIM, RAD, BOX, true>(g, ht, wide, wdev, src, dst, stream)
+                               : launch_p<NDIM, RAD, BOX, false>(g, ht, wide, wdev, src, dst, stream);
 }
 
 }  // namespace
@@ -203,23 +303,20 @@ cudaError_t launch_nt(int mode, const Geom& g, const HostTaps& ht, const WideTap
 cudaError_t launch_direct(int ndim, int radius, Shape shape, int boundary, const Geom& g,
                           const HostTaps& taps, const WideTaps& wide, const double* wdev, const double* src, double* dst,
                           cudaStream_t stream) {
-  int mode = 0;
-  if (boundary == kPeriodic) {
-    bool small = g.nx < radius || (ndim >= 2 && g.ny < radius) || (ndim >= 3 && g.nz < radius);
-    mode = small ? 2 : 1;
-  }
-  switch (taps.n) {
-    case 3: return launch_nt<3>(mode, g, taps, wide, wdev, src, dst, stream);
-    case 5: return launch_nt<5>(mode, g, taps, wide, wdev, src, dst, stream);
-    case 7: return launch_nt<7>(mode, g, taps, wide, wdev, src, dst, stream);
-    case 9: return launch_nt<9>(mode, g, taps, wide, wdev, src, dst, stream);
-    case 13: return launch_nt<13>(mode, g, taps, wide, wdev, src, dst, stream);
-    case 25: return launch_nt<25>(mode, g, taps, wide, wdev, src, dst, stream);
-    case 27: return launch_nt<27>(mode, g, taps, wide, wdev, src, dst, stream);
-    case 125: return launch_nt<125>(mode, g, taps, wide, wdev, src, dst, stream);
+  const bool box = shape == Shape::kBox;
+  switch (ndim * 10 + radius) {
+    case 11: return launch_c<1, 1, false>(boundary, g, taps, wide, wdev, src, dst, stream);
+    case 12: return launch_c<1, 2, false>(boundary, g, taps, wide, wdev, src, dst, stream);
+    case 21: return box ? launch_c<2, 1, true>(boundary, g, taps, wide, wdev, src, dst, stream)
+                        : launch_c<2, 1, false>(boundary, g, taps, wide, wdev, src, dst, stream);
+    case 22: return box ? launch_c<2, 2, true>(boundary, g, taps, wide, wdev, src, dst, stream)
+                        : launch_c<2, 2, false>(boundary, g, taps, wide, wdev, src, dst, stream);
+    case 31: return box ? launch_c<3, 1, true>(boundary, g, taps, wide, wdev, src, dst, stream)
+                        : launch_c<3, 1, false>(boundary, g, taps, wide, wdev, src, dst, stream);
+    case 32: return box ? launch_c<3, 2, true>(boundary, g, taps, wide, wdev, src, dst, stream)
+                        : launch_c<3, 2, false>(boundary, g, taps, wide, wdev, src, dst, stream);
     default: return cudaErrorInvalidValue;
   }
-  (void)shape;
 }
 
 cudaError_t launch_direct_f32(int ndim, int radius, int boundary, const Geom& g, const HostTaps& taps,

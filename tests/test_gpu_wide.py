@@ -257,3 +257,34 @@ def test_a_few_values_among_zeros(st, shape, kind, radius, tuning, boundary):
     # relative to what a cell's neighbourhood holds: the largest value that reaches it
     top = oracle.run(np.abs(u0), (w > 0).astype(float), radius, boundary, T, nthreads=0)
     assert (np.abs(got - ref) <= T * (2 * taps + 2) * EPS * top + 60 * T * 5e-324).all()
+
+
+# axes of one, two and three cells (shorter than the radius and as long), and of a block and one more
+SHORT = [(1,), (2,), (257,), (1, 1), (2, 33), (9, 2), (3, 65), (1, 1, 1), (2, 1, 33), (1, 9, 2), (3, 2, 3), (4, 9, 33)]
+
+
+@pytest.mark.parametrize("kind", ["star", "box"])
+@pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
+@pytest.mark.parametrize("shape", SHORT)
+def test_cell_by_cell_on_short_axes(st, shape, boundary, kind):
+    for radius in (1, 2):
+        w = weights(kind, len(shape), radius)
+        u0 = synth.normal(34, shape)
+        T, taps = 3, int(np.count_nonzero(w))
+        ref = oracle.run(u0, w, radius, boundary, T, nthreads=0)
+        tol = T * (2 * taps + 2) * EPS * np.abs(u0).max()
+        got = run(st, u0, w, radius, boundary, T, (1, st.VARIANT_DIRECT))
+        assert np.abs(got - ref).max() <= tol, radius
+
+
+# the smallest that are streamed since, and the first with tiles of 16 rows
+@pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
+@pytest.mark.parametrize("shape,kind,radius", [((257, 129, 127), "star", 1), ((101, 103, 101), "box", 1),
+                                               ((257, 256), "star", 2), ((331, 297), "box", 2)])
+def test_smallest_streamed(st, shape, boundary, kind, radius):
+    w = weights(kind, len(shape), radius)
+    u0 = synth.normal(35, shape)
+    T, taps = 2, int(np.count_nonzero(w))
+    ref = oracle.run(u0, w, radius, boundary, T, nthreads=0)
+    got = run(st, u0, w, radius, boundary, T, (1, st.VARIANT_DIRECT))
+    assert np.abs(got - ref).max() <= T * (2 * taps + 2) * EPS * np.abs(u0).max()
