@@ -696,7 +696,7 @@ int run_steps(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, int variant,
       if (v == kVariantStream && p->ndim == 3 && p->wide.n)
         e = launch_wide3d(p->shape, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, tile_y, true,
                           chained);
-      else if (v == kVariantStream && p->ndim == 2 && p->wide.n && !(equal_box && p->radius == 1))
+      else if (v == kVariantStream && p->ndim == 2 && p->wide.n)
         e = launch_wide2d(p->shape, p->radius, p->boundary, p->g, p->wide, p->d_w, a, b, p->d_status, sms, s, true,
                           chained);
       else if (v == kVariantStream && p->ndim == 3)

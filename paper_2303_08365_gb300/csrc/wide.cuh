@@ -140,6 +140,21 @@ __device__ __forceinline__ long long wide_align(const WideVal& u, int d) {
   return a;
 }
 
+// R 2^x, rounded once to a double.
+__device__ __forceinline__ double wide_double(long long R, int x) {
+  // R to double: (2^84 + 2^63 + high) - (2^84 + 2^63 + 2^52) exactly, then one
+  // rounding when the low word (2^52 + low) is added.  As FMAs on registers,
+  // which run at the full FP64 rate (additions at 83%)
+  double one, off;
+  asm("mov.f64 %0, 0d3FF0000000000000;" : "=d"(one));
+  asm("mov.f64 %0, 0dC530000080100000;" : "=d"(off));
+  const double dh = __hiloint2double(0x45300000, (int)(R >> 32) ^ (int)0x80000000);
+  const double dl = __hiloint2double(0x43300000, (int)(unsigned int)R);
+  const double r = fma(dl, one, fma(dh, one, off));
+  const int h = __double2hiint(r);
+  return __hiloint2double(h != 0 ? h + (x << 20) : h, __double2loint(r));
+}
+
 // The accumulators of a cell: hh, hl, lh and ll count units of 2^57, 2^32, 2^26 and
 // 1 of S (27 taps: below 2^63 each).
 struct WideAcc {
@@ -194,18 +209,7 @@ struct WideAcc {
   // The sum as a double.
   template <class Taps>
   __device__ __forceinline__ double get(int E, const Taps& T) const {
-    const long long R = rounded();
-    // R to double: (2^84 + 2^63 + high) - (2^84 + 2^63 + 2^52) exactly, then one
-    // rounding when the low word (2^52 + low) is added.  As FMAs on registers,
-    // which run at the full FP64 rate (additions at 83%)
-    double one, off;
-    asm("mov.f64 %0, 0d3FF0000000000000;" : "=d"(one));
-    asm("mov.f64 %0, 0dC530000080100000;" : "=d"(off));
-    const double dh = __hiloint2double(0x45300000, (int)(R >> 32) ^ (int)0x80000000);
-    const double dl = __hiloint2double(0x43300000, (int)(unsigned int)R);
-    const double r = fma(dl, one, fma(dh, one, off));
-    const int h = __double2hiint(r);
-    return __hiloint2double(h != 0 ? h + ((E - T.bias) << 20) : h, __double2loint(r));
+    return wide_double(rounded(), E - T.bias);
   }
 };
 
@@ -259,6 +263,36 @@ __device__ __forceinline__ double wide_sum_heat(const WideVal (&u)[NT], const Ta
   const int E = wide_acc_heat<NT>(u, T, acc);
   ok = wide_covers(E, T);
   return acc.get(E, T);
+}
+
+// Boxes whose weights are all equal: the values of a block of cells are aligned to one
+// exponent E, the largest of the block, and added as integers; a cell's sum S takes one
+// multiplication.  S counts units of 2^-(61 - kEqualShift) of the largest value, up to
+// (2 RAD + 1)^2 < 2^(kEqualShift + 2) of which fit; the bits that the values lose, a unit at
+// most each, are centred by the first summand (half a unit for every
+// value), which also lets values that cancel exactly sum to zero.
+template <int RAD>
+constexpr int kEqualShift = RAD == 1 ? 3 : 4;
+template <int RAD>
+constexpr int kEqualFirst = RAD == 1 ? 4 : 12;
+// How far below the block's a cell's own largest exponent may lie.  Then a unit is 2^-55
+// (RAD 1) or 2^-55 (RAD 2) of the cell's own largest value, and the 9 (25) lost parts add
+// up to 0.9 (1.4) units on average, against half a unit of 2^-52 of the result that its
+// rounding takes.
+template <int RAD>
+constexpr int kEqualGap = RAD == 1 ? 3 : 2;
+
+// w S as a double, w the weights' one value.
+template <int RAD, class Taps>
+__device__ __forceinline__ double wide_equal(long long S, int E, const Taps& T) {
+  const int ah = (int)(S >> 32), lo = T.lo[0];
+  const unsigned int al = (unsigned int)S;
+  // units of 2^56, 2^32, 2^26 and 1 of S W
+  const long long hh = (long long)ah * (2 * T.hi2[0]);
+  const unsigned long long ll = (unsigned long long)al * (unsigned int)lo;
+  const unsigned long long lh = (unsigned long long)al * (unsigned int)T.hi[0] + (ll >> 26);
+  const long long hl = (long long)ah * lo + ((1 << 23) + (long long)(lh >> 6));
+  return wide_double(hh + (hl >> 24), E - T.bias + kEqualShift<RAD> - 1);
 }
 
 // The same with the FMA chain in its place where it has to be.

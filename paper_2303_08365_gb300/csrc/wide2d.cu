@@ -16,7 +16,10 @@
 // The rows between two tiles are unpacked twice (18 or 20 rows for 16).
 //
 // Measured at 8192^2, periodic, general weights (FMA chain before): 25-point box
-// 52 GStencil/s (23.6), radius-2 star 113 (67).
+// 52 GStencil/s (23.6), radius-2 star 113 (67).  Boxes whose weights are all equal
+// share alignments and partial sums among a lane's four cells (wide_equal): 9-point
+// box at 16384^2 225 GStencil/s (140 with shared sums on the FP64 pipe), 25-point box
+// at 8192^2 139 (24), 512^2 43 (14).
 //
 // Work split: the tiles are cut into equal contiguous ranges, one per CTA.
 #include <cudaTypedefs.h>
@@ -153,11 +156,44 @@ __device__ __noinline__ void chain_cells(const Plane<RAD>& u, int row0, int rows
     }
 }
 
-template <bool BOX, int RAD>
-constexpr int wide2d_ctas() { return RAD == 1 && !BOX ? 3 : 2; }
+// A lane's cells one by one, each aligned to its own largest exponent: where the block's
+// lies too far above.  Out of line: rarely run.
+template <int RAD>
+__device__ __noinline__ void own_cells(const Plane<RAD>& u, int row0, int rows, int c0, const WideTaps& T,
+                                       const double* wdev, double* out, int nx) {
+  for (int r = 0; r < rows; ++r)
+    for (int i = 0; i < 2; ++i) {
+      const int row = row0 + r, c = c0 + i;
+      unsigned int any = 0;
+      int E = 0;
+      for (int dy = -RAD; dy <= RAD; ++dy)
+        for (int dx = -RAD; dx <= RAD; ++dx) {
+          const WideVal x = get(&u.m[row + dy][c + dx], &u.e[row + dy][c + dx]);
+          any |= wide_nonzero(x);
+          E = max(E, x.e);
+        }
+      double v = 0.0;
+      if (any != 0 && !wide_covers(E, T)) {
+        v = chain_cell<true, RAD>(u, row, c, wdev);
+      } else if (any != 0) {
+        WideAcc acc;
+        for (int dy = -RAD; dy <= RAD; ++dy)
+          for (int dx = -RAD; dx <= RAD; ++dx) {
+            const WideVal x = get(&u.m[row + dy][c + dx], &u.e[row + dy][c + dx]);
+            acc.add(x, 0, E - x.e, T);
+          }
+        v = acc.get(E, T);
+      }
+      out[(int64_t)r * nx + i] = v;
+    }
+}
 
+template <bool BOX, int RAD, bool HEAT>
+constexpr int wide2d_ctas() { return RAD == 1 && (!BOX || HEAT) ? 3 : 2; }
+
+// HEAT: a star whose weights wide_sum_heat takes; a box whose weights are all equal.
 template <bool BOX, int RAD, bool HEAT, bool PERIODIC, bool TMA>
-__global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(const __grid_constant__ Params P) {
+__global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_wide2d(const __grid_constant__ Params P) {
   constexpr int kRows = kTC + 2 * RAD;
   constexpr unsigned long long kWaitNs = (unsigned long long)kSpinLimitNs;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -376,6 +412,63 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(
           }
           store(r, v[0], v[1]);
         }
+      } else if constexpr (HEAT) {
+        // equal weights, the lane's two rows and columns as one block: each value is
+        // aligned once for the four cells, and rows (mid: their common columns) and
+        // columns share their partial sums
+        constexpr int N = 2 * RAD + 2;
+        static_assert(kR == 2 && TMA, "the block; columns and rows outside the grid hold values or zeros");
+        int E = 0, own[2][2], e[N][N];  // the block's largest exponent, the cells' own
+#pragma unroll
+        for (int r = 0; r < N; ++r) {
+          const int* er = &u.e[row0 - RAD + r][c];
+#pragma unroll
+          for (int k = 0; k < RAD + 1; ++k) {
+            if (RAD == 1 && k != 0) continue;
+            const int2 m = *reinterpret_cast<const int2*>(er + (RAD == 1 ? 0 : 2 * k - 2));
+            e[r][RAD == 1 ? 1 : 2 * k] = m.x;
+            e[r][RAD == 1 ? 2 : 2 * k + 1] = m.y;
+          }
+          if (RAD == 1) {
+            e[r][0] = er[-1];
+            e[r][3] = er[2];
+          }
+          int mid = e[r][1];
+#pragma unroll
+          for (int k = 2; k < N - 1; ++k) mid = max(mid, e[r][k]);
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int h = max(mid, e[r][i * (N - 1)]);
+            if (r < N - 1) own[0][i] = r == 0 ? h : max(own[0][i], h);
+            if (r > 0) own[1][i] = r == 1 ? h : max(own[1][i], h);
+          }
+        }
+        E = max(max(own[0][0], own[0][1]), max(own[1][0], own[1][1]));
+        int least = min(own[0][0], own[0][1]);
+        if (rows > 1) least = min(least, min(own[1][0], own[1][1]));
+        all = rows <= 0 || (wide_covers(E, P.wide) && wide_covers(least, P.wide) && E - least <= kEqualGap<RAD>);
+        long long S[2][2], both[2] = {kEqualFirst<RAD>, kEqualFirst<RAD>};  // both: of the rows that both read
+        E += kEqualShift<RAD>;
+        if (RAD > 1) asm volatile("" ::: "memory");  // 36 exponents would not fit the registers: read again
+#pragma unroll
+        for (int r = 0; r < N; ++r) {
+          WideVal v[N];
+          get_row<RAD>(u, row0 - RAD + r, c, v);
+          long long mid = wide_align(v[1], E - v[1].e);
+#pragma unroll
+          for (int k = 2; k < N - 1; ++k) mid += wide_align(v[k], E - v[k].e);
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const long long h = mid + wide_align(v[i * (N - 1)], E - v[i * (N - 1)].e);
+            if (r == 0) S[0][i] = h;
+            else if (r < N - 1) both[i] += h;
+            else S[1][i] = h;
+          }
+        }
+        E -= kEqualShift<RAD>;
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+          store(r, wide_equal<RAD>(S[r][0] + both[0], E, P.wide), wide_equal<RAD>(S[r][1] + both[1], E, P.wide));
       } else {
         // row by row; the largest exponents first, then the sums: a pair's values would
         // not fit the registers, so their rows are read twice
@@ -420,8 +513,10 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD>())) k_wide2d(
           store(r, acc[0].get(E[0], P.wide), acc[1].get(E[1], P.wide));
         }
       }
-      if (!all && !zero_cells<BOX, RAD>(u, row0, rows, min(2, P.nx - xa), c, out, P.nx))
-        chain_cells<BOX, RAD>(u, row0, rows, min(2, P.nx - xa), c, P.wide, P.wdev, out, P.nx);
+      if (!all && !zero_cells<BOX, RAD>(u, row0, rows, min(2, P.nx - xa), c, out, P.nx)) {
+        if constexpr (BOX && HEAT) own_cells<RAD>(u, row0, rows, c, P.wide, P.wdev, out, P.nx);
+        else chain_cells<BOX, RAD>(u, row0, rows, min(2, P.nx - xa), c, P.wide, P.wdev, out, P.nx);
+      }
       __syncwarp();
     }
     if (t < t1) next();
@@ -494,8 +589,15 @@ cudaError_t launch_wide2d(Shape shape, int radius, int boundary, const Geom& g, 
                           const double* wdev, const double* src, double* dst, int* status, int sms,
                           cudaStream_t stream, bool tma, bool chained) {
   const bool per = boundary == kPeriodic, box = shape == Shape::kBox;
-  const int side = 2 * radius + 1;
+  const int side = 2 * radius + 1, mid = wide.n / 2;
   if (wide.n != (box ? side * side : 4 * radius + 1)) return cudaErrorInvalidValue;
+  if (box && tma && wide.heat && wide.hi[mid] == wide.hi[0] && wide.lo[mid] == wide.lo[0] && wide.ex[mid] == wide.ex[0]) {
+    if (radius == 2)
+      return per ? launch_t<true, 2, true, true, true>(g, wide, wdev, src, dst, status, sms, stream, chained)
+                 : launch_t<true, 2, true, false, true>(g, wide, wdev, src, dst, status, sms, stream, chained);
+    return per ? launch_t<true, 1, true, true, true>(g, wide, wdev, src, dst, status, sms, stream, chained)
+               : launch_t<true, 1, true, false, true>(g, wide, wdev, src, dst, status, sms, stream, chained);
+  }
   if (radius == 2)
     return box ? launch_p<true, 2, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained)
                : launch_p<false, 2, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained);

@@ -288,3 +288,56 @@ def test_smallest_streamed(st, shape, boundary, kind, radius):
     ref = oracle.run(u0, w, radius, boundary, T, nthreads=0)
     got = run(st, u0, w, radius, boundary, T, (1, st.VARIANT_DIRECT))
     assert np.abs(got - ref).max() <= T * (2 * taps + 2) * EPS * np.abs(u0).max()
+
+
+def equal_weights(ndim, radius):
+    return np.full((2 * radius + 1,) * ndim, 1.0 / (2 * radius + 1) ** ndim)
+
+
+@pytest.mark.parametrize("spread", [0, 3, 60])
+@pytest.mark.parametrize("radius", [1, 2])
+def test_equal_box_against_exact_arithmetic(st, radius, spread):
+    """The equal-weight boxes align the values of four cells to one exponent, at most 3 (2)
+    above a cell's own: 5 (13) units of 2^-55 and half a unit of the product, 2^-52, of the
+    cell's largest product, and one rounding of the result."""
+    rng = np.random.default_rng(spread + radius)
+    u0 = rng.standard_normal((19, 70)) * 2.0 ** rng.integers(-spread, spread + 1, (19, 70))
+    u0[rng.random(u0.shape) < 0.1] = 0.0
+    w = equal_weights(2, radius)
+    got = run(st, u0, w, radius, DIRICHLET, 1, (1, st.VARIANT_STREAM))
+    slack = Fraction((5 if radius == 1 else 13) * 2.0 ** -55 + 2.0 ** -52)
+    for at in np.ndindex(*u0.shape):
+        want, top = exact_sum(u0, w, at, radius)
+        assert abs(Fraction(float(got[at])) - want) <= abs(want) * Fraction(EPS) + top * slack, at
+
+
+@pytest.mark.parametrize("shape,boundary", [((1, 2), DIRICHLET), ((17, 66), DIRICHLET), ((15, 62), DIRICHLET),
+                                            ((16, 64), PERIODIC), ((48, 192), PERIODIC), ((643, 1286), DIRICHLET)])
+@pytest.mark.parametrize("radius", [1, 2])
+def test_equal_box_tiles(st, shape, boundary, radius):
+    w = equal_weights(2, radius)
+    taps, T = w.size, 3
+    for u0 in (synth.normal(36, shape), np.where(synth.uniform(37, shape) < 0.003, synth.normal(38, shape), 0.0)):
+        ref = oracle.run(u0, w, radius, boundary, T, nthreads=0)
+        got = run(st, u0, w, radius, boundary, T, (1, st.VARIANT_STREAM))
+        assert np.abs(got - ref).max() <= T * (2 * taps + 2) * EPS * np.abs(u0).max()
+        assert np.array_equal(got == 0.0, ref == 0.0)
+
+
+@pytest.mark.parametrize("radius", [1, 2])
+def test_equal_box_values_outside_the_integer_range(st, radius):
+    rng = np.random.default_rng(10)
+    w = equal_weights(2, radius)
+    for values in ([np.inf, 1.0], [np.nan, 1.0], [-np.inf, np.inf, 0.0], [1.7e308, -1.2e308, 3.0],
+                   [5e-324, -3e-310, 0.0], [2.3e-308, 0.0], [0.0, -0.0]):
+        u0 = np.zeros((19, 70))
+        mask = rng.random(u0.shape) < 0.05
+        u0[mask] = rng.choice(values, int(mask.sum()))
+        with np.errstate(all="ignore"):
+            ref = oracle.run(u0, w, radius, DIRICHLET, 1, nthreads=1)
+            got = run(st, u0, w, radius, DIRICHLET, 1, (1, st.VARIANT_STREAM))
+            assert np.array_equal(np.isnan(got), np.isnan(ref)), values
+            fine = np.isfinite(ref)
+            assert np.array_equal(got[~fine & ~np.isnan(ref)], ref[~fine & ~np.isnan(ref)]), values
+            top = np.abs(u0[np.isfinite(u0)]).max() if np.isfinite(u0).any() else 0.0
+            assert np.abs(got[fine] - ref[fine]).max(initial=0.0) <= max(60 * EPS * top, 60 * 5e-324), values
