@@ -225,7 +225,7 @@ void build_taps(stencil_plan_s* p, const double* w) {
 // The stencil classes whose kernels have the integer form of the sum.  All
 // kernels of a class take it, so its results do not depend on the kernel.
 bool uses_wide(int ndim, int radius) {
-  return (ndim == 3 && radius == 1) || ndim == 2;
+  return (ndim == 3 && radius == 1) || ndim <= 2;
 }
 
 // Whether a grid that the TMA-fed kernels do not take is streamed all the same
@@ -389,7 +389,7 @@ int default_variant(const stencil_plan_s* p, int* Tb = nullptr) {
   }
   if (p->ndim == 2 && p->radius == 2) return stream2d ? kVariantStream : kVariantDirect;
   if (p->ndim == 1) {
-    if (Tb) *Tb = 8;  // 8 steps per launch in shared memory, 0.4-0.8% halo recompute
+    if (Tb) *Tb = 8;  // 8 steps per launch
     return kVariantTemporal;
   }
   return kVariantDirect;
@@ -686,6 +686,11 @@ int run_steps(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, int variant,
       if (rc) return rc;
       e = cudaSuccess;
       steps = Tb;
+    } else if (variant == kVariantTemporal && p->ndim == 1 && p->wide.n) {
+      WideTapsOf<5> wide;
+      make_wide(p->taps.w, p->taps.n, wide);
+      steps = (int)std::min<int64_t>(Tb, T - t);
+      e = launch_wide1d(p->radius, p->boundary, steps, p->g, wide, p->d_w, a, b, sms, s);
     } else if (variant == kVariantTemporal && T - t >= Tb) {
       e = launch_temporal(p->ndim, p->radius, p->shape, p->boundary, Tb, p->g, p->wide, p->d_w, a, b, sms, s,
                           equal_box && p->ndim == 2 && p->radius == 1);

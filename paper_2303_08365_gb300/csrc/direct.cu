@@ -266,7 +266,7 @@ cudaError_t launch_p(const Geom& g, const HostTaps& ht, const WideTaps& wide, co
   DirectParams P{src, dst, g.nz, g.ny, g.nx, 1, wdev};
   direct_shape(g, grid, block, P.zper);
   bool done = false;
-  if constexpr (NDIM == 2 || (NDIM == 3 && RAD == 1)) {  // the classes that have the integer form
+  if constexpr (NDIM <= 2 || RAD == 1) {  // the classes that have the integer form
     if (wide.n) {
       done = true;
       if constexpr (!BOX && RAD == 1) {

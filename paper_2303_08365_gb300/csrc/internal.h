@@ -131,6 +131,12 @@ cudaError_t launch_wide2d(Shape shape, int radius, int boundary, const Geom& g, 
                           const double* wdev, const double* src, double* dst, int* status, int sms,
                           cudaStream_t stream, bool tma, bool chained = false);
 
+// 1D sweep (radius 1 or 2) with the weighted sum in the integer form (wide.n != 0),
+// `steps` fused steps (at most kWide1dSteps).
+constexpr int kWide1dSteps = 8;
+cudaError_t launch_wide1d(int radius, int boundary, int steps, const Geom& g, const WideTapsOf<5>& wide,
+                          const double* wdev, const double* src, double* dst, int sms, cudaStream_t stream);
+
 // Temporal blocking: Tb fused steps per launch (2D and 3D: radius 1, any
 // shape and boundary; 1D: radius 1 or 2; Tb in {2, 4, 8}).
 bool temporal_supported(int ndim, int radius, int Tb);

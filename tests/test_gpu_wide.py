@@ -341,3 +341,37 @@ def test_equal_box_values_outside_the_integer_range(st, radius):
             assert np.array_equal(got[~fine & ~np.isnan(ref)], ref[~fine & ~np.isnan(ref)]), values
             top = np.abs(u0[np.isfinite(u0)]).max() if np.isfinite(u0).any() else 0.0
             assert np.abs(got[fine] - ref[fine]).max(initial=0.0) <= max(60 * EPS * top, 60 * 5e-324), values
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 31, 47, 48, 49, 385, 65535, 65537, 65536 + 7 * 8 * 112, (1 << 20) - 1, (1 << 20) + 12345])
+@pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
+def test_fused_1d_equals_single_steps(st, n, boundary):
+    """Warps of 64, 128 and 256 cells, the last one ragged; 11 steps as 8 and 3."""
+    for radius, w in ((1, synth.heat_weights(1, 0.2)), (1, weights("star", 1, 1)), (2, weights("star", 1, 2))):
+        u0 = synth.normal(39, (n,))
+        got = run(st, u0, w, radius, boundary, 11)
+        assert np.array_equal(got, run(st, u0, w, radius, boundary, 11, (1, st.VARIANT_DIRECT))), radius
+        ref = oracle.run(u0, w, radius, boundary, 11, nthreads=0)
+        assert np.abs(got - ref).max() <= 11 * (2 * w.size + 2) * EPS * np.abs(u0).max(), radius
+
+
+@pytest.mark.parametrize("values", [[np.inf, 1.0], [np.nan, 1.0], [-np.inf, np.inf, 0.0], [1.7e308, -1.2e308, 3.0],
+                                    [5e-324, -3e-310, 0.0], [2.3e-308, 0.0], [0.0, -0.0]])
+def test_fused_1d_values_outside_the_integer_range(st, values):
+    rng = np.random.default_rng(11)
+    for radius in (1, 2):
+        w = weights("star", 1, radius)
+        u0 = np.zeros(1500)
+        mask = rng.random(u0.shape) < 0.02
+        u0[mask] = rng.choice(values, int(mask.sum()))
+        for T in (1, 8):
+            got = run(st, u0, w, radius, DIRICHLET, T)
+            assert same(got, run(st, u0, w, radius, DIRICHLET, T, (1, st.VARIANT_DIRECT))), (radius, T)
+        with np.errstate(all="ignore"):
+            ref = oracle.run(u0, w, radius, DIRICHLET, 1, nthreads=1)
+            got = run(st, u0, w, radius, DIRICHLET, 1)
+            assert np.array_equal(np.isnan(got), np.isnan(ref))
+            fine = np.isfinite(ref)
+            assert np.array_equal(got[~fine & ~np.isnan(ref)], ref[~fine & ~np.isnan(ref)])
+            top = np.abs(u0[np.isfinite(u0)]).max() if np.isfinite(u0).any() else 0.0
+            assert np.abs(got[fine] - ref[fine]).max(initial=0.0) <= max(60 * EPS * top, 60 * 5e-324)
