@@ -508,19 +508,24 @@ void tune_on_first_run(stencil_plan_s* p, const double* d_grid, cudaStream_t s) 
   cudaFree(scratch);
 }
 
+// The flags (progress words) of up to `tiles` tiles (grown on demand).
+int ensure_flags(stencil_plan_s* p, int tiles) {
+  if (p->flags_cap >= tiles) return STENCIL_OK;
+  cudaFree(p->d_flags);
+  p->d_flags = nullptr;
+  p->flags_cap = 0;
+  CUDA_TRY(dev_malloc(&p->d_flags, (size_t)tiles * kFlagWords * sizeof(unsigned int)), "allocating the tile flags");
+  p->flags_cap = tiles;
+  return STENCIL_OK;
+}
+
 // Persistent temporal kernel: Tb steps in shared memory per exchange, tiles
 // synchronised by per-tile flags, one launch for all T steps.
 int run_persistent_tb(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, cudaStream_t s) {
   PersistTbLaunch L;
   persist_tiling(p->g.ny, p->g.nx, Tb, sm_count(), &L.tiles_y, &L.tiles_x, &L.reach_y, &L.reach_x);
   const int ntiles = L.tiles_y * L.tiles_x;
-  if (p->flags_cap < ntiles) {
-    cudaFree(p->d_flags);
-    p->d_flags = nullptr;
-    p->flags_cap = 0;
-    CUDA_TRY(dev_malloc(&p->d_flags, (size_t)ntiles * kFlagWords * sizeof(unsigned int)), "allocating the tile flags");
-    p->flags_cap = ntiles;
-  }
+  if (const int rc = ensure_flags(p, ntiles)) return rc;
   CUDA_TRY(cudaMemsetAsync(p->d_flags, 0, (size_t)ntiles * kFlagWords * sizeof(unsigned int), s), "clearing the tile flags");
   L.a = d_grid;
   L.b = p->d_tmp;
@@ -562,6 +567,43 @@ int run_wide_steps(stencil_plan_s* p, double* d_grid, int64_t T, cudaStream_t s)
   L.spin_limit = kSpinLimitNs;
   cudaError_t e = launch_wide_steps(L, L.one.ntiles, p->boundary, sm_count(), s);
   if (e != cudaSuccess) return cuda_fail(e, "launching the persistent step kernel");
+  return STENCIL_OK;
+}
+
+// Whether a 3D run whose kernel nobody chose takes all its steps in one persistent launch
+// (steps3d.cu): 7-point grids of at most a brick per SM (us a step: 64^3 4.3 against 7.1,
+// 24^3 2.5 / 4.4; of three steps 10 / 12 and 8.3 / 9.8, so that two are left as they
+// were).  z: the brick's cells per thread.
+// The progress words are allocated by the first run of whatever length; a stream that is
+// being captured before there was one takes a launch per step.
+bool steps3d_anyway(stencil_plan_s* p, bool tuned, int tile_y, cudaStream_t s, Steps3dLaunch& L, int& z) {
+  if (tuned || tile_y || p->user_Tb > 0 || p->user_variant > 0 || p->ndim != 3 || p->wide.n != 7) return false;
+  z = steps3d_cut(p->g, sm_count(), L.bricks);
+  if (z == 0) return false;
+  const int bricks = L.bricks[0] * L.bricks[1] * L.bricks[2];
+  if (p->flags_cap >= bricks) return true;
+  cudaStreamCaptureStatus capture;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return false;
+  return ensure_flags(p, bricks) == STENCIL_OK;
+}
+
+int run_steps3d(stencil_plan_s* p, double* d_grid, int64_t T, Steps3dLaunch& L, int z, cudaStream_t s) {
+  const size_t bytes = (size_t)L.bricks[0] * L.bricks[1] * L.bricks[2] * kFlagWords * sizeof(unsigned int);
+  CUDA_TRY(cudaMemsetAsync(p->d_flags, 0, bytes, s), "clearing the progress words");
+  L.a = d_grid;
+  L.b = p->d_tmp;
+  L.nz = p->g.nz;
+  L.ny = p->g.ny;
+  L.nx = p->g.nx;
+  L.periodic = p->boundary == kPeriodic;
+  L.T = (int)T;
+  L.wdev = p->d_w;
+  make_wide(p->taps.w, 7, L.wide);
+  L.progress = p->d_flags;
+  L.status = p->d_status;
+  L.spin_limit = kSpinLimitNs;
+  cudaError_t e = launch_steps3d(L, z, s);
+  if (e != cudaSuccess) return cuda_fail(e, "launching the persistent 3D kernel");
   return STENCIL_OK;
 }
 
@@ -768,6 +810,10 @@ int run_const(stencil_plan_s* p, double* d_grid, int64_t T, cudaStream_t s) {
     variant = kVariantDirect;
   }
   if (!tuned && streams_anyway(p, Tb, variant, stream_ok)) variant = kVariantStream;
+  Steps3dLaunch steps3d;
+  int z;
+  if (steps3d_anyway(p, tuned, tile_y, s, steps3d, z) && T > 2 && T <= (1 << 30))
+    return run_steps3d(p, d_grid, T, steps3d, z, s);
   if (variant == kVariantPersistent && Tb > 1) {
     if (p->ndim == 2 && p->radius == 1 && (p->taps.n == 5 || p->taps.n == 9) && Tb <= 8)
       return run_persistent_tb(p, d_grid, T, Tb, s);

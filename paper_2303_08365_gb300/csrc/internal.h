@@ -137,6 +137,25 @@ constexpr int kWide1dSteps = 8;
 cudaError_t launch_wide1d(int radius, int boundary, int steps, const Geom& g, const WideTapsOf<5>& wide,
                           const double* wdev, const double* src, double* dst, int sms, cudaStream_t stream);
 
+// All steps of a small 3D 7-point grid in one cooperative launch, one brick per SM (wide.n == 7).
+struct Steps3dLaunch {
+  double* a;        // the caller's grid
+  double* b;        // partner buffer
+  int nz, ny, nx;
+  int periodic;
+  int T;
+  int bricks[3];    // along x, y, z
+  const double* wdev;
+  WideTapsOf<7> wide;
+  unsigned int* progress;  // kFlagWords words for each brick, zero before the launch
+  int* status;
+  long long spin_limit;    // ns
+};
+// Cuts a grid into at most `sms` bricks; returns their cells per thread (launch_steps3d's
+// z), 0 when the grid is too large.
+int steps3d_cut(const Geom& g, int sms, int (&bricks)[3]);
+cudaError_t launch_steps3d(const Steps3dLaunch& L, int z, cudaStream_t stream);
+
 // Temporal blocking: Tb fused steps per launch (2D and 3D: radius 1, any
 // shape and boundary; 1D: radius 1 or 2; Tb in {2, 4, 8}).
 bool temporal_supported(int ndim, int radius, int Tb);

@@ -375,3 +375,56 @@ def test_fused_1d_values_outside_the_integer_range(st, values):
             assert np.array_equal(got[~fine & ~np.isnan(ref)], ref[~fine & ~np.isnan(ref)])
             top = np.abs(u0[np.isfinite(u0)]).max() if np.isfinite(u0).any() else 0.0
             assert np.abs(got[fine] - ref[fine]).max(initial=0.0) <= max(60 * EPS * top, 60 * 5e-324)
+
+
+# one brick of 32 x 8 x 16 cells and less, bricks of unequal sizes, every depth (2 to 16), the
+# largest cuts that are taken in one launch (152 bricks) and one beyond
+BRICKS = [(1, 1, 1), (1, 1, 2), (2, 3, 4), (3, 9, 33), (16, 8, 32), (17, 8, 32), (5, 17, 65), (64, 64, 64), (65, 65, 65),
+          (33, 47, 61), (40, 150, 127), (299, 16, 31), (70, 80, 90), (113, 28, 118)]
+
+
+@pytest.mark.parametrize("kind", ["heat", "star"])
+@pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
+@pytest.mark.parametrize("shape", BRICKS)
+def test_persistent_bricks_equal_single_steps(st, shape, boundary, kind):
+    w = synth.heat_weights(3, 0.12) if kind == "heat" else weights("star", 3, 1)
+    u0 = synth.normal(40, shape)
+    for T in (3, 8, 31):
+        want = run(st, u0, w, 1, boundary, T, (1, st.VARIANT_DIRECT))
+        for offset in (0, 1):
+            assert np.array_equal(run(st, u0, w, 1, boundary, T, (0, 0), offset), want), (T, offset)
+
+
+@pytest.mark.parametrize("values", [[np.inf, 1.0], [np.nan, 1.0], [-np.inf, np.inf, 0.0], [1.7e308, -1.2e308, 3.0],
+                                    [5e-324, -3e-310, 0.0], [2.3e-308, 0.0], [0.0, -0.0], [1.0, 0.0]])
+def test_persistent_bricks_values_outside_the_integer_range(st, values):
+    rng = np.random.default_rng(12)
+    w = weights("star", 3, 1)
+    u0 = np.zeros((11, 13, 40))
+    mask = rng.random(u0.shape) < 0.01
+    u0[mask] = rng.choice(values, int(mask.sum()))
+    for T in (3, 4):
+        got = run(st, u0, w, 1, DIRICHLET, T)
+        assert same(got, run(st, u0, w, 1, DIRICHLET, T, (1, st.VARIANT_DIRECT))), T
+
+
+def test_persistent_bricks_under_capture(st):
+    """A graph captured after a run, replayed on new data; and one captured before there was any."""
+    import torch
+    w = synth.heat_weights(3, 0.12)
+    fields = [synth.uniform(41 + k, (33, 20, 40)) for k in range(2)]
+    g = torch.from_numpy(fields[0].copy()).cuda()
+    p = st.Plan(fields[0].shape, 1, w, PERIODIC)
+    p.run(g, 1)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        p.run(g, 9)
+    for u in fields:
+        g.copy_(torch.from_numpy(u))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(g.cpu().numpy(), run(st, u, w, 1, PERIODIC, 9, (1, st.VARIANT_DIRECT)))
+    assert p.status() == 0
+    p.close()
