@@ -3,7 +3,7 @@
 //
 // Operation: steps of u'(x) = sum_o w_o u~(x+o) (paper Sec. 2.1, Listing 1), blocked in
 // time (Sec. 4.1).  The integer pipes bound it (112 instructions a cell and step, two thirds
-// of them on the ALU pipe, 64% busy), where the FMA chain was bound by the FP64 pipe.
+// of them on the ALU pipe), where the FMA chain was bound by the FP64 pipe.
 // Values stay unpacked, in registers, from the first step to the last: a warp owns 32 C consecutive cells, C on each lane,
 // steps * R of them on either side a halo that goes wrong from the outside in; a
 // lane takes the R values beyond its ends from its neighbours by shuffles, and the sums are
@@ -12,9 +12,10 @@
 // time within 1%.)  Shared memory only turns the rows of 32 that global memory likes into the lanes' runs of C.
 //
 // Us a step, radius 1 (before, by the FMA chain from shared memory, single steps at the end of
-// a run): 10^3 cells 1.2 (2.8), 60 000 1.3 (3.0), 220 000 2.5 (3.0), 10^6 6.3 (7.4), 10^7
-// 50 (55).  C, us a step at radius 1: 20 000 cells 2: 1.0, 4: 1.5; 220 000 2.4 / 2.6 (radius
-// 2 4.0 / 3.4); 10^6 4: 6.3, 8: 6.4; 10^7 51.5 / 49.7, 16: 51.7.
+// a run): 10^3 cells 1.2 (2.8), 60 000 1.3 (3.0), 220 000 2.5 (3.0), 10^6 5.3 (7.4), 10^7
+// 43 (55; 50 with the cells that the integer form does not take told apart one by one).
+// C, us a step at radius 1: 20 000 cells 2: 1.0, 4: 1.5; 220 000 2.4 / 2.6 (radius
+// 2 4.0 / 3.4); 10^6 4: 5.3, 8: 5.8 (radius 2 8.5 / 7.7); 10^7 42.8 / 43.2 (74.9 / 63.9).
 #include "internal.h"
 #include "wide.cuh"
 
@@ -72,29 +73,43 @@ __global__ void __launch_bounds__(kThreads1d, 2)
       const WideVal& h = u[r];
       after[r] = {__shfl_down_sync(kAll, h.hi, 1), __shfl_down_sync(kAll, h.lo, 1), __shfl_down_sync(kAll, h.e, 1)};
     }
+    auto near = [&](int j, WideVal (&v)[NT]) {  // the values that cell j reads
+#pragma unroll
+      for (int k = 0; k < NT; ++k) {
+        const int q = j + k - R;
+        v[k] = q < 0 ? before[q < 0 ? q + R : 0] : q < C ? u[q < 0 || q >= C ? 0 : q] : after[q < C ? 0 : q - C];
+      }
+    };
+    // all cells first, without a branch between them, which would keep them apart
+    WideVal w[C];
+    unsigned int other = 0;
 #pragma unroll
     for (int j = 0; j < C; ++j) {
       WideVal v[NT];
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        v[r] = before[r];
-        v[R + 1 + r] = j + 1 + r < C ? u[j + 1 + r < C ? j + 1 + r : 0] : after[j + 1 + r < C ? 0 : j + 1 + r - C];
-      }
-      v[R] = u[j];
-#pragma unroll
-      for (int r = 0; r + 1 < R; ++r) before[r] = before[r + 1];
-      before[R - 1] = u[j];
+      near(j, v);
       WideAcc acc;
       int E;
       if constexpr (HEAT) E = wide_acc_heat<NT>(v, T, acc);
       else E = wide_acc<NT>(v, T, acc);
-      WideVal w = acc.val(E, T);
-      if (!wide_covers(E, T)) w = wide_zeros<NT>(v) ? wide_unpack(0.0) : chain_cell<NT>(v, wdev);
+      w[j] = acc.val(E, T);
+      if (!wide_covers(E, T)) other |= 1u << j;
+    }
+    if (other != 0) {
+#pragma unroll
+      for (int j = 0; j < C; ++j)
+        if (other >> j & 1) {
+          WideVal v[NT];
+          near(j, v);
+          w[j] = wide_zeros<NT>(v) ? wide_unpack(0.0) : chain_cell<NT>(v, wdev);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+      u[j] = w[j];
       if (!PERIODIC && !inside) {
         const long long x = x0 + lane * C + j;
-        if (x < 0 || x >= n) w = wide_unpack(0.0);  // a ghost stays zero
+        if (x < 0 || x >= n) u[j] = wide_unpack(0.0);  // a ghost stays zero
       }
-      u[j] = w;
     }
   }
 #pragma unroll
