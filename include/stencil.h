@@ -145,6 +145,21 @@ int stencil_adjoint_vjp(stencil_plan p, const double* d_u0, const double* d_kapp
                         int64_t T, int ckpt_every, const double* d_lambda_T, double* d_grad_u0,
                         double* d_grad_kappa, void* cuda_stream);
 
+/* The pair for a caller that needs u^T first and the gradients later (an
+ * autograd forward and backward): the forward sweep of a variable-coefficient
+ * plan from d_u0, which it leaves alone, to d_uT, keeping the checkpoints
+ * u^c, u^2c, ... < u^T in d_kept (device, caller-owned, stencil_kept_states
+ * grids one after another; may be NULL when that is 0; c as above), and the
+ * reverse sweep that reads them there instead of sweeping forward again.
+ * Same bits as stencil_run and stencil_adjoint_vjp; scratch of the second:
+ * c + 8 grids.  Both asynchronous on cuda_stream. */
+int64_t stencil_kept_states(int64_t T, int ckpt_every);
+int stencil_run_kept(stencil_plan p, const double* d_u0, double* d_uT, int64_t T, const double* d_kappa,
+                     double dt, int ckpt_every, double* d_kept, void* cuda_stream);
+int stencil_adjoint_vjp_kept(stencil_plan p, const double* d_u0, const double* d_kappa, double dt,
+                             int64_t T, int ckpt_every, const double* d_kept, const double* d_lambda_T,
+                             double* d_grad_u0, double* d_grad_kappa, void* cuda_stream);
+
 /* ----------------------------------------------------------- batched form */
 
 /* One independent 2D heat grid of a batch: ny x nx cells (row-major, device,

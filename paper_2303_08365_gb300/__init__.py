@@ -59,6 +59,10 @@ SIGNATURES = [
                                        _VP, _VP, _DP, _VP]),
     ("stencil_adjoint_vjp", ctypes.c_int, [_VP, _VP, _VP, ctypes.c_double, ctypes.c_int64, ctypes.c_int,
                                            _VP, _VP, _VP, _VP]),
+    ("stencil_kept_states", ctypes.c_int64, [ctypes.c_int64, ctypes.c_int]),
+    ("stencil_run_kept", ctypes.c_int, [_VP, _VP, _VP, ctypes.c_int64, _VP, ctypes.c_double, ctypes.c_int, _VP, _VP]),
+    ("stencil_adjoint_vjp_kept", ctypes.c_int, [_VP, _VP, _VP, ctypes.c_double, ctypes.c_int64, ctypes.c_int, _VP,
+                                                _VP, _VP, _VP, _VP]),
     ("stencil_batch_create", ctypes.c_int, [ctypes.POINTER(BatchItem), ctypes.c_int, ctypes.c_int,
                                             ctypes.POINTER(_VP)]),
     ("stencil_batch_run", ctypes.c_int, [_VP, _VP]),
@@ -231,6 +235,32 @@ def stencil_adjoint_vjp(h, u0, kappa, dt, T, ckpt_every, lambda_T, grad_u0, grad
                                      int(T), int(ckpt_every), _dev_ptr(lambda_T, "lambda_T", shape),
                                      _dev_ptr(grad_u0, "grad_u0", shape),
                                      _dev_ptr(grad_kappa, "grad_kappa", shape), _stream(stream)))
+
+
+def stencil_kept_states(T, ckpt_every=0):
+    """How many states stencil_run_kept keeps."""
+    return lib().stencil_kept_states(int(T), int(ckpt_every))
+
+
+def stencil_run_kept(h, u0, uT, T, kappa, dt, ckpt_every, kept, stream=None):
+    """u^T from u0 (left alone) into uT, the checkpoints into kept (stencil_kept_states
+    grids, one after another; unused when that is 0)."""
+    shape = tuple(u0.shape)
+    n = stencil_kept_states(T, ckpt_every)
+    _check(lib().stencil_run_kept(h, _dev_ptr(u0, "u0"), _dev_ptr(uT, "uT", shape), int(T),
+                                  _dev_ptr(kappa, "kappa", shape), float(dt), int(ckpt_every),
+                                  _dev_ptr(kept, "kept", (n,) + shape) if n else None, _stream(stream)))
+
+
+def stencil_adjoint_vjp_kept(h, u0, kappa, dt, T, ckpt_every, kept, lambda_T, grad_u0, grad_kappa, stream=None):
+    """stencil_adjoint_vjp with the checkpoints of stencil_run_kept; asynchronous."""
+    shape = tuple(u0.shape)
+    n = stencil_kept_states(T, ckpt_every)
+    _check(lib().stencil_adjoint_vjp_kept(h, _dev_ptr(u0, "u0"), _dev_ptr(kappa, "kappa", shape), float(dt), int(T),
+                                          int(ckpt_every), _dev_ptr(kept, "kept", (n,) + shape) if n else None,
+                                          _dev_ptr(lambda_T, "lambda_T", shape),
+                                          _dev_ptr(grad_u0, "grad_u0", shape),
+                                          _dev_ptr(grad_kappa, "grad_kappa", shape), _stream(stream)))
 
 
 def _batch_items(grids, alphas, steps):

@@ -11,39 +11,65 @@ field after T explicit steps of du/dt = div(kappa grad u) (the paper's Eq. 1
 with a per-cell diffusivity).  Its backward takes the upstream gradient
 dL/du^T as lambda^T and sweeps the transposed stencil backward in time
 (stencil_adjoint_vjp), recomputing the forward states from checkpoints every
-ckpt_every steps (0: every state kept when it fits in half of the free
-device memory, else about sqrt(T)).  dt is a constant (no gradient).  Every
-step runs in the library's CUDA kernels.
+ckpt_every steps (0: about sqrt(T)).  dt is a constant (no gradient).  Every
+step runs in the library's CUDA kernels.  diffuse() lets the forward pass keep
+those checkpoints, about T / ckpt_every grids until the graph is freed, where a
+gradient is asked for and the memory is there, so that the backward pass does
+not sweep forward again.
 """
 import numpy as np
 import torch
 
-from . import Plan, stencil_adjoint_vjp, stencil_run
+from . import (Plan, stencil_adjoint_vjp, stencil_adjoint_vjp_kept, stencil_kept_states, stencil_run,
+               stencil_run_kept)
 
 
 class StencilAdjointFn(torch.autograd.Function):
     @staticmethod
-    def forward(ctx, u0, kappa, plan, dt, T, ckpt_every=0):
-        u = u0.detach().clone().contiguous()
-        stencil_run(plan.handle, u, T, kappa.detach().contiguous(), dt)
-        ctx.save_for_backward(u0.detach(), kappa.detach())
+    def forward(ctx, u0, kappa, plan, dt, T, ckpt_every=0, keep=False):
         ctx.plan, ctx.dt, ctx.T, ctx.ckpt = plan, float(dt), int(T), int(ckpt_every)
+        kept = _room_for_states(u0, ctx.T, ctx.ckpt) if keep else None
+        if kept is None:
+            u = u0.detach().clone().contiguous()
+            stencil_run(plan.handle, u, T, kappa.detach().contiguous(), dt)
+            ctx.save_for_backward(u0.detach(), kappa.detach())
+            return u
+        u = torch.empty_like(u0, memory_format=torch.contiguous_format)
+        stencil_run_kept(plan.handle, u0.detach().contiguous(), u, ctx.T, kappa.detach().contiguous(), ctx.dt, ctx.ckpt,
+                         kept)
+        ctx.save_for_backward(u0.detach(), kappa.detach(), kept)
         return u
 
     @staticmethod
     def backward(ctx, grad_out):
-        u0, kappa = ctx.saved_tensors
+        u0, kappa, *kept = ctx.saved_tensors
         lam = grad_out.detach().contiguous()
         gu = torch.empty_like(u0)
         gk = torch.empty_like(u0)
-        stencil_adjoint_vjp(ctx.plan.handle, u0.contiguous(), kappa.contiguous(), ctx.dt, ctx.T,
-                            ctx.ckpt, lam, gu, gk)
-        return gu, gk, None, None, None, None
+        if kept:
+            stencil_adjoint_vjp_kept(ctx.plan.handle, u0.contiguous(), kappa.contiguous(), ctx.dt, ctx.T, ctx.ckpt,
+                                     kept[0], lam, gu, gk)
+        else:
+            stencil_adjoint_vjp(ctx.plan.handle, u0.contiguous(), kappa.contiguous(), ctx.dt, ctx.T,
+                                ctx.ckpt, lam, gu, gk)
+        return gu, gk, None, None, None, None, None
+
+
+def _room_for_states(u0, T, ckpt_every):
+    """An uninitialised tensor for the checkpoints of a forward pass; None when the device
+    has no room for it, or u0 is not what the sweep takes (it says so itself)."""
+    if u0.device.type != "cuda" or u0.dtype != torch.float64 or T < 0 or ckpt_every < 0:
+        return None
+    try:
+        return torch.empty((stencil_kept_states(T, ckpt_every), *u0.shape), dtype=u0.dtype, device=u0.device)
+    except torch.OutOfMemoryError:
+        return None
 
 
 def diffuse(u0, kappa, plan, dt, T, ckpt_every=0):
     """u^T with autograd support for u0 and kappa."""
-    return StencilAdjointFn.apply(u0, kappa, plan, dt, T, ckpt_every)
+    keep = torch.is_grad_enabled() and (u0.requires_grad or kappa.requires_grad)
+    return StencilAdjointFn.apply(u0, kappa, plan, dt, T, ckpt_every, keep)
 
 
 def reflected(weights):

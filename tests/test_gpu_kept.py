@@ -1,0 +1,67 @@
+"""The forward sweep that keeps its checkpoints for the reverse sweep: the same
+bits as the pair that does not, for every interval, and the autograd function
+with and without room for them."""
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+PERIODIC, DIRICHLET = 1, 0
+
+
+@pytest.fixture(scope="module")
+def st():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2303_08365_gb300 import build
+    build.build()
+    import paper_2303_08365_gb300 as st
+    return st
+
+
+def inputs(shape, seed):
+    import torch
+    u0, kappa, lam = synth.uniform(seed, shape), synth.lognormal(seed + 1, shape, 0.5), synth.normal(seed + 2, shape)
+    return [torch.from_numpy(a).cuda() for a in (u0, kappa, lam)] + [0.1 / float(kappa.max())]
+
+
+@pytest.mark.parametrize("shape,boundary", [((9, 13, 11), PERIODIC), ((15, 21), DIRICHLET), ((7, 1, 9), DIRICHLET),
+                                            ((1, 40), PERIODIC)])
+@pytest.mark.parametrize("T", [0, 1, 2, 12, 17])
+def test_kept_states_give_the_same_bits(st, shape, boundary, T):
+    import torch
+    u0, kappa, lam, dt = inputs(shape, 51)
+    p = st.Plan.varcoef(shape, boundary)
+    want = u0.clone()
+    p.run(want, T, kappa, dt)
+    gu, gk, hu, hk, uT = (torch.empty_like(u0) for _ in range(5))
+    for ckpt in (0, 1, 3, 4, T + 1, T + 5):
+        n = st.stencil_kept_states(T, ckpt)
+        buf = torch.full((n + 2, *shape), 7.0, dtype=torch.float64, device="cuda")
+        kept, before = buf[1:n + 1], u0.clone()
+        st.stencil_run_kept(p.handle, u0, uT, T, kappa, dt, ckpt, kept)
+        assert torch.equal(uT, want) and torch.equal(u0, before), ckpt
+        st.stencil_adjoint_vjp_kept(p.handle, u0, kappa, dt, T, ckpt, kept, lam, gu, gk)
+        st.stencil_adjoint_vjp(p.handle, u0, kappa, dt, T, ckpt, lam, hu, hk)
+        assert torch.equal(gu, hu) and torch.equal(gk, hk), ckpt
+        assert bool((buf[0] == 7.0).all()) and bool((buf[-1] == 7.0).all()), ckpt
+    p.close()
+
+
+def test_autograd_with_and_without_room(st, monkeypatch):
+    import torch
+    from paper_2303_08365_gb300 import autograd
+    shape = (12, 10, 14)
+    u0, kappa, lam, dt = inputs(shape, 61)
+    p = st.Plan.varcoef(shape, DIRICHLET)
+    got = []
+    for room in (True, False):
+        if not room:
+            monkeypatch.setattr(autograd, "_room_for_states", lambda *a: None)
+        u, k = u0.clone().requires_grad_(), kappa.clone().requires_grad_()
+        out = autograd.diffuse(u, k, p, dt, 19)
+        got.append([out.detach(), *torch.autograd.grad(out, (u, k), lam)])
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+    with torch.no_grad():
+        assert torch.equal(autograd.diffuse(u0, kappa, p, dt, 19), got[0][0])
+    p.close()
