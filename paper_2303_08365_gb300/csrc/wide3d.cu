@@ -148,8 +148,11 @@ __device__ __noinline__ void chain_cells(const Plane<TC>& um, const Plane<TC>& u
     }
 }
 
+// Three CTAs of nine warps per SM where 72 registers are enough (199 x 251 x 301 by bulk
+// copies, us a step, three against two: heat 124 / 137; general weights, which spill,
+// 167 / 148).
 template <bool BOX, bool HEAT, bool PERIODIC, bool TMA, int TC>
-__global__ void __launch_bounds__(kThreads, BOX || !TMA ? 2 : 3) k_wide3d(const __grid_constant__ Params P) {
+__global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wide3d(const __grid_constant__ Params P) {
   constexpr int R = TC / kWarps;  // rows of a consumer warp
   constexpr int kU = ring<BOX>();
   constexpr int kLag = BOX ? 2 : 1;  // the middle plane is kLag planes behind the one being unpacked
