@@ -265,25 +265,24 @@ __device__ __forceinline__ double wide_sum_heat(const WideVal (&u)[NT], const Ta
   return acc.get(E, T);
 }
 
-// Boxes whose weights are all equal: the values of a block of cells are aligned to one
-// exponent E, the largest of the block, and added as integers; a cell's sum S takes one
+// Boxes of N taps whose weights are all equal: the values of a block of cells are aligned to
+// one exponent E, the largest of the block, and added as integers; a cell's sum S takes one
 // multiplication.  S counts units of 2^-(61 - kEqualShift) of the largest value, up to
-// (2 RAD + 1)^2 < 2^(kEqualShift + 2) of which fit; the bits that the values lose, a unit at
-// most each, are centred by the first summand (half a unit for every
-// value), which also lets values that cancel exactly sum to zero.
-template <int RAD>
-constexpr int kEqualShift = RAD == 1 ? 3 : 4;
-template <int RAD>
-constexpr int kEqualFirst = RAD == 1 ? 4 : 12;
+// N of which fit 63 bits; the bits that the values lose, a unit at
+// most each, are centred by the first summand (about half a unit for every value, and
+// such that values that cancel in pairs sum to zero once rounded).
+template <int N>
+constexpr int kEqualShift = N == 9 ? 3 : 4;
+template <int N>
+constexpr int kEqualFirst = N == 9 ? 4 : N == 25 ? 12 : 11;
 // How far below the block's a cell's own largest exponent may lie.  Then a unit is 2^-55
-// (RAD 1) or 2^-55 (RAD 2) of the cell's own largest value, and the 9 (25) lost parts add
-// up to 0.9 (1.4) units on average, against half a unit of 2^-52 of the result that its
-// rounding takes.
-template <int RAD>
-constexpr int kEqualGap = RAD == 1 ? 3 : 2;
+// of the cell's own largest value, and the lost parts add up to 0.9 (9 taps) or 1.4 to 1.5
+// units on average, against half a unit of 2^-52 of the result that its rounding takes.
+template <int N>
+constexpr int kEqualGap = N == 9 ? 3 : 2;
 
 // w S as a double, w the weights' one value.
-template <int RAD, class Taps>
+template <int N, class Taps>
 __device__ __forceinline__ double wide_equal(long long S, int E, const Taps& T) {
   const int ah = (int)(S >> 32), lo = T.lo[0];
   const unsigned int al = (unsigned int)S;
@@ -292,7 +291,7 @@ __device__ __forceinline__ double wide_equal(long long S, int E, const Taps& T) 
   const unsigned long long ll = (unsigned long long)al * (unsigned int)lo;
   const unsigned long long lh = (unsigned long long)al * (unsigned int)T.hi[0] + (ll >> 26);
   const long long hl = (long long)ah * lo + ((1 << 23) + (long long)(lh >> 6));
-  return wide_double(hh + (hl >> 24), E - T.bias + kEqualShift<RAD> - 1);
+  return wide_double(hh + (hl >> 24), E - T.bias + kEqualShift<N> - 1);
 }
 
 // The same with the FMA chain in its place where it has to be.

@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
         // equal weights, the lane's two rows and columns as one block: each value is
         // aligned once for the four cells, and rows (mid: their common columns) and
         // columns share their partial sums
-        constexpr int N = 2 * RAD + 2;
+        constexpr int N = 2 * RAD + 2, NT = (2 * RAD + 1) * (2 * RAD + 1);
         static_assert(kR == 2 && TMA, "the block; columns and rows outside the grid hold values or zeros");
         int E = 0, own[2][2], e[N][N];  // the block's largest exponent, the cells' own
 #pragma unroll
@@ -446,9 +446,9 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
         E = max(max(own[0][0], own[0][1]), max(own[1][0], own[1][1]));
         int least = min(own[0][0], own[0][1]);
         if (rows > 1) least = min(least, min(own[1][0], own[1][1]));
-        all = rows <= 0 || (wide_covers(E, P.wide) && wide_covers(least, P.wide) && E - least <= kEqualGap<RAD>);
-        long long S[2][2], both[2] = {kEqualFirst<RAD>, kEqualFirst<RAD>};  // both: of the rows that both read
-        E += kEqualShift<RAD>;
+        all = rows <= 0 || (wide_covers(E, P.wide) && wide_covers(least, P.wide) && E - least <= kEqualGap<NT>);
+        long long S[2][2], both[2] = {kEqualFirst<NT>, kEqualFirst<NT>};  // both: of the rows that both read
+        E += kEqualShift<NT>;
         if (RAD > 1) asm volatile("" ::: "memory");  // 36 exponents would not fit the registers: read again
 #pragma unroll
         for (int r = 0; r < N; ++r) {
@@ -465,10 +465,10 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
             else S[1][i] = h;
           }
         }
-        E -= kEqualShift<RAD>;
+        E -= kEqualShift<NT>;
 #pragma unroll
         for (int r = 0; r < 2; ++r)
-          store(r, wide_equal<RAD>(S[r][0] + both[0], E, P.wide), wide_equal<RAD>(S[r][1] + both[1], E, P.wide));
+          store(r, wide_equal<NT>(S[r][0] + both[0], E, P.wide), wide_equal<NT>(S[r][1] + both[1], E, P.wide));
       } else {
         // row by row; the largest exponents first, then the sums: a pair's values would
         // not fit the registers, so their rows are read twice

@@ -25,6 +25,8 @@
 // bound is the FP64 pipe).  Registers instead of shared memory for the three
 // planes (1.5 unpacks per cell, rows of 4) ran at 142 and spilled; a converter
 // warp that loads and unpacks everything for the consumers at 94.
+// Box, 384^3, zero outside: general weights 48 GStencil/s (22.7 for the FMA chain), equal
+// ones (wide_equal) 63.
 // Work split: the (tile, z) planes are cut into equal contiguous ranges, one per CTA.
 #include <cudaTypedefs.h>
 
@@ -148,6 +150,42 @@ __device__ __noinline__ void chain_cells(const Plane<TC>& um, const Plane<TC>& u
     }
 }
 
+// A lane's cells of an equal-weight box one by one, each aligned to its own largest
+// exponent: where the block's lies too far above.  Out of line: rarely run.
+template <int TC>
+__device__ __noinline__ void own_cells(const Plane<TC>& um, const Plane<TC>& u0, const Plane<TC>& up, int row0, int rows,
+                                       int c0, const WideTaps& T, const double* wdev, double* out, int nx) {
+  const Plane<TC>* const pl[3] = {&um, &u0, &up};
+  for (int r = 0; r < rows; ++r)
+    for (int i = 0; i < 2; ++i) {
+      const int row = row0 + r, c = c0 + i;
+      auto at = [&](int k) {
+        const int y = row + k / 3 % 3 - 1, x = c + k % 3 - 1;
+        return get(&pl[k / 9]->m[y][x], &pl[k / 9]->e[y][x]);
+      };
+      unsigned int any = 0;
+      int E = 0;
+      for (int k = 0; k < 27; ++k) {
+        const WideVal u = at(k);
+        any |= wide_nonzero(u);
+        E = max(E, u.e);
+      }
+      double v = 0.0;
+      if (any != 0 && !wide_covers(E, T)) {
+        v = chain_cell<true, TC>(um, u0, up, row, c, wdev);
+      } else if (any != 0) {
+        WideAcc acc;
+        for (int k = 0; k < 27; ++k) {
+          const WideVal u = at(k);
+          acc.add(u, 0, E - u.e, T);
+        }
+        v = acc.get(E, T);
+      }
+      out[(int64_t)r * nx + i] = v;
+    }
+}
+
+// HEAT: a star whose weights wide_sum_heat takes; a box whose weights are all equal.
 // Three CTAs of nine warps per SM where 72 registers are enough (199 x 251 x 301 by bulk
 // copies, us a step, three against two: heat 124 / 137; general weights, which spill,
 // 167 / 148).
@@ -378,6 +416,66 @@ __global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wid
             }
             store(r, v[0], v[1]);
           }
+        } else if constexpr (HEAT) {
+          // equal weights, the lane's rows and two columns as one block: each value is
+          // aligned once for all cells, and rows (mid: their common columns) share their
+          // partial sums.  Exponents first: a block's values would not fit the registers.
+          static_assert(TMA, "columns and rows outside the grid hold values or zeros");
+          int own[R][2];
+#pragma unroll
+          for (int r = 0; r < R; ++r) own[r][0] = own[r][1] = 0;
+#pragma unroll 1
+          for (int p = 0; p < 3; ++p) {
+            const Plane<TC>& u = p == 0 ? um : p == 1 ? u0 : up;
+#pragma unroll
+            for (int q = 0; q < R + 2; ++q) {  // the block's row: read by cells q-2 .. q
+              const int* er = &u.e[row0 - 1 + q][c];
+              const int2 m = *reinterpret_cast<const int2*>(er);
+              const int mid = max(m.x, m.y), h0 = max(mid, er[-1]), h1 = max(mid, er[2]);
+#pragma unroll
+              for (int r = 0; r < R; ++r)
+                if (q - 2 <= r && r <= q) {
+                  own[r][0] = max(own[r][0], h0);
+                  own[r][1] = max(own[r][1], h1);
+                }
+            }
+          }
+          int E = 0, least = max(own[0][0], own[0][1]);
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            E = max(E, max(own[r][0], own[r][1]));
+            if (r < rows) least = min(least, min(own[r][0], own[r][1]));
+          }
+          all = rows <= 0 || (wide_covers(E, P.wide) && wide_covers(least, P.wide) && E - least <= kEqualGap<27>);
+          long long sum[R][2], both[2] = {kEqualFirst<27>, kEqualFirst<27>};  // both: of the rows that all cells read
+#pragma unroll
+          for (int r = 0; r < R; ++r) sum[r][0] = sum[r][1] = 0;
+          E += kEqualShift<27>;
+#pragma unroll 1
+          for (int p = 0; p < 3; ++p) {
+            const Plane<TC>& u = p == 0 ? um : p == 1 ? u0 : up;
+#pragma unroll
+            for (int q = 0; q < R + 2; ++q) {
+              WideVal v[4];
+              get_row<TC>(u, row0 - 1 + q, c, v);
+              const long long mid = wide_align(v[1], E - v[1].e) + wide_align(v[2], E - v[2].e);
+              const long long h[2] = {mid + wide_align(v[0], E - v[0].e), mid + wide_align(v[3], E - v[3].e)};
+#pragma unroll
+              for (int i = 0; i < 2; ++i) {
+                if (R <= q + 1 && q <= 2) {
+                  both[i] += h[i];
+                } else {
+#pragma unroll
+                  for (int r = 0; r < R; ++r)
+                    if (q - 2 <= r && r <= q) sum[r][i] += h[i];
+                }
+              }
+            }
+          }
+          E -= kEqualShift<27>;
+#pragma unroll
+          for (int r = 0; r < R; ++r)
+            store(r, wide_equal<27>(sum[r][0] + both[0], E, P.wide), wide_equal<27>(sum[r][1] + both[1], E, P.wide));
         } else {
           // row by row; the largest exponents first, then the sums: the 36 values of
           // a pair would not fit the registers, so their rows are read twice
@@ -416,8 +514,10 @@ __global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wid
             store(r, acc[0].get(E[0], P.wide), acc[1].get(E[1], P.wide));
           }
         }
-        if (!all && !zero_cells<BOX, TC>(um, u0, up, row0, rows, min(2, P.nx - xa), c, out, P.nx))
-          chain_cells<BOX, TC>(um, u0, up, row0, rows, min(2, P.nx - xa), c, P.wide, P.wdev, out, P.nx);
+        if (!all && !zero_cells<BOX, TC>(um, u0, up, row0, rows, min(2, P.nx - xa), c, out, P.nx)) {
+          if constexpr (BOX && HEAT) own_cells<TC>(um, u0, up, row0, rows, c, P.wide, P.wdev, out, P.nx);
+          else chain_cells<BOX, TC>(um, u0, up, row0, rows, min(2, P.nx - xa), c, P.wide, P.wdev, out, P.nx);
+        }
         __syncwarp();
         out += plane;
       }
@@ -491,6 +591,13 @@ cudaError_t launch_wide3d(Shape shape, int boundary, const Geom& g, const WideTa
   const bool per = boundary == kPeriodic, low = tile_y == 8;
   if (shape == Shape::kBox) {
     if (wide.n != 27) return cudaErrorInvalidValue;
+    if (tma && wide.heat && wide.hi[13] == wide.hi[0] && wide.lo[13] == wide.lo[0] && wide.ex[13] == wide.ex[0]) {
+      if (low)
+        return per ? launch_t<true, true, true, true, 8>(g, wide, wdev, src, dst, status, sms, stream, chained)
+                   : launch_t<true, true, false, true, 8>(g, wide, wdev, src, dst, status, sms, stream, chained);
+      return per ? launch_t<true, true, true, true, 16>(g, wide, wdev, src, dst, status, sms, stream, chained)
+                 : launch_t<true, true, false, true, 16>(g, wide, wdev, src, dst, status, sms, stream, chained);
+    }
     return per ? launch_p<true, false, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained)
                : launch_p<true, false, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained);
   }

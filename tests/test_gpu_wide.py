@@ -428,3 +428,44 @@ def test_persistent_bricks_under_capture(st):
         assert np.array_equal(g.cpu().numpy(), run(st, u, w, 1, PERIODIC, 9, (1, st.VARIANT_DIRECT)))
     assert p.status() == 0
     p.close()
+
+
+@pytest.mark.parametrize("spread", [0, 3, 60])
+def test_equal_box_against_exact_arithmetic_3d(st, spread):
+    """As in two dimensions, at most 2 exponents apart: 16 units of 2^-55 and half a unit of
+    the product, 2^-52, of the cell's largest product, and one rounding of the result."""
+    rng = np.random.default_rng(spread + 7)
+    u0 = rng.standard_normal((4, 11, 34)) * 2.0 ** rng.integers(-spread, spread + 1, (4, 11, 34))
+    u0[rng.random(u0.shape) < 0.1] = 0.0
+    w = equal_weights(3, 1)
+    got = run(st, u0, w, 1, DIRICHLET, 1, (1, st.VARIANT_STREAM))
+    slack = Fraction(16 * 2.0 ** -55 + 2.0 ** -52)
+    for at in np.ndindex(*u0.shape):
+        want, top = exact_sum(u0, w, at, 1)
+        assert abs(Fraction(float(got[at])) - want) <= abs(want) * Fraction(EPS) + top * slack, at
+
+
+@pytest.mark.parametrize("shape,boundary,tile", [((1, 1, 2), DIRICHLET, 16), ((3, 17, 66), DIRICHLET, 16),
+                                                 ((5, 15, 62), DIRICHLET, 8), ((4, 16, 64), PERIODIC, 16),
+                                                 ((9, 24, 192), PERIODIC, 8), ((61, 97, 130), DIRICHLET, 16)])
+def test_equal_box_tiles_3d(st, shape, boundary, tile):
+    w = equal_weights(3, 1)
+    T = 3
+    for u0 in (synth.normal(44, shape), np.where(synth.uniform(45, shape) < 0.001, synth.normal(46, shape), 0.0),
+               np.where(synth.uniform(47, shape) < 0.001, np.inf, 1.0)):
+        with np.errstate(all="ignore"):
+            ref = oracle.run(u0, w, 1, boundary, T, nthreads=0)
+        import torch
+        g = torch.from_numpy(u0.copy()).cuda()
+        p = st.Plan(shape, 1, w, boundary)
+        p.set_tuning(1, st.VARIANT_STREAM)
+        p.set_tile(64, tile)
+        p.run(g, T)
+        assert p.status() == 0
+        p.close()
+        got = g.cpu().numpy()
+        fine = np.isfinite(ref)
+        assert np.array_equal(fine, np.isfinite(got))
+        top = np.abs(u0[np.isfinite(u0)]).max()
+        assert np.abs(got[fine] - ref[fine]).max(initial=0.0) <= T * (2 * w.size + 2) * EPS * top
+        assert np.array_equal(got == 0.0, ref == 0.0)
