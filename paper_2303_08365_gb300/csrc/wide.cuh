@@ -93,6 +93,25 @@ __device__ __forceinline__ WideVal wide_unpack(double v) {
   return u;
 }
 
+// The same with negative values in two's complement, for sums of integers whose units are not
+// far below the result's (wide_equal): a one's complement is a bias there (half of it taken
+// back by a constant, 79 steps of a 9-point box ended 4.1e-16 off; so, 3.3e-16).
+__device__ __forceinline__ WideVal wide_unpack_twos(double v) {
+  WideVal u = wide_unpack(v);
+  const unsigned int s = (unsigned int)(u.hi >> 31);
+  const long long m = (long long)(((unsigned long long)(unsigned int)u.hi << 32) | u.lo) - (int)s;
+  u.hi = (int)(m >> 32);
+  u.lo = (unsigned int)m;
+  return u;
+}
+__device__ __forceinline__ WideVal wide_ones(WideVal u) {  // back to wide_unpack's form
+  const long long v = (long long)(((unsigned long long)(unsigned int)u.hi << 32) | u.lo);
+  const long long m = v + (v >> 63);
+  u.hi = (int)(m >> 32);
+  u.lo = (unsigned int)m;
+  return u;
+}
+
 // Zero bits when the value is a zero.  Neighbourhoods of zeros, which the integer form
 // does not take, are told apart first: whole grids of them are ordinary input (512^3 with
 // one hot cell: 134 GStencil/s, the FMA chain for each 17; no zeros 170).
@@ -265,19 +284,16 @@ __device__ __forceinline__ double wide_sum_heat(const WideVal (&u)[NT], const Ta
   return acc.get(E, T);
 }
 
-// Boxes of N taps whose weights are all equal: the values of a block of cells are aligned to
-// one exponent E, the largest of the block, and added as integers; a cell's sum S takes one
-// multiplication.  S counts units of 2^-(61 - kEqualShift) of the largest value, up to
-// N of which fit 63 bits; the bits that the values lose, a unit at
-// most each, are centred by the first summand (about half a unit for every value, and
-// such that values that cancel in pairs sum to zero once rounded).
+// Boxes of N taps whose weights are all equal: the values of a block of cells (two's
+// complement) are aligned to one exponent E, the largest of the block, and added as integers;
+// a cell's sum S takes one multiplication.  S counts units of 2^-(61 - kEqualShift) of the
+// largest value, N of which fit 63 bits.  A value within 2^(9 - kEqualShift) of the
+// largest loses nothing, one below that less than a unit.
 template <int N>
 constexpr int kEqualShift = N == 9 ? 3 : 4;
-template <int N>
-constexpr int kEqualFirst = N == 9 ? 4 : N == 25 ? 12 : 11;
-// How far below the block's a cell's own largest exponent may lie.  Then a unit is 2^-55
-// of the cell's own largest value, and the lost parts add up to 0.9 (9 taps) or 1.4 to 1.5
-// units on average, against half a unit of 2^-52 of the result that its rounding takes.
+// How far below the block's a cell's own largest exponent may lie: then a unit is 2^-55
+// of the cell's own largest value, half a unit of 2^-52 of the result being what its
+// rounding takes.
 template <int N>
 constexpr int kEqualGap = N == 9 ? 3 : 2;
 

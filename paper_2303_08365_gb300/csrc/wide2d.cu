@@ -120,14 +120,15 @@ __device__ __noinline__ bool zero_cells(const Plane<RAD>& u, int row0, int rows,
 }
 
 // One cell by the FMA chain.
-template <bool BOX, int RAD>
+template <bool BOX, int RAD, bool TWOS = false>
 __device__ __noinline__ double chain_cell(const Plane<RAD>& u, int row, int c, const double* wdev) {
   constexpr int NT = BOX ? (2 * RAD + 1) * (2 * RAD + 1) : 4 * RAD + 1;
   double v[NT];
   for (int dy = -RAD; dy <= RAD; ++dy)
     for (int dx = -RAD; dx <= RAD; ++dx) {
       if (!BOX && dy != 0 && dx != 0) continue;
-      v[tap_at<BOX, RAD>(dy, dx)] = wide_repack(get(&u.m[row + dy][c + dx], &u.e[row + dy][c + dx]));
+      const WideVal x = get(&u.m[row + dy][c + dx], &u.e[row + dy][c + dx]);
+      v[tap_at<BOX, RAD>(dy, dx)] = wide_repack(TWOS ? wide_ones(x) : x);
     }
   return wide_chain(v, wdev, NT);
 }
@@ -168,18 +169,18 @@ __device__ __noinline__ void own_cells(const Plane<RAD>& u, int row0, int rows, 
       int E = 0;
       for (int dy = -RAD; dy <= RAD; ++dy)
         for (int dx = -RAD; dx <= RAD; ++dx) {
-          const WideVal x = get(&u.m[row + dy][c + dx], &u.e[row + dy][c + dx]);
+          const WideVal x = wide_ones(get(&u.m[row + dy][c + dx], &u.e[row + dy][c + dx]));
           any |= wide_nonzero(x);
           E = max(E, x.e);
         }
       double v = 0.0;
       if (any != 0 && !wide_covers(E, T)) {
-        v = chain_cell<true, RAD>(u, row, c, wdev);
+        v = chain_cell<true, RAD, true>(u, row, c, wdev);
       } else if (any != 0) {
         WideAcc acc;
         for (int dy = -RAD; dy <= RAD; ++dy)
           for (int dx = -RAD; dx <= RAD; ++dx) {
-            const WideVal x = get(&u.m[row + dy][c + dx], &u.e[row + dy][c + dx]);
+            const WideVal x = wide_ones(get(&u.m[row + dy][c + dx], &u.e[row + dy][c + dx]));
             acc.add(x, 0, E - x.e, T);
           }
         v = acc.get(E, T);
@@ -323,14 +324,14 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
       for (int q = 0; q < HN; ++q) {
         const int k = lane + 32 * q, j = k / HR, row = H0 + k % HR;
         const int c = 2 + (j < RAD ? j - RAD : cols + (j - RAD));
-        if (k < HALL) put(&u.m[row][c], &u.e[row][c], wide_unpack(h[q]));
+        if (k < HALL) put(&u.m[row][c], &u.e[row][c], BOX && HEAT ? wide_unpack_twos(h[q]) : wide_unpack(h[q]));
       }
       if (!wait(&S.full[pos.s], pos.ph)) return leave(t);
       WideVal v[2];
 #pragma unroll
       for (int r = 0; r < RAD; ++r) {
-        unpack_row<TMA, kRows>(S.raw[pos.s], S.shift[pos.s], u, r, lane, cols, v);
-        unpack_row<TMA, kRows>(S.raw[pos.s], S.shift[pos.s], u, kTC + RAD + r, lane, cols, v);
+        unpack_row<TMA, kRows, BOX && HEAT>(S.raw[pos.s], S.shift[pos.s], u, r, lane, cols, v);
+        unpack_row<TMA, kRows, BOX && HEAT>(S.raw[pos.s], S.shift[pos.s], u, kTC + RAD + r, lane, cols, v);
       }
       __syncwarp();
       if (lane == 0) {
@@ -358,7 +359,7 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
       WideVal v[2];
 #pragma unroll
       for (int r = 0; r < kR; ++r)
-        unpack_row<TMA, kRows>(S.raw[pos.s], S.shift[pos.s], S.u[pos.s], row0 + r, lane, cols, v);
+        unpack_row<TMA, kRows, BOX && HEAT>(S.raw[pos.s], S.shift[pos.s], S.u[pos.s], row0 + r, lane, cols, v);
       __syncwarp();
       if (lane == 0) {
         mbar_arrive(&S.empty[pos.s]);
@@ -447,7 +448,7 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
         int least = min(own[0][0], own[0][1]);
         if (rows > 1) least = min(least, min(own[1][0], own[1][1]));
         all = rows <= 0 || (wide_covers(E, P.wide) && wide_covers(least, P.wide) && E - least <= kEqualGap<NT>);
-        long long S[2][2], both[2] = {kEqualFirst<NT>, kEqualFirst<NT>};  // both: of the rows that both read
+        long long S[2][2], both[2] = {0, 0};  // both: of the rows that both read
         E += kEqualShift<NT>;
         if (RAD > 1) asm volatile("" ::: "memory");  // 36 exponents would not fit the registers: read again
 #pragma unroll

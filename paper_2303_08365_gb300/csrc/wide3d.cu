@@ -26,7 +26,8 @@
 // planes (1.5 unpacks per cell, rows of 4) ran at 142 and spilled; a converter
 // warp that loads and unpacks everything for the consumers at 94.
 // Box, 384^3, zero outside: general weights 48 GStencil/s (22.7 for the FMA chain), equal
-// ones (wide_equal) 63.
+// ones (wide_equal) 63 (each plane's sums kept in registers for the next two planes:
+// 66, but they spill, and small grids lose, 64^3 10.9 us a step to 16).
 // Work split: the (tile, z) planes are cut into equal contiguous ranges, one per CTA.
 #include <cudaTypedefs.h>
 
@@ -109,7 +110,7 @@ __device__ __noinline__ bool zero_cells(const Plane<TC>& um, const Plane<TC>& u0
 }
 
 // One cell by the FMA chain.
-template <bool BOX, int TC>
+template <bool BOX, int TC, bool TWOS = false>
 __device__ __noinline__ double chain_cell(const Plane<TC>& um, const Plane<TC>& u0, const Plane<TC>& up, int row, int c,
                                           const double* wdev) {
   constexpr int NT = BOX ? 27 : 7;
@@ -118,7 +119,8 @@ __device__ __noinline__ double chain_cell(const Plane<TC>& um, const Plane<TC>& 
   for (int k = 0; k < 27; ++k) {
     const int dz = k / 9 - 1, dy = k / 3 % 3 - 1, dx = k % 3 - 1;
     if (!BOX && (dz != 0) + (dy != 0) + (dx != 0) > 1) continue;
-    v[tap_at<BOX>(dz, dy, dx)] = wide_repack(get(&pl[dz + 1]->m[row + dy][c + dx], &pl[dz + 1]->e[row + dy][c + dx]));
+    const WideVal x = get(&pl[dz + 1]->m[row + dy][c + dx], &pl[dz + 1]->e[row + dy][c + dx]);
+    v[tap_at<BOX>(dz, dy, dx)] = wide_repack(TWOS ? wide_ones(x) : x);
   }
   return wide_chain(v, wdev, NT);
 }
@@ -161,7 +163,7 @@ __device__ __noinline__ void own_cells(const Plane<TC>& um, const Plane<TC>& u0,
       const int row = row0 + r, c = c0 + i;
       auto at = [&](int k) {
         const int y = row + k / 3 % 3 - 1, x = c + k % 3 - 1;
-        return get(&pl[k / 9]->m[y][x], &pl[k / 9]->e[y][x]);
+        return wide_ones(get(&pl[k / 9]->m[y][x], &pl[k / 9]->e[y][x]));
       };
       unsigned int any = 0;
       int E = 0;
@@ -172,7 +174,7 @@ __device__ __noinline__ void own_cells(const Plane<TC>& um, const Plane<TC>& u0,
       }
       double v = 0.0;
       if (any != 0 && !wide_covers(E, T)) {
-        v = chain_cell<true, TC>(um, u0, up, row, c, wdev);
+        v = chain_cell<true, TC, true>(um, u0, up, row, c, wdev);
       } else if (any != 0) {
         WideAcc acc;
         for (int k = 0; k < 27; ++k) {
@@ -339,11 +341,11 @@ __global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wid
         Plane<TC>& u = S.u[con().s];
 #pragma unroll
         for (int q = 0; q < HN; ++q)
-          if (hrow[q] >= 0) put(&u.m[hrow[q]][hcol[q]], &u.e[hrow[q]][hcol[q]], wide_unpack(h[q]));
+          if (hrow[q] >= 0) put(&u.m[hrow[q]][hcol[q]], &u.e[hrow[q]][hcol[q]], BOX && HEAT ? wide_unpack_twos(h[q]) : wide_unpack(h[q]));
         if (!wait(&S.full[raw.s], raw.ph)) return leave(j);
         WideVal v[2];
-        unpack_row<TMA, TC + 2>(S.raw[raw.s], S.shift[raw.s], u, 0, lane, cols, v);
-        unpack_row<TMA, TC + 2>(S.raw[raw.s], S.shift[raw.s], u, TC + 1, lane, cols, v);
+        unpack_row<TMA, TC + 2, BOX && HEAT>(S.raw[raw.s], S.shift[raw.s], u, 0, lane, cols, v);
+        unpack_row<TMA, TC + 2, BOX && HEAT>(S.raw[raw.s], S.shift[raw.s], u, TC + 1, lane, cols, v);
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(&S.empty[raw.s]);
@@ -379,7 +381,7 @@ __global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wid
       if (j < nplanes) {
         if (!wait(&S.full[raw.s], raw.ph)) return;
 #pragma unroll
-        for (int r = 0; r < R; ++r) unpack_row<TMA, TC + 2>(S.raw[raw.s], S.shift[raw.s], S.u[con().s], row0 + r, lane, cols, zp[r]);
+        for (int r = 0; r < R; ++r) unpack_row<TMA, TC + 2, BOX && HEAT>(S.raw[raw.s], S.shift[raw.s], S.u[con().s], row0 + r, lane, cols, zp[r]);
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(&S.empty[raw.s]);
@@ -447,7 +449,7 @@ __global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wid
             if (r < rows) least = min(least, min(own[r][0], own[r][1]));
           }
           all = rows <= 0 || (wide_covers(E, P.wide) && wide_covers(least, P.wide) && E - least <= kEqualGap<27>);
-          long long sum[R][2], both[2] = {kEqualFirst<27>, kEqualFirst<27>};  // both: of the rows that all cells read
+          long long sum[R][2], both[2] = {0, 0};  // both: of the rows that all cells read
 #pragma unroll
           for (int r = 0; r < R; ++r) sum[r][0] = sum[r][1] = 0;
           E += kEqualShift<27>;

@@ -298,14 +298,14 @@ def equal_weights(ndim, radius):
 @pytest.mark.parametrize("radius", [1, 2])
 def test_equal_box_against_exact_arithmetic(st, radius, spread):
     """The equal-weight boxes align the values of four cells to one exponent, at most 3 (2)
-    above a cell's own: 5 (13) units of 2^-55 and half a unit of the product, 2^-52, of the
+    above a cell's own: 8 (24) units of 2^-55 and half a unit of the product, 2^-52, of the
     cell's largest product, and one rounding of the result."""
     rng = np.random.default_rng(spread + radius)
     u0 = rng.standard_normal((19, 70)) * 2.0 ** rng.integers(-spread, spread + 1, (19, 70))
     u0[rng.random(u0.shape) < 0.1] = 0.0
     w = equal_weights(2, radius)
     got = run(st, u0, w, radius, DIRICHLET, 1, (1, st.VARIANT_STREAM))
-    slack = Fraction((5 if radius == 1 else 13) * 2.0 ** -55 + 2.0 ** -52)
+    slack = Fraction((8 if radius == 1 else 24) * 2.0 ** -55 + 2.0 ** -52)
     for at in np.ndindex(*u0.shape):
         want, top = exact_sum(u0, w, at, radius)
         assert abs(Fraction(float(got[at])) - want) <= abs(want) * Fraction(EPS) + top * slack, at
@@ -432,14 +432,14 @@ def test_persistent_bricks_under_capture(st):
 
 @pytest.mark.parametrize("spread", [0, 3, 60])
 def test_equal_box_against_exact_arithmetic_3d(st, spread):
-    """As in two dimensions, at most 2 exponents apart: 16 units of 2^-55 and half a unit of
+    """As in two dimensions, at most 2 exponents apart: 26 units of 2^-55 and half a unit of
     the product, 2^-52, of the cell's largest product, and one rounding of the result."""
     rng = np.random.default_rng(spread + 7)
     u0 = rng.standard_normal((4, 11, 34)) * 2.0 ** rng.integers(-spread, spread + 1, (4, 11, 34))
     u0[rng.random(u0.shape) < 0.1] = 0.0
     w = equal_weights(3, 1)
     got = run(st, u0, w, 1, DIRICHLET, 1, (1, st.VARIANT_STREAM))
-    slack = Fraction(16 * 2.0 ** -55 + 2.0 ** -52)
+    slack = Fraction(26 * 2.0 ** -55 + 2.0 ** -52)
     for at in np.ndindex(*u0.shape):
         want, top = exact_sum(u0, w, at, 1)
         assert abs(Fraction(float(got[at])) - want) <= abs(want) * Fraction(EPS) + top * slack, at
@@ -469,3 +469,15 @@ def test_equal_box_tiles_3d(st, shape, boundary, tile):
         top = np.abs(u0[np.isfinite(u0)]).max()
         assert np.abs(got[fine] - ref[fine]).max(initial=0.0) <= T * (2 * w.size + 2) * EPS * top
         assert np.array_equal(got == 0.0, ref == 0.0)
+
+
+@pytest.mark.parametrize("ndim,radius,shape", [(2, 1, (64, 128)), (2, 2, (64, 128)), (3, 1, (16, 32, 64))])
+def test_equal_boxes_lean_to_no_side(st, ndim, radius, shape):
+    """A field and its negative over many steps: sums that lose or gain a unit of 2^-58 a value and
+    step on one side would end 160 of them apart, 5e-16; roundings to nearest differ cell by
+    cell at most, which the mean of some thousand cells does not show."""
+    w, T = equal_weights(ndim, radius), 160
+    u0 = synth.uniform(48, shape)
+    a, b = (run(st, sign * u0, w, radius, PERIODIC, T, (1, st.VARIANT_STREAM)) for sign in (1.0, -1.0))
+    total = sum(Fraction(float(x)) for x in a.flat)
+    assert abs(total + sum(Fraction(float(x)) for x in b.flat)) <= total * Fraction(EPS) / 2
