@@ -425,11 +425,14 @@ int one_step_variant(const stencil_plan_s* p) {
 
 // Whether a run that would take its steps one at a time in one persistent launch, by
 // default and not by a caller's or the tuner's choice, takes one launch per step instead:
-// in the integer form each of those is set up while the step before runs, and TMA copies
-// whole tiles (heat, GStencil/s, streamed against persistent: 1000^2 107 / 90, 600^2 73 / 60,
-// 1536^2 157 / 118).  Rows off 16 bytes, which TMA does not take, stay (1001^2).
+// in the integer form each of those is set up while the step before runs.  By TMA copies
+// (heat, GStencil/s, streamed against persistent: 1000^2 107 / 90, 600^2 73 / 60, 1536^2
+// 157 / 118), or by bulk copies where the grid fills its tiles (us a step of 60, streamed
+// against persistent: 331 x 1101 5.8 / 7.3, 1001^2 12.0 / 13.3, 3804 x 314 12.5 / 13.7,
+// 1024 x 2050 17.6 / 20.0).
 bool streams_anyway(const stencil_plan_s* p, int Tb, int variant, bool stream_ok) {
-  return variant == kVariantPersistent && Tb == 1 && p->user_variant == 0 && p->wide.n && stream_ok;
+  return variant == kVariantPersistent && Tb == 1 && p->user_variant == 0 && p->wide.n &&
+         (stream_ok || (streamed_any_shape(p) && wide_steps_worth(p->g.ny, p->g.nx)));
 }
 
 // Resolved (Tb, variant, streaming tile height; 0 = the kernel's default) for
@@ -809,7 +812,7 @@ int run_const(stencil_plan_s* p, double* d_grid, int64_t T, cudaStream_t s) {
                   "height (16; 32 for the 3D star)");
     variant = kVariantDirect;
   }
-  if (!tuned && streams_anyway(p, Tb, variant, stream_ok)) variant = kVariantStream;
+  if (!tuned && streams_anyway(p, Tb, variant, stream_ok)) variant = stream_ok ? kVariantStream : kVariantDirect;
   Steps3dLaunch steps3d;
   int z;
   if (steps3d_anyway(p, tuned, tile_y, s, steps3d, z) && T > 2 && T <= (1 << 30))

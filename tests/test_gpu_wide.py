@@ -481,3 +481,16 @@ def test_equal_boxes_lean_to_no_side(st, ndim, radius, shape):
     a, b = (run(st, sign * u0, w, radius, PERIODIC, T, (1, st.VARIANT_STREAM)) for sign in (1.0, -1.0))
     total = sum(Fraction(float(x)) for x in a.flat)
     assert abs(total + sum(Fraction(float(x)) for x in b.flat)) <= total * Fraction(EPS) / 2
+
+
+# more cells than the temporal kernel takes, rows that TMA does not take: one row or column more
+# than a tile, tiles four fifths full and a little less
+@pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
+@pytest.mark.parametrize("shape", [(513, 513), (600, 602), (331, 1101), (4097, 65), (2600, 103), (2600, 102)])
+def test_stars_by_default_equal_the_persistent_kernel(st, shape, boundary):
+    w = synth.heat_weights(2, 0.2)
+    u0 = synth.normal(49, shape)
+    for T in (1, 6):
+        for offset in (0, 1):
+            got = run(st, u0, w, 1, boundary, T, (0, 0), offset)
+            assert np.array_equal(got, run(st, u0, w, 1, boundary, T, (1, st.VARIANT_PERSISTENT), offset)), (T, offset)
