@@ -256,7 +256,7 @@ __device__ __forceinline__ void unit_rows(const XSlot& sl, const RegWeights<NT>&
 // see unit_chain).  The values are unpacked from the unit's planes, their rows
 // read twice: for the largest exponents, then for the sums (the 36 values of a
 // box's pair would not fit the registers).
-template <int NT, bool BOX>
+template <int NT, bool BOX, bool HEAT>
 __device__ __forceinline__ bool unit_row_wide(const XSlot& sl, const WideTaps& T, int r, int lane, double (&out)[2]) {
   auto row = [&](int dz, int dy, double (&v)[4]) {  // columns x-1 .. x+2
     const double2 p = *reinterpret_cast<const double2*>(&sl.plane[dz + 1][r + 1 + dy][2 * lane]);
@@ -285,7 +285,8 @@ __device__ __forceinline__ bool unit_row_wide(const XSlot& sl, const WideTaps& T
       const WideVal u[7] = {wide_unpack(zm[1 + i]), wide_unpack(n[1 + i]), x[i], x[i + 1], x[i + 2],
                             wide_unpack(s[1 + i]), wide_unpack(zp[1 + i])};
       bool ok;
-      out[i] = wide_sum<7>(u, T, ok);
+      if constexpr (HEAT) out[i] = wide_sum_heat<7>(u, T, ok);
+      else out[i] = wide_sum<7>(u, T, ok);
       all = all && ok;
     }
     return all;
@@ -450,7 +451,7 @@ __device__ int build_segs(const XParams& P, int ra, int rb, int ytop, int wrap, 
   return ns;
 }
 
-template <int NT, bool BOX, bool PERIODIC, bool WIDE>
+template <int NT, bool BOX, bool PERIODIC, int WIDE>
 __global__ void __launch_bounds__(kThreadsX, 1) k_exchange3d(const __grid_constant__ XParams P) {
   const int K = P.K;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -716,14 +717,24 @@ __global__ void __launch_bounds__(kThreadsX, 1) k_exchange3d(const __grid_consta
         else if (y0 + r >= P.own_lo && y0 + r < P.own_hi) st_global_v2_cs(P.dst + off, v0, v1);
       };
       if constexpr (WIDE) {
+        auto finish = [&](int r, const double (&v)[2], bool all) {
+          if (!xin) return;
+          put(r, v[0], v[1]);
+          if (!all && (!last || (y0 + r >= P.own_lo && y0 + r < P.own_hi)))
+            unit_chain<NT, BOX>(sl, P.wide, P.wdev, r, lane, (last ? P.dst : P.ring) + base + (int64_t)r * P.nx);
+        };
+        if (!BOX && r0 + kWarps < h) {  // the star's two rows together: four sums in flight
+          double v[2][2];
+          const bool all0 = unit_row_wide<NT, BOX, WIDE == kHeat>(sl, P.wide, r0, lane, v[0]);
+          const bool all1 = unit_row_wide<NT, BOX, WIDE == kHeat>(sl, P.wide, r0 + kWarps, lane, v[1]);
+          finish(r0, v[0], all0);
+          finish(r0 + kWarps, v[1], all1);
+        } else {
 #pragma unroll 1
-        for (int r = r0; r < h; r += kWarps) {
-          double v[2];
-          const bool all = unit_row_wide<NT, BOX>(sl, P.wide, r, lane, v);
-          if (xin) {
-            put(r, v[0], v[1]);
-            if (!all && (!last || (y0 + r >= P.own_lo && y0 + r < P.own_hi)))
-              unit_chain<NT, BOX>(sl, P.wide, P.wdev, r, lane, (last ? P.dst : P.ring) + base + (int64_t)r * P.nx);
+          for (int r = r0; r < h; r += kWarps) {
+            double v[2];
+            const bool all = unit_row_wide<NT, BOX, WIDE == kHeat>(sl, P.wide, r, lane, v);
+            finish(r, v, all);
           }
         }
       } else if (r0 + kWarps < h) {
@@ -782,7 +793,7 @@ bool encode_ring(CUtensorMap* map, const double* base, int nx, int nyb, int K, i
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int NT, bool BOX, bool PERIODIC, bool WIDE>
+template <int NT, bool BOX, bool PERIODIC, int WIDE>
 int x_occupancy() {
   static std::atomic<int> cache[kMaxDeviceOrdinals];
   return cached_per_device(cache, [] {
@@ -796,7 +807,7 @@ int x_occupancy() {
   });
 }
 
-template <int NT, bool BOX, bool PERIODIC, bool WIDE>
+template <int NT, bool BOX, bool PERIODIC, int WIDE>
 cudaError_t launch_x(const ExchangeLaunch& L, cudaStream_t stream) {
   if (x_occupancy<NT, BOX, PERIODIC, WIDE>() < 1) return cudaErrorInvalidConfiguration;
   XParams P;
@@ -905,11 +916,13 @@ cudaError_t launch_exchange(Shape shape, int boundary, const ExchangeLaunch& L, 
   const bool per = boundary == kPeriodic;
   if (L.Tb < 2 || L.Tb > kMaxStages || L.tiles_x < 1 || L.band.tiles_y < 1) return cudaErrorInvalidValue;
   if (shape == Shape::kBox)
-    return L.wide.n ? (per ? launch_x<27, true, true, true>(L, stream) : launch_x<27, true, false, true>(L, stream))
-                    : (per ? launch_x<27, true, true, false>(L, stream) : launch_x<27, true, false, false>(L, stream));
+    return L.wide.n ? (per ? launch_x<27, true, true, kWide>(L, stream) : launch_x<27, true, false, kWide>(L, stream))
+                    : (per ? launch_x<27, true, true, kChain>(L, stream) : launch_x<27, true, false, kChain>(L, stream));
+  if (L.wide.heat)
+    return per ? launch_x<7, false, true, kHeat>(L, stream) : launch_x<7, false, false, kHeat>(L, stream);
   if (L.wide.n)
-    return per ? launch_x<7, false, true, true>(L, stream) : launch_x<7, false, false, true>(L, stream);
-  return per ? launch_x<7, false, true, false>(L, stream) : launch_x<7, false, false, false>(L, stream);
+    return per ? launch_x<7, false, true, kWide>(L, stream) : launch_x<7, false, false, kWide>(L, stream);
+  return per ? launch_x<7, false, true, kChain>(L, stream) : launch_x<7, false, false, kChain>(L, stream);
 }
 
 }  // namespace gbst
