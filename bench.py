@@ -41,15 +41,15 @@ HEADLINE = dict(name="heat3d-7pt", shape=(512, 512, 512), T=1000, alpha=0.1, bou
 # update (13) plus 3 faces x (2 differences, 1 product, 1 sum) = 25.
 FLOPS = {"heat3d-7pt": 13, "box2d-9pt": 17, "box3d-27pt": 53, "heat2d-5pt": 9,
          "varcoef-7pt": 13, "adjoint-7pt": 13 + 25, "star2d-9pt": 17, "box2d-25pt": 49,
-         "heat1d-3pt": 5, "star1d-5pt": 9}
+         "heat1d-3pt": 5, "star1d-5pt": 9, "box2d-9pt-general": 17}
 NOMINAL_FP64_TFLOPS = 2 * 152 * 2.07e9 * 2 / 1e12   # 2 DFMA/clk/SM x 152 SMs x 2.07 GHz x 2 flop
-# FP64 instructions the kernels issue per cell update (one pipe slot each):
+# FP64 instructions the FMA-chain kernels issue per cell update (one pipe slot each):
 # K for a K-tap chain; 4.25 for the equal-weight 9-point box with shared
 # partial sums (17 warp instructions per 2 rows x 64 columns, strip edges
 # included); adjoint: forward 7 + recompute 7 + transposed step 7 + 3 faces x 3.
 INSTR = {"heat3d-7pt": 7, "box3d-27pt": 27, "box2d-9pt": 4.25, "heat2d-5pt": 5,
          "varcoef-7pt": 7, "adjoint-7pt": 7 + 7 + 7 + 9, "star2d-9pt": 9, "box2d-25pt": 25,
-         "heat1d-3pt": 3 * (2048 + 8) / 2048, "star1d-5pt": 5 * (2048 + 16) / 2048}
+         "box2d-9pt-general": 9, "heat1d-3pt": 3 * (2048 + 8) / 2048, "star1d-5pt": 5 * (2048 + 16) / 2048}
 
 
 # ------------------------------------------------------------------ helpers
@@ -173,7 +173,14 @@ KERNEL_SOURCES = {"stream3d": ["stream.cu", "ptx.cuh", "taps.cuh"],
                   "batched": ["batched.cu"],
                   "persistent": ["batched.cu"],
                   "varcoef": ["varcoef.cu", "taps.cuh"],
-                  "adjoint": ["varcoef.cu", "taps.cuh"]}
+                  "adjoint": ["varcoef.cu", "taps.cuh"],
+                  # the kernels (or forms of kernels) that take the weighted sum in integer arithmetic
+                  "wide3d": ["wide3d.cu", "widestream.cuh", "wide.cuh", "ptx.cuh"],
+                  "wide2d": ["wide2d.cu", "widestream.cuh", "wide.cuh", "ptx.cuh"],
+                  "wide1d": ["wide1d.cu", "wide.cuh"],
+                  "exchange-wide": ["exchange.cu", "wide.cuh", "ptx.cuh", "taps.cuh"],
+                  "persistent-wide": ["batched.cu", "wide.cuh"],
+                  "batched-wide": ["batched.cu", "widesteps.cu", "widestream.cuh", "wide.cuh", "ptx.cuh"]}
 
 
 def _code_only(text):
@@ -238,6 +245,72 @@ def variant_kernel(variant, ndim):
     return variant
 
 
+def running_kernel(variant, ndim):
+    """The kernel that a constant-weight plan with positive weights (every one here) runs
+    as this variant: the integer form where the variant has one."""
+    if variant == "temporal":
+        return "wide1d" if ndim == 1 else "temporal"
+    k = variant_kernel(variant, ndim)
+    return {"stream3d": "wide3d", "stream2d": "wide2d", "exchange": "exchange-wide",
+            "persistent": "persistent-wide"}.get(k, k)
+
+
+ISSUE_PEAK = 152 * 4 * 32 * 2.07e9   # lane instructions per second: 4 warp instructions a clock and SM
+
+
+def recorded_issue(kernel, workload):
+    """(instructions issued, FP64 instructions) per cell update of an integer-form kernel, counted by
+    ncu (profiles/int_instr.txt) on its current sources; None otherwise."""
+    path = os.path.join(ROOT, "profiles", "int_instr.txt")
+    if not os.path.exists(path) or kernel not in KERNEL_SOURCES:
+        return None
+    cur = kernel_source_hash(kernel)
+    for ln in open(path):
+        parts = ln.split()
+        if len(parts) >= 5 and not ln.startswith("#") and parts[0] == kernel and parts[1] == workload and \
+                parts[4] == cur:
+            return float(parts[2]), float(parts[3])
+    return None
+
+
+def integer_roofline(name, cells, T, ms, launches, kernel, Tb, bytes_per_cell, traffic_key, peak_tflops):
+    """The roofline of a kernel that takes the sum in integer arithmetic: the rate at which it could
+    issue its instructions (ncu count per cell), or the HBM bandwidth where that is lower."""
+    counted = recorded_issue(kernel, f"{name}@tb{Tb}" if Tb > 1 else name)
+    rate = cells * T / (ms * 1e-3)
+    hbm = HBM_GBS * 1e9 * Tb / bytes_per_cell
+    issue = ISSUE_PEAK / counted[0] if counted else None
+    gbs = rate * bytes_per_cell / Tb / 1e9
+    if issue is not None and issue <= hbm:
+        out = {"bound": "alu", "achieved": round(rate * counted[0] / 1e12, 4), "peak": round(ISSUE_PEAK / 1e12, 4),
+               "unit": "Tinstr/s", "frac": round(rate / issue, 4),
+               "frac_basis": f"{counted[0]:g} instructions per cell (ncu count) / 152 SMs x 4 x 32 lanes at 2.07 GHz: "
+                             "the weighted sum is taken in integer arithmetic"}
+    else:
+        out = {"bound": "hbm", "achieved": round(gbs, 2), "peak": round(HBM_GBS, 1), "unit": "GB/s",
+               "frac": round(gbs / HBM_GBS, 4),
+               "frac_basis": f"algorithmic bytes ({bytes_per_cell} per cell per Tb block) / measured HBM copy" +
+                             ("" if counted else "; no current instruction count of this kernel")}
+    F = FLOPS[name]
+    fp64 = peak_tflops * 1e12 / F
+    out.update({
+        "issue_ceiling_gstencil_per_s": None if issue is None else round(issue / 1e9, 3),
+        "hbm_ceiling_gstencil_per_s": round(hbm / 1e9, 3),
+        # what a chain of FP64 multiply-adds could reach: these kernels go past it
+        "fp64_ceiling_gstencil_per_s": round(fp64 / 1e9, 3),
+        "frac_of_stated_roofline": out["frac"],
+        "instr_per_cell": None if counted is None else counted[0],
+        "fp64_instr_per_cell": None if counted is None else counted[1],
+        "fp64_instr_source": "ncu count, profiles/int_instr.txt" if counted else "none (kernel changed since the count)",
+        "fp64_pipe_frac": None if counted is None else round(counted[1] * rate / (peak_tflops * 1e12 / 2), 4),
+        "traffic": recorded_traffic(kernel, traffic_key or (name if Tb == 1 else f"{name}@tb{Tb}")),
+        "algorithmic_flops_per_launch": F * cells * T / max(launches, 1),
+        "algorithmic_bytes_per_launch": bytes_per_cell * cells * T / Tb / max(launches, 1),
+        "peak_source": "152 SMs x 4 warp instructions a clock at the maximum SM clock; FP64 peak: DFMA "
+                       "microbenchmark measured in this run, best of 3 (x2 flop/FMA)"})
+    return out
+
+
 def _measured_hbm_gbs(default=6681.8):
     """HBM copy bandwidth (GB/s) from MEASURED_PEAKS.json beside this script
     when present (a STREAM-style copy measured on GB300), else `default`,
@@ -258,6 +331,8 @@ def roofline(name, cells, T, ms, launches, peak_tflops, kernel, Tb=1, bytes_per_
     cell) in cell updates per second; `frac` = achieved FP64 flops / peak
     (the FP64 term binds for every workload here).  `traffic_key` names the
     DRAM-traffic record when it is not the workload name (plus "@tb<Tb>")."""
+    if kernel.startswith("wide") or kernel.endswith("-wide"):
+        return integer_roofline(name, cells, T, ms, launches, kernel, Tb, bytes_per_cell, traffic_key, peak_tflops)
     F = FLOPS[name] if flops is None else flops
     achieved = F * cells * T / (ms * 1e-3) / 1e12
     per_launch = F * cells * T / max(launches, 1)
@@ -419,18 +494,23 @@ def form_const(st, name, shape, radius, weights, boundary, T, u0, stream, peak, 
     sweep = None
     if tb_sweep:
         sweep = {}
-        fp64_ceiling = peak * 1e12 / FLOPS[name] / 1e9
         for tbs, vs in tb_sweep:
             plan.set_tuning(tbs, vs)
             ms_s, _ = time_plan(st, plan, grid, T, 1, stream)
             rate = cells * T / (ms_s * 1e-3) / 1e9
-            ceiling = min(fp64_ceiling, HBM_GBS * tbs / 16)
-            entry = {"gstencil_per_s": round(rate, 3), "frac_of_stated_roofline": round(rate / ceiling, 4)}
+            entry = {"gstencil_per_s": round(rate, 3)}
             instr = shared_sum_instr(name, st.stencil_variant_name(vs), tbs)
-            if instr is not None and rate / ceiling > 1.0:
+            kernel = running_kernel(st.stencil_variant_name(vs), len(shape))
+            if "wide" in kernel:
+                r = roofline(name, cells, T, ms_s, T // tbs, peak, kernel, Tb=tbs)
+                entry.update(frac_of_stated_roofline=r["frac"], frac_basis=r["frac_basis"])
+            elif instr is not None:
                 # shared partial sums: F over-counts the work, report the executed fraction
                 entry["frac_of_stated_roofline"] = round(rate * 1e9 * instr / (peak * 1e12 / 2), 4)
                 entry["frac_basis"] = f"executed FP64 instructions ({instr:.3f} per cell) / peak"
+            else:  # the integer form too, not counted: against the HBM bandwidth
+                entry["frac_of_stated_roofline"] = round(rate / (HBM_GBS * tbs / 16), 4)
+                entry["frac_basis"] = "algorithmic bytes / measured HBM copy"
             sweep[f"Tb={tbs} {st.stencil_variant_name(vs)}"] = entry
         plan.set_tuning(0, 0)
     plan.close()
@@ -443,7 +523,7 @@ def form_const(st, name, shape, radius, weights, boundary, T, u0, stream, peak, 
            "tile": list(tile) if tile[0] else None,
            "launches": launches,
            "roofline": roofline(name, cells, T, ms, launches, peak,
-                                variant_kernel(st.stencil_variant_name(v), len(shape)), Tb=tb)}
+                                running_kernel(st.stencil_variant_name(v), len(shape)), Tb=tb)}
     if sweep is not None:
         out["tb_sweep_gstencil_per_s"] = sweep
     return out
@@ -466,10 +546,9 @@ def shared_sum_instr(name, variant, Tb):
 
 def form_forced(st, name, shape, radius, weights, boundary, T, u0, stream, peak, Tb, variant, reps=1,
                 traffic_key=None):
-    """One constant-weight workload on a forced (Tb, variant), with its roofline:
-    FP64 instructions per cell include what the exchange kernel computes
-    twice (the periodic z-halo, (Tb-1)/nz of the planes, and the margin rows
-    of a plane cut into bands).  `u0`: the initial grid, or a seed for a
+    """One constant-weight workload on a forced (Tb, variant), with its roofline (the
+    instruction counts include what the exchange kernel computes twice: the
+    periodic z-halo and the margin rows of a plane cut into bands).  `u0`: the initial grid, or a seed for a
     uniform grid drawn on the device."""
     import torch
     if isinstance(u0, np.ndarray):
@@ -488,17 +567,11 @@ def form_forced(st, name, shape, radius, weights, boundary, T, u0, stream, peak,
     del grid
     torch.cuda.empty_cache()
     cells = int(np.prod(shape))
-    counted = recorded_instr(variant_kernel(vname, len(shape)), name)
-    instr = INSTR[name] if counted is None else counted
-    if vname == "exchange":
-        if boundary == 1:
-            instr *= 1 + (Tb - 1) / shape[0]  # the stage skew's extra planes
-        instr *= bands[1] / shape[1]          # margin rows that two bands both compute
     out = {"workload": f"{name} {'x'.join(map(str, shape))} T={T} {'periodic' if boundary else 'dirichlet0'}",
            "gstencil_per_s": round(cells * T / (ms * 1e-3) / 1e9, 3), "ms": round(ms, 3), "Tb": Tb,
            "variant": vname, "launches": launches,
-           "roofline": roofline(name, cells, T, ms, launches, peak, variant_kernel(vname, len(shape)), Tb=Tb,
-                                instr=instr, traffic_key=traffic_key)}
+           "roofline": roofline(name, cells, T, ms, launches, peak, running_kernel(vname, len(shape)), Tb=Tb,
+                                traffic_key=traffic_key)}
     if bands is not None:
         out["bands"] = {"count": bands[0], "rows_computed": bands[1], "rows": shape[1]}
     return out
@@ -570,10 +643,10 @@ def form_table1(st, stream, peak):
         ms, launches = time_plan(st, plan, grid, T, 1, stream)
         tb, v = plan.get_tuning()
         cells = int(np.prod(shape))
-        # the shared-partial-sum count of INSTR holds only for equal box weights
-        instr = 9 if name == "box2d-9pt" and not np.all(w == w.flat[0]) else None
-        r = roofline(name, cells, T, ms, max(launches, 1), peak,
-                     variant_kernel(st.stencil_variant_name(v), len(shape)), Tb=tb, instr=instr)
+        # the count of the equal-weight box does not hold for general weights
+        key = "box2d-9pt-general" if name == "box2d-9pt" and not np.all(w == w.flat[0]) else name
+        r = roofline(key, cells, T, ms, max(launches, 1), peak,
+                     running_kernel(st.stencil_variant_name(v), len(shape)), Tb=tb)
         out[label] = {"shape": list(shape), "T": T, "variant": st.stencil_variant_name(v), "Tb": tb,
                       "gstencil_per_s": round(cells * T / (ms * 1e-3) / 1e9, 3),
                       "frac": r["frac"], "fp64_pipe_frac": r["fp64_pipe_frac"]}
@@ -632,7 +705,7 @@ def form_batched(st, stream, peak, rank=0, world=1):
             "plain_sweep_ms": round(ms_plain, 3),
             "plain_sweep_gstencil_per_s": round(updates / (ms_plain * 1e-3) / 1e9, 3),
             "speedup_vs_plain": round(ms_plain / ms, 3),
-            "roofline": roofline("heat2d-5pt", updates, 1, ms, max(launches, 1), peak, "batched")}
+            "roofline": roofline("heat2d-5pt", updates, 1, ms, max(launches, 1), peak, "batched-wide")}
 
 
 def form_adjoint(st, stream, peak):
@@ -825,7 +898,7 @@ def thermal_case(st, n, T, stream, fp32=True, peak=None):
     rate = n * n * T / (ms * 1e-3)
     if peak:
         out["roofline"] = roofline("heat2d-5pt", n * n, T, ms, T, peak,
-                                   variant_kernel(st.stencil_variant_name(v), 2), Tb=tb,
+                                   running_kernel(st.stencil_variant_name(v), 2), Tb=tb,
                                    traffic_key=f"heat2d-5pt-{n}sq" if tb == 1 else None)
     if n == THERMAL["n"]:
         full = THERMAL["n"] ** 2 * THERMAL["T_full"] / rate
@@ -999,7 +1072,7 @@ def main():
                             "direct": "one cell per thread, 32 x 8 threads"}.get(h["variant"], h["variant"]),
                    "l2_flush": "none needed: each launch streams 2 GiB > 129 MB L2"},
         "roofline": roofline("heat3d-7pt", cells, T, h["ms"], h["launches"] // args.steps,
-                             peak_tflops, variant_kernel(h["variant"], 3), Tb=h["Tb"]),
+                             peak_tflops, running_kernel(h["variant"], 3), Tb=h["Tb"]),
         "fp64_peak_tflops_measured": round(peak_tflops, 4),
         "e2e": {"value": round(e2e_value, 4), "unit": "GStencil/s",
                 "h2d_bytes_per_step": h["h2d"], "d2h_bytes_per_step": h["d2h"],
