@@ -590,6 +590,7 @@ bool steps3d_anyway(stencil_plan_s* p, bool tuned, int tile_y, cudaStream_t s, S
   return ensure_flags(p, bricks) == STENCIL_OK;
 }
 
+constexpr int kNotHere = 1;  // nothing was enqueued that matters: another kernel takes the run
 int run_steps3d(stencil_plan_s* p, double* d_grid, int64_t T, Steps3dLaunch& L, int z, cudaStream_t s) {
   const size_t bytes = (size_t)L.bricks[0] * L.bricks[1] * L.bricks[2] * kFlagWords * sizeof(unsigned int);
   CUDA_TRY(cudaMemsetAsync(p->d_flags, 0, bytes, s), "clearing the progress words");
@@ -606,6 +607,10 @@ int run_steps3d(stencil_plan_s* p, double* d_grid, int64_t T, Steps3dLaunch& L, 
   L.status = p->d_status;
   L.spin_limit = kSpinLimitNs;
   cudaError_t e = launch_steps3d(L, z, s);
+  if (e == cudaErrorCooperativeLaunchTooLarge) {  // (a process that may not use every SM)
+    cudaGetLastError();
+    return kNotHere;
+  }
   if (e != cudaSuccess) return cuda_fail(e, "launching the persistent 3D kernel");
   return STENCIL_OK;
 }
@@ -815,8 +820,10 @@ int run_const(stencil_plan_s* p, double* d_grid, int64_t T, cudaStream_t s) {
   if (!tuned && streams_anyway(p, Tb, variant, stream_ok)) variant = stream_ok ? kVariantStream : kVariantDirect;
   Steps3dLaunch steps3d;
   int z;
-  if (steps3d_anyway(p, tuned, tile_y, s, steps3d, z) && T > 2 && T <= (1 << 30))
-    return run_steps3d(p, d_grid, T, steps3d, z, s);
+  if (steps3d_anyway(p, tuned, tile_y, s, steps3d, z) && T > 2 && T <= (1 << 30)) {
+    rc = run_steps3d(p, d_grid, T, steps3d, z, s);
+    if (rc != kNotHere) return rc;
+  }
   if (variant == kVariantPersistent && Tb > 1) {
     if (p->ndim == 2 && p->radius == 1 && (p->taps.n == 5 || p->taps.n == 9) && Tb <= 8)
       return run_persistent_tb(p, d_grid, T, Tb, s);

@@ -245,7 +245,7 @@ cudaError_t launch_z(const Steps3dLaunch& L, cudaStream_t stream) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, L);
-  g_launches.fetch_add(1, std::memory_order_relaxed);
+  if (e == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
   return e;
 }
 

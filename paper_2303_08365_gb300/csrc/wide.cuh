@@ -310,19 +310,6 @@ __device__ __forceinline__ double wide_equal(long long S, int E, const Taps& T) 
   return wide_double(hh + (hl >> 24), E - T.bias + kEqualShift<N> - 1);
 }
 
-// The same with the FMA chain in its place where it has to be.
-template <int NT, class Taps>
-__device__ __forceinline__ double wide_sum(const WideVal (&u)[NT], const Taps& T, const double* __restrict__ wdev) {
-  bool ok;
-  const double r = wide_sum<NT>(u, T, ok);
-  if (ok) return r;
-  if (wide_zeros<NT>(u)) return 0.0;
-  double v[NT];
-#pragma unroll
-  for (int k = 0; k < NT; ++k) v[k] = wide_repack(u[k]);
-  return wide_chain(v, wdev, NT);
-}
-
 // How a kernel takes the weighted sum of a cell, collected tap by tap: the FMA
 // chain in tap order, or the integer form once every value is there (kHeat: for
 // weights that wide_sum_heat takes).
