@@ -248,6 +248,23 @@ int any_shape_tile_y(const stencil_plan_s* p) {
   return p->shape == Shape::kBox && p->cells() < (int64_t)1 << 20 ? 8 : 16;
 }
 
+// The plan's split weights for a kernel that takes fewer of them (a split anew would
+// cost each short run a microsecond).
+template <int N>
+void narrow(const WideTaps& w, WideTapsOf<N>& t) {
+  t.n = w.n <= N ? w.n : 0;
+  for (int k = 0; k < t.n; ++k) {
+    t.hi[k] = w.hi[k];
+    t.hi2[k] = w.hi2[k];
+    t.lo[k] = w.lo[k];
+    t.ex[k] = w.ex[k];
+  }
+  t.heat = w.heat;
+  t.bias = w.bias;
+  t.e_min = w.e_min;
+  t.e_span = w.e_span;
+}
+
 std::string device_name();
 
 std::string plan_key(const stencil_plan_s* p) {
@@ -536,7 +553,7 @@ int run_persistent_tb(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, cuda
   L.nx = p->g.nx;
   L.T = T;
   L.wdev = p->d_w;
-  if (p->wide.n) make_wide(p->taps.w, p->taps.n, L.wide);
+  narrow(p->wide, L.wide);
   L.flags = p->d_flags;
   L.status = p->d_status;
   L.spin_limit = kSpinLimitNs;
@@ -558,7 +575,7 @@ int run_wide_steps(stencil_plan_s* p, double* d_grid, int64_t T, cudaStream_t s)
   it.nx = p->g.nx;
   it.T = (int)T;
   for (int k = 0; k < 5; ++k) it.w[k] = p->taps.w[k];
-  make_wide(it.w, 5, it.wide);
+  narrow(p->wide, it.wide);
   WideStepsLaunch L;
   wide_step_item(L.one, it, 0);
   L.nitems = 1;
@@ -602,7 +619,7 @@ int run_steps3d(stencil_plan_s* p, double* d_grid, int64_t T, Steps3dLaunch& L, 
   L.periodic = p->boundary == kPeriodic;
   L.T = (int)T;
   L.wdev = p->d_w;
-  make_wide(p->taps.w, 7, L.wide);
+  narrow(p->wide, L.wide);
   L.progress = p->d_flags;
   L.status = p->d_status;
   L.spin_limit = kSpinLimitNs;
@@ -738,7 +755,7 @@ int run_steps(stencil_plan_s* p, double* d_grid, int64_t T, int Tb, int variant,
       steps = Tb;
     } else if (variant == kVariantTemporal && p->ndim == 1 && p->wide.n) {
       WideTapsOf<5> wide;
-      make_wide(p->taps.w, p->taps.n, wide);
+      narrow(p->wide, wide);
       steps = (int)std::min<int64_t>(Tb, T - t);
       e = launch_wide1d(p->radius, p->boundary, steps, p->g, wide, p->d_w, a, b, sms, s);
     } else if (variant == kVariantTemporal && T - t >= Tb) {
