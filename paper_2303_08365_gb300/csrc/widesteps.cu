@@ -128,6 +128,14 @@ __device__ __noinline__ void chain_cells(const Plane& u, int row0, int rows, int
 
 constexpr int kProgressStride = kProgressWords / kWideStepCtas;  // half a line for each CTA's word
 
+// Whether all lanes' waits ended well; what each of them has acquired holds for all from
+// here on (the vote alone orders no memory).
+__device__ __forceinline__ bool joined(bool ok) {
+  ok = __all_sync(0xffffffffu, ok);
+  __syncwarp();
+  return ok;
+}
+
 // Waits until CTAs first[k]..last[k] (k < 3) have done `steps` steps (false: gave up:
 // the limit is on the time in which none of a lane's makes a step).  All 32 lanes; a
 // lane's loads are in flight together.
@@ -160,7 +168,7 @@ __device__ bool wait_progress(const unsigned int* progress, const int (&first)[3
         if (!ok) break;
       }
     }
-    return __all_sync(0xffffffffu, ok);
+    return joined(ok);
   }
   for (int k0 = (int)(threadIdx.x & 31); ok && k0 < n; k0 += 32 * kLoads) {
     const unsigned int* p[kLoads];
@@ -201,7 +209,7 @@ __device__ bool wait_progress(const unsigned int* progress, const int (&first)[3
     }
   }
   asm volatile("fence.acq_rel.gpu;" ::: "memory");
-  return __all_sync(0xffffffffu, ok);
+  return joined(ok);
 }
 
 // The CTA whose range of `tiles` tiles over n CTAs holds tile j.
