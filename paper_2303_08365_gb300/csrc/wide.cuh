@@ -136,13 +136,14 @@ __device__ __forceinline__ double wide_repack(const WideVal& u) {
 }
 
 // The FMA chain for the neighbourhoods that the integer form does not take
-// (wdev: the weights as doubles).  Out of line: it is rarely run.
+// (wdev: the weights as doubles, in global memory or among a kernel's parameters, so by plain
+// loads: the read-only path takes global addresses alone).  Out of line: it is rarely run.
 static __device__ __noinline__ double wide_chain(const double* v, const double* wdev, int n) {
   long long any = 0;
   for (int k = 0; k < n; ++k) any |= __double_as_longlong(v[k]) << 1;
   if (any == 0) return 0.0;  // every value is a zero
   double acc = 0.0;
-  for (int k = 0; k < n; ++k) acc = fma(__ldg(wdev + k), v[k], acc);
+  for (int k = 0; k < n; ++k) acc = fma(wdev[k], v[k], acc);
   return acc;
 }
 

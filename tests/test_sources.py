@@ -23,3 +23,13 @@ def test_a_vote_on_waits_is_followed_by_a_warp_barrier():
                 seen += 1
                 assert code[k + 1] == "__syncwarp()", (os.path.basename(path), s)
     assert seen >= 2
+
+
+def test_the_fma_chain_reads_its_weights_by_plain_loads():
+    """wide_chain's weights may lie among a kernel's parameters (a single grid's tile kernel):
+    __ldg is a load from global memory and undefined there."""
+    code = statements(os.path.join(CSRC, "wide.cuh"))
+    at = next(k for k, s in enumerate(code) if re.search(r"double wide_chain\(", s))
+    body = code[at + 1:code.index("return acc", at)]
+    assert any("fma(wdev[k], v[k], acc)" in s for s in body)
+    assert not any("__ldg" in s for s in body)
