@@ -223,7 +223,8 @@ void build_taps(stencil_plan_s* p, const double* w) {
 }
 
 // The stencil classes whose kernels have the integer form of the sum.  All
-// kernels of a class take it, so its results do not depend on the kernel.
+// kernels of a class take it, so its results do not depend on the kernel (but for the overlapped
+// temporal kernel's 2D box of equal weights).
 bool uses_wide(int ndim, int radius) {
   return (ndim == 3 && radius == 1) || ndim <= 2;
 }
@@ -260,6 +261,7 @@ void narrow(const WideTaps& w, WideTapsOf<N>& t) {
     t.ex[k] = w.ex[k];
   }
   t.heat = w.heat;
+  t.equal = w.equal;
   t.bias = w.bias;
   t.e_min = w.e_min;
   t.e_span = w.e_span;
@@ -1178,7 +1180,7 @@ int stencil_create(int ndim, const int64_t* dims, int radius, const double* weig
   p->boundary = boundary;
   p->shape = (star || ndim == 1) ? Shape::kStar : Shape::kBox;
   build_taps(p, weights);
-  if (uses_wide(ndim, radius)) make_wide(p->taps.w, p->taps.n, p->wide);
+  if (uses_wide(ndim, radius)) make_wide(p->taps.w, p->taps.n, p->wide, p->shape == Shape::kBox);
   *out = p;
   return STENCIL_OK;
 }

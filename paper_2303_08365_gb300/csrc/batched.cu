@@ -551,12 +551,20 @@ __global__ void __launch_bounds__(kPThreads, 2) k_persist_tb_wide(const __grid_c
               const int k = BOX ? (dy + 1) * 3 + (dx + 1) : (dy < 0 ? 0 : dy > 0 ? 4 : 2 + dx);
               u[k] = in.get(at + dy * RW + dx);
             }
-          WideAcc acc;
+          long long R;
           int E;
-          if constexpr (HEAT) E = wide_acc_heat<NT>(u, L.wide, acc);
-          else E = wide_acc<NT>(u, L.wide, acc);
-          if (m > 0) out.put(at, acc.val(E, L.wide));
-          else dst[(int64_t)y * nx + x] = acc.get(E, L.wide);
+          if constexpr (HEAT && BOX) {
+            WideSum S;
+            E = wide_acc_equal<NT>(u, S);
+            R = wide_equal(S, L.wide);
+          } else {
+            WideAcc acc;
+            if constexpr (HEAT) E = wide_acc_heat<NT>(u, L.wide, acc);
+            else E = wide_acc<NT>(u, L.wide, acc);
+            R = acc.rounded();
+          }
+          if (m > 0) out.put(at, wide_val(R, E - L.wide.bias));
+          else dst[(int64_t)y * nx + x] = wide_double(R, E - L.wide.bias);
           if (!wide_covers(E, L.wide)) {
             const double v = wide_zeros<NT>(u) ? 0.0 : ptb_chain_wide<NT, TB>(in, at, L.wdev);
             if (m > 0) out.put(at, wide_unpack(v));
@@ -816,6 +824,8 @@ cudaError_t launch_persist_tb(Shape shape, int boundary, int Tb, const PersistTb
                               cudaStream_t stream) {
   const bool per = boundary == kPeriodic;
   if (shape == Shape::kBox) {
+    if (L.wide.equal)
+      return per ? ptb_by_tb<9, true, true, kHeat>(Tb, L, sms, stream) : ptb_by_tb<9, true, false, kHeat>(Tb, L, sms, stream);
     if (L.wide.n)
       return per ? ptb_by_tb<9, true, true, kWide>(Tb, L, sms, stream) : ptb_by_tb<9, true, false, kWide>(Tb, L, sms, stream);
     return per ? ptb_by_tb<9, true, true, kChain>(Tb, L, sms, stream) : ptb_by_tb<9, true, false, kChain>(Tb, L, sms, stream);

@@ -147,7 +147,8 @@ __global__ void __launch_bounds__(256) k_direct_box125(const __grid_constant__ D
   }
 }
 
-// The same sweep with the weighted sum in the integer form (wide.cuh).
+// The same sweep with the weighted sum in the integer form (wide.cuh; HEAT: a star whose
+// weights wide_sum_heat takes, a box whose weights are all equal).
 template <int NDIM, int RAD, bool BOX, bool PERIODIC, bool HEAT>
 __global__ void __launch_bounds__(256) k_direct_wide(const __grid_constant__ DirectParams P,
                                                      const __grid_constant__ WideTaps wide) {
@@ -158,7 +159,8 @@ __global__ void __launch_bounds__(256) k_direct_wide(const __grid_constant__ Dir
     for (int k = 0; k < NT; ++k) u[k] = wide_unpack(v[k]);
     bool ok;
     double r;
-    if constexpr (HEAT) r = wide_sum_heat<NT>(u, wide, ok);
+    if constexpr (HEAT && BOX) r = wide_sum_equal<NT>(u, wide, ok);
+    else if constexpr (HEAT) r = wide_sum_heat<NT>(u, wide, ok);
     else r = wide_sum<NT>(u, wide, ok);
     if (ok) return r;
     if (wide_zeros<NT>(u)) return 0.0;
@@ -269,8 +271,8 @@ cudaError_t launch_p(const Geom& g, const HostTaps& ht, const WideTaps& wide, co
   if constexpr (NDIM <= 2 || RAD == 1) {  // the classes that have the integer form
     if (wide.n) {
       done = true;
-      if constexpr (!BOX && RAD == 1) {
-        if (wide.heat) k_direct_wide<NDIM, RAD, BOX, PERIODIC, true><<<grid, block, 0, stream>>>(P, wide);
+      if constexpr (BOX || RAD == 1) {
+        if (BOX ? wide.equal : wide.heat) k_direct_wide<NDIM, RAD, BOX, PERIODIC, true><<<grid, block, 0, stream>>>(P, wide);
         else k_direct_wide<NDIM, RAD, BOX, PERIODIC, false><<<grid, block, 0, stream>>>(P, wide);
       } else {
         k_direct_wide<NDIM, RAD, BOX, PERIODIC, false><<<grid, block, 0, stream>>>(P, wide);

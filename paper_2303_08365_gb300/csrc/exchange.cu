@@ -306,33 +306,55 @@ __device__ __forceinline__ bool unit_row_wide(const XSlot& sl, const WideTaps& T
             if (k - i >= 0 && k - i <= 2) E[i] = max(E[i], e + T.ex[tap_at<BOX>(dz, dy, k - i - 1)]);
         }
       }
-    WideAcc acc[2];
+    if constexpr (HEAT) {  // equal weights
+      E[0] |= 3;
+      E[1] |= 3;
+      WideSum S[2];
 #pragma unroll
-    for (int dz = -1; dz <= 1; ++dz)
+      for (int dz = -1; dz <= 1; ++dz)
 #pragma unroll
-      for (int dy = -1; dy <= 1; ++dy) {
-        double v[4];
-        row(dz, dy, v);
+        for (int dy = -1; dy <= 1; ++dy) {
+          double v[4];
+          row(dz, dy, v);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const WideVal u = wide_unpack(v[k]);
+          for (int k = 0; k < 4; ++k) {
+            const WideVal u = wide_unpack(v[k]);
 #pragma unroll
-          for (int i = 0; i < 2; ++i)
-            if (k - i >= 0 && k - i <= 2) {
-              const int t = tap_at<BOX>(dz, dy, k - i - 1);
-              acc[i].add(u, t, E[i] - u.e - T.ex[t], T);
-            }
+            for (int i = 0; i < 2; ++i)
+              if (k - i >= 0 && k - i <= 2) S[i] += wide_part(wide_twos(u), E[i]);
+          }
         }
-      }
-    out[0] = acc[0].get(E[0], T);
-    out[1] = acc[1].get(E[1], T);
+      out[0] = wide_equal_double(S[0], E[0], T);
+      out[1] = wide_equal_double(S[1], E[1], T);
+    } else {
+      WideAcc acc[2];
+#pragma unroll
+      for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+        for (int dy = -1; dy <= 1; ++dy) {
+          double v[4];
+          row(dz, dy, v);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const WideVal u = wide_unpack(v[k]);
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+              if (k - i >= 0 && k - i <= 2) {
+                const int t = tap_at<BOX>(dz, dy, k - i - 1);
+                acc[i].add(u, t, E[i] - u.e - T.ex[t], T);
+              }
+          }
+        }
+      out[0] = acc[0].get(E[0], T);
+      out[1] = acc[1].get(E[1], T);
+    }
     return wide_covers(E[0], T) && wide_covers(E[1], T);
   }
 }
 
 // Those of the two cells that the integer form does not take, by the FMA chain,
 // written at out.  Out of line: rarely run.
-template <int NT, bool BOX>
+template <int NT, bool BOX, bool EQUAL>
 __device__ __noinline__ void unit_chain(const XSlot& sl, const WideTaps& T, const double* wdev, int r, int lane,
                                         double* out) {
   {  // a pair of zeros among zeros: ordinary input
@@ -366,7 +388,7 @@ __device__ __noinline__ void unit_chain(const XSlot& sl, const WideTaps& T, cons
                                                                  : sl.plane[dz + 1][r + 1 + dy][x];
       E = max(E, wide_unpack(v[t]).e + T.ex[t]);
     }
-    if (!wide_covers(E, T)) out[i] = wide_chain(v, wdev, NT);
+    if (!wide_covers(EQUAL ? E | 3 : E, T)) out[i] = wide_chain(v, wdev, NT);
   }
 }
 
@@ -721,7 +743,7 @@ __global__ void __launch_bounds__(kThreadsX, 1) k_exchange3d(const __grid_consta
           if (!xin) return;
           put(r, v[0], v[1]);
           if (!all && (!last || (y0 + r >= P.own_lo && y0 + r < P.own_hi)))
-            unit_chain<NT, BOX>(sl, P.wide, P.wdev, r, lane, (last ? P.dst : P.ring) + base + (int64_t)r * P.nx);
+            unit_chain<NT, BOX, BOX && WIDE == kHeat>(sl, P.wide, P.wdev, r, lane, (last ? P.dst : P.ring) + base + (int64_t)r * P.nx);
         };
         if (!BOX && r0 + kWarps < h) {  // the star's two rows together: four sums in flight
           double v[2][2];
@@ -915,6 +937,8 @@ size_t exchange_ring_cells(const Geom& g, int Tb, int band_rows) {
 cudaError_t launch_exchange(Shape shape, int boundary, const ExchangeLaunch& L, cudaStream_t stream) {
   const bool per = boundary == kPeriodic;
   if (L.Tb < 2 || L.Tb > kMaxStages || L.tiles_x < 1 || L.band.tiles_y < 1) return cudaErrorInvalidValue;
+  if (shape == Shape::kBox && L.wide.equal)
+    return per ? launch_x<27, true, true, kHeat>(L, stream) : launch_x<27, true, false, kHeat>(L, stream);
   if (shape == Shape::kBox)
     return L.wide.n ? (per ? launch_x<27, true, true, kWide>(L, stream) : launch_x<27, true, false, kWide>(L, stream))
                     : (per ? launch_x<27, true, true, kChain>(L, stream) : launch_x<27, true, false, kChain>(L, stream));

@@ -67,6 +67,7 @@ struct WideTapsOf {
   int hi2[N];                              // 2 * hi
   int ex[N];                               // exponent below the largest weight's (<= 0)
   int heat;                                // one weight at the centre tap (n / 2), one at all others
+  int equal;                               // a box whose weights are all equal
   int bias;                                // exponent of the result: E - bias above R's
   int e_min;                               // E in [e_min, e_min + e_span], else the FMA chain
   unsigned int e_span;

@@ -478,6 +478,9 @@ cudaError_t launch_temporal(int ndim, int radius, Shape shape, int boundary, int
                : launch_1d<1, false>(Tb, g, wdev, src, dst, stream);
   }
   if (ndim == 3) {
+    if (box && wide.equal)
+      return per ? by_tb<3, 27, true, true, false, kHeat>(Tb, g, wide, wdev, src, dst, sms, stream)
+                 : by_tb<3, 27, true, false, false, kHeat>(Tb, g, wide, wdev, src, dst, sms, stream);
     if (box && wide.n) return per ? by_tb<3, 27, true, true, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream)
                                   : by_tb<3, 27, true, false, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream);
     if (box) return per ? by_tb<3, 27, true, true>(Tb, g, wide, wdev, src, dst, sms, stream)
@@ -491,7 +494,7 @@ cudaError_t launch_temporal(int ndim, int radius, Shape shape, int boundary, int
                                : by_tb<2, 9, true, false, true>(Tb, g, wide, wdev, src, dst, sms, stream);
   if (box && wide.n) return per ? by_tb<2, 9, true, true, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream)
                                 : by_tb<2, 9, true, false, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream);
-  if (wide.heat) return per ? by_tb<2, 5, false, true, false, kHeat>(Tb, g, wide, wdev, src, dst, sms, stream)
+  if (!box && wide.heat) return per ? by_tb<2, 5, false, true, false, kHeat>(Tb, g, wide, wdev, src, dst, sms, stream)
                             : by_tb<2, 5, false, false, false, kHeat>(Tb, g, wide, wdev, src, dst, sms, stream);
   if (wide.n) return per ? by_tb<2, 5, false, true, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream)
                          : by_tb<2, 5, false, false, false, kWide>(Tb, g, wide, wdev, src, dst, sms, stream);

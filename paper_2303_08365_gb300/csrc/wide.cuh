@@ -18,7 +18,16 @@
 // (half a unit of R, and K/16 units from the bits that the alignment drops),
 // against K roundings of partial sums in an FMA chain.  The result is
 // a function of the K values alone: every kernel that takes it gives the same
-// bits, whatever its tiles.
+// bits, whatever its tiles.  (One kernel of a class that has it does not: the overlapped temporal
+// kernel for 2D boxes of equal weights, temporal.cu.)
+//
+// Boxes whose weights are all equal take one multiplication a cell, and share the alignment of
+// a value between cells where a kernel can (WideSum).  For their results to be a function of
+// the K values alone all the same, E is the next number of the form 4 n + 3 from the largest
+// exponent on: neighbouring cells seldom differ in that.  (In the largest exponent itself they
+// would differ wherever a field passes a power of two.)  With up to three bits fewer, the unit
+// of A that a negative value's one's complement is short by would show over many steps (160 of
+// a 9-point box: 2.2e-16 between a field and its negative), so theirs is a two's complement.
 //
 // It covers weights > 0.  Values whose largest exponent is out of the range in
 // which that is safe (infinities, NaN, products near the largest or the
@@ -37,8 +46,8 @@ namespace gbst {
 // them: a weight that is not positive, or weights so far apart or so extreme
 // that no range of exponents is left.
 template <int N>
-inline bool make_wide(const double* w, int n, WideTapsOf<N>& t) {
-  t.n = 0;
+inline bool make_wide(const double* w, int n, WideTapsOf<N>& t, bool box = false) {
+  t.n = t.heat = t.equal = 0;
   if (n < 1 || n > N) return false;
   int xmax = -100000, x[N];
   for (int k = 0; k < n; ++k) {
@@ -68,6 +77,7 @@ inline bool make_wide(const double* w, int n, WideTapsOf<N>& t) {
   t.heat = n >= 3 && n % 2 == 1;
   for (int k = 1; k < n; ++k)
     if (k != n / 2 && w[k] != w[0]) t.heat = 0;
+  t.equal = box && t.heat && w[n / 2] == w[0];
   t.n = n;
   return true;
 }
@@ -93,18 +103,15 @@ __device__ __forceinline__ WideVal wide_unpack(double v) {
   return u;
 }
 
-// The same with negative values in two's complement, for sums of integers whose units are not
-// far below the result's (wide_equal): a one's complement is a bias there (half of it taken
-// back by a constant, 79 steps of a 9-point box ended 4.1e-16 off; so, 3.3e-16).
-__device__ __forceinline__ WideVal wide_unpack_twos(double v) {
-  WideVal u = wide_unpack(v);
-  const unsigned int s = (unsigned int)(u.hi >> 31);
-  const long long m = (long long)(((unsigned long long)(unsigned int)u.hi << 32) | u.lo) - (int)s;
+// From and to two's complement for negative values (boxes of equal weights).
+__device__ __forceinline__ WideVal wide_twos(WideVal u) {
+  const int s = u.hi >> 31;
+  const long long m = (long long)(((unsigned long long)(unsigned int)u.hi << 32) | u.lo) - s;
   u.hi = (int)(m >> 32);
   u.lo = (unsigned int)m;
   return u;
 }
-__device__ __forceinline__ WideVal wide_ones(WideVal u) {  // back to wide_unpack's form
+__device__ __forceinline__ WideVal wide_ones(WideVal u) {
   const long long v = (long long)(((unsigned long long)(unsigned int)u.hi << 32) | u.lo);
   const long long m = v + (v >> 63);
   u.hi = (int)(m >> 32);
@@ -175,6 +182,25 @@ __device__ __forceinline__ double wide_double(long long R, int x) {
   return __hiloint2double(h != 0 ? h + (x << 20) : h, __double2loint(r));
 }
 
+// The same, rounded alike, unpacked: for a value that the next step reads, without the two FP64
+// instructions (64 cycles each) between.
+__device__ __forceinline__ WideVal wide_val(long long R, int x) {
+  const long long s = R >> 63;
+  const unsigned long long a = (unsigned long long)((R ^ s) - s);
+  if (a == 0) return wide_unpack(0.0);
+  const int lz = __clzll((long long)a);
+  const unsigned long long n = a << lz;  // leading bit 63; 53 bits stay
+  unsigned long long r = n + 0x3ff + ((n >> 11) & 1);
+  const bool carry = r < n;
+  r = carry ? 1ull << 63 : r;
+  const unsigned long long m = ((r & ~0x7ffull) >> 2) ^ (unsigned long long)s;
+  WideVal u;
+  u.hi = (int)(m >> 32);
+  u.lo = (unsigned int)m;
+  u.e = x + (1023 + 63) - lz + (carry ? 1 : 0);
+  return u;
+}
+
 // The accumulators of a cell: hh, hl, lh and ll count units of 2^57, 2^32, 2^26 and
 // 1 of S (27 taps: below 2^63 each).
 struct WideAcc {
@@ -205,25 +231,9 @@ struct WideAcc {
     return hh + ((hl + (long long)((lh + (ll >> 26)) >> 6)) >> 25);
   }
 
-  // The sum rounded to a double as get() rounds it, unpacked: for a value that the
-  // next step reads, without the two FP64 instructions (64 cycles each) between.
   template <class Taps>
   __device__ __forceinline__ WideVal val(int E, const Taps& T) const {
-    const long long R = rounded();
-    const long long s = R >> 63;
-    const unsigned long long a = (unsigned long long)((R ^ s) - s);
-    if (a == 0) return wide_unpack(0.0);
-    const int lz = __clzll((long long)a);
-    const unsigned long long n = a << lz;  // leading bit 63; 53 bits stay
-    unsigned long long r = n + 0x3ff + ((n >> 11) & 1);
-    const bool carry = r < n;
-    r = carry ? 1ull << 63 : r;
-    const unsigned long long m = ((r & ~0x7ffull) >> 2) ^ (unsigned long long)s;
-    WideVal u;
-    u.hi = (int)(m >> 32);
-    u.lo = (unsigned int)m;
-    u.e = E - T.bias + (1023 + 63) - lz + (carry ? 1 : 0);
-    return u;
+    return wide_val(rounded(), E - T.bias);
   }
 
   // The sum as a double.
@@ -285,35 +295,74 @@ __device__ __forceinline__ double wide_sum_heat(const WideVal (&u)[NT], const Ta
   return acc.get(E, T);
 }
 
-// Boxes of N taps whose weights are all equal: the values of a block of cells (two's
-// complement) are aligned to one exponent E, the largest of the block, and added as integers;
-// a cell's sum S takes one multiplication.  S counts units of 2^-(61 - kEqualShift) of the
-// largest value, N of which fit 63 bits.  A value within 2^(9 - kEqualShift) of the
-// largest loses nothing, one below that less than a unit.
-template <int N>
-constexpr int kEqualShift = N == 9 ? 3 : 4;
-// How far below the block's a cell's own largest exponent may lie: then a unit is 2^-55
-// of the cell's own largest value, half a unit of 2^-52 of the result being what its
-// rounding takes.
-template <int N>
-constexpr int kEqualGap = N == 9 ? 3 : 2;
+// The sum of aligned values (two's complement) of a box whose weights are all equal: up to 27
+// of 63 bits, so the sum modulo 2^64, and the sum of the values' top bits (units of 2^37), which
+// has the rest.  (Values cut to 58 bits, whose sum fits 64, lean to one side: by 2^-54 a step
+// where they are spread over a few powers of two.)
+struct WideSum {
+  long long s;
+  int top;
+  __device__ __forceinline__ WideSum() : s(0), top(0) {}
+  __device__ __forceinline__ explicit WideSum(long long a) : s(a), top((int)(a >> 37)) {}
+  __device__ __forceinline__ WideSum& operator+=(const WideSum& o) {
+    s += o.s;
+    top += o.top;
+    return *this;
+  }
+  friend __device__ __forceinline__ WideSum operator+(WideSum a, const WideSum& o) { return a += o; }
+  // The sum's bits from the 37th on: the values' fall short of them by one a value at most.
+  __device__ __forceinline__ int high() const {
+    return top + (((int)((unsigned long long)s >> 37) - top) & ((1 << 27) - 1));
+  }
+  // Times 2^g, g < 37.
+  __device__ __forceinline__ void shift(int g) {
+    top = (high() << g) | ((int)((unsigned long long)s >> (37 - g)) & ((1 << g) - 1));
+    s <<= g;
+  }
+};
 
-// w S as a double, w the weights' one value.
-template <int N, class Taps>
-__device__ __forceinline__ double wide_equal(long long S, int E, const Taps& T) {
-  const int ah = (int)(S >> 32), lo = T.lo[0];
-  const unsigned int al = (unsigned int)S;
-  // units of 2^56, 2^32, 2^26 and 1 of S W
-  const long long hh = (long long)ah * (2 * T.hi2[0]);
-  const unsigned long long ll = (unsigned long long)al * (unsigned int)lo;
-  const unsigned long long lh = (unsigned long long)al * (unsigned int)T.hi[0] + (ll >> 26);
-  const long long hl = (long long)ah * lo + ((1 << 23) + (long long)(lh >> 6));
-  return wide_double(hh + (hl >> 24), E - T.bias + kEqualShift<N> - 1);
+// A value's share of a sum of exponent E.
+__device__ __forceinline__ WideSum wide_part(const WideVal& u, int E) { return WideSum(wide_align(u, E - u.e)); }
+
+// R = w S / 2^57 rounded, w the weights' one value.
+template <class Taps>
+__device__ __forceinline__ long long wide_equal(const WideSum& S, const Taps& T) {
+  const int ext = S.high() >> 27;  // S = ext 2^64 + s
+  const unsigned int ah = (unsigned int)((unsigned long long)S.s >> 32), al = (unsigned int)S.s;
+  const unsigned int lo = (unsigned int)T.lo[0], hi = (unsigned int)T.hi[0], hi2 = (unsigned int)T.hi2[0];
+  // units of 2^57, 2^32, 2^26 and 1 of S W
+  const unsigned long long lh = (unsigned long long)al * hi + ((unsigned long long)al * lo >> 26);
+  const unsigned long long hl = (unsigned long long)ah * lo + (1 << 24) + (lh >> 6);
+  const long long top = (long long)(ext << 7) * (int)lo + ((long long)(ext * (int)hi2) << 32);
+  return (long long)((unsigned long long)ah * hi2 + (hl >> 25)) + top;
+}
+template <class Taps>
+__device__ __forceinline__ double wide_equal_double(const WideSum& S, int E, const Taps& T) {
+  return wide_double(wide_equal(S, T), E - T.bias);
+}
+
+// One cell: S and E.
+template <int NT>
+__device__ __forceinline__ int wide_acc_equal(const WideVal (&u)[NT], WideSum& S) {
+  int E = u[0].e;
+#pragma unroll
+  for (int k = 1; k < NT; ++k) E = max(E, u[k].e);
+  E |= 3;
+#pragma unroll
+  for (int k = 0; k < NT; ++k) S += wide_part(wide_twos(u[k]), E);
+  return E;
+}
+template <int NT, class Taps>
+__device__ __forceinline__ double wide_sum_equal(const WideVal (&u)[NT], const Taps& T, bool& ok) {
+  WideSum S;
+  const int E = wide_acc_equal<NT>(u, S);
+  ok = wide_covers(E, T);
+  return wide_equal_double(S, E, T);
 }
 
 // How a kernel takes the weighted sum of a cell, collected tap by tap: the FMA
 // chain in tap order, or the integer form once every value is there (kHeat: for
-// weights that wide_sum_heat takes).
+// weights that wide_sum_heat takes, or a box whose weights are all equal).
 enum SumForm : int { kChain = 0, kWide = 1, kHeat = 2 };
 
 template <int NT, int FORM, class Taps = WideTaps>
@@ -327,7 +376,8 @@ struct TapSum {
   __device__ __forceinline__ void tap(Acc& acc, int k, double v, int) const { acc.u[k] = wide_unpack(v); }
   // ok = false: the FMA chain has to take the cell
   __device__ __forceinline__ double get(const Acc& acc, bool& ok) const {
-    if constexpr (FORM == kHeat) return wide_sum_heat<NT>(acc.u, T, ok);
+    if constexpr (FORM == kHeat && NT >= 9) return wide_sum_equal<NT>(acc.u, T, ok);
+    else if constexpr (FORM == kHeat) return wide_sum_heat<NT>(acc.u, T, ok);
     else return wide_sum<NT>(acc.u, T, ok);
   }
   __device__ __forceinline__ double get(const Acc& acc) const {

@@ -17,9 +17,11 @@
 //
 // Measured at 8192^2, periodic, general weights (FMA chain before): 25-point box
 // 52 GStencil/s (23.6), radius-2 star 113 (67).  Boxes whose weights are all equal
-// share alignments and partial sums among a lane's four cells (wide_equal): 9-point
-// box at 16384^2 225 GStencil/s (140 with shared sums on the FP64 pipe), 25-point box
-// at 8192^2 139 (24), 512^2 43 (14).
+// share alignments and partial sums among a lane's four cells (WideSum), with the bits that each
+// cell has alone: 9-point box at 16384^2 210 GStencil/s (140 with shared sums on the FP64 pipe; 225
+// with values cut to 58 bits at the four cells' common exponent, which made the bits depend on
+// where a tile begins), 25-point box at 8192^2 147 (24; 139 cut), 512^2 49 (14).  Zero-mean noise,
+// whose cells differ in exponent and lie further apart than 2^9, takes own_cells: 146, 91, 39.
 //
 // Work split: the tiles are cut into equal contiguous ranges, one per CTA.
 #include <cudaTypedefs.h>
@@ -157,36 +159,52 @@ __device__ __noinline__ void chain_cells(const Plane<RAD>& u, int row0, int rows
     }
 }
 
-// A lane's cells one by one, each aligned to its own largest exponent: where the block's
-// lies too far above.  Out of line: rarely run.
+// An equal-weight box's cells of a lane, each aligned to its own exponent E (or by the FMA
+// chain).  Out of line: where they differ in E and are not within 2^9 of each other.
 template <int RAD>
-__device__ __noinline__ void own_cells(const Plane<RAD>& u, int row0, int rows, int c0, const WideTaps& T,
+__device__ __noinline__ void own_cells(const Plane<RAD>& u, int row0, int rows, int cols, int c, const WideTaps& T,
                                        const double* wdev, double* out, int nx) {
-  for (int r = 0; r < rows; ++r)
-    for (int i = 0; i < 2; ++i) {
-      const int row = row0 + r, c = c0 + i;
-      unsigned int any = 0;
-      int E = 0;
-      for (int dy = -RAD; dy <= RAD; ++dy)
-        for (int dx = -RAD; dx <= RAD; ++dx) {
-          const WideVal x = wide_ones(get(&u.m[row + dy][c + dx], &u.e[row + dy][c + dx]));
-          any |= wide_nonzero(x);
-          E = max(E, x.e);
-        }
-      double v = 0.0;
-      if (any != 0 && !wide_covers(E, T)) {
-        v = chain_cell<true, RAD, true>(u, row, c, wdev);
-      } else if (any != 0) {
-        WideAcc acc;
-        for (int dy = -RAD; dy <= RAD; ++dy)
-          for (int dx = -RAD; dx <= RAD; ++dx) {
-            const WideVal x = wide_ones(get(&u.m[row + dy][c + dx], &u.e[row + dy][c + dx]));
-            acc.add(x, 0, E - x.e, T);
-          }
-        v = acc.get(E, T);
+#pragma unroll 1
+  for (int r = 0; r < rows; ++r) {
+    const int row = row0 + r;
+    int E[2] = {0, 0};
+#pragma unroll
+    for (int dy = -RAD; dy <= RAD; ++dy)
+#pragma unroll
+      for (int dx = -RAD; dx <= RAD + 1; ++dx) {
+        const int e = u.e[row + dy][c + dx];
+        if (dx <= RAD) E[0] = max(E[0], e);
+        if (dx > -RAD) E[1] = max(E[1], e);
       }
-      out[(int64_t)r * nx + i] = v;
+    E[0] |= 3;
+    E[1] |= 3;
+    WideSum S[2];
+#pragma unroll
+    for (int dy = -RAD; dy <= RAD; ++dy) {
+      WideVal v[2 * RAD + 2];
+      get_row<RAD>(u, row + dy, c, v);
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int k = 0; k < 2 * RAD + 1; ++k) S[i] += wide_part(v[i + k], E[i]);
     }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (i < cols)
+        out[(int64_t)r * nx + i] =
+            wide_covers(E[i], T) ? wide_equal_double(S[i], E[i], T) : chain_cell<true, RAD, true>(u, row, c + i, wdev);
+  }
+}
+
+// The smallest exponent of the values that an equal-weight box's lane reads.
+template <int RAD>
+__device__ __forceinline__ int least_exponent(const Plane<RAD>& u, int row0, int c) {
+  int e = 0x7fffffff;
+#pragma unroll
+  for (int r = -RAD; r < kR + RAD; ++r)
+#pragma unroll
+    for (int x = -RAD; x < 2 + RAD; ++x) e = min(e, u.e[row0 + r][c + x]);
+  return e;
 }
 
 template <bool BOX, int RAD, bool HEAT>
@@ -324,7 +342,7 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
       for (int q = 0; q < HN; ++q) {
         const int k = lane + 32 * q, j = k / HR, row = H0 + k % HR;
         const int c = 2 + (j < RAD ? j - RAD : cols + (j - RAD));
-        if (k < HALL) put(&u.m[row][c], &u.e[row][c], BOX && HEAT ? wide_unpack_twos(h[q]) : wide_unpack(h[q]));
+        if (k < HALL) put(&u.m[row][c], &u.e[row][c], BOX && HEAT ? wide_twos(wide_unpack(h[q])) : wide_unpack(h[q]));
       }
       if (!wait(&S.full[pos.s], pos.ph)) return leave(t);
       WideVal v[2];
@@ -382,7 +400,7 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
         }
       };
       // the integer form takes every cell that is stored (the others may hold anything)
-      bool all = true;
+      bool all = true, zeros = true;  // (zeros: there may be nothing else)
       auto covers = [&](bool ok, int r, int i) { return ok || r >= rows || (!TMA && i == 1 && xa + 1 >= P.nx); };
       if constexpr (!BOX) {
 #pragma unroll
@@ -417,9 +435,9 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
         // equal weights, the lane's two rows and columns as one block: each value is
         // aligned once for the four cells, and rows (mid: their common columns) and
         // columns share their partial sums
-        constexpr int N = 2 * RAD + 2, NT = (2 * RAD + 1) * (2 * RAD + 1);
-        static_assert(kR == 2 && TMA, "the block; columns and rows outside the grid hold values or zeros");
-        int E = 0, own[2][2], e[N][N];  // the block's largest exponent, the cells' own
+        constexpr int N = 2 * RAD + 2;
+        static_assert(kR == 2, "the block");
+        int own[2][2], e[N][N];  // the cells' largest exponents
 #pragma unroll
         for (int r = 0; r < N; ++r) {
           const int* er = &u.e[row0 - RAD + r][c];
@@ -444,32 +462,67 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
             if (r > 0) own[1][i] = r == 1 ? h : max(own[1][i], h);
           }
         }
-        E = max(max(own[0][0], own[0][1]), max(own[1][0], own[1][1]));
-        int least = min(own[0][0], own[0][1]);
-        if (rows > 1) least = min(least, min(own[1][0], own[1][1]));
-        all = rows <= 0 || (wide_covers(E, P.wide) && wide_covers(least, P.wide) && E - least <= kEqualGap<NT>);
-        long long S[2][2], both[2] = {0, 0};  // both: of the rows that both read
-        E += kEqualShift<NT>;
-        if (RAD > 1) asm volatile("" ::: "memory");  // 36 exponents would not fit the registers: read again
-#pragma unroll
-        for (int r = 0; r < N; ++r) {
-          WideVal v[N];
-          get_row<RAD>(u, row0 - RAD + r, c, v);
-          long long mid = wide_align(v[1], E - v[1].e);
-#pragma unroll
-          for (int k = 2; k < N - 1; ++k) mid += wide_align(v[k], E - v[k].e);
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const long long h = mid + wide_align(v[i * (N - 1)], E - v[i * (N - 1)].e);
-            if (r == 0) S[0][i] = h;
-            else if (r < N - 1) both[i] += h;
-            else S[1][i] = h;
-          }
+        // (what is not stored may hold anything)
+        if (!TMA && xa + 1 >= P.nx) {
+          own[0][1] = own[0][0];
+          own[1][1] = own[1][0];
         }
-        E -= kEqualShift<NT>;
+        if (rows < 2) {
+          own[1][0] = own[0][0];
+          own[1][1] = own[0][1];
+        }
+        int E = max(max(own[0][0], own[0][1]), max(own[1][0], own[1][1])) | 3;
+        const int least = min(min(own[0][0], own[0][1]), min(own[1][0], own[1][1])) | 3;
+        zeros = E == 3;
+        // Where cells differ in E (a field passes a power of 16), no bit is cut as long as all
+        // values are within the 2^9 that the integers have room for: the sums are exact then,
+        // and those of each cell's own alignment follow.  Else the warp takes own_cells.
+        all = wide_covers(E, P.wide) && (E == least || (wide_covers(least, P.wide) && least_exponent<RAD>(u, row0, c) + 9 >= E));
+        const bool fits = __all_sync(0xffffffffu, all || rows <= 0);
+        all = rows <= 0 || fits;
+        if (fits) {
+          WideSum S[2][2], both[2];  // both: of the rows that both read
+          if (RAD > 1) asm volatile("" ::: "memory");  // 36 exponents would not fit the registers: read again
+          // (two values fit 64 bits: by pairs, side by side or one below the other)
+          auto part = [&](const WideVal& x, const WideVal& y) {
+            return WideSum(wide_align(x, E - x.e) + wide_align(y, E - y.e));
+          };
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
-          store(r, wide_equal<NT>(S[r][0] + both[0], E, P.wide), wide_equal<NT>(S[r][1] + both[1], E, P.wide));
+          for (int q = 0; q < 2; ++q) {
+            WideVal v[N];
+            get_row<RAD>(u, row0 - RAD + q * (N - 1), c, v);
+            WideSum mid = part(v[1], v[2]);
+#pragma unroll
+            for (int k = 3; k < N - 1; k += 2) mid += part(v[k], v[k + 1]);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) S[q][i] = mid + wide_part(v[i * (N - 1)], E);
+          }
+#pragma unroll
+          for (int r = 1; r < N - 1; r += 2) {
+            WideVal v[N], w[N];
+            get_row<RAD>(u, row0 - RAD + r, c, v);
+            get_row<RAD>(u, row0 - RAD + r + 1, c, w);
+            WideSum mid = part(v[1], w[1]);
+#pragma unroll
+            for (int k = 2; k < N - 1; ++k) mid += part(v[k], w[k]);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) both[i] += mid + part(v[i * (N - 1)], w[i * (N - 1)]);
+          }
+          int Ec[2][2] = {{E, E}, {E, E}};
+#pragma unroll
+          for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              S[r][i] += both[i];
+              if (E != least) {
+                Ec[r][i] = own[r][i] | 3;
+                S[r][i].shift(E - Ec[r][i]);
+              }
+            }
+#pragma unroll
+          for (int r = 0; r < 2; ++r)
+            store(r, wide_equal_double(S[r][0], Ec[r][0], P.wide), wide_equal_double(S[r][1], Ec[r][1], P.wide));
+        }
       } else {
         // row by row; the largest exponents first, then the sums: a pair's values would
         // not fit the registers, so their rows are read twice
@@ -514,8 +567,8 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
           store(r, acc[0].get(E[0], P.wide), acc[1].get(E[1], P.wide));
         }
       }
-      if (!all && !zero_cells<BOX, RAD>(u, row0, rows, min(2, P.nx - xa), c, out, P.nx)) {
-        if constexpr (BOX && HEAT) own_cells<RAD>(u, row0, rows, c, P.wide, P.wdev, out, P.nx);
+      if (!all && (!zeros || !zero_cells<BOX, RAD>(u, row0, rows, min(2, P.nx - xa), c, out, P.nx))) {
+        if constexpr (BOX && HEAT) own_cells<RAD>(u, row0, rows, min(2, P.nx - xa), c, P.wide, P.wdev, out, P.nx);
         else chain_cells<BOX, RAD>(u, row0, rows, min(2, P.nx - xa), c, P.wide, P.wdev, out, P.nx);
       }
       __syncwarp();
@@ -590,15 +643,11 @@ cudaError_t launch_wide2d(Shape shape, int radius, int boundary, const Geom& g, 
                           const double* wdev, const double* src, double* dst, int* status, int sms,
                           cudaStream_t stream, bool tma, bool chained) {
   const bool per = boundary == kPeriodic, box = shape == Shape::kBox;
-  const int side = 2 * radius + 1, mid = wide.n / 2;
+  const int side = 2 * radius + 1;
   if (wide.n != (box ? side * side : 4 * radius + 1)) return cudaErrorInvalidValue;
-  if (box && tma && wide.heat && wide.hi[mid] == wide.hi[0] && wide.lo[mid] == wide.lo[0] && wide.ex[mid] == wide.ex[0]) {
-    if (radius == 2)
-      return per ? launch_t<true, 2, true, true, true>(g, wide, wdev, src, dst, status, sms, stream, chained)
-                 : launch_t<true, 2, true, false, true>(g, wide, wdev, src, dst, status, sms, stream, chained);
-    return per ? launch_t<true, 1, true, true, true>(g, wide, wdev, src, dst, status, sms, stream, chained)
-               : launch_t<true, 1, true, false, true>(g, wide, wdev, src, dst, status, sms, stream, chained);
-  }
+  if (box && wide.equal)
+    return radius == 2 ? launch_p<true, 2, true>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained)
+                       : launch_p<true, 1, true>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained);
   if (radius == 2)
     return box ? launch_p<true, 2, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained)
                : launch_p<false, 2, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained);

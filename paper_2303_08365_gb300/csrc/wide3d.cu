@@ -26,8 +26,8 @@
 // planes (1.5 unpacks per cell, rows of 4) ran at 142 and spilled; a converter
 // warp that loads and unpacks everything for the consumers at 94.
 // Box, 384^3, zero outside: general weights 48 GStencil/s (22.7 for the FMA chain), equal
-// ones (wide_equal) 63 (each plane's sums kept in registers for the next two planes:
-// 66, but they spill, and small grids lose, 64^3 10.9 us a step to 16).
+// ones (WideSum) 102, 64 where a warp takes own_cells (zero-mean noise).  Each plane's sums kept
+// in registers for the next two planes spilled.
 // Work split: the (tile, z) planes are cut into equal contiguous ranges, one per CTA.
 #include <cudaTypedefs.h>
 
@@ -152,39 +152,42 @@ __device__ __noinline__ void chain_cells(const Plane<TC>& um, const Plane<TC>& u
     }
 }
 
-// A lane's cells of an equal-weight box one by one, each aligned to its own largest
-// exponent: where the block's lies too far above.  Out of line: rarely run.
+// An equal-weight box's cells of a lane, each aligned to its own exponent E (or by the FMA
+// chain).  Out of line: where they differ in E and are not within 2^9 of each other.
 template <int TC>
 __device__ __noinline__ void own_cells(const Plane<TC>& um, const Plane<TC>& u0, const Plane<TC>& up, int row0, int rows,
-                                       int c0, const WideTaps& T, const double* wdev, double* out, int nx) {
+                                       int cols, int c, const WideTaps& T, const double* wdev, double* out, int nx) {
   const Plane<TC>* const pl[3] = {&um, &u0, &up};
-  for (int r = 0; r < rows; ++r)
-    for (int i = 0; i < 2; ++i) {
-      const int row = row0 + r, c = c0 + i;
-      auto at = [&](int k) {
-        const int y = row + k / 3 % 3 - 1, x = c + k % 3 - 1;
-        return wide_ones(get(&pl[k / 9]->m[y][x], &pl[k / 9]->e[y][x]));
-      };
-      unsigned int any = 0;
-      int E = 0;
-      for (int k = 0; k < 27; ++k) {
-        const WideVal u = at(k);
-        any |= wide_nonzero(u);
-        E = max(E, u.e);
-      }
-      double v = 0.0;
-      if (any != 0 && !wide_covers(E, T)) {
-        v = chain_cell<true, TC, true>(um, u0, up, row, c, wdev);
-      } else if (any != 0) {
-        WideAcc acc;
-        for (int k = 0; k < 27; ++k) {
-          const WideVal u = at(k);
-          acc.add(u, 0, E - u.e, T);
-        }
-        v = acc.get(E, T);
-      }
-      out[(int64_t)r * nx + i] = v;
+#pragma unroll 1
+  for (int r = 0; r < rows; ++r) {
+    const int row = row0 + r;
+    int E[2] = {0, 0};
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const int* er = &pl[k / 3]->e[row + k % 3 - 1][c];
+      const int2 m = *reinterpret_cast<const int2*>(er);
+      const int mid = max(m.x, m.y);
+      E[0] = max(E[0], max(mid, er[-1]));
+      E[1] = max(E[1], max(mid, er[2]));
     }
+    E[0] |= 3;
+    E[1] |= 3;
+    WideSum S[2];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      WideVal v[4];
+      get_row<TC>(*pl[k / 3], row + k % 3 - 1, c, v);
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int x = 0; x < 3; ++x) S[i] += wide_part(v[i + x], E[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (i < cols)
+        out[(int64_t)r * nx + i] =
+            wide_covers(E[i], T) ? wide_equal_double(S[i], E[i], T) : chain_cell<true, TC, true>(um, u0, up, row, c + i, wdev);
+  }
 }
 
 // HEAT: a star whose weights wide_sum_heat takes; a box whose weights are all equal.
@@ -341,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wid
         Plane<TC>& u = S.u[con().s];
 #pragma unroll
         for (int q = 0; q < HN; ++q)
-          if (hrow[q] >= 0) put(&u.m[hrow[q]][hcol[q]], &u.e[hrow[q]][hcol[q]], BOX && HEAT ? wide_unpack_twos(h[q]) : wide_unpack(h[q]));
+          if (hrow[q] >= 0) put(&u.m[hrow[q]][hcol[q]], &u.e[hrow[q]][hcol[q]], BOX && HEAT ? wide_twos(wide_unpack(h[q])) : wide_unpack(h[q]));
         if (!wait(&S.full[raw.s], raw.ph)) return leave(j);
         WideVal v[2];
         unpack_row<TMA, TC + 2, BOX && HEAT>(S.raw[raw.s], S.shift[raw.s], u, 0, lane, cols, v);
@@ -394,7 +397,7 @@ __global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wid
         const Plane<TC>& up = S.u[BOX ? u1 : con().s];
         // the integer form takes every cell that is stored (the others may hold
         // anything, and one CTA that calls chain_cells for them delays the rest)
-        bool all = true;
+        bool all = true, zeros = true;  // (zeros: there may be nothing else)
         auto covers = [&](bool ok, int r, int i) {
           return ok || r >= rows || (!TMA && i == 1 && xa + 1 >= P.nx);
         };
@@ -419,10 +422,10 @@ __global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wid
             store(r, v[0], v[1]);
           }
         } else if constexpr (HEAT) {
+          static_assert(R <= 2, "the block");
           // equal weights, the lane's rows and two columns as one block: each value is
           // aligned once for all cells, and rows (mid: their common columns) share their
           // partial sums.  Exponents first: a block's values would not fit the registers.
-          static_assert(TMA, "columns and rows outside the grid hold values or zeros");
           int own[R][2];
 #pragma unroll
           for (int r = 0; r < R; ++r) own[r][0] = own[r][1] = 0;
@@ -442,42 +445,77 @@ __global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wid
                 }
             }
           }
-          int E = 0, least = max(own[0][0], own[0][1]);
+          // (what is not stored may hold anything)
+          int E = own[0][0], least = own[0][0];
 #pragma unroll
           for (int r = 0; r < R; ++r) {
+            if (r > 0 && r >= rows) own[r][0] = own[0][0];
+            if ((!TMA && xa + 1 >= P.nx) || (r > 0 && r >= rows)) own[r][1] = own[0][0];
             E = max(E, max(own[r][0], own[r][1]));
-            if (r < rows) least = min(least, min(own[r][0], own[r][1]));
+            least = min(least, min(own[r][0], own[r][1]));
           }
-          all = rows <= 0 || (wide_covers(E, P.wide) && wide_covers(least, P.wide) && E - least <= kEqualGap<27>);
-          long long sum[R][2], both[2] = {0, 0};  // both: of the rows that all cells read
-#pragma unroll
-          for (int r = 0; r < R; ++r) sum[r][0] = sum[r][1] = 0;
-          E += kEqualShift<27>;
+          E |= 3;
+          least |= 3;
+          zeros = E == 3;
+          // Where cells differ in E (a field passes a power of 16), no bit is cut as long as all
+          // values are within the 2^9 that the integers have room for: the sums are exact then,
+          // and those of each cell's own alignment follow.  Else the warp takes own_cells.
+          all = wide_covers(E, P.wide);
+          if (all && E != least) {
+            int low = 0x7fffffff;
 #pragma unroll 1
-          for (int p = 0; p < 3; ++p) {
-            const Plane<TC>& u = p == 0 ? um : p == 1 ? u0 : up;
+            for (int p = 0; p < 3; ++p) {
+              const Plane<TC>& u = p == 0 ? um : p == 1 ? u0 : up;
 #pragma unroll
-            for (int q = 0; q < R + 2; ++q) {
-              WideVal v[4];
-              get_row<TC>(u, row0 - 1 + q, c, v);
-              const long long mid = wide_align(v[1], E - v[1].e) + wide_align(v[2], E - v[2].e);
-              const long long h[2] = {mid + wide_align(v[0], E - v[0].e), mid + wide_align(v[3], E - v[3].e)};
+              for (int q = 0; q < R + 2; ++q)
+#pragma unroll
+                for (int x = -1; x < 3; ++x) low = min(low, u.e[row0 - 1 + q][c + x]);
+            }
+            all = wide_covers(least, P.wide) && low + 9 >= E;
+          }
+          const bool fits = __all_sync(0xffffffffu, all || rows <= 0);
+          all = rows <= 0 || fits;
+          if (fits) {
+            WideSum sum[R][2], both[2];  // both: of the rows that all cells read
+            // (two values fit 64 bits: by pairs, side by side or one below the other)
+            auto part = [&](const WideVal& x, const WideVal& y) {
+              return WideSum(wide_align(x, E - x.e) + wide_align(y, E - y.e));
+            };
+#pragma unroll 1
+            for (int p = 0; p < 3; ++p) {
+              const Plane<TC>& u = p == 0 ? um : p == 1 ? u0 : up;
+              auto one = [&](int q, WideSum (&to)[2]) {
+                WideVal v[4];
+                get_row<TC>(u, row0 - 1 + q, c, v);
+                const WideSum mid = part(v[1], v[2]);
+                to[0] += mid + wide_part(v[0], E);
+                to[1] += mid + wide_part(v[3], E);
+              };
+              one(R == 2 ? 0 : 2, R == 2 ? sum[0] : both);
+              if constexpr (R == 2) one(3, sum[R - 1]);
+              WideVal v[4], w[4];
+              get_row<TC>(u, row0 + R - 2, c, v);
+              get_row<TC>(u, row0 + R - 1, c, w);
+              const WideSum mid = part(v[1], w[1]) + part(v[2], w[2]);
+              both[0] += mid + part(v[0], w[0]);
+              both[1] += mid + part(v[3], w[3]);
+            }
+            int Ec[R][2];
+#pragma unroll
+            for (int r = 0; r < R; ++r)
 #pragma unroll
               for (int i = 0; i < 2; ++i) {
-                if (R <= q + 1 && q <= 2) {
-                  both[i] += h[i];
-                } else {
-#pragma unroll
-                  for (int r = 0; r < R; ++r)
-                    if (q - 2 <= r && r <= q) sum[r][i] += h[i];
+                sum[r][i] += both[i];
+                Ec[r][i] = E;
+                if (E != least) {
+                  Ec[r][i] = own[r][i] | 3;
+                  sum[r][i].shift(E - Ec[r][i]);
                 }
               }
-            }
-          }
-          E -= kEqualShift<27>;
 #pragma unroll
-          for (int r = 0; r < R; ++r)
-            store(r, wide_equal<27>(sum[r][0] + both[0], E, P.wide), wide_equal<27>(sum[r][1] + both[1], E, P.wide));
+            for (int r = 0; r < R; ++r)
+              store(r, wide_equal_double(sum[r][0], Ec[r][0], P.wide), wide_equal_double(sum[r][1], Ec[r][1], P.wide));
+          }
         } else {
           // row by row; the largest exponents first, then the sums: the 36 values of
           // a pair would not fit the registers, so their rows are read twice
@@ -516,8 +554,8 @@ __global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wid
             store(r, acc[0].get(E[0], P.wide), acc[1].get(E[1], P.wide));
           }
         }
-        if (!all && !zero_cells<BOX, TC>(um, u0, up, row0, rows, min(2, P.nx - xa), c, out, P.nx)) {
-          if constexpr (BOX && HEAT) own_cells<TC>(um, u0, up, row0, rows, c, P.wide, P.wdev, out, P.nx);
+        if (!all && (!zeros || !zero_cells<BOX, TC>(um, u0, up, row0, rows, min(2, P.nx - xa), c, out, P.nx))) {
+          if constexpr (BOX && HEAT) own_cells<TC>(um, u0, up, row0, rows, min(2, P.nx - xa), c, P.wide, P.wdev, out, P.nx);
           else chain_cells<BOX, TC>(um, u0, up, row0, rows, min(2, P.nx - xa), c, P.wide, P.wdev, out, P.nx);
         }
         __syncwarp();
@@ -593,13 +631,9 @@ cudaError_t launch_wide3d(Shape shape, int boundary, const Geom& g, const WideTa
   const bool per = boundary == kPeriodic, low = tile_y == 8;
   if (shape == Shape::kBox) {
     if (wide.n != 27) return cudaErrorInvalidValue;
-    if (tma && wide.heat && wide.hi[13] == wide.hi[0] && wide.lo[13] == wide.lo[0] && wide.ex[13] == wide.ex[0]) {
-      if (low)
-        return per ? launch_t<true, true, true, true, 8>(g, wide, wdev, src, dst, status, sms, stream, chained)
-                   : launch_t<true, true, false, true, 8>(g, wide, wdev, src, dst, status, sms, stream, chained);
-      return per ? launch_t<true, true, true, true, 16>(g, wide, wdev, src, dst, status, sms, stream, chained)
-                 : launch_t<true, true, false, true, 16>(g, wide, wdev, src, dst, status, sms, stream, chained);
-    }
+    if (wide.equal)
+      return per ? launch_p<true, true, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained)
+                 : launch_p<true, true, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained);
     return per ? launch_p<true, false, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained)
                : launch_p<true, false, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained);
   }

@@ -86,7 +86,7 @@ __device__ __forceinline__ void get_pair(const long long* m, const int* e, WideV
 }
 
 // Unpacks row `row` of a raw plane (two columns per lane; those at or beyond
-// column `cols` of the tile are the producer's or nobody's; TWOS: wide_unpack_twos).
+// column `cols` of the tile are the producer's or nobody's; TWOS: in two's complement).
 template <bool TMA, int ROWS, bool TWOS = false>
 __device__ __forceinline__ void unpack_row(const double (&raw)[ROWS][raw_col<TMA>()], const int (&shift)[ROWS],
                                            WidePlane<ROWS>& u, int row, int lane, int cols, WideVal (&v)[2]) {
@@ -97,8 +97,8 @@ __device__ __forceinline__ void unpack_row(const double (&raw)[ROWS][raw_col<TMA
     const double* r = &raw[row][2 * lane + shift[row]];
     p = make_double2(r[0], r[1]);
   }
-  v[0] = TWOS ? wide_unpack_twos(p.x) : wide_unpack(p.x);
-  v[1] = TWOS ? wide_unpack_twos(p.y) : wide_unpack(p.y);
+  v[0] = TWOS ? wide_twos(wide_unpack(p.x)) : wide_unpack(p.x);
+  v[1] = TWOS ? wide_twos(wide_unpack(p.y)) : wide_unpack(p.y);
   if (TMA || 2 * lane + 1 < cols) {
     *reinterpret_cast<int4*>(&u.m[row][2 + 2 * lane]) = make_int4((int)v[0].lo, v[0].hi, (int)v[1].lo, v[1].hi);
     *reinterpret_cast<int2*>(&u.e[row][2 + 2 * lane]) = make_int2(v[0].e, v[1].e);

@@ -23,8 +23,8 @@ r*Tb planes each way per block:
     the array's own edge (wrong there), but the owned planes depend only on
     planes within r*s <= H of them, which were all correct at the start of
     the block: the owned planes are exactly the single-grid result.  The
-    kernels apply the same per-cell multiply-add chain whatever the array's
-    shape, so they are bitwise equal to it too;
+    kernels take the same per-cell sum whatever the array's shape and wherever
+    in the grid it begins, so they are bitwise equal to it too;
   - the halo is recomputed by both neighbours (2H planes per slab and step):
     the price of one message per block instead of one per step.
 

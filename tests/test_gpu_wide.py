@@ -494,3 +494,63 @@ def test_stars_by_default_equal_the_persistent_kernel(st, shape, boundary):
         for offset in (0, 1):
             got = run(st, u0, w, 1, boundary, T, (0, 0), offset)
             assert np.array_equal(got, run(st, u0, w, 1, boundary, T, (1, st.VARIANT_PERSISTENT), offset)), (T, offset)
+
+
+def equal_box_fields(shape):
+    """Values of one binade, of many, at the ends of the binades that share an alignment, and among
+    zeros and values that the integer form does not take."""
+    rng = np.random.default_rng(50)
+    yield synth.uniform(51, shape)
+    yield rng.uniform(1.0, 4.0, shape) * rng.choice([1.0, -1.0], shape)
+    yield rng.uniform(0.02, 4.0, shape)
+    yield rng.standard_normal(shape) * 2.0 ** rng.integers(-4, 5, shape)
+    yield rng.choice([2.0, np.nextafter(2.0, 0), -2.0, 0.125, 0.0, -0.0], shape)
+    u0 = rng.standard_normal(shape) * 2.0 ** rng.integers(-60, 61, shape)
+    u0[rng.random(shape) < 0.3] = 0.0
+    mask = rng.random(shape) < 1e-3
+    u0[mask] = rng.choice([np.inf, -np.inf, np.nan, 1.7e308, 5e-324, 1e-300], int(mask.sum()))
+    yield u0
+
+
+# cell by cell against tiles (TMA; tiles of 8 and 16 rows), Tb steps on the chip and handed over
+# between CTAs; and as many cells as bulk copies take (3D: 8 and 16 rows)
+EQUAL_BOXES = [((64, 128), 1, ["direct", "persistent", "stream"]), ((512, 320), 1, ["direct", "persistent", "stream"]),
+               ((64, 192), 2, ["direct", "stream"]), ((512, 256), 2, ["direct", "stream"]),
+               ((5, 32, 128), 1, ["direct", "stream", "temporal", "exchange"]),
+               ((34, 64, 64), 1, ["direct", "stream"]), ((260, 64, 64), 1, ["direct", "stream"])]
+
+
+@pytest.mark.parametrize("boundary", [DIRICHLET, PERIODIC])
+@pytest.mark.parametrize("shape,radius,kernels", EQUAL_BOXES)
+def test_equal_boxes_have_the_same_bits_in_every_kernel(st, shape, radius, kernels, boundary):
+    import torch
+    w, T = equal_weights(len(shape), radius), 4
+    for u0 in equal_box_fields(shape):
+        want = run(st, u0, w, radius, boundary, T, (1, st.VARIANT_DIRECT), 1)
+        ways = [("direct", 1, 0), *(("stream", 1, ty) for ty in ((0, 8, 16) if len(shape) == 3 else (0,))),
+                *((k, Tb, 0) for k in ("persistent", "temporal", "exchange") for Tb in (2, 4))]
+        for kernel, Tb, tile in ways:
+            if kernel not in kernels:
+                continue
+            g = torch.from_numpy(u0.copy()).cuda()
+            p = st.Plan(shape, radius, w, boundary)
+            p.set_tuning(Tb, getattr(st, "VARIANT_" + kernel.upper()))
+            if tile:
+                p.set_tile(64, tile)
+            p.run(g, T)
+            assert p.status() == 0
+            p.close()
+            assert same(g.cpu().numpy(), want), (kernel, Tb, tile)
+
+
+@pytest.mark.parametrize("radius", [1, 2])
+def test_equal_boxes_have_the_same_bits_in_a_part_of_the_grid(st, radius):
+    """Rows that start at any row and columns that start at any column of the whole grid."""
+    w = equal_weights(2, radius)
+    for u0 in equal_box_fields((48, 130)):
+        want = run(st, u0, w, radius, DIRICHLET, 1, (1, st.VARIANT_STREAM))
+        for y, x in ((1, 0), (3, 1), (4, 2), (7, 5)):
+            part = np.ascontiguousarray(u0[y:y + 33, x:x + 100])
+            got = run(st, part, w, radius, DIRICHLET, 1, (1, st.VARIANT_STREAM))
+            inner = (slice(radius, -radius),) * 2
+            assert same(got[inner], want[y:y + 33, x:x + 100][inner]), (y, x)
