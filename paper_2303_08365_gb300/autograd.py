@@ -14,29 +14,33 @@ dL/du^T as lambda^T and sweeps the transposed stencil backward in time
 ckpt_every steps (0: about sqrt(T)).  dt is a constant (no gradient).  Every
 step runs in the library's CUDA kernels.  diffuse() lets the forward pass keep
 those checkpoints, about T / ckpt_every grids until the graph is freed, where a
-gradient is asked for and the memory is there, so that the backward pass does
-not sweep forward again.
+gradient is asked for, so that the backward pass does not sweep forward again.
+It keeps them only as long as that leaves half of the device's memory free (a
+sixteenth of the device, all graphs together, goes without the question), for
+the sweeps' own scratch and whatever else the program is yet to allocate.
+Otherwise a pass keeps u0 and kappa alone.
 """
+import functools
+import threading
+
 import numpy as np
 import torch
 
-from . import (Plan, stencil_adjoint_vjp, stencil_adjoint_vjp_kept, stencil_kept_states, stencil_run,
-               stencil_run_kept)
+from . import (ERR_OOM, Plan, StencilError, stencil_adjoint_vjp, stencil_adjoint_vjp_kept, stencil_kept_states,
+               stencil_run, stencil_run_kept)
 
 
 class StencilAdjointFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, u0, kappa, plan, dt, T, ckpt_every=0, keep=False):
         ctx.plan, ctx.dt, ctx.T, ctx.ckpt = plan, float(dt), int(T), int(ckpt_every)
-        kept = _room_for_states(u0, ctx.T, ctx.ckpt) if keep else None
-        if kept is None:
+        done = _run_kept(u0, kappa, plan, ctx.dt, ctx.T, ctx.ckpt) if keep else None
+        if done is None:
             u = u0.detach().clone().contiguous()
             stencil_run(plan.handle, u, T, kappa.detach().contiguous(), dt)
             ctx.save_for_backward(u0.detach(), kappa.detach())
             return u
-        u = torch.empty_like(u0, memory_format=torch.contiguous_format)
-        stencil_run_kept(plan.handle, u0.detach().contiguous(), u, ctx.T, kappa.detach().contiguous(), ctx.dt, ctx.ckpt,
-                         kept)
+        u, kept, ctx.held = done
         ctx.save_for_backward(u0.detach(), kappa.detach(), kept)
         return u
 
@@ -55,15 +59,59 @@ class StencilAdjointFn(torch.autograd.Function):
         return gu, gk, None, None, None, None, None
 
 
+class _Held:
+    """The bytes that a graph's checkpoints take, summed per device over the graphs alive."""
+    alive = {}
+    lock = threading.Lock()
+
+    def __init__(self, device, n):
+        self.device, self.n = device, n
+        with self.lock:
+            self.alive[device] = self.alive.get(device, 0) + n
+
+    def __del__(self):
+        with self.lock:
+            self.alive[self.device] -= self.n
+
+
+def _run_kept(u0, kappa, plan, dt, T, ckpt_every):
+    """(u^T, its checkpoints, their _Held); None where there is no room for them."""
+    try:
+        kept = _room_for_states(u0, T, ckpt_every)
+        if kept is None:
+            return None
+        u = torch.empty_like(u0, memory_format=torch.contiguous_format)
+        stencil_run_kept(plan.handle, u0.detach().contiguous(), u, T, kappa.detach().contiguous(), dt, ckpt_every, kept)
+        return u, kept, _Held(kept.device, 8 * kept.numel())
+    except torch.OutOfMemoryError:
+        return None
+    except StencilError as e:
+        if e.code != ERR_OOM:
+            raise
+        return None
+
+
+@functools.lru_cache
+def _total_memory(device):
+    return torch.cuda.get_device_properties(device).total_memory
+
+
 def _room_for_states(u0, T, ckpt_every):
     """An uninitialised tensor for the checkpoints of a forward pass; None when the device
     has no room for it, or u0 is not what the sweep takes (it says so itself)."""
     if u0.device.type != "cuda" or u0.dtype != torch.float64 or T < 0 or ckpt_every < 0:
         return None
-    try:
-        return torch.empty((stencil_kept_states(T, ckpt_every), *u0.shape), dtype=u0.dtype, device=u0.device)
-    except torch.OutOfMemoryError:
-        return None
+    n = stencil_kept_states(T, ckpt_every)
+    # with the sweeps' scratch (5 grids forward, 8 and a segment's states backward) and the
+    # outputs, 3 grids
+    need = 8 * u0.numel() * (n + (T // n if n else T) + 16)
+    total = _total_memory(u0.device)
+    # the driver's answer takes 15 to 20 us, a small pass 370: asked from a thousandth of the
+    # device on, and once the graphs alive hold a sixteenth
+    if need > total // 1024 or need + _Held.alive.get(u0.device, 0) > total // 16:
+        if torch.cuda.mem_get_info(u0.device)[0] < total // 2 + need:
+            return None
+    return torch.empty((n, *u0.shape), dtype=u0.dtype, device=u0.device)
 
 
 def diffuse(u0, kappa, plan, dt, T, ckpt_every=0):

@@ -65,3 +65,53 @@ def test_autograd_with_and_without_room(st, monkeypatch):
     with torch.no_grad():
         assert torch.equal(autograd.diffuse(u0, kappa, p, dt, 19), got[0][0])
     p.close()
+
+
+@pytest.mark.parametrize("short", ["driver", "states", "output", "scratch"])
+def test_autograd_short_of_memory(st, monkeypatch, short):
+    """Where the checkpoints would take what the rest needs, the passes go without them, with
+    the same results: too little free memory, or an allocation of the kept pass that fails."""
+    import torch
+    from paper_2303_08365_gb300 import autograd
+    shape, T = (12, 10, 14), 19
+    u0, kappa, lam, dt = inputs(shape, 71)
+    p = st.Plan.varcoef(shape, DIRICHLET)
+
+    def forward():
+        u, k = u0.clone().requires_grad_(), kappa.clone().requires_grad_()
+        out = autograd.diffuse(u, k, p, dt, T)
+        return out, u, k, len(out.grad_fn.saved_tensors) == 3
+
+    def fails(error):
+        def f(*args, **kwargs):
+            raise error
+        return f
+
+    def results(out, u, k, kept):
+        return [out.detach(), *torch.autograd.grad(out, (u, k), lam)]
+
+    plenty = forward()
+    assert plenty[-1]
+    with monkeypatch.context() as m:
+        if short == "driver":  # other graphs hold a sixteenth, and half of the device is not free any more
+            total = torch.cuda.get_device_properties(0).total_memory
+            n = st.stencil_kept_states(T)  # and a segment of at most T / n, scratch and outputs
+            need = 8 * u0.numel() * (n + T // n + 16)
+            m.setitem(autograd._Held.alive, u0.device, total // 16)
+            m.setattr(torch.cuda, "mem_get_info", lambda *a: (total // 2 + need, total))
+            assert forward()[-1]
+            m.setattr(torch.cuda, "mem_get_info", lambda *a: (total // 2 + need - 1, total))
+        elif short == "states":
+            m.setattr(torch, "empty", fails(torch.OutOfMemoryError("no room")))
+        elif short == "output":
+            m.setattr(torch, "empty_like", fails(torch.OutOfMemoryError("no room")))
+        else:
+            m.setattr(autograd, "stencil_run_kept", fails(st.StencilError(st.ERR_OOM, "no room")))
+        without = forward()
+    assert not without[-1]
+    held = autograd._Held.alive[u0.device]
+    assert held >= 8 * u0.numel() * st.stencil_kept_states(T)
+    assert all(torch.equal(a, b) for a, b in zip(results(*plenty), results(*without)))
+    del plenty
+    assert autograd._Held.alive[u0.device] == held - 8 * u0.numel() * st.stencil_kept_states(T)
+    p.close()
