@@ -197,7 +197,7 @@ void stencil_batch_destroy(stencil_batch b);
  * barrier, with cells_per_thread (1, 2 or 4; a tile is 256 *
  * cells_per_thread consecutive cells of one item) and cooperative blocks per
  * SM (1 .. the kernel's occupancy; 0 restores the defaults 2, or 4 from 2^22
- * cells on, and min(occupancy, 4)).  With both at their defaults, a batch with
+ * cells on, and min(occupancy, 4)).  With both 0, a batch with
  * positive weights whose items fill tiles of 64 x 16 cells to 80 % or more, 1000
  * tiles at least, runs tile by tile instead, every tile as soon as its
  * neighbours have made the step before.  Tb = 2, 4 or 8: Tb steps in shared memory per
@@ -208,7 +208,8 @@ void stencil_batch_destroy(stencil_batch b);
  * the device.  Results do not depend on it (bitwise). */
 int stencil_batch_set_tuning(stencil_batch b, int Tb, int cells_per_thread, int blocks_per_sm);
 
-/* Reports the batch's Tb, cells per thread (0 when Tb > 1) and blocks per SM. */
+/* Reports the batch's Tb, cells per thread (0 when Tb > 1) and blocks per SM; (1, 0, 0) for a
+ * batch that runs tile by tile. */
 int stencil_batch_get_tuning(stencil_batch b, int* Tb, int* cells_per_thread, int* blocks_per_sm);
 
 /* The batch autotuner: times every configuration (Tb = 1 with each

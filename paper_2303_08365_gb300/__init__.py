@@ -471,7 +471,7 @@ class Batch:
         _check(lib().stencil_batch_set_tuning(self.handle, int(Tb), int(cells_per_thread), int(blocks_per_sm)))
 
     def get_tuning(self):
-        """(Tb, cells per thread, blocks per SM) of the batch's kernel."""
+        """(Tb, cells per thread, blocks per SM) of the batch's kernel; (1, 0, 0): tile by tile."""
         t, c, b = ctypes.c_int(0), ctypes.c_int(0), ctypes.c_int(0)
         _check(lib().stencil_batch_get_tuning(self.handle, ctypes.byref(t), ctypes.byref(c), ctypes.byref(b)))
         return t.value, c.value, b.value

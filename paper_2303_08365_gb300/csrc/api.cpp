@@ -1018,18 +1018,14 @@ int batch_init(stencil_batch_s* b, const std::vector<BatchItemDev>& hi, int boun
   std::vector<int> order(n);
   for (int i = 0; i < n; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return hi[a].T > hi[c].T; });
-  // the defaults, asked for or as stencil_batch_get_tuning reports them: tiles where
-  // they are worth it, else cells per thread
+  // nothing asked for: tiles where they are worth it, else cells per thread
   b->any_wide = 0;
   int64_t cells = 0;
   for (const BatchItemDev& it : hi) {
     b->any_wide |= it.wide.n != 0;
     cells += (int64_t)it.ny * it.nx;
   }
-  const bool tiles_wanted = b->Tb == 1 && (b->cpt == 0 || b->cpt == batched_default_cpt()) &&
-                            (b->per_sm == 0 || b->per_sm == 4);
-  // (400 grids of 64..256 in the integer form: 102 GStencil/s with 4 cells per thread, 97 with 2)
-  if (b->cpt == 0) b->cpt = b->any_wide && cells >= (int64_t)1 << 22 ? 4 : batched_default_cpt();
+  const bool tiles_wanted = b->Tb == 1 && b->cpt == 0 && b->per_sm == 0;
   b->hi = hi;
   CUDA_TRY(dev_malloc(&b->d_ctl, (4 + kProgressWords) * sizeof(unsigned int)), "allocating the barrier words");
   CUDA_TRY(cudaMemset(b->d_ctl, 0, 4 * sizeof(unsigned int)), "clearing the barrier words");
@@ -1038,12 +1034,12 @@ int batch_init(stencil_batch_s* b, const std::vector<BatchItemDev>& hi, int boun
     const int rc = batch_init_steps(b, hi, order);
     if (rc) return rc;
     if (b->nsteps > 0) {
-      b->cpt = batched_default_cpt();
-      b->blocks = 4 * sm_count();  // (what get_tuning reports)
       b->ready = true;
       return STENCIL_OK;
     }
   }
+  // (400 grids of 64..256 in the integer form: 102 GStencil/s with 4 cells per thread, 97 with 2)
+  if (b->cpt == 0) b->cpt = b->any_wide && cells >= (int64_t)1 << 22 ? 4 : batched_default_cpt();
   std::vector<BatchTile> tiles;
   const int tc = batched_tile_cells(b->cpt);
   for (int i : order) {
@@ -1756,7 +1752,7 @@ int stencil_batch_get_tuning(stencil_batch b, int* Tb, int* cells_per_thread, in
   if (!b || !Tb || !cells_per_thread || !blocks_per_sm) return fail(STENCIL_ERR_ARG, "NULL argument");
   *Tb = b->Tb;
   *cells_per_thread = b->Tb > 1 ? 0 : b->cpt;
-  *blocks_per_sm = (b->blocks + sm_count() - 1) / std::max(1, sm_count());
+  *blocks_per_sm = b->nsteps > 0 ? 0 : (b->blocks + sm_count() - 1) / std::max(1, sm_count());
   return STENCIL_OK;
 }
 

@@ -554,3 +554,27 @@ def test_equal_boxes_have_the_same_bits_in_a_part_of_the_grid(st, radius):
             got = run(st, part, w, radius, DIRICHLET, 1, (1, st.VARIANT_STREAM))
             inner = (slice(radius, -radius),) * 2
             assert same(got[inner], want[y:y + 33, x:x + 100][inner]), (y, x)
+
+
+def test_batch_runs_the_kernel_that_is_asked_for(st):
+    """Tiles by default where the grids fill them; the cells per thread and blocks per SM that a
+    caller names otherwise, the default ones among them.  The same bits; what is reported can be set."""
+    import torch
+    u0 = [synth.uniform(60 + i, s) for i, s in enumerate([(900, 1300), (1024, 640), (700, 900)])]
+    grids = [torch.from_numpy(u.copy()).cuda() for u in u0]
+    with st.Batch(grids, [0.1, 0.2, 0.15], [7, 12, 3]) as b:
+        assert b.get_tuning() == (1, 0, 0)
+        b.run()
+        assert b.status() == 0
+        want = [g.cpu().numpy().copy() for g in grids]
+        for tuning in ((1, 2, 4), (1, 2, 0), (1, 0, 4), (1, 4, 2), (1, 0, 0)):
+            for g, u in zip(grids, u0):
+                g.copy_(torch.from_numpy(u))
+            b.set_tuning(*tuning)
+            got = b.get_tuning()
+            assert got == tuning if tuning in ((1, 2, 4), (1, 4, 2), (1, 0, 0)) else got[1] > 0 and got[2] > 0, tuning
+            b.set_tuning(*got)
+            assert b.get_tuning() == got
+            b.run()
+            assert b.status() == 0
+            assert all(np.array_equal(g.cpu().numpy(), w) for g, w in zip(grids, want)), tuning
