@@ -1406,6 +1406,7 @@ int64_t stencil_kept_states(int64_t T, int ckpt_every) {
 
 int stencil_run_kept(stencil_plan p, const double* d_u0, double* d_uT, int64_t T, const double* d_kappa, double dt,
                      int ckpt_every, double* d_kept, void* cuda_stream) {
+  g_err.clear();
   if (!p) return fail(STENCIL_ERR_ARG, "plan is NULL");
   if (!p->varcoef) return fail(STENCIL_ERR_ARG, "keeping the states needs a variable-coefficient plan");
   if (!d_u0 || !d_uT || !d_kappa || d_u0 == d_uT) return fail(STENCIL_ERR_ARG, "NULL buffer, or u0 and uT the same");
@@ -1440,6 +1441,7 @@ int stencil_run_kept(stencil_plan p, const double* d_u0, double* d_uT, int64_t T
 int stencil_adjoint_vjp_kept(stencil_plan p, const double* d_u0, const double* d_kappa, double dt, int64_t T,
                              int ckpt_every, const double* d_kept, const double* d_lambda_T, double* d_grad_u0,
                              double* d_grad_kappa, void* cuda_stream) {
+  g_err.clear();
   if (!p) return fail(STENCIL_ERR_ARG, "plan is NULL");
   if (!d_lambda_T) return fail(STENCIL_ERR_ARG, "NULL buffer");
   if (!d_kept && stencil_kept_states(T, ckpt_every) > 0) return fail(STENCIL_ERR_ARG, "NULL buffer for the states");

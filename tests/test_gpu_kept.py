@@ -115,3 +115,19 @@ def test_autograd_short_of_memory(st, monkeypatch, short):
     del plenty
     assert autograd._Held.alive[u0.device] == held - 8 * u0.numel() * st.stencil_kept_states(T)
     p.close()
+
+
+def test_kept_calls_leave_no_earlier_message(st):
+    import torch
+    u0, kappa, lam, dt = inputs((5, 6, 7), 81)
+    p = st.Plan.varcoef((5, 6, 7), DIRICHLET)
+    uT, gu, gk = (torch.empty_like(u0) for _ in range(3))
+    kept = torch.empty((st.stencil_kept_states(9), 5, 6, 7), dtype=torch.float64, device="cuda")
+    for call in (lambda: st.stencil_run_kept(p.handle, u0, uT, 9, kappa, dt, 0, kept),
+                 lambda: st.stencil_adjoint_vjp_kept(p.handle, u0, kappa, dt, 9, 0, kept, lam, gu, gk)):
+        with pytest.raises(st.StencilError):
+            p.run(uT, 1, kappa, -1.0)
+        assert st.last_error() != ""
+        call()
+        assert st.last_error() == ""
+    p.close()
