@@ -298,8 +298,8 @@ int stencil_get_tuning(stencil_plan p, int* Tb, int* variant);
 /* Tile shape of the 3D TMA-fed streaming kernel (STENCIL_VARIANT_STREAM,
  * radius 1): tiles of tile_x = 64 columns (one warp's 32 lanes x 2 cells; 0
  * also means 64) by tile_y rows, tile_y in {8, 16, 32}, or 0 for the default
- * (32 for a star, 16 for a box).  Periodic grids need ny a multiple of
- * tile_y (STENCIL_ERR_UNSUPPORTED at the next run otherwise).  The paper's
+ * (16; 32 for a star whose weights are not all positive).  Periodic grids need ny a multiple of
+ * tile_y, the star's by default of 32 (STENCIL_ERR_UNSUPPORTED at the next run otherwise).  The paper's
  * blocking sizes are per-benchmark tuning parameters too (Table 1); results
  * do not depend on the tile (bitwise).  The temporal kernels' tiles follow
  * from Tb and, for STENCIL_VARIANT_EXCHANGE, from the SM count (one

@@ -243,6 +243,12 @@ bool streamed_any_shape(const stencil_plan_s* p) {
   return p->ndim == 3 && p->radius == 1 && p->cells() >= (int64_t)1 << (box ? 17 : 22);
 }
 
+// The 3D streaming kernel's tile height for a choice of tile_y (0: its default): 16 rows in the
+// integer form; the FMA chain's kernel has 32 for a star.
+int stream_tile_y(const stencil_plan_s* p, int tile_y) {
+  return tile_y == 0 && p->wide.n ? 16 : stream3d_tile_y(p->shape, tile_y);
+}
+
 // The tile height of those: 16 rows, 8 for small 27-point boxes, whose planes are too
 // few for the chip otherwise (16 against 8 rows: 65^3 28.4 / 22.8 us a step, 97^3 44.4 / 41.0).
 int any_shape_tile_y(const stencil_plan_s* p) {
@@ -1515,7 +1521,7 @@ int stencil_get_tile(stencil_plan p, int* tile_x, int* tile_y) {
   *tile_y = 0;
   if (v == kVariantStream && p->ndim == 3 && p->radius == 1) {
     *tile_x = 64;
-    *tile_y = stream3d_tile_y(p->shape, ty);
+    *tile_y = stream_tile_y(p, ty);
   }
   return STENCIL_OK;
 }
@@ -1556,7 +1562,7 @@ int stencil_autotune(stencil_plan p, double* d_grid, int64_t probe_steps, void* 
                              {2, kVariantExchange, 0}, {4, kVariantExchange, 0}, {8, kVariantExchange, 0}};
   if (p->ndim == 3 && p->radius == 1)  // the streaming kernel's tile heights
     for (int ty : {8, 16, 32})
-      if (ty != stream3d_tile_y(p->shape, 0)) cands.push_back({1, kVariantStream, ty});
+      if (ty != stream_tile_y(p, 0)) cands.push_back({1, kVariantStream, ty});
   cudaEvent_t e0, e1;
   CUDA_TRY(cudaEventCreate(&e0), "creating an event");
   CUDA_TRY(cudaEventCreate(&e1), "creating an event");

@@ -105,7 +105,7 @@ cudaError_t launch_stream3d(Shape shape, int boundary, const Geom& g, const Host
                             long long skip_plane = -1, int tile_y = 0);
 
 // 3D radius-1 sweep with the weighted sum in the integer form (wide.n != 0):
-// tiles of 64 columns by 16 rows (8 for tile_y = 8).  tma: the grid is one that
+// tiles of 64 columns by 16 rows (tile_y = 8: 8, and with tma 32: 32).  tma: the grid is one that
 // stream3d_eligible takes; false: any shape, alignment and boundary.  chained: the
 // stream's last launch is a step of the same run by this kernel or launch_wide2d's
 // (launch_step in widestream.cuh).

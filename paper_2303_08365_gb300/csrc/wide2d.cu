@@ -622,7 +622,7 @@ cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, co
   P.wide = wide;
   int64_t grid = (int64_t)sms * occ;
   if (grid > work) grid = work;
-  if (const cudaError_t e = launch_step(kern, (unsigned)grid, bytes, stream, chained, P)) return e;
+  if (const cudaError_t e = launch_step(kern, (unsigned)grid, kThreads, bytes, stream, chained, P)) return e;
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
 }

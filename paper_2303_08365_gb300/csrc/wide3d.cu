@@ -43,7 +43,14 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();  // stream.cu
 
 namespace {
 
-constexpr int kTX = kWTX, kRaw = kWRaw, kWarps = kWWarps, kThreads = kWThreads;
+constexpr int kTX = kWTX, kRaw = kWRaw;
+// Consumer warps: two rows each of a tile of 16, one of 8; of 32 rows (a caller's or the tuner's
+// choice) twice as many, one CTA to an SM.  GStencil/s at 8, 16 and 32 rows: heat 512^3 138, 170.5,
+// 173.5, 128^3 96, 106, 118, general box 384^3 46, 48.7, 50.5, equal box 77, 108, 110.
+template <int TC>
+constexpr int warps() { return TC == 32 ? 2 * kWWarps : kWWarps; }
+template <int TC>
+constexpr int threads() { return 32 * (warps<TC>() + 1); }
 template <int TC>
 using Plane = WidePlane<TC + 2>;
 
@@ -97,7 +104,7 @@ __device__ __forceinline__ constexpr int tap_at(int dz, int dy, int dx) {
 template <bool BOX, int TC>
 __device__ __noinline__ bool zero_cells(const Plane<TC>& um, const Plane<TC>& u0, const Plane<TC>& up, int row0,
                                         int rows, int cols, int c0, double* out, int nx) {
-  constexpr int R = TC / kWarps;
+  constexpr int R = TC / warps<TC>();
   if (!zero_rows<R, 1>(u0, row0, c0, cols)) return false;
   if (BOX ? !zero_rows<1, 1>(u0, row0 - 1, c0, cols) || !zero_rows<1, 1>(u0, row0 + R, c0, cols) ||
                 !zero_rows<R + 2, 1>(um, row0 - 1, c0, cols) || !zero_rows<R + 2, 1>(up, row0 - 1, c0, cols)
@@ -195,8 +202,10 @@ __device__ __noinline__ void own_cells(const Plane<TC>& um, const Plane<TC>& u0,
 // copies, us a step, three against two: heat 124 / 137; general weights, which spill,
 // 167 / 148).
 template <bool BOX, bool HEAT, bool PERIODIC, bool TMA, int TC>
-__global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wide3d(const __grid_constant__ Params P) {
-  constexpr int R = TC / kWarps;  // rows of a consumer warp
+__global__ void __launch_bounds__(threads<TC>(), TC == 32 ? 1 : BOX || !(TMA || HEAT) ? 2 : 3)
+    k_wide3d(const __grid_constant__ Params P) {
+  constexpr int kWarps = warps<TC>(), R = TC / kWarps;  // R: rows of a consumer warp
+  static_assert(TMA || TC < 32, "by bulk copies, a lane copies a row");
   constexpr int kU = ring<BOX>();
   constexpr int kLag = BOX ? 2 : 1;  // the middle plane is kLag planes behind the one being unpacked
   constexpr unsigned long long kWaitNs = (unsigned long long)kSpinLimitNs;
@@ -422,7 +431,6 @@ __global__ void __launch_bounds__(kThreads, BOX || !(TMA || HEAT) ? 2 : 3) k_wid
             store(r, v[0], v[1]);
           }
         } else if constexpr (HEAT) {
-          static_assert(R <= 2, "the block");
           // equal weights, the lane's rows and two columns as one block: each value is
           // aligned once for all cells, and rows (mid: their common columns) share their
           // partial sums.  Exponents first: a block's values would not fit the registers.
@@ -587,7 +595,7 @@ cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, co
   const int occ = cached_per_device(cache, [kern] {
     int n = 0;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kThreads, bytes) != cudaSuccess)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads<TC>(), bytes) != cudaSuccess)
       n = 0;
     return n;
   });
@@ -608,14 +616,16 @@ cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, co
   P.wide = wide;
   long long grid = (long long)sms * occ;
   if (grid > P.work) grid = P.work;
-  if (const cudaError_t e = launch_step(kern, (unsigned)grid, bytes, stream, chained, P)) return e;
+  if (const cudaError_t e = launch_step(kern, (unsigned)grid, threads<TC>(), bytes, stream, chained, P)) return e;
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
 }
 
 template <bool BOX, bool HEAT, bool PERIODIC>
 cudaError_t launch_p(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst,
-                     int* status, int sms, cudaStream_t stream, bool tma, bool low, bool chained) {
+                     int* status, int sms, cudaStream_t stream, bool tma, int tile_y, bool chained) {
+  const bool low = tile_y == 8;
+  if (tma && tile_y == 32) return launch_t<BOX, HEAT, PERIODIC, true, 32>(g, wide, wdev, src, dst, status, sms, stream, chained);
   if (tma)
     return low ? launch_t<BOX, HEAT, PERIODIC, true, 8>(g, wide, wdev, src, dst, status, sms, stream, chained)
                : launch_t<BOX, HEAT, PERIODIC, true, 16>(g, wide, wdev, src, dst, status, sms, stream, chained);
@@ -628,21 +638,21 @@ cudaError_t launch_p(const Geom& g, const WideTaps& wide, const double* wdev, co
 cudaError_t launch_wide3d(Shape shape, int boundary, const Geom& g, const WideTaps& wide, const double* wdev,
                           const double* src, double* dst, int* status, int sms, cudaStream_t stream, int tile_y,
                           bool tma, bool chained) {
-  const bool per = boundary == kPeriodic, low = tile_y == 8;
+  const bool per = boundary == kPeriodic;
   if (shape == Shape::kBox) {
     if (wide.n != 27) return cudaErrorInvalidValue;
     if (wide.equal)
-      return per ? launch_p<true, true, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained)
-                 : launch_p<true, true, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained);
-    return per ? launch_p<true, false, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained)
-               : launch_p<true, false, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained);
+      return per ? launch_p<true, true, true>(g, wide, wdev, src, dst, status, sms, stream, tma, tile_y, chained)
+                 : launch_p<true, true, false>(g, wide, wdev, src, dst, status, sms, stream, tma, tile_y, chained);
+    return per ? launch_p<true, false, true>(g, wide, wdev, src, dst, status, sms, stream, tma, tile_y, chained)
+               : launch_p<true, false, false>(g, wide, wdev, src, dst, status, sms, stream, tma, tile_y, chained);
   }
   if (wide.n != 7) return cudaErrorInvalidValue;
   if (wide.heat)
-    return per ? launch_p<false, true, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained)
-               : launch_p<false, true, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained);
-  return per ? launch_p<false, false, true>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained)
-             : launch_p<false, false, false>(g, wide, wdev, src, dst, status, sms, stream, tma, low, chained);
+    return per ? launch_p<false, true, true>(g, wide, wdev, src, dst, status, sms, stream, tma, tile_y, chained)
+               : launch_p<false, true, false>(g, wide, wdev, src, dst, status, sms, stream, tma, tile_y, chained);
+  return per ? launch_p<false, false, true>(g, wide, wdev, src, dst, status, sms, stream, tma, tile_y, chained)
+             : launch_p<false, false, false>(g, wide, wdev, src, dst, status, sms, stream, tma, tile_y, chained);
 }
 
 }  // namespace gbst

@@ -169,10 +169,10 @@ __device__ __forceinline__ void step_begins() {
 // Launches a step's kernel.  chained: what the stream holds last is the step
 // before of the same run (any other launch takes the stream's plain order).
 template <class Kernel, class P>
-cudaError_t launch_step(Kernel kern, unsigned int grid, size_t smem, cudaStream_t stream, bool chained, const P& p) {
+cudaError_t launch_step(Kernel kern, unsigned int grid, int threads, size_t smem, cudaStream_t stream, bool chained, const P& p) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kWThreads);
+  cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];

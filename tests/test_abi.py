@@ -154,6 +154,21 @@ def test_tile_setting_is_checked_on_host(stencil):
     p.close()
 
 
+def test_the_tile_reported_is_the_tile_run(stencil):
+    """The streaming kernel's own heights: 16 by default in the integer form, 32 for a star on the
+    FMA chain; what is set otherwise."""
+    heat = np.zeros(27)
+    heat[[4, 10, 12, 13, 14, 16, 22]] = [.1, .1, .1, .4, .1, .1, .1]
+    cold = heat.copy()
+    cold[13] = -.4
+    for w, default in ((heat, 16), (cold, 32), (np.ones(27) / 27, 16)):
+        with stencil.Plan((8, 64, 128), 1, w, stencil.PERIODIC) as p:
+            assert p.get_tile() == (64, default)
+            for ty in (8, 16, 32):
+                p.set_tile(64, ty)
+                assert p.get_tile() == (64, ty)
+
+
 def test_old_four_field_tuning_records_are_read(tmp_path):
     """Records written before the tile field (key Tb variant rate) still apply."""
     import subprocess

@@ -512,7 +512,7 @@ def equal_box_fields(shape):
     yield u0
 
 
-# cell by cell against tiles (TMA; tiles of 8 and 16 rows), Tb steps on the chip and handed over
+# cell by cell against tiles (TMA; tiles of 8, 16 and 32 rows), Tb steps on the chip and handed over
 # between CTAs; and as many cells as bulk copies take (3D: 8 and 16 rows)
 EQUAL_BOXES = [((64, 128), 1, ["direct", "persistent", "stream"]), ((512, 320), 1, ["direct", "persistent", "stream"]),
                ((64, 192), 2, ["direct", "stream"]), ((512, 256), 2, ["direct", "stream"]),
@@ -527,7 +527,7 @@ def test_equal_boxes_have_the_same_bits_in_every_kernel(st, shape, radius, kerne
     w, T = equal_weights(len(shape), radius), 4
     for u0 in equal_box_fields(shape):
         want = run(st, u0, w, radius, boundary, T, (1, st.VARIANT_DIRECT), 1)
-        ways = [("direct", 1, 0), *(("stream", 1, ty) for ty in ((0, 8, 16) if len(shape) == 3 else (0,))),
+        ways = [("direct", 1, 0), *(("stream", 1, ty) for ty in ((0, 8, 16, 32) if len(shape) == 3 else (0,))),
                 *((k, Tb, 0) for k in ("persistent", "temporal", "exchange") for Tb in (2, 4))]
         for kernel, Tb, tile in ways:
             if kernel not in kernels:
