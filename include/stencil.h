@@ -321,10 +321,10 @@ int stencil_get_tile(stencil_plan p, int* tile_x, int* tile_y);
  * take the plan. */
 int stencil_exchange_layout(stencil_plan p, int Tb, int* nbands, int64_t* rows_computed);
 
-/* Times the candidate (Tb, variant) pairs -- and, for the 3D streaming
+/* Times the default choice, the candidate (Tb, variant) pairs -- and, for the 3D streaming
  * kernel, each tile height -- on d_grid (device, contents are destroyed) for
  * probe_steps steps each, after a warm-up, and keeps the fastest for p (and
- * in the tuning record: key Tb variant tile_y rate).  Synchronous.
+ * in the tuning record: key Tb variant tile_y rate; Tb and variant 0 for the default).  Synchronous.
  * *best_gstencils (may be NULL) receives its rate in 1e9 cell updates per
  * second. */
 int stencil_autotune(stencil_plan p, double* d_grid, int64_t probe_steps, void* cuda_stream,

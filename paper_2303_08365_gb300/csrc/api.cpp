@@ -150,6 +150,8 @@ struct stencil_plan_s {
   // tuning
   int user_Tb = 0, user_variant = 0;
   int tuned_Tb = 0, tuned_variant = 0;
+  bool tuned_default = false;  // the tuner's choice is the library's default
+  bool probing = false;        // the tuner is timing that: records do not count
   int user_tile_y = 0, tuned_tile_y = 0;  // streaming kernel's tile height (0: its default)
 
   int64_t cells() const { return g.cells(); }
@@ -285,6 +287,13 @@ std::string plan_key(const stencil_plan_s* p) {
   return buf;
 }
 
+// The key that this plan's own choices are recorded under: with the form of its sum, where its class
+// has two, as the weights' signs select other kernels.  (Records of earlier versions, without it,
+// are read where there is none with.)
+std::string plan_form_key(const stencil_plan_s* p) {
+  return plan_key(p) + (!uses_wide(p->ndim, p->radius) ? "" : p->wide.n ? "/int" : "/fma");
+}
+
 int ensure(double** buf, size_t count, const char* what) {
   if (*buf) return STENCIL_OK;
   cudaError_t e = dev_malloc(buf, count * sizeof(double));
@@ -314,8 +323,9 @@ int sm_count() {
 // ------------------------------------------------------------ tuning record
 // Process-wide record of autotuned choices, keyed by the GPU name and the
 // plan's shape (ndim, dims, radius, stencil class, equal-weight box,
-// boundary).  STENCIL_TUNE_CACHE=<file> persists it across processes (one
-// line per key: key Tb variant rate); STENCIL_TUNE=off ignores it,
+// boundary; form of the sum).  STENCIL_TUNE_CACHE=<file> persists it across processes (one
+// line per key: key Tb variant tile_y rate; Tb and variant 0: the library's default);
+// STENCIL_TUNE=off ignores it,
 // STENCIL_TUNE=full tunes a plan on its first run when no record exists.
 struct TuneRec {
   int Tb, variant, tile_y;
@@ -360,7 +370,7 @@ void tune_load_locked() {
     double rate = 0.0;
     const int got = std::sscanf(line, "%511s %d %d %d %lf", key, &tb, &v, &ty, &rate);
     if (got == 4) ty = 0;  // key Tb variant rate
-    if (got >= 4 && tb > 0 && v > 0 && v < kVariantCount && ty >= 0) g_tune[key] = {tb, v, ty};
+    if (got >= 4 && tb >= 0 && v >= 0 && (tb > 0) == (v > 0) && v < kVariantCount && ty >= 0) g_tune[key] = {tb, v, ty};
   }
   std::fclose(f);
 }
@@ -377,10 +387,11 @@ void tune_store(const std::string& key, int tb, int v, int ty, double rate) {
   std::fclose(f);
 }
 
-bool tune_lookup(const std::string& key, int& tb, int& v, int& ty) {
+bool tune_lookup(const stencil_plan_s* p, int& tb, int& v, int& ty) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
   tune_load_locked();
-  auto it = g_tune.find(key);
+  auto it = g_tune.find(plan_form_key(p));
+  if (it == g_tune.end()) it = g_tune.find(plan_key(p));
   if (it == g_tune.end()) return false;
   tb = it->second.Tb;
   v = it->second.variant;
@@ -471,14 +482,14 @@ void choose(const stencil_plan_s* p, int& Tb, int& variant, int& tile_y, bool& t
     return;
   }
   tuned = true;
-  if (p->tuned_Tb > 0) {
+  if (p->tuned_Tb > 0 && !p->probing) {
     Tb = p->tuned_Tb;
     variant = p->tuned_variant;
     if (!tile_y) tile_y = p->tuned_tile_y;
     return;
   }
   int ty = 0;
-  if (tune_mode() != "off" && tune_lookup(plan_key(p), Tb, variant, ty)) {
+  if (!p->probing && !p->tuned_default && tune_mode() != "off" && tune_lookup(p, Tb, variant, ty) && Tb > 0) {
     if (!tile_y) tile_y = ty;
     return;
   }
@@ -522,9 +533,11 @@ int ensure_status(stencil_plan_s* p) {
 // STENCIL_TUNE=full: the first run of an untuned shape times the candidates
 // on a scratch copy of the grid (their runs destroy it) and records the best.
 void tune_on_first_run(stencil_plan_s* p, const double* d_grid, cudaStream_t s) {
-  if (tune_mode() != "full" || p->user_Tb != 0 || p->user_variant != 0 || p->tuned_Tb != 0) return;
+  if (tune_mode() != "full" || p->user_Tb != 0 || p->user_variant != 0 || p->tuned_Tb != 0 || p->tuned_default ||
+      p->probing)
+    return;
   int tb0, v0, ty0;
-  if (tune_lookup(plan_key(p), tb0, v0, ty0)) return;
+  if (tune_lookup(p, tb0, v0, ty0)) return;
   double* scratch = nullptr;
   if (dev_malloc(&scratch, (size_t)p->cells() * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
@@ -1556,7 +1569,8 @@ int stencil_autotune(stencil_plan p, double* d_grid, int64_t probe_steps, void* 
   if (probe_steps < 1) return fail(STENCIL_ERR_ARG, "probe_steps must be >= 1");
   cudaStream_t s = (cudaStream_t)cuda_stream;
   struct Cand { int Tb, variant, tile_y; };
-  std::vector<Cand> cands = {{1, kVariantDirect, 0}, {1, kVariantStream, 0}, {1, kVariantPersistent, 0},
+  // first the default, which has kernels that no variant names
+  std::vector<Cand> cands = {{0, 0, 0}, {1, kVariantDirect, 0}, {1, kVariantStream, 0}, {1, kVariantPersistent, 0},
                              {2, kVariantPersistent, 0}, {4, kVariantPersistent, 0}, {8, kVariantPersistent, 0},
                              {2, kVariantTemporal, 0}, {4, kVariantTemporal, 0}, {8, kVariantTemporal, 0},
                              {2, kVariantExchange, 0}, {4, kVariantExchange, 0}, {8, kVariantExchange, 0}};
@@ -1573,7 +1587,8 @@ int stencil_autotune(stencil_plan p, double* d_grid, int64_t probe_steps, void* 
     p->user_Tb = c.Tb;
     p->user_variant = c.variant;
     p->user_tile_y = c.tile_y;
-    int rc = stencil_run(p, d_grid, c.Tb, nullptr, 0.0, cuda_stream);  // warm-up
+    p->probing = c.Tb == 0;
+    int rc = stencil_run(p, d_grid, c.Tb > 0 ? c.Tb : probe_steps, nullptr, 0.0, cuda_stream);  // warm-up
     if (rc == STENCIL_ERR_UNSUPPORTED) continue;
     if (rc) break;
     cudaEventRecord(e0, s);
@@ -1589,6 +1604,7 @@ int stencil_autotune(stencil_plan p, double* d_grid, int64_t probe_steps, void* 
       best_c = c;
     }
   }
+  p->probing = false;
   p->user_Tb = saved_Tb;
   p->user_variant = saved_v;
   p->user_tile_y = saved_ty;
@@ -1598,7 +1614,8 @@ int stencil_autotune(stencil_plan p, double* d_grid, int64_t probe_steps, void* 
   p->tuned_Tb = best_c.Tb;
   p->tuned_variant = best_c.variant;
   p->tuned_tile_y = best_c.tile_y;
-  tune_store(plan_key(p), best_c.Tb, best_c.variant, best_c.tile_y, best);
+  p->tuned_default = best_c.Tb == 0;
+  tune_store(plan_form_key(p), best_c.Tb, best_c.variant, best_c.tile_y, best);
   if (best_gstencils) *best_gstencils = best;
   return STENCIL_OK;
 }

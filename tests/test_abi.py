@@ -186,6 +186,32 @@ def test_old_four_field_tuning_records_are_read(tmp_path):
     assert out.stdout.split() == ["4", "3"]
 
 
+def test_tuning_records_name_the_form_of_the_sum_and_the_default(tmp_path):
+    """A choice timed with positive weights (another kernel) is not taken for others, nor the other way;
+    0 0 is the default; a record without the form serves where there is none with."""
+    import subprocess
+    import sys
+    code = ("import numpy as np, paper_2303_08365_gb300 as st\n"
+            "for w in (np.ones(27) / 27, -np.ones(27) / 27):\n"
+            "    print(*st.stencil_get_tuning(st.stencil_create((16, 32, 64), 1, w, st.PERIODIC)))\n")
+    key = "unknown/d3/16x32x64/r1/boxeq/b1"
+
+    def choices(*records):
+        cache = tmp_path / "tune.txt"
+        cache.write_text("".join(r + "\n" for r in records))
+        env = dict(os.environ, STENCIL_TUNE_CACHE=str(cache), PYTHONPATH=ROOT)
+        out = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, cwd=ROOT)
+        assert out.returncode == 0, out.stderr
+        return out.stdout.splitlines()
+
+    if choices(key + " 2 3 0 12.5") == ["1 2", "1 2"]:
+        pytest.skip("a CUDA device is visible: the key carries its name")
+    assert choices(key + " 2 3 0 12.5") == ["2 3", "2 3"]
+    assert choices(key + "/int 4 3 0 9.5") == ["4 3", "1 2"]
+    assert choices(key + "/fma 4 3 0 9.5") == ["1 2", "4 3"]
+    assert choices(key + " 2 3 0 12.5", key + "/int 0 0 0 20.0") == ["1 2", "2 3"]
+
+
 def test_fixed_tb_without_variant_keeps_its_tb(stencil):
     """set_tuning(Tb, 0) keeps the Tb: a fused kernel for Tb > 1 (the
     exchange kernel where its tiling fits -- on a host without a GPU the SM

@@ -578,3 +578,18 @@ def test_batch_runs_the_kernel_that_is_asked_for(st):
             b.run()
             assert b.status() == 0
             assert all(np.array_equal(g.cpu().numpy(), w) for g, w in zip(grids, want)), tuning
+
+
+def test_autotune_keeps_a_default_that_no_variant_names(st):
+    """A small 3D star runs all its steps in one launch, by default alone: the tuner times that too, and
+    what it records serves other plans of the key.  20 steps of one launch each take more than twice as long."""
+    import torch
+    shape, w = (64, 64, 64), synth.heat_weights(3, 0.11)
+    g = torch.from_numpy(synth.uniform(70, shape)).cuda()
+    with st.Plan(shape, 1, w, PERIODIC) as a, st.Plan(shape, 1, w, PERIODIC) as b:
+        a.autotune(g.clone(), 20)
+        for p in (a, b):
+            before = st.stencil_launch_count()
+            p.run(g, 20)
+            assert st.stencil_launch_count() - before == 1
+            assert p.status() == 0
