@@ -402,6 +402,7 @@ def headline(st, steps, warmup, world, stream):
     grid = torch.from_numpy(u0).cuda()
     plan = st.Plan(shape, 1, synth.heat_weights(3, HEADLINE["alpha"]), st.PERIODIC)
     tb, variant = plan.get_tuning()
+    tile = plan.get_tile()
     uuid = None
     try:
         uuid = str(torch.cuda.get_device_properties(torch.cuda.current_device()).uuid)
@@ -463,7 +464,21 @@ def headline(st, steps, warmup, world, stream):
     torch.cuda.empty_cache()
     return dict(ms=ms / steps, launches=launches, clocks=clocks, e2e_ms=e2e_ms, e2e_clocks=e2e_clocks,
                 h2d=h2d, d2h=h2d, copy_gbs=copy_gbs, e2e_calls=e2e_calls,
-                Tb=tb, variant=st.stencil_variant_name(variant), u0=u0, checks=checks)
+                Tb=tb, variant=st.stencil_variant_name(variant), tile=tile, u0=u0, checks=checks)
+
+
+def short_forms(forms):
+    """The forms as the line carries them: rates, the kernel's choice and the fraction of its bound."""
+    def short(r):
+        keys = ("gstencil_per_s", "ms", "Tb", "variant", "frac", "speedup_vs_plain", "ratio_vs_forward",
+                "forward_gstencil_per_s")
+        out = {k: r[k] for k in keys if r.get(k) is not None}
+        if isinstance(r.get("roofline"), dict):
+            out.update(bound=r["roofline"]["bound"], frac=r["roofline"]["frac"])
+        if isinstance(r.get("tb_sweep_gstencil_per_s"), dict):
+            out["tb_sweep"] = {k: v["gstencil_per_s"] for k, v in r["tb_sweep_gstencil_per_s"].items()}
+        return out or {k: short(v) for k, v in r.items() if isinstance(v, dict)}
+    return {name: short(r) for name, r in forms.items()}
 
 
 def time_plan(st, plan, grid, T, reps, stream, warm=1):
@@ -1018,6 +1033,8 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--forms", default="all", help="all | none | comma list of "
                     "box2d,box3d,heat2d,batched,adjoint,radius2,onedim,thermal,heat3d_tb,temporal,table1")
+    ap.add_argument("--forms-out", default=os.path.join(ROOT, "bench_forms.json"),
+                    help="where the forms' full records go (the line has their rates)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--case", default=None,
                     help="profiling mode: heat3d | box3d | heat2d | box2d | star2d9 | box2d25 | heat1d | "
@@ -1064,7 +1081,8 @@ def main():
                    "shape": list(HEADLINE["shape"]), "T": T, "grids": world,
                    "parallelism": "replicas" if world > 1 else "single GPU",
                    "Tb": h["Tb"], "variant": h["variant"],
-                   "tile": {"stream": "64 x 32 cells of (x, y), streamed along z, 4-plane TMA ring",
+                   "tile": {"stream": f"{h['tile'][0]} x {h['tile'][1]} cells of (x, y), streamed along z, raw planes "
+                                      "by TMA and unpacked planes in rings of three",
                             "temporal": "64 x 32 (Tb 2), 32 x 32 (Tb 4) or 16 x 16 (Tb 8) cells of (x, y) "
                                         "plus a Tb halo, streamed along z",
                             "exchange": "64 columns x 26-27 rows of (x, y) per co-resident CTA, streamed "
@@ -1170,7 +1188,10 @@ def main():
                                         autotune_steps=8)
         if "adjoint" in want:
             forms["adjoint"] = form_adjoint(st, stream, peak_tflops)
-        line["forms"] = forms
+        # every form in full goes to a file: the line stays short enough to be read as one
+        with open(args.forms_out, "w", encoding="utf-8") as f:
+            json.dump(forms, f, indent=1)
+        line["forms"] = short_forms(forms)
         print(json.dumps(line))
     barrier(world)
     if world > 1:

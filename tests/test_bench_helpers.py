@@ -131,3 +131,20 @@ def test_source_hash_ignores_comments_only():
     c = "int f(int x) {\n  return 3 * x;\n}\n"
     assert bench._code_only(a) == bench._code_only(b)
     assert bench._code_only(a) != bench._code_only(c)
+
+
+def test_the_line_carries_the_forms_rates_and_stays_short():
+    """Full records of some twenty kilobytes made the one line unreadable; a form's rate, choice and
+    fraction of its bound stay in it."""
+    roof = bench.roofline("heat3d-7pt", 512 ** 3, 10, 8.0, 10, 1.256, "wide3d")
+    full = {"workload": "w" * 80, "gstencil_per_s": 170.5, "ms": 787.1, "Tb": 1, "variant": "stream", "tile": [64, 16],
+            "launches": 1000, "roofline": roof,
+            "tb_sweep_gstencil_per_s": {f"Tb={t} exchange": {"gstencil_per_s": 80.0 + t, "frac_basis": "b" * 150}
+                                        for t in (1, 2, 4, 8)}}
+    forms = {f"form{k}": full for k in range(16)}
+    forms["table1"] = {"Heat-3D": {"shape": [1024] * 3, "gstencil_per_s": 171.0, "variant": "stream", "Tb": 1, "frac": 0.5}}
+    short = bench.short_forms(forms)
+    assert short["form3"]["gstencil_per_s"] == 170.5 and short["form3"]["frac"] == roof["frac"]
+    assert short["form3"]["bound"] == roof["bound"] and short["form3"]["tb_sweep"]["Tb=8 exchange"] == 88.0
+    assert short["table1"]["Heat-3D"]["gstencil_per_s"] == 171.0
+    assert len(json.dumps(short)) < 5000 < len(json.dumps(forms)) / 4
