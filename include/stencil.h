@@ -238,14 +238,22 @@ int stencil_plan_status(stencil_plan p, void* cuda_stream);
  * tuned: 3D radius 1 -> STREAM; 2D radius 1 -> PERSISTENT with Tb = 4 up to
  * 2^18 cells (positive weights: a star Tb = 8 up to 2^16, a box of unequal
  * weights up to 2^17), PERSISTENT with Tb = 1 (5-point star) up to 3 * 2^20
- * cells -- by default, with positive weights and a grid that STREAM takes, run
- * as STREAM, which is faster --, else STREAM; 2D radius 2 -> STREAM; 1D ->
- * TEMPORAL with Tb = 8; anything else -> DIRECT.  STREAM needs an even nx and, for periodic grids, nx a
+ * cells, else STREAM; 2D radius 2 -> STREAM; 1D -> TEMPORAL with Tb = 8;
+ * anything else -> DIRECT.  STREAM needs an even nx and, for periodic grids, nx a
  * multiple of 64 and ny a multiple of the tile height (32 for the 3D star,
  * 16 otherwise); other shapes default to DIRECT.  A variant a plan cannot
  * use (including STREAM on buffers not 16-byte aligned) falls back to DIRECT
  * unless it was forced, in which case stencil_run returns
- * STENCIL_ERR_UNSUPPORTED. */
+ * STENCIL_ERR_UNSUPPORTED.
+ *
+ * With positive weights, where something else is faster for the same results
+ * (bitwise), a run takes it without another name for it:
+ *   - by default, a 2D PERSISTENT run with Tb = 1 goes one launch per step where
+ *     STREAM takes the grid or the grid fills tiles of 64 x 16 cells to 80 %;
+ *   - by default, a 7-point star of at most one brick of 32 x 8 x 16 cells per SM
+ *     runs three steps and more in one persistent launch;
+ *   - DIRECT streams grids that STREAM does not take by bulk copies, from 2^16 to
+ *     2^22 cells on, by class. */
 typedef enum {
   STENCIL_VARIANT_AUTO = 0,
   STENCIL_VARIANT_DIRECT = 1,     /* one launch per step, any shape */
@@ -292,7 +300,8 @@ typedef enum {
  * nor a fixed Tb is dropped silently. */
 int stencil_set_tuning(stencil_plan p, int Tb, int variant);
 
-/* Reports the Tb and variant the next stencil_run of p will use. */
+/* Reports the Tb and variant chosen for the next stencil_run of p (forced, tuned or
+ * default; stencil_variant says where a run takes another kernel in their place). */
 int stencil_get_tuning(stencil_plan p, int* Tb, int* variant);
 
 /* Tile shape of the 3D TMA-fed streaming kernel (STENCIL_VARIANT_STREAM,
