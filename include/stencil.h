@@ -426,6 +426,13 @@ int stencil_selftest_flag_timeout(double limit_ms, void* cuda_stream);
  * reported it as designed.  Synchronous; allocates and frees about 0.5 MB. */
 int stencil_selftest_tma_timeout(double limit_ms, void* cuda_stream);
 
+/* The same for the kernels that take positive weights: 0 and 1, the 3D and the 2D
+ * streaming kernel (copies left out, as above), 2, the 2D persistent tile kernel,
+ * and 3, the 3D persistent brick kernel (one CTA does not publish the steps that
+ * its neighbours wait for).  Small grids of the library's own; the waits end by
+ * their wall-time limit.  Synchronous; allocates and frees about 0.6 MB. */
+int stencil_selftest_wide_timeout(int kernel, double limit_ms, void* cuda_stream);
+
 /* Host-side fault injection for tests: after `after` more device allocations
  * by this library succeed, every later one fails as if the device were out
  * of memory, without calling the driver, until the injection is turned off

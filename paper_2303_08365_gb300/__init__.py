@@ -87,6 +87,7 @@ SIGNATURES = [
     ("stencil_debug_fail_allocations", None, [ctypes.c_int]),
     ("stencil_selftest_flag_timeout", ctypes.c_int, [ctypes.c_double, _VP]),
     ("stencil_selftest_tma_timeout", ctypes.c_int, [ctypes.c_double, _VP]),
+    ("stencil_selftest_wide_timeout", ctypes.c_int, [ctypes.c_int, ctypes.c_double, _VP]),
     ("stencil_run_2d_static", ctypes.c_int, [ctypes.c_int64, ctypes.c_int64, _DP, ctypes.c_int, _VP,
                                              ctypes.c_int64, _VP]),
     ("stencil_static_status", ctypes.c_int, [_VP]),
@@ -353,6 +354,12 @@ def stencil_selftest_tma_timeout(limit_ms=20.0, stream=None):
     """Runs the streaming kernel's starved-mbarrier failure path; returns the
     status code (ERR_TIMEOUT when it behaved)."""
     return lib().stencil_selftest_tma_timeout(float(limit_ms), _stream(stream))
+
+
+def stencil_selftest_wide_timeout(kernel, limit_ms=20.0, stream=None):
+    """Runs the failure path of a positive-weight kernel's bounded waits (0, 1: 3D, 2D streaming;
+    2, 3: 2D, 3D persistent); returns the status code (ERR_TIMEOUT when it behaved)."""
+    return lib().stencil_selftest_wide_timeout(int(kernel), float(limit_ms), _stream(stream))
 
 
 def stencil_debug_fail_allocations(after):

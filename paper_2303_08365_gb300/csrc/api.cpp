@@ -2083,6 +2083,95 @@ int stencil_selftest_tma_timeout(double limit_ms, void* cuda_stream) {
   return st;
 }
 
+int stencil_selftest_wide_timeout(int kernel, double limit_ms, void* cuda_stream) {
+  g_err.clear();
+  if (kernel < 0 || kernel > 3) return fail(STENCIL_ERR_ARG, "kernel must be 0, 1, 2 or 3 (got %d)", kernel);
+  if (!(limit_ms > 0.0) || limit_ms > 2000.0) return fail(STENCIL_ERR_ARG, "limit_ms must be in (0, 2000]");
+  cudaStream_t s = (cudaStream_t)cuda_stream;
+  // 0, 1: the streaming kernels, without copies that their consumers wait for; 2, 3: the persistent
+  // ones of two CTAs or more, one of which does not publish the steps that its neighbours wait for
+  const bool flat = kernel == 1 || kernel == 2;
+  const Geom g = flat ? Geom{1, 64, 128} : Geom{8, 32, 128};
+  const int n = flat ? 5 : 7;
+  const size_t cells = (size_t)g.cells(), words = std::max<size_t>(kProgressWords, 64 * kFlagWords);
+  double *a = nullptr, *b = nullptr, *w = nullptr;
+  unsigned int* ctl = nullptr;  // the status word, a line on the progress words
+  auto cleanup = [&]() {
+    cudaFree(a);
+    cudaFree(b);
+    cudaFree(w);
+    cudaFree(ctl);
+  };
+  if (dev_malloc(&a, cells * sizeof(double)) != cudaSuccess || dev_malloc(&b, cells * sizeof(double)) != cudaSuccess ||
+      dev_malloc(&w, (n + kExtraSlots) * sizeof(double)) != cudaSuccess ||
+      dev_malloc(&ctl, (kFlagWords + words) * sizeof(unsigned int)) != cudaSuccess) {
+    cleanup();
+    return fail(STENCIL_ERR_OOM, "allocating the self-test buffers");
+  }
+  std::vector<double> hw(n + kExtraSlots, 0.0);
+  for (int k = 0; k < n; ++k) hw[k] = k == n / 2 ? 0.5 : 0.5 / (n - 1);
+  for (int k = 0; k < kOneSlots; ++k) hw[n + kZeroSlots + k] = 1.0;
+  WideTaps wide;
+  make_wide(hw.data(), n, wide);
+  cudaMemsetAsync(a, 0, cells * sizeof(double), s);
+  cudaMemsetAsync(ctl, 0, (kFlagWords + words) * sizeof(unsigned int), s);
+  cudaMemcpyAsync(w, hw.data(), hw.size() * sizeof(double), cudaMemcpyHostToDevice, s);
+  int* status = (int*)ctl;
+  const long long limit_ns = (long long)(limit_ms * 1e6);
+  cudaError_t e;
+  if (kernel == 0) {
+    e = launch_wide3d_starved(g, wide, w, a, b, status, sm_count(), s, (unsigned long long)limit_ns);
+  } else if (kernel == 1) {
+    e = launch_wide2d_starved(g, wide, w, a, b, status, sm_count(), s, (unsigned long long)limit_ns);
+  } else if (kernel == 2) {
+    BatchItemDev it;
+    it.a = a;
+    it.b = b;
+    it.ny = g.ny;
+    it.nx = g.nx;
+    it.T = 4;
+    for (int k = 0; k < 5; ++k) it.w[k] = hw[k];
+    narrow(wide, it.wide);
+    WideStepsLaunch L;
+    wide_step_item(L.one, it, 0);
+    L.nitems = 1;
+    L.max_T = it.T;
+    L.any_odd = 0;
+    L.heat = it.wide.heat;
+    L.progress = ctl + kFlagWords;
+    L.status = status;
+    L.spin_limit = limit_ns;
+    L.mute = 1;
+    e = launch_wide_steps(L, L.one.ntiles, kPeriodic, sm_count(), s);
+  } else {
+    Steps3dLaunch L;
+    L.a = a;
+    L.b = b;
+    L.nz = g.nz;
+    L.ny = g.ny;
+    L.nx = g.nx;
+    L.periodic = 1;
+    L.T = 4;
+    const int z = steps3d_cut(g, std::min(sm_count(), 64), L.bricks);
+    L.wdev = w;
+    narrow(wide, L.wide);
+    L.progress = ctl + kFlagWords;
+    L.status = status;
+    L.spin_limit = limit_ns;
+    L.mute = 1;
+    e = launch_steps3d(L, z, s);
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  int st = 0;
+  if (e == cudaSuccess) e = cudaMemcpy(&st, status, sizeof(int), cudaMemcpyDeviceToHost);
+  const int rc = e == cudaSuccess ? STENCIL_OK : cuda_fail(e, "running the self-test");
+  cleanup();
+  if (rc) return rc;
+  if (st != STENCIL_ERR_TIMEOUT)
+    return fail(STENCIL_ERR_CUDA, "the bounded waits did not report a timeout (status %d)", st);
+  return st;
+}
+
 // ------------------------------------------------------------ measurement
 
 int stencil_fp64_peak(double millis, double* dfma_per_s, void* cuda_stream) {

@@ -132,6 +132,13 @@ cudaError_t launch_wide2d(Shape shape, int radius, int boundary, const Geom& g, 
                           const double* wdev, const double* src, double* dst, int* status, int sms,
                           cudaStream_t stream, bool tma, bool chained = false);
 
+// Self-tests of those kernels' bounded waits (a star with wide.heat on a periodic grid that TMA takes):
+// the producers leave copies out, so that waits run out after wait_ns.
+cudaError_t launch_wide3d_starved(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst,
+                                  int* status, int sms, cudaStream_t stream, unsigned long long wait_ns);
+cudaError_t launch_wide2d_starved(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst,
+                                  int* status, int sms, cudaStream_t stream, unsigned long long wait_ns);
+
 // 1D sweep (radius 1 or 2) with the weighted sum in the integer form (wide.n != 0),
 // `steps` fused steps (at most kWide1dSteps).
 constexpr int kWide1dSteps = 8;
@@ -151,6 +158,7 @@ struct Steps3dLaunch {
   unsigned int* progress;  // kFlagWords words for each brick, zero before the launch
   int* status;
   long long spin_limit;    // ns
+  int mute = -1;           // self-test: the brick that does not publish its steps
 };
 // Cuts a grid into at most `sms` bricks; returns their cells per thread (launch_steps3d's
 // z), 0 when the grid is too large.
@@ -288,6 +296,7 @@ struct WideStepsLaunch {
   unsigned int* progress;  // kProgressWords words, zero before the launch: steps done by every CTA
   int* status;
   long long spin_limit;    // ns
+  int mute = -1;           // self-test: the CTA that does not publish its steps
 };
 constexpr int kWideStepCtas = 512;  // most CTAs of a launch
 constexpr int kProgressWords = 16 * kWideStepCtas;  // half a line for each

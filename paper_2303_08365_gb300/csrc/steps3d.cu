@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kStepThreads) k_steps3d(const __grid_constant_
     return ok;
   };
   auto publish = [&](unsigned int steps) {  // (after a CTA barrier)
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && (int)blockIdx.x != L.mute) {
       __threadfence();
       asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(L.progress + (int64_t)blockIdx.x * kFlagWords), "r"(steps)
                    : "memory");

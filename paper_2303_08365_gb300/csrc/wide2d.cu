@@ -67,6 +67,7 @@ struct Params {
   int work;  // tiles
   int vec;   // rows start on 16 bytes
   int* status;
+  unsigned long long wait_ns;  // of STARVED
   const double* wdev;
   WideTaps wide;
 };
@@ -211,10 +212,12 @@ template <bool BOX, int RAD, bool HEAT>
 constexpr int wide2d_ctas() { return RAD == 1 && (!BOX || HEAT) ? 3 : 2; }
 
 // HEAT: a star whose weights wide_sum_heat takes; a box whose weights are all equal.
-template <bool BOX, int RAD, bool HEAT, bool PERIODIC, bool TMA>
+// STARVED: the self-test of the bounded waits: no copy (and no arrival that announces one) for a
+// CTA's tiles, and waits of P.wait_ns.
+template <bool BOX, int RAD, bool HEAT, bool PERIODIC, bool TMA, bool STARVED = false>
 __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_wide2d(const __grid_constant__ Params P) {
   constexpr int kRows = kTC + 2 * RAD;
-  constexpr unsigned long long kWaitNs = (unsigned long long)kSpinLimitNs;
+  const unsigned long long kWaitNs = STARVED ? P.wait_ns : (unsigned long long)kSpinLimitNs;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   Smem<RAD, TMA>& S = *reinterpret_cast<Smem<RAD, TMA>*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -263,12 +266,12 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
       if (TMA) {
         const bool whole = !PERIODIC || (y0 >= RAD && y0 + kTC + RAD <= P.ny);
         fence_proxy_async_smem();
-        if (lane == 0) {
+        if (lane == 0 && !STARVED) {
           mbar_arrive_expect_tx(&S.full[post.s], (uint32_t)sizeof(S.raw[0]));
           if (whole) tma_load_2d(&S.raw[post.s][0][0], &P.map_tile, x0, y0 - RAD, &S.full[post.s]);
         }
         __syncwarp();
-        if (!whole && r < kRows)
+        if (!whole && r < kRows && !STARVED)
           tma_load_2d(&S.raw[post.s][r][0], &P.map_row, x0, wrap_near(y, P.ny), &S.full[post.s]);
       } else {
         bool in = r < kRows;
@@ -591,10 +594,10 @@ bool encode_2d(CUtensorMap* map, const double* base, const Geom& g, int rows) {
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <bool BOX, int RAD, bool HEAT, bool PERIODIC, bool TMA>
+template <bool BOX, int RAD, bool HEAT, bool PERIODIC, bool TMA, bool STARVED = false>
 cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst,
-                     int* status, int sms, cudaStream_t stream, bool chained) {
-  auto kern = k_wide2d<BOX, RAD, HEAT, PERIODIC, TMA>;
+                     int* status, int sms, cudaStream_t stream, bool chained, unsigned long long wait_ns = 0) {
+  auto kern = k_wide2d<BOX, RAD, HEAT, PERIODIC, TMA, STARVED>;
   constexpr size_t bytes = sizeof(Smem<RAD, TMA>);
   static std::atomic<int> cache[kMaxDeviceOrdinals];
   const int occ = cached_per_device(cache, [kern] {
@@ -618,6 +621,7 @@ cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, co
   P.work = (int)work;
   P.vec = g.nx % 2 == 0 && ((uintptr_t)dst & 15) == 0;
   P.status = status;
+  P.wait_ns = wait_ns;
   P.wdev = wdev;
   P.wide = wide;
   int64_t grid = (int64_t)sms * occ;
@@ -654,6 +658,11 @@ cudaError_t launch_wide2d(Shape shape, int radius, int boundary, const Geom& g, 
   if (box) return launch_p<true, 1, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained);
   return wide.heat ? launch_p<false, 1, true>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained)
                    : launch_p<false, 1, false>(per, tma, g, wide, wdev, src, dst, status, sms, stream, chained);
+}
+
+cudaError_t launch_wide2d_starved(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst,
+                                  int* status, int sms, cudaStream_t stream, unsigned long long wait_ns) {
+  return launch_t<false, 1, true, true, true, true>(g, wide, wdev, src, dst, status, sms, stream, false, wait_ns);
 }
 
 }  // namespace gbst

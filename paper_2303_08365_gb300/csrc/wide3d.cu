@@ -80,6 +80,7 @@ struct Params {
   long long work;  // tiles * nz
   int vec;         // rows start on 16 bytes
   int* status;
+  unsigned long long wait_ns;  // of STARVED
   const double* wdev;
   WideTaps wide;
 };
@@ -201,14 +202,16 @@ __device__ __noinline__ void own_cells(const Plane<TC>& um, const Plane<TC>& u0,
 // Three CTAs of nine warps per SM where 72 registers are enough (199 x 251 x 301 by bulk
 // copies, us a step, three against two: heat 124 / 137; general weights, which spill,
 // 167 / 148).
-template <bool BOX, bool HEAT, bool PERIODIC, bool TMA, int TC>
+// STARVED: the self-test of the bounded waits: no copy (and no arrival that announces one) for a
+// CTA's second plane, and waits of P.wait_ns.
+template <bool BOX, bool HEAT, bool PERIODIC, bool TMA, int TC, bool STARVED = false>
 __global__ void __launch_bounds__(threads<TC>(), TC == 32 ? 1 : BOX || !(TMA || HEAT) ? 2 : 3)
     k_wide3d(const __grid_constant__ Params P) {
   constexpr int kWarps = warps<TC>(), R = TC / kWarps;  // R: rows of a consumer warp
   static_assert(TMA || TC < 32, "by bulk copies, a lane copies a row");
   constexpr int kU = ring<BOX>();
   constexpr int kLag = BOX ? 2 : 1;  // the middle plane is kLag planes behind the one being unpacked
-  constexpr unsigned long long kWaitNs = (unsigned long long)kSpinLimitNs;
+  const unsigned long long kWaitNs = STARVED ? P.wait_ns : (unsigned long long)kSpinLimitNs;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   Smem<BOX, TMA, TC>& S = *reinterpret_cast<Smem<BOX, TMA, TC>*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -272,7 +275,7 @@ __global__ void __launch_bounds__(threads<TC>(), TC == 32 ? 1 : BOX || !(TMA || 
         if (!wait(&S.empty[post.s], post.ph ^ 1)) return false;
         const int z = wrap1(za - 1 + j, P.nz, PERIODIC);
         if (TMA) {
-          if (lane == 0) {
+          if (lane == 0 && !(STARVED && j == 1)) {
             fence_proxy_async_smem();
             mbar_arrive_expect_tx(&S.full[post.s], (uint32_t)sizeof(S.raw[0]));
             tma_load_3d(&S.raw[post.s][0][0], &P.map_row, x0, wrap1(y0 - 1, P.ny, PERIODIC), z, &S.full[post.s]);
@@ -586,10 +589,10 @@ bool encode_3d(CUtensorMap* map, const double* base, const Geom& g, int box_y) {
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <bool BOX, bool HEAT, bool PERIODIC, bool TMA, int TC>
+template <bool BOX, bool HEAT, bool PERIODIC, bool TMA, int TC, bool STARVED = false>
 cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst,
-                     int* status, int sms, cudaStream_t stream, bool chained) {
-  auto kern = k_wide3d<BOX, HEAT, PERIODIC, TMA, TC>;
+                     int* status, int sms, cudaStream_t stream, bool chained, unsigned long long wait_ns = 0) {
+  auto kern = k_wide3d<BOX, HEAT, PERIODIC, TMA, TC, STARVED>;
   constexpr size_t bytes = sizeof(Smem<BOX, TMA, TC>);
   static std::atomic<int> cache[kMaxDeviceOrdinals];
   const int occ = cached_per_device(cache, [kern] {
@@ -612,6 +615,7 @@ cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, co
   P.work = (long long)P.tiles_x * P.tiles_y * g.nz;
   P.vec = g.nx % 2 == 0 && ((uintptr_t)dst & 15) == 0;
   P.status = status;
+  P.wait_ns = wait_ns;
   P.wdev = wdev;
   P.wide = wide;
   long long grid = (long long)sms * occ;
@@ -653,6 +657,11 @@ cudaError_t launch_wide3d(Shape shape, int boundary, const Geom& g, const WideTa
                : launch_p<false, true, false>(g, wide, wdev, src, dst, status, sms, stream, tma, tile_y, chained);
   return per ? launch_p<false, false, true>(g, wide, wdev, src, dst, status, sms, stream, tma, tile_y, chained)
              : launch_p<false, false, false>(g, wide, wdev, src, dst, status, sms, stream, tma, tile_y, chained);
+}
+
+cudaError_t launch_wide3d_starved(const Geom& g, const WideTaps& wide, const double* wdev, const double* src, double* dst,
+                                  int* status, int sms, cudaStream_t stream, unsigned long long wait_ns) {
+  return launch_t<false, true, true, true, 16, true>(g, wide, wdev, src, dst, status, sms, stream, false, wait_ns);
 }
 
 }  // namespace gbst

@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_wide_steps(const __grid_constan
         if (!wait(&S.done, done_ph)) return false;
         done_ph ^= 1;
       }
-      if (lane == 0) {
+      if (lane == 0 && (int)blockIdx.x != L.mute) {
         asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(L.progress + blockIdx.x * kProgressStride), "r"(steps)
                      : "memory");
       }

@@ -593,3 +593,22 @@ def test_autotune_keeps_a_default_that_no_variant_names(st):
             p.run(g, 20)
             assert st.stencil_launch_count() - before == 1
             assert p.status() == 0
+
+
+# (kernel of the self-test, a grid that it takes, its variant)
+STARVED = [(0, (8, 32, 128), 2), (1, (64, 128), 2), (2, (512, 640), 4), (3, (8, 32, 128), 0)]
+
+
+@pytest.mark.parametrize("kernel,shape,variant", STARVED)
+def test_waits_that_run_out_report_it_and_the_context_survives(st, kernel, shape, variant):
+    """Every bounded wait of the kernels for positive weights: copies that never come, steps that a
+    neighbour never publishes.  They end by their limit of 20 ms, and the next sweep is right."""
+    import time
+    t0 = time.perf_counter()
+    assert st.stencil_selftest_wide_timeout(kernel, 20.0) == st.ERR_TIMEOUT
+    assert time.perf_counter() - t0 < 5.0
+    w, u0 = synth.heat_weights(len(shape), 0.1), synth.normal(71, shape)
+    got = run(st, u0, w, 1, PERIODIC, 5, (1, variant) if variant else (0, 0))
+    assert np.array_equal(got, run(st, u0, w, 1, PERIODIC, 5, (1, st.VARIANT_DIRECT), 1))
+    with pytest.raises(st.StencilError):
+        st._check(st.lib().stencil_selftest_wide_timeout(4, 20.0, None))
