@@ -275,8 +275,8 @@ typedef enum {
                                      intermediate time levels handed between
                                      tiles through an L2-resident ring of
                                      (Tb-1) x K grid planes (plan-owned; K =
-                                     5 for a star, 6 for a box, 9 / 10 at
-                                     Tb = 2).
+                                     9, 7 and 5 for a star at Tb = 2, 4 and 8,
+                                     10, 8 and 6 for a box).
                                      Needs nx even (a multiple of 64 on a
                                      periodic grid) and at most one 64-column
                                      tile column per SM.  A plane taller

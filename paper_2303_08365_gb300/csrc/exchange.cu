@@ -22,7 +22,7 @@
 //     an L2-resident ring of K planes per stage (the whole plane of the band
 //     of rows the launch covers, so neighbouring tiles can read their halo
 //     from it), stage Tb writes the
-//     output grid.  The stage skew of L >= 2 planes (2; 4 at Tb = 2) means a
+//     output grid.  The stage skew of L planes (4, 3 and 2 at Tb = 2, 4 and 8) means a
 //     stage only reads planes written in earlier iterations: unit (i, s)
 //     needs unit (i-L+1, s-1);
 //   - a consumer thread fences its stores into the async proxy and bumps its
@@ -71,11 +71,11 @@
 //     s >= 2, is posted once every neighbour has finished (i-L+1, s-1), so all
 //     of iteration i-L; unit (i, 1) after the wait of the last such unit of
 //     iteration i-1, so all of iteration i-L-1: K = 2L+1 planes (star) or
-//     2L+2 (box) keep every read ahead of the rewrite (5 / 6 at L = 2, 9 / 10
-//     at L = 4).
-// Each cell applies its taps in the direct kernel's lexicographic order with
-// register-resident weights, so a Tb-fused sweep is bitwise equal to Tb
-// single steps.  Every wait is bounded (2 s of wall time): a CTA that gives up
+//     2L+2 (box) keep every read ahead of the rewrite (5 / 6 at L = 2, 7 / 8
+//     at L = 3, 9 / 10 at L = 4).
+// Each cell takes the direct kernel's sum (the integer form, or the FMA chain in
+// lexicographic order with register-resident weights), so a Tb-fused sweep is
+// bitwise equal to Tb single steps.  Every wait is bounded (2 s of wall time): a CTA that gives up
 // writes STENCIL_ERR_TIMEOUT to the status word, lets its posted copies land
 // and returns; the others see the status word and return too.
 #include <cudaTypedefs.h>

@@ -67,10 +67,10 @@ struct WideTapsOf {
   int hi2[N];                              // 2 * hi
   int ex[N];                               // exponent below the largest weight's (<= 0)
   int heat;                                // one weight at the centre tap (n / 2), one at all others
-  int equal;                               // a box whose weights are all equal
   int bias;                                // exponent of the result: E - bias above R's
   int e_min;                               // E in [e_min, e_min + e_span], else the FMA chain
   unsigned int e_span;
+  int equal;                               // a box whose weights are all equal
 };
 using WideTaps = WideTapsOf<kWideMaxTaps>;
 
@@ -177,7 +177,7 @@ cudaError_t launch_temporal(int ndim, int radius, Shape shape, int boundary, int
 // Temporal blocking without recomputation (3D radius 1, star or box, Tb >= 2):
 // one co-resident CTA per 64-column tile of a band of rows of the (y, x)
 // plane, intermediate time levels handed between tiles through a ring of
-// Tb-1 x K band planes (K = 5 / 6 for the star / box; 9 / 10 at Tb = 2).  A
+// Tb-1 x K band planes (K = 9 / 10, 7 / 8 and 5 / 6 for the star / box at Tb = 2, 4 and 8).  A
 // plane taller than the co-resident tiles cover (32 rows each) is cut into
 // bands, one launch each, every band with a margin of Tb-1 rows toward each
 // neighbouring band: the rows its last stage may get wrong at an edge whose

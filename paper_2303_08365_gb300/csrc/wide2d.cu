@@ -67,9 +67,10 @@ struct Params {
   int work;  // tiles
   int vec;   // rows start on 16 bytes
   int* status;
-  unsigned long long wait_ns;  // of STARVED
   const double* wdev;
   WideTaps wide;
+  WideEqualTaps equal;         // of a box with wide.equal
+  unsigned long long wait_ns;  // of STARVED
 };
 
 // First column and row of a tile, advanced tile by tile (a division per warp and tile
@@ -480,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
         // Where cells differ in E (a field passes a power of 16), no bit is cut as long as all
         // values are within the 2^9 that the integers have room for: the sums are exact then,
         // and those of each cell's own alignment follow.  Else the warp takes own_cells.
-        all = wide_covers(E, P.wide) && (E == least || (wide_covers(least, P.wide) && least_exponent<RAD>(u, row0, c) + 9 >= E));
+        all = wide_covers(E, P.equal) && (E == least || (wide_covers(least, P.equal) && least_exponent<RAD>(u, row0, c) + 9 >= E));
         const bool fits = __all_sync(0xffffffffu, all || rows <= 0);
         all = rows <= 0 || fits;
         if (fits) {
@@ -524,7 +525,7 @@ __global__ void __launch_bounds__(kThreads, (wide2d_ctas<BOX, RAD, HEAT>())) k_w
             }
 #pragma unroll
           for (int r = 0; r < 2; ++r)
-            store(r, wide_equal_double(S[r][0], Ec[r][0], P.wide), wide_equal_double(S[r][1], Ec[r][1], P.wide));
+            store(r, wide_equal_double(S[r][0], Ec[r][0], P.equal), wide_equal_double(S[r][1], Ec[r][1], P.equal));
         }
       } else {
         // row by row; the largest exponents first, then the sums: a pair's values would
@@ -624,6 +625,7 @@ cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, co
   P.wait_ns = wait_ns;
   P.wdev = wdev;
   P.wide = wide;
+  P.equal = wide;
   int64_t grid = (int64_t)sms * occ;
   if (grid > work) grid = work;
   if (const cudaError_t e = launch_step(kern, (unsigned)grid, kThreads, bytes, stream, chained, P)) return e;

@@ -80,9 +80,10 @@ struct Params {
   long long work;  // tiles * nz
   int vec;         // rows start on 16 bytes
   int* status;
-  unsigned long long wait_ns;  // of STARVED
   const double* wdev;
   WideTaps wide;
+  WideEqualTaps equal;         // of a box with wide.equal
+  unsigned long long wait_ns;  // of STARVED
 };
 
 // Columns c-1 .. c+2 of a row.
@@ -471,7 +472,7 @@ __global__ void __launch_bounds__(threads<TC>(), TC == 32 ? 1 : BOX || !(TMA || 
           // Where cells differ in E (a field passes a power of 16), no bit is cut as long as all
           // values are within the 2^9 that the integers have room for: the sums are exact then,
           // and those of each cell's own alignment follow.  Else the warp takes own_cells.
-          all = wide_covers(E, P.wide);
+          all = wide_covers(E, P.equal);
           if (all && E != least) {
             int low = 0x7fffffff;
 #pragma unroll 1
@@ -482,7 +483,7 @@ __global__ void __launch_bounds__(threads<TC>(), TC == 32 ? 1 : BOX || !(TMA || 
 #pragma unroll
                 for (int x = -1; x < 3; ++x) low = min(low, u.e[row0 - 1 + q][c + x]);
             }
-            all = wide_covers(least, P.wide) && low + 9 >= E;
+            all = wide_covers(least, P.equal) && low + 9 >= E;
           }
           const bool fits = __all_sync(0xffffffffu, all || rows <= 0);
           all = rows <= 0 || fits;
@@ -525,7 +526,7 @@ __global__ void __launch_bounds__(threads<TC>(), TC == 32 ? 1 : BOX || !(TMA || 
               }
 #pragma unroll
             for (int r = 0; r < R; ++r)
-              store(r, wide_equal_double(sum[r][0], Ec[r][0], P.wide), wide_equal_double(sum[r][1], Ec[r][1], P.wide));
+              store(r, wide_equal_double(sum[r][0], Ec[r][0], P.equal), wide_equal_double(sum[r][1], Ec[r][1], P.equal));
           }
         } else {
           // row by row; the largest exponents first, then the sums: the 36 values of
@@ -618,6 +619,7 @@ cudaError_t launch_t(const Geom& g, const WideTaps& wide, const double* wdev, co
   P.wait_ns = wait_ns;
   P.wdev = wdev;
   P.wide = wide;
+  P.equal = wide;
   long long grid = (long long)sms * occ;
   if (grid > P.work) grid = P.work;
   if (const cudaError_t e = launch_step(kern, (unsigned)grid, threads<TC>(), bytes, stream, chained, P)) return e;
