@@ -297,8 +297,8 @@ __device__ __forceinline__ double wide_sum_heat(const WideVal (&u)[NT], const Ta
 
 // The sum of aligned values (two's complement) of a box whose weights are all equal: up to 27
 // of 63 bits, so the sum modulo 2^64, and the sum of the values' top bits (units of 2^37), which
-// has the rest.  (Values cut to 58 bits, whose sum fits 64, lean to one side: by 2^-54 a step
-// where they are spread over a few powers of two.)
+// has the rest.  (Values cut to 58 bits, whose sum fits 64, lean to one side: spread from e^-4 to
+// e^4, by 0.10 of 2^-53 a step of a 27-point box; so, 0.02.)
 struct WideSum {
   long long s;
   int top;
